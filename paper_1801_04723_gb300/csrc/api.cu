@@ -788,19 +788,19 @@ __global__ void synth_sdd_kernel(double* A, int64_t n, uint64_t seed) {
 //   t = launch + max(ceil(tiles / 152) * 2 * TM * TM * k / P_sm, 2 m n k / P_gpu)
 // with the product kernel's TM x TM tiles (64, 32 or 16) and P_sm = 4 flops/clock at 2.07 GHz (P_gpu = 152 P_sm,
 // 1.259 TFLOP/s, the measured DFMA rate); per leaf of order L on C = min(16,
-// 2^ceil(log2 L)) CTAs with R = ceil(L / C) rows each, L pivot steps of
-//   a + b L + R L / (2 FMA/clock)     (rows in shared memory)
+// 2^ceil(log2 L)) CTAs, L pivot steps of
+//   a + b T                           (L <= 256: columns over the cluster, T
+//                                      = 1, 2, 4, 8 rows per lane)
+//   a + b L + R L / (2 FMA/clock)     (R = ceil(L / C) rows per CTA in shared memory)
 //   a + b L + R L g                   (rows in L2-resident global memory)
-// with a = 1.55 us, b = 5 ns for L <= 256 (candidate rows pushed to every
-// CTA) and a = 1.8 us, b = 14 ns above (pivot row read from its owner), and
-// g = 0.55 ns per element: per-step times of one leaf on its 16-CTA cluster
-// (bench.py --leaf-times, L = 32 ... 2048).  It reproduces the measured sweeps at n = 1024,
-// 4096 and 8192 (leaf 64 ... 2048) within 8 %.
+// with a = 0.36 us, b = 0.125 us for the first (per-step times of one leaf:
+// 0.58 / 0.61 / 0.82 / 1.39 us at L = 32 / 64 / 128 / 256), a = 3.46 us, b =
+// 6.4 ns for the others and g = 0.44 ns per element (bench.py --leaf-times).
 constexpr double kModelClock = 2.07e9;
 constexpr double kModelPsm = 4.0 * kModelClock;
 constexpr double kModelPgpu = 152.0 * kModelPsm;
 constexpr double kModelLaunch = 4e-6;
-constexpr double kModelAPush = 1.85e-6, kModelBPush = 0.0, kModelAPull = 3.46e-6, kModelBPull = 6.4e-9;
+constexpr double kModelACol = 0.36e-6, kModelBCol = 0.125e-6, kModelAPull = 3.46e-6, kModelBPull = 6.4e-9;
 constexpr double kModelG = 0.44e-9;
 
 double model_gemm(int64_t m, int64_t n, int64_t k) {
@@ -815,7 +815,7 @@ double model_leaf(int64_t L) {
     while (C < 16 && C < L) C <<= 1;
     const int64_t R = (L + C - 1) / C;
     const double fma_time = (double)R * L / (2.0 * kModelClock);
-    if (L <= 256) return (double)L * (kModelAPush + kModelBPush * (double)L + fma_time);
+    if (L <= 256) return (double)L * (kModelACol + kModelBCol * (L <= 32 ? 1.0 : L <= 64 ? 2.0 : L <= 128 ? 4.0 : 8.0));
     const bool smem = (double)R * L * 8 + 16.0 * R + 64.0 * C + 16.0 * L <= 200.0 * 1024;
     return (double)L * (kModelAPull + kModelBPull * (double)L + (smem ? fma_time : (double)R * L * kModelG));
 }

@@ -10,31 +10,30 @@
 // in reverse order.
 //
 // GB300 mapping.  FP64 runs at ~2 FMA/clock/SM, so one L x L leaf on one SM
-// takes ~L^3 cycles; the leaf is spread over a thread-block cluster of C
-// CTAs (C <= 16) whose rows stay put: every CTA owns R = ceil(L/C) rows in
-// shared memory when they fit (global memory, L2-resident, otherwise).  Row
-// interchanges are bookkeeping only (position <-> physical row tables
-// replicated in every CTA).  A pivot step is latency-bound at these sizes:
-// each SM sub-partition's FP64 unit takes one warp instruction per 64
-// cycles, a dependent FP64 operation waits behind every one queued before
-// it (~250 cycles in a step), so a step keeps remote reads, fences and FP64
-// work off its critical path:
-//  - the pivot search compares the bit patterns of |a_ik| as integers
-//    (redux.sync argmax), and each candidate's reciprocal is computed once,
-//    by the CTA that publishes it;
-//  - every CTA publishes its candidate for the next column into every other
-//    CTA's shared memory, double-buffered by step parity (a CTA writes step
-//    k+1's slot while a slower one may still read step k's; the slot it
-//    overwrites was last read in step k-1);
-//  - the multipliers of step k+1 (column k+1 after step k) go to a second
-//    buffer, written by the threads that compute them;
-//  - the pivot row of step k is left raw; its scaling by 1/pivot is folded
-//    into step k+1's update of that row.
-// Two forms (leaf_gj_push_body, leaf_gj_pull_body below): for L <= 256 the
-// candidate rows travel with the candidates (st.async and bulk copies that
-// complete on per-slot mbarriers, with the bulk of each step overlapping the
-// exchange); above, the pivot row is read from its owner and a step ends at
-// a cluster barrier.
+// takes ~L^3 cycles; a single inversion's leaf is spread over a thread-block
+// cluster of C CTAs (C <= 16).  A pivot step is latency-bound at these
+// sizes: each SM sub-partition's FP64 unit takes one warp instruction per 64
+// cycles and a dependent FP64 operation waits behind every one queued before
+// it, so every form keeps the pivot search on integers (redux.sync argmax of
+// the bit patterns of |a_ik|) and takes 1/pivot once per step.  Row
+// interchanges are bookkeeping only.
+//  - leaf_gj_col_kernel (leaf_col.cuh), single inversions with L <= 256:
+//    columns over the cluster, one warp each.
+//  - leaf_gj_pull_body, L > 256: every CTA owns R = ceil(L/C) rows in shared
+//    memory when they fit (global memory, L2-resident, otherwise); the pivot
+//    row is read from its owner and a step ends at a cluster barrier.
+//  - leaf_gj_cta_body (leaf_core.cuh), the batched paths with L <= 128: one
+//    CTA per leaf.
+//  - leaf_gj_push_body, the batched paths with 128 < L <= 256: rows over the
+//    narrowest cluster that holds them, candidate rows pushed to every CTA
+//    (st.async and bulk copies that complete on per-slot mbarriers).
+// The pull and push forms publish every CTA's candidate for the next column
+// into every other CTA's shared memory, double-buffered by step parity (a
+// CTA writes step k+1's slot while a slower one may still read step k's; the
+// slot it overwrites was last read in step k-1); the multipliers of step k+1
+// (column k+1 after step k) go to a second buffer, written by the threads
+// that compute them; the pivot row of step k is left raw and its scaling by
+// 1/pivot folded into step k+1's update of that row.
 #include <cooperative_groups.h>
 #include <limits.h>
 
@@ -42,6 +41,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "leaf_col.cuh"
 #include "leaf_core.cuh"
 #include "tc_ptx.cuh"
 
@@ -100,28 +100,6 @@ __device__ __forceinline__ Cand warp_candidate(const double* M, int L, int nrows
     }
     return warp_argmax(key, val, 0.0, pos, phys);
 }
-
-// Bounded wait for a slot barrier (a step takes microseconds; the limit
-// only turns a broken exchange into an error instead of a hang).
-constexpr uint64_t kLeafWaitLimitNs = 4000000000ull;
-
-// Exchange settings of the pushed-row form: the wait limit, and (tests
-// only) a CTA that sends nothing, so that the others' waits run out.
-struct LeafWait {
-    uint64_t limit_ns = kLeafWaitLimitNs;
-    int mute_rank = -1;
-};
-
-__device__ __forceinline__ bool slot_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
-    if (tc::mbar_try_wait_cluster(bar, parity)) return true;
-    const uint64_t t0 = tc::globaltimer_ns();
-    for (uint32_t spins = 1;; spins++) {
-        if (tc::mbar_try_wait_cluster(bar, parity)) return true;
-        if ((spins & 63u) == 0 && tc::globaltimer_ns() - t0 > limit_ns) return false;
-    }
-}
-
-
 
 // Winner of step k among the C published candidates (every warp computes it).
 __device__ __forceinline__ Cand cluster_winner(const Cand* slot, int C) {
@@ -309,7 +287,7 @@ __device__ __forceinline__ void leaf_gj_pull_body(const double* __restrict__ src
 // row, so that every step delivers the same byte count.
 __device__ __forceinline__ void leaf_gj_push_body(const double* __restrict__ src, int64_t lds,
                                                   double* __restrict__ dst, int64_t ldd, int L, int R, int32_t* info,
-                                                  int leaf_index, LeafWait lw) {
+                                                  int leaf_index) {
     const int C = (int)tc::cluster_nctarank();
     const int rank = (int)tc::cluster_ctarank();
     const int tid = threadIdx.x;
@@ -343,9 +321,8 @@ __device__ __forceinline__ void leaf_gj_push_body(const double* __restrict__ src
     // fenced for the copy engine by the compute threads before a barrier the
     // messenger has passed) to the other CTAs' slot s: one bulk copy per
     // peer, by the messenger lanes.
-    const bool muted = rank == lw.mute_rank;
     auto send_row = [&](int s) {
-        if (mt >= 0 && mt < C && mt != rank && !muted) {
+        if (mt >= 0 && mt < C && mt != rank) {
             const uint32_t src_row = tc::smem_u32(slots + ((size_t)s * C + rank) * LS);
             tc::bulk_copy_to_peer(tc::mapa_u32(src_row, (uint32_t)mt), src_row, row_bytes,
                                   tc::mapa_u32(tc::smem_u32(&bars[s]), (uint32_t)mt));
@@ -362,7 +339,7 @@ __device__ __forceinline__ void leaf_gj_push_body(const double* __restrict__ src
                 mine.inv = inv;
                 mine.pos = c.pos;
                 mine.phys = c.phys;
-            } else if (!muted) {
+            } else {
                 const uint32_t a = tc::mapa_u32(tc::smem_u32(&infos[s * C + rank]), (uint32_t)mt);
                 const uint32_t b = tc::mapa_u32(tc::smem_u32(&bars[s]), (uint32_t)mt);
                 tc::st_async_v2_b64(a, c.key, (uint64_t)__double_as_longlong(c.val), b);
@@ -411,7 +388,7 @@ __device__ __forceinline__ void leaf_gj_push_body(const double* __restrict__ src
     double prev_inv = 0.0;
     for (int k = 0; k < L; k++) {
         const int s = k & 1;
-        const bool ok = slot_wait(&bars[s], (uint32_t)(k >> 1) & 1u, lw.limit_ns);
+        const bool ok = slot_wait(&bars[s], (uint32_t)(k >> 1) & 1u, kLeafWaitLimitNs);
         if (__syncthreads_or(!ok)) {  // also makes this CTA's own slot entries visible
             if (tid == 0) record_failure(info, SPIN_ERR_TIMEOUT, leaf_index, k);
             break;
@@ -531,18 +508,18 @@ leaf_gj_cta_kernel(BatchView srcv, BatchView dstv, int L, int32_t* info_base, in
 template <bool ROWS_IN_SMEM, bool PUSH>
 __device__ __forceinline__ void leaf_gj_body(const double* __restrict__ src, int64_t lds, double* __restrict__ dst,
                                              int64_t ldd, double* __restrict__ gwork, int L, int R, int32_t* info,
-                                             int leaf_index, LeafWait lw) {
+                                             int leaf_index) {
     if constexpr (PUSH)
-        leaf_gj_push_body(src, lds, dst, ldd, L, R, info, leaf_index, lw);
+        leaf_gj_push_body(src, lds, dst, ldd, L, R, info, leaf_index);
     else
         leaf_gj_pull_body<ROWS_IN_SMEM>(src, lds, dst, ldd, gwork, L, R, info, leaf_index);
 }
 
-template <bool ROWS_IN_SMEM, bool PUSH>
-__global__ void __launch_bounds__(PUSH ? NT + kMessengers : NT, 1)
+template <bool ROWS_IN_SMEM>
+__global__ void __launch_bounds__(NT, 1)
 leaf_gj_kernel(const double* __restrict__ src, int64_t lds, double* __restrict__ dst, int64_t ldd,
-               double* __restrict__ gwork, int L, int R, int32_t* info, int leaf_index, LeafWait lw) {
-    leaf_gj_body<ROWS_IN_SMEM, PUSH>(src, lds, dst, ldd, gwork, L, R, info, leaf_index, lw);
+               double* __restrict__ gwork, int L, int R, int32_t* info, int leaf_index) {
+    leaf_gj_pull_body<ROWS_IN_SMEM>(src, lds, dst, ldd, gwork, L, R, info, leaf_index);
 }
 
 // Batched form: cluster blockIdx.y inverts problem z = blockIdx.y.  Many
@@ -551,12 +528,12 @@ leaf_gj_kernel(const double* __restrict__ src, int64_t lds, double* __restrict__
 template <bool ROWS_IN_SMEM, bool PUSH>
 __global__ void __launch_bounds__(PUSH ? NT + kMessengers : NT, 2)
 leaf_gj_batched_kernel(BatchView src, BatchView dst, double* __restrict__ gwork, int64_t gwork_stride, int L, int R,
-                       int32_t* info, int leaf_index, LeafWait lw) {
+                       int32_t* info, int leaf_index) {
     const int z = blockIdx.y;
     const int64_t lds = src.ld_of(z), ldd = dst.ld_of(z);
     leaf_gj_body<ROWS_IN_SMEM, PUSH>(src.ptr(z, lds), lds, const_cast<double*>(dst.ptr(z, ldd)), ldd,
                                      ROWS_IN_SMEM ? nullptr : gwork + (int64_t)z * gwork_stride, L, R,
-                                     info + (int64_t)z * INFO_WORDS, leaf_index, lw);
+                                     info + (int64_t)z * INFO_WORDS, leaf_index);
 }
 
 struct LeafConfig {
@@ -573,7 +550,7 @@ int max_cluster_size() {
     static int cached = 0;
     if (cached) return cached;
     cached = 8;
-    auto kern = leaf_gj_kernel<true, false>;
+    auto kern = leaf_gj_kernel<true>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         cudaGetLastError();
@@ -600,13 +577,10 @@ size_t leaf_smem_bytes(int64_t L, int C, bool rows, bool push) {
     return leaf_layout((int)L, (int)((L + C - 1) / C), C, rows, push).total;
 }
 
-// Cluster shape.  A pivot step costs a barrier's latency plus R*L FMAs on
-// each CTA at ~2 FP64 FMA/clock: measured per-step times at L = 128 are
-// 12.2 / 7.4 / 4.5 / 3.2 / 2.9 us on 1 / 2 / 4 / 8 / 16 CTAs, and 2.0 us at
-// L = 32 on 16.  A single inversion waits on its leaves,
-// so it takes the widest cluster (latency); a batch runs many leaves side
-// by side, so it takes the narrowest that fits shared memory (SM time).
-// Rows are pushed to every CTA when L <= 256 and the slots fit.
+// Cluster shape.  A single inversion waits on its leaves, so it takes the
+// widest cluster (latency); a batch runs many leaves side by side, so it
+// takes the narrowest that fits shared memory (SM time).  Batched rows are
+// pushed to every CTA when L <= 256 and the slots fit.
 // SPIN_LEAF_CLUSTER_MAX caps the single inversions' cluster width (1..16,
 // for measurement: a narrower cluster takes longer per leaf but holds fewer
 // SMs while other work could use them); read once.
@@ -622,7 +596,7 @@ int leaf_cluster_cap() {
 LeafConfig leaf_config(int64_t L, bool have_scratch, bool batched = false) {
     LeafConfig c;
     const int cmax = batched ? max_cluster_size() : std::min(max_cluster_size(), leaf_cluster_cap());
-    const bool push_ok = L <= kPushMaxL;
+    const bool push_ok = batched && L <= kPushMaxL;
     c.C = 1;
     if (batched) {
         while (c.C < cmax && leaf_smem_bytes(L, c.C, true, push_ok) > kSmemBudget) c.C <<= 1;
@@ -654,29 +628,73 @@ int prepare_leaf_kernel(K kern) {
     return SPIN_OK;
 }
 
-template <bool S, bool P>
-int launch_leaf_impl(const double* A, int64_t lda, double* X, int64_t ldx, const LeafConfig& c, int64_t L,
-                     double* scratch, int32_t* info, int leaf_index, cudaStream_t s, LeafWait lw = LeafWait()) {
-    static PerDeviceOnce attrs;
-    auto kern = leaf_gj_kernel<S, P>;
-    {
-        const int rc = attrs.run([&] { return prepare_leaf_kernel(kern); });
-        if (rc != SPIN_OK) return rc;
-    }
+// Launch kern on one cluster of C CTAs.
+template <typename K, typename... Args>
+int launch_cluster(K kern, int C, int threads, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)c.C, 1, 1);
-    cfg.blockDim = dim3(P ? NT + kMessengers : NT, 1, 1);
-    cfg.dynamicSmemBytes = c.smem;
+    cfg.gridDim = dim3((unsigned)C, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)c.C;
+    attr[0].val.clusterDim.x = (unsigned)C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    SPIN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, A, lda, X, ldx, scratch, (int)L, c.R, info, leaf_index, lw));
+    SPIN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
     return SPIN_OK;
+}
+
+template <bool S>
+int launch_leaf_pull(const double* A, int64_t lda, double* X, int64_t ldx, const LeafConfig& c, int64_t L,
+                     double* scratch, int32_t* info, int leaf_index, cudaStream_t s) {
+    static PerDeviceOnce attrs;
+    auto kern = leaf_gj_kernel<S>;
+    const int rc = attrs.run([&] { return prepare_leaf_kernel(kern); });
+    if (rc != SPIN_OK) return rc;
+    return launch_cluster(kern, c.C, NT, c.smem, s, A, lda, X, ldx, scratch, (int)L, c.R, info, leaf_index);
+}
+
+// The column form's cluster for order L: w columns per CTA, and the CTAs (a
+// power of two; those past the last column only take part in the barriers).
+// false when the block does not fit the cluster (L > 256, or fewer CTAs
+// than 16 available for L > 128): the pull form runs then.
+struct ColConfig {
+    int T, w, C;
+};
+bool col_config(int64_t L, ColConfig* c) {
+    if (L < 1 || L > kColMaxL) return false;
+    const int cmax = std::min({max_cluster_size(), leaf_cluster_cap(), kColMaxCtas});
+    c->T = col_rows((int)L);
+    c->w = col_panel((int)L, cmax);
+    if (c->w > std::max(2 * c->T, kColMinPanel)) return false;
+    const int nact = (int)((L + c->w - 1) / c->w);
+    c->C = 1;
+    while (c->C < nact) c->C <<= 1;
+    return c->C <= cmax;
+}
+
+template <int T>
+int launch_leaf_col_t(const double* A, int64_t lda, double* X, int64_t ldx, const ColConfig& c, int64_t L,
+                      int32_t* info, int leaf_index, cudaStream_t s, LeafWait lw) {
+    static PerDeviceOnce attrs;
+    auto kern = leaf_gj_col_kernel<T>;
+    const int rc = attrs.run([&] { return prepare_leaf_kernel(kern); });
+    if (rc != SPIN_OK) return rc;
+    return launch_cluster(kern, c.C, 32 * (c.w + 1), col_layout((int)L, c.w).total, s, A, lda, X, ldx, (int)L, c.w, info,
+                          leaf_index, lw);
+}
+
+int launch_leaf_col(const double* A, int64_t lda, double* X, int64_t ldx, const ColConfig& c, int64_t L,
+                    int32_t* info, int leaf_index, cudaStream_t s, LeafWait lw = LeafWait()) {
+    switch (c.T) {
+        case 1: return launch_leaf_col_t<1>(A, lda, X, ldx, c, L, info, leaf_index, s, lw);
+        case 2: return launch_leaf_col_t<2>(A, lda, X, ldx, c, L, info, leaf_index, s, lw);
+        case 4: return launch_leaf_col_t<4>(A, lda, X, ldx, c, L, info, leaf_index, s, lw);
+        default: return launch_leaf_col_t<8>(A, lda, X, ldx, c, L, info, leaf_index, s, lw);
+    }
 }
 
 template <bool S, bool P>
@@ -701,8 +719,7 @@ int launch_leaf_batched_impl(const BatchView& src, const BatchView& dst, const L
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    SPIN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, src, dst, scratch, stride, (int)L, c.R, info, leaf_index,
-                                     LeafWait()));
+    SPIN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, src, dst, scratch, stride, (int)L, c.R, info, leaf_index));
     return SPIN_OK;
 }
 
@@ -742,11 +759,12 @@ int launch_leaf_gj(const double* A, int64_t lda, double* X, int64_t ldx, int64_t
                    int32_t* info, int leaf_index, cudaStream_t s) {
     if (L <= 0) return SPIN_OK;
     if (L > kMaxLeaf) return SPIN_ERR_INVALID_ARG;
+    ColConfig cc;
+    if (col_config(L, &cc)) return launch_leaf_col(A, lda, X, ldx, cc, L, info, leaf_index, s);
     const LeafConfig c = leaf_config(L, scratch != nullptr);
     if (c.smem > kSmemBudget) return SPIN_ERR_INVALID_ARG;
-    if (c.push) return launch_leaf_impl<true, true>(A, lda, X, ldx, c, L, nullptr, info, leaf_index, s);
-    if (c.smem_rows) return launch_leaf_impl<true, false>(A, lda, X, ldx, c, L, nullptr, info, leaf_index, s);
-    return launch_leaf_impl<false, false>(A, lda, X, ldx, c, L, scratch, info, leaf_index, s);
+    if (c.smem_rows) return launch_leaf_pull<true>(A, lda, X, ldx, c, L, nullptr, info, leaf_index, s);
+    return launch_leaf_pull<false>(A, lda, X, ldx, c, L, scratch, info, leaf_index, s);
 }
 
 }  // namespace spin
@@ -759,9 +777,9 @@ int launch_leaf_gj(const double* A, int64_t lda, double* X, int64_t ldx, int64_t
 // exchange, while every CTA still waits.  Returns the recorded status.
 extern "C" int spin_test_leaf_timeout(int64_t L, int mute_rank, double limit_ms) {
     using namespace spin;
-    if (L < 2 || L > kPushMaxL || !(limit_ms > 0.0) || limit_ms > 4000.0) return SPIN_ERR_INVALID_ARG;
-    const LeafConfig c = leaf_config(L, false);
-    if (!c.push || mute_rank < 0 || mute_rank >= c.C) return SPIN_ERR_INVALID_ARG;
+    if (L < 2 || L > kColMaxL || !(limit_ms > 0.0) || limit_ms > 4000.0) return SPIN_ERR_INVALID_ARG;
+    ColConfig c;
+    if (!col_config(L, &c) || mute_rank < 0 || mute_rank * c.w >= L) return SPIN_ERR_INVALID_ARG;
     double* A = nullptr;
     double* X = nullptr;
     int32_t* info = nullptr;
@@ -782,7 +800,7 @@ extern "C" int spin_test_leaf_timeout(int64_t L, int mute_rank, double limit_ms)
     LeafWait lw;
     lw.limit_ns = (uint64_t)(limit_ms * 1e6);
     lw.mute_rank = mute_rank;
-    int rc = launch_leaf_impl<true, true>(A, L, X, L, c, L, nullptr, info, 0, 0, lw);
+    int rc = launch_leaf_col(A, L, X, L, c, L, info, 0, 0, lw);
     int32_t h[INFO_WORDS] = {0, 0, 0, 0};
     if (rc == SPIN_OK) {
         if (cudaMemcpy(h, info, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) rc = SPIN_ERR_CUDA;

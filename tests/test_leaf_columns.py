@@ -1,0 +1,53 @@
+"""The single inversions' leaf with its columns over a cluster (orders up to
+256) at the edges of its layout (rows per lane, columns per CTA, panels in the
+slot ring) and of its pivot search and reciprocal: bit for bit the batched
+paths' leaf, which shares none of that code (rows in one CTA up to 128, rows
+over a cluster above), with the same status."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def spin():
+    import paper_1801_04723_gb300 as s
+
+    s.build()
+    s.lib()
+    return s
+
+
+def matrix(kind, L, rng):
+    if kind == "uniform":
+        return rng.uniform(-1, 1, (L, L))
+    if kind == "ties":  # equal magnitudes everywhere: the lowest position wins
+        return rng.choice([-1.0, 1.0], (L, L)) + np.diag(np.full(L, 2.0))
+    if kind == "low_words":  # rows that differ in the last bits of |a| only
+        return rng.choice([-1.0, 1.0], (L, L)) * (1.0 + rng.integers(0, 4, (L, L)) * 2.0 ** -52) + np.diag(
+            np.full(L, 3.0))
+    if kind == "range":  # pivots near both ends of the exponent range
+        d = 2.0 ** rng.choice([-1015.0, -1000.0, -3.0, 0.0, 7.0, 1000.0, 1022.0], L)
+        return rng.uniform(0.5, 1, (L, L)) * 2.0 ** -1020 + np.diag(d)
+    if kind == "powers":  # reciprocals that are exact, and significands of all ones
+        return np.diag(rng.choice([2.0 ** -60, 1.0, 2.0 - 2.0 ** -52, -(2.0 - 2.0 ** -52) * 2.0 ** 40], L))
+    A = rng.uniform(-1, 1, (L, L))
+    if kind == "zero_column":
+        A[:, L // 2] = 0.0
+    else:
+        A[L // 3, L // 2] = np.nan if kind == "nan" else np.inf
+    return A
+
+
+@pytest.mark.parametrize("kind", ["uniform", "ties", "low_words", "range", "powers", "zero_column", "nan", "inf"])
+@pytest.mark.parametrize("L", [1, 2, 4, 5, 16, 17, 31, 32, 33, 63, 64, 65, 80, 127, 128, 129, 144, 145, 255, 256])
+def test_same_bits_as_the_batched_leaf(spin, L, kind):
+    A = torch.from_numpy(np.ascontiguousarray(matrix(kind, L, np.random.default_rng(1000 * L + len(kind))))).cuda()
+    info = torch.zeros(4, dtype=torch.int32, device="cuda:0")
+    X = spin.leaf_inverse(A, info_dev=info)
+    Y, status = spin.invert_batched([A], leaf=L, schedule="lockstep")
+    torch.cuda.synchronize()
+    assert info[0].item() == status[0].item()
+    if info[0].item() == 0:
+        assert torch.equal(X, Y[0])
