@@ -64,8 +64,8 @@ typedef enum {
     SPIN_MIXED_BF16X3 = 1, /* products on BF16 tensor cores with 3-term splits, FP32 accumulate,
                               then Newton-Schulz refinement to opts.tol                       */
     /* 2 is not a precision (a call passing it gets SPIN_ERR_INVALID_ARG)                     */
-    SPIN_MIXED_DIGITS = 3  /* products on BF16 tensor cores as 4-slice fixed-point digit
-                              products with exact FP32 runs (~2^-30 relative), then the same
+    SPIN_MIXED_DIGITS = 3  /* products on BF16 tensor cores in fixed point as accurate as 4
+                              8-bit digit slices (~2^-30 relative), then the same
                               refinement -- which usually stops at its first, certifying
                               residual                                                    */
 } spin_precision;
@@ -534,7 +534,12 @@ int spin_gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha,
  * digit slices of 8 bits (balanced digits of magnitude <= 128, exact in
  * BF16; 8 * slices - 1 bits in all); digit products (<= 2^14) are summed
  * exactly in FP32 runs of 1024, the runs in int32, and each slice-pair group
- * is scaled into the FP64 result (slice pairs (t, u) with t + u < slices).  The refinement residual
+ * is scaled into the FP64 result (slice pairs (t, u) with t + u < slices).
+ * For 4 slices and more (and k <= 98304) the same fixed-point integers, at
+ * least 8 * slices - 4 bits of them, are multiplied modulo several coprime
+ * numbers instead and the whole sum is put together from its residues: fewer
+ * tensor-core products, no pair left out, a smaller error; a row of A or a
+ * column of B that holds an infinity or NaN then gives NaN.  The refinement residual
  * R = I - A X of the mixed method is this call with alpha = -1, beta = 0,
  * add_identity = 1.  sumsq_dev (device double, optional) receives
  * += sum of squares of D.

@@ -250,7 +250,7 @@ int leaf_prof(Run& r, int depth, const double* A, int64_t lda, double* X, int64_
 
 // One level product D = beta*C + alpha*(A B).  FP64 for the plain method
 // (and for small products in mixed mode); in mixed mode bf16x3 on the
-// tensor cores, or FP64-class digit slices for the Schur complement of the
+// tensor cores, or the FP64-class product for the Schur complement of the
 // top fp64_levels levels.
 // Smallest m and n a mixed-mode product takes to the tensor cores
 // (SPIN_TC_MIN overrides it, for measurement; read once).
@@ -271,24 +271,13 @@ int level_gemm(Run& r, int depth, bool schur, int64_t m, int64_t n, int64_t k, d
         return gemm_f64_prof(r, depth, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd);
     const double f = 2.0 * (double)m * (double)n * (double)k;
     SplitPlan sp;
-    int rc;
     const bool fp64_schur = schur && depth < r.fp64_levels;
     if (fp64_schur || r.precision == SPIN_MIXED_DIGITS) {
         const int sl = fp64_schur ? kSchurSlices : kLevelSlices;
-        RET(plan_ozaki(m, n, k, sl, r.scratch, r.scratch_bytes, &sp));
-        {
-            ProfScope ps(r.prof, r.s, SPIN_KERNEL_SPLIT, depth, m, k, 0, 0.0, 8.0 * m * k + 2.0 * sl * m * k);
-            RET(split_a_ozaki(sp, A, lda, m, k, nullptr, r.s));
-        }
-        {
-            ProfScope ps(r.prof, r.s, SPIN_KERNEL_SPLIT, depth, k, n, 0, 0.0, 8.0 * k * n + 2.0 * sl * k * n);
-            RET(split_b_ozaki(sp, B, ldb, k, n, nullptr, r.s));
-        }
-        const int pairs = sl * (sl + 1) / 2;
-        ProfScope ps(r.prof, r.s, SPIN_KERNEL_GEMM_TC, depth, m, n, k, pairs * f,
-                     2.0 * sl * (m * k + k * n) + 8.0 * m * n * (beta != 0.0 ? 2 : 1));
-        rc = product_ozaki(sp, m, n, k, alpha, beta, C, ldc, D, ldd, 0, nullptr, r.err, r.s);
-        return rc;
+        ProfScope ps(r.prof, r.s, SPIN_KERNEL_GEMM_TC, depth, m, n, k, fp64_class_products(k, sl) * f,
+                     8.0 * (m * k + k * n) + 8.0 * m * n * (beta != 0.0 ? 2 : 1));
+        return gemm_fp64_class(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, sl, 0, Fp64ClassExtra(),
+                               r.scratch, r.scratch_bytes, r.err, r.s);
     }
     RET(plan_bf16x3(m, n, k, r.scratch, r.scratch_bytes, &sp));
     {
@@ -444,21 +433,24 @@ int read_info(StreamState* st, cudaStream_t s, spin_info* info) {
 }
 
 // Workspace of the mixed-precision form: the FP64 recursion workspace (later
-// reused for the residual R), the split arena, and the cached digit planes
-// of A for the refinement residual.
+// reused for the residual R), the norms, the row exponents of A (kept over
+// the refinement's rounds), the side stream's split arena, and the split
+// arena, which takes whatever the workspace holds beyond `total`.
 struct MixLayout {
-    size_t region0, scratch, apl, off_scratch, off_apl, off_norms, total;
-    size_t side_scratch, off_side;  // split arena of the side stream (overlapped schedule), else 0
-    int sr;  // digit slices of the certifying residuals (and of A's cached planes)
-    int s0;  // slices of the first residual's pairs (<= sr)
+    size_t region0, off_norms, off_exps, off_side, off_scratch, total;
+    size_t scratch;       // least bytes of the split arena
+    size_t side_scratch;  // split arena of the side stream (overlapped schedule), else 0
+    size_t preferred;     // total, and an arena in which the refinement's products need no panels
+    int sr;  // digit slices that the certifying residuals stand for
+    int s0;  // those of the first residual (<= sr)
 };
 
 size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 MixLayout mix_layout(int64_t n, int64_t leaf, const spin_opts& o) {
     MixLayout L;
-    // 9-bit digits relative to the largest entry of each row (column): the
-    // residual's error is ~0.6 sqrt(n) 2^-(9s-1) in the normalised measure
+    // digits relative to the largest entry of each row (column): the
+    // residual's error is ~0.6 sqrt(n) 2^-(8s-1) in the normalised measure
     // (residual_error_model); slices per round from that model
     L.sr = o.residual_slices > 0 ? o.residual_slices : residual_slices_for(n, o.tol);
     L.s0 = o.residual_slices > 0 ? o.residual_slices : first_residual_slices_for(n, o.tol, L.sr);
@@ -474,8 +466,9 @@ MixLayout mix_layout(int64_t n, int64_t leaf, const spin_opts& o) {
     }
     sc = std::max(sc, ozaki_scratch_bytes(0, n, n, L.sr));
     sc = std::max(sc, bf16x6_scratch_bytes(n, n, n));
-    L.scratch = round256(sc);
-    L.apl = round256((size_t)L.sr * (size_t)n * (size_t)tc_ld(n) * 2 + (size_t)n * 4 + 512);
+    // both operands of the residual
+    sc = round256(sc) + round256((size_t)L.sr * (size_t)n * (size_t)tc_ld(n) * 2);
+    L.scratch = sc;
     // the side stream's products (II and C21 of every level: at most n2 x n1 x n1)
     size_t side = 0;
     if (overlap) {
@@ -484,11 +477,13 @@ MixLayout mix_layout(int64_t n, int64_t leaf, const spin_opts& o) {
         if (o.precision == SPIN_MIXED_DIGITS) side = std::max(side, ozaki_scratch_bytes(n1, n1, n1, kLevelSlices));
     }
     L.side_scratch = round256(side);
-    L.off_scratch = L.region0;
-    L.off_apl = L.off_scratch + L.scratch;
-    L.off_norms = L.off_apl + L.apl;
-    L.off_side = L.off_norms + 256;
-    L.total = L.off_side + L.side_scratch;
+    L.off_norms = L.region0;
+    L.off_exps = L.off_norms + 256;
+    L.off_side = L.off_exps + round256((size_t)n * sizeof(int));
+    L.off_scratch = L.off_side + L.side_scratch;
+    L.total = L.off_scratch + L.scratch;
+    const size_t full = round256(fp64_class_bytes(n, n, n, L.sr));
+    L.preferred = L.off_scratch + std::max(L.scratch, std::min(full, kFp64ClassArena));
     return L;
 }
 
@@ -496,6 +491,12 @@ size_t inner_bytes(int64_t n, int64_t leaf, const spin_opts& o) {
     if (o.precision == SPIN_FP64)
         return ws_fp64_elems(n, leaf, n > leaf && overlap_schedule(n, o.precision, o.schedule)) * sizeof(double);
     return mix_layout(n, leaf, o).total;
+}
+
+// What the library's own buffer is made when the device has the memory.
+size_t preferred_bytes(int64_t n, int64_t leaf, const spin_opts& o, size_t need) {
+    if (o.precision == SPIN_FP64 || o.pretransform != 0) return need;
+    return std::max(need, mix_layout(n, leaf, o).preferred);
 }
 
 // Butterfly transform: [diagonals | Ar (np x np) | Y (np x np) | the
@@ -524,8 +525,7 @@ size_t workspace_bytes_for(int64_t n, int64_t leaf, const spin_opts& o) {
 
 // Newton-Schulz refinement X <- X + X (I - A X) (Bailey-style stabilisation
 // of Strassen's inversion, cited in Sec. 2.1): every residual R = I - A X is
-// FP64-class (digit slices of A, split once and cached, and of X), the
-// correction X R is a six-product BF16 form.  Every residual is recomputed
+// FP64-class (A's row exponents taken once), the correction X R is a six-product BF16 form.  Every residual is recomputed
 // in full: after a step the true residual is dominated by the previous
 // residual's own rounding error, which an update of the form R - A (dX)
 // cannot see.  Stops when ||AX - I||_F / (||A||_F ||X||_F) <= tol.
@@ -534,40 +534,34 @@ size_t workspace_bytes_for(int64_t n, int64_t leaf, const spin_opts& o) {
 // 0 .. max_refine are all enqueued, each gated on the stream's active flag,
 // so the call never waits for the host between steps.
 int refine(Run& r, StreamState* st, const double* A, int64_t lda, double* X, int64_t ldx, int64_t n,
-           const spin_opts& o, const MixLayout& L, unsigned char* ws) {
+           const spin_opts& o, const MixLayout& L, unsigned char* ws, size_t ws_bytes) {
     cudaStream_t s = r.s;
     double* R = (double*)ws;
     double* norms = (double*)(ws + L.off_norms);
     int* act = st->active();
-    const int64_t ld = tc_ld(n);
-    OzakiCachedA ca{(uint16_t*)(ws + L.off_apl), (int*)(ws + L.off_apl + (size_t)L.sr * n * ld * 2)};
+    int* exps = (int*)(ws + L.off_exps);
     void* scratch = ws + L.off_scratch;
+    const size_t scratch_bytes = ws_bytes - L.off_scratch;
     // a leaf that failed leaves the matrix switched off: nothing below runs
     RET(launch_refine_init(st->info_dev, 1, act, st->rel(), st->iters(), s));
     SPIN_CUDA_TRY(cudaMemsetAsync(norms, 0, 3 * sizeof(double), s));
-    {
-        ProfScope ps(r.prof, s, SPIN_KERNEL_SPLIT, -1, n, n, 0, 0.0, 8.0 * n * n + 2.0 * L.sr * n * n, act);
-        RET(ozaki_split_a(A, lda, n, n, L.sr, &ca, &norms[0], s, act));
-    }
     const double f = 2.0 * (double)n * n * n;
-    const int sr = L.sr;
     for (int it = 0; it <= o.max_refine; it++) {
-        // the first residual only feeds the update: fewer slice pairs
-        const int s_it = it == 0 ? L.s0 : sr;
-        const int pairs = s_it * (s_it + 1) / 2;
-        SPIN_CUDA_TRY(cudaMemsetAsync(norms + 1, 0, 2 * sizeof(double), s));
-        SplitPlan sp;
-        RET(plan_ozaki(0, n, n, sr, scratch, L.scratch, &sp));
-        sp.a = ca.planes;
-        sp.ea = ca.exps;
+        // the first residual only feeds the update: fewer slices
+        const int s_it = it == 0 ? L.s0 : L.sr;
+        if (it > 0) SPIN_CUDA_TRY(cudaMemsetAsync(norms + 1, 0, 2 * sizeof(double), s));
         {
-            ProfScope ps(r.prof, s, SPIN_KERNEL_SPLIT, -1, n, n, 0, 0.0, 8.0 * n * n + 2.0 * sr * n * n, act);
-            RET(split_b_ozaki(sp, X, ldx, n, n, &norms[1], s, act));
-        }
-        {
-            ProfScope ps(r.prof, s, SPIN_KERNEL_RESIDUAL, -1, n, n, n, pairs * f, 2.0 * sr * 2.0 * n * n + 8.0 * n * n,
+            Fp64ClassExtra x;
+            x.active = act;
+            x.sumsq_a = &norms[0];
+            x.sumsq_b = &norms[1];
+            x.sumsq_d = &norms[2];
+            x.a_exps = exps;
+            x.a_known = it > 0;
+            ProfScope ps(r.prof, s, SPIN_KERNEL_RESIDUAL, -1, n, n, n, fp64_class_products(n, s_it) * f, 24.0 * n * n,
                          act);
-            RET(product_ozaki(sp, n, n, n, -1.0, 0.0, nullptr, 0, R, n, 1, &norms[2], r.err, s, act, s_it));
+            RET(gemm_fp64_class(n, n, n, -1.0, A, lda, X, ldx, 0.0, nullptr, 0, R, n, s_it, 1, x, scratch,
+                                scratch_bytes, r.err, s));
         }
         RET(launch_refine_decide(norms, norms + 1, norms + 2, 1, o.tol, residual_error_model(n, s_it), it,
                                  o.max_refine, act, st->rel(), st->iters(), st->info_dev, s));
@@ -576,7 +570,7 @@ int refine(Run& r, StreamState* st, const double* A, int64_t lda, double* X, int
         // relative): the correction's own error enters the next residual
         // amplified by ~kappa * rel, so it needs more than bf16x3's ~2^-16.
         SplitPlan up;
-        RET(plan_bf16x6(n, n, n, scratch, L.scratch, &up));
+        RET(plan_bf16x6(n, n, n, scratch, scratch_bytes, &up));
         {
             ProfScope ps(r.prof, s, SPIN_KERNEL_SPLIT, -1, n, n, 0, 0.0, 28.0 * n * n, act);
             RET(split_a_bf16x6(up, X, ldx, n, n, s, act));
@@ -592,7 +586,7 @@ int refine(Run& r, StreamState* st, const double* A, int64_t lda, double* X, int
 // transform undone afterwards (pretransform 1); mixed modes then refine
 // X against A itself.
 int enqueue_once(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, int64_t leaf, const spin_opts& o,
-                 bool rbt, StreamState* st, cudaStream_t s, unsigned char* ws) {
+                 bool rbt, StreamState* st, cudaStream_t s, unsigned char* ws, size_t ws_bytes) {
     const bool mixed = o.precision != SPIN_FP64;
     st->last_mixed = mixed ? 1 : 0;
     st->last_pretransformed = rbt ? 1 : 0;
@@ -616,6 +610,7 @@ int enqueue_once(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n
         Xout = (double*)(ws + R.off_y);
         ldx_out = R.np;
         inner = ws + R.off_inner;
+        ws_bytes -= R.off_inner;
     }
     if (!mixed) {
         if (overlap_schedule(n_in, o.precision, o.schedule) && n_in > leaf) {
@@ -631,7 +626,7 @@ int enqueue_once(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n
     r.precision = o.precision;
     r.fp64_levels = o.fp64_levels;
     r.scratch = inner + Lin.off_scratch;
-    r.scratch_bytes = Lin.scratch;
+    r.scratch_bytes = ws_bytes - Lin.off_scratch;
     if (Lin.side_scratch > 0) {
         if (st->side == nullptr) SPIN_CUDA_TRY(cudaStreamCreateWithFlags(&st->side, cudaStreamNonBlocking));
         r.side = st->side;
@@ -644,7 +639,7 @@ int enqueue_once(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n
     RET(inv_rec(r, 0, Ain, lda_in, Xout, ldx_out, n_in, (double*)inner));
     if (rbt) RET(launch_rbt_backward(Xout, R.np, kRbtDepth, (const double*)ws, X, ldx, n, s));
     // the refinement's layout for order n fits in the recursion's (order >= n)
-    return refine(r, st, A, lda, X, ldx, n, o, mix_layout(n, leaf, o), inner);
+    return refine(r, st, A, lda, X, ldx, n, o, mix_layout(n, leaf, o), inner, ws_bytes);
 }
 
 // Whether repeated calls replay a captured graph (SPIN_GRAPH=0 turns it
@@ -666,18 +661,18 @@ uint64_t bits_of(double x) {
 
 // Every argument that shapes the launch sequence or its operands.
 std::vector<uint64_t> call_key(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, int64_t leaf,
-                               const spin_opts& o, const void* ws) {
+                               const spin_opts& o, const void* ws, size_t ws_bytes) {
     return {(uint64_t)(uintptr_t)A, (uint64_t)lda, (uint64_t)(uintptr_t)X, (uint64_t)ldx, (uint64_t)n,
             (uint64_t)leaf, (uint64_t)o.precision, bits_of(o.tol), (uint64_t)o.max_refine,
             (uint64_t)o.fp64_levels, (uint64_t)o.residual_slices, (uint64_t)o.pretransform, o.rbt_seed,
             (uint64_t)(int64_t)o.schedule,
-            (uint64_t)(uintptr_t)ws};
+            (uint64_t)(uintptr_t)ws, (uint64_t)ws_bytes};
 }
 
 // Capture the whole schedule of one call (every launch enqueue_once makes,
 // on this stream and on the side stream) into a graph on a private stream.
 int capture_schedule(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, int64_t leaf,
-                     const spin_opts& o, StreamState* st, unsigned char* ws) {
+                     const spin_opts& o, StreamState* st, unsigned char* ws, size_t ws_bytes) {
     if (st->cap == nullptr) SPIN_CUDA_TRY(cudaStreamCreateWithFlags(&st->cap, cudaStreamNonBlocking));
     if (st->exec) {
         cudaGraphExecDestroy(st->exec);
@@ -685,7 +680,7 @@ int capture_schedule(const double* A, int64_t lda, double* X, int64_t ldx, int64
         st->graph_key.clear();
     }
     SPIN_CUDA_TRY(cudaStreamBeginCapture(st->cap, cudaStreamCaptureModeThreadLocal));
-    const int rc = enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, st->cap, ws);
+    const int rc = enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, st->cap, ws, ws_bytes);
     cudaGraph_t graph = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(st->cap, &graph);
     if (rc != SPIN_OK) {
@@ -716,25 +711,29 @@ int enqueue(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, con
     if (o.schedule < SPIN_SCHEDULE_DEFAULT || o.schedule > SPIN_SCHEDULE_PERSISTENT) return SPIN_ERR_INVALID_ARG;
     const size_t need = workspace_bytes_for(n, leaf, o);
     unsigned char* ws;
+    size_t ws_bytes;  // mixed forms: what lies beyond `need` saves panels (crt.cu), the results are the same
     if (o.workspace != nullptr) {
         if (o.workspace_bytes < need || ((uintptr_t)o.workspace & 255u) != 0) return SPIN_ERR_INVALID_ARG;
         ws = (unsigned char*)o.workspace;
+        ws_bytes = o.workspace_bytes;
     } else {
-        RET(ensure_ws(st, need));
+        const size_t want = preferred_bytes(n, leaf, o, need);
+        if (want == need || ensure_ws(st, want) != SPIN_OK) RET(ensure_ws(st, need));
         ws = (unsigned char*)st->ws;
+        ws_bytes = std::min(st->ws_bytes, want);
     }
     if (o.pretransform != 2) {
-        if (!graph_mode() || st->prof.on) return enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, s, ws);
+        if (!graph_mode() || st->prof.on) return enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, s, ws, ws_bytes);
         // The second call with the same arguments captures the schedule;
         // later ones replay it (one graph launch, dependencies resolved on
         // the device); any other call runs the launches directly.
-        std::vector<uint64_t> key = call_key(A, lda, X, ldx, n, leaf, o, ws);
+        std::vector<uint64_t> key = call_key(A, lda, X, ldx, n, leaf, o, ws, ws_bytes);
         if (st->exec == nullptr || key != st->graph_key) {
             if (key != st->prev_key) {
                 st->prev_key = key;
-                return enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, s, ws);
+                return enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, s, ws, ws_bytes);
             }
-            RET(capture_schedule(A, lda, X, ldx, n, leaf, o, st, ws));
+            RET(capture_schedule(A, lda, X, ldx, n, leaf, o, st, ws, ws_bytes));
             st->graph_key = key;
         }
         st->last_mixed = st->graph_mixed;
@@ -745,12 +744,12 @@ int enqueue(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, con
     }
     // plain first; a zero or non-finite pivot (A11 or a Schur complement
     // singular in working precision) sends the call through the transform
-    RET(enqueue_once(A, lda, X, ldx, n, leaf, o, false, st, s, ws));
+    RET(enqueue_once(A, lda, X, ldx, n, leaf, o, false, st, s, ws, ws_bytes));
     SPIN_CUDA_TRY(cudaMemcpyAsync(st->info_host, st->info_dev, INFO_WORDS * sizeof(int32_t),
                                   cudaMemcpyDeviceToHost, s));
     SPIN_CUDA_TRY(cudaStreamSynchronize(s));
     if (st->info_host[INFO_STATUS] != SPIN_ERR_SINGULAR) return SPIN_OK;
-    return enqueue_once(A, lda, X, ldx, n, leaf, o, true, st, s, ws);
+    return enqueue_once(A, lda, X, ldx, n, leaf, o, true, st, s, ws, ws_bytes);
 }
 
 // ---- leaf autotuning ----

@@ -1,0 +1,791 @@
+// FP64-class products on the BF16 tensor cores by residues.
+//
+// The digit form (tc_gemm.cu, exact mode) cuts every operand into s digits
+// and needs the s (s + 1) / 2 digit products of the leading weights.  Here
+// the same fixed-point integers a' = round(a 2^(b - e)) (e the row's, for B
+// the column's exponent) are taken modulo N pairwise coprime numbers p <=
+// 256 instead, one product per modulus gives sum_k a'_ik b'_kj modulo p
+// exactly, and the Chinese remainder theorem gives the whole sum, as long as
+// the product of the moduli exceeds twice its largest magnitude (Ozaki,
+// Uchino and Imamura, "Ozaki Scheme II", 2025, on INT8 units, whose rate on
+// GB300 is far below BF16's).  Nothing is left out of the sum, so fewer bits
+// give the same error (crt_bits_for_slices), and the number of tensor-core
+// products falls from 21 to 13 or 14 for s = 6, from 28 to 15 or 16 for s = 7.
+//
+// Three kernels:
+//   split    FP64 -> N BF16 planes of signed residues (|r| <= 128, exact):
+//            the integer is cut into balanced 14-bit pieces, and a residue is
+//            one FP32 dot product of 4 or 5 pieces with the powers of 2^14
+//            modulo p (every partial sum below 2^24, exact) and one rounded
+//            quotient: six FP32 operations per residue.
+//   product  per modulus and 128 x 256 tile, exact FP32 runs of 1024 products
+//            (|r r'| <= 2^14, sums <= 2^24) drained into int32, reduced
+//            modulo p and written as one byte per output.  A tile of one
+//            modulus is a work item of its own, so small products still fill
+//            the SMs, and the drain is a conversion and an add per run.
+//   combine  sum / P = frac(sum_l c_l u_l / p_l) with u_l the inverse of P /
+//            p_l modulo p_l: one 128-bit fixed-point accumulation per output
+//            with the constants u_l 2^128 / p_l (four 32-bit limbs, no carries
+//            between moduli), then times P 2^(e + f - 2 b), rounded once to
+//            FP64, and the product's epilogue (alpha, beta C, identity, sum of
+//            squares).
+// The integers are exact and every output depends on its row and column
+// only, so the result does not depend on the panels the arena allows.
+#include <math.h>
+#include <string.h>
+
+#include <algorithm>
+
+#include "crt.h"
+#include "tc_pipe.cuh"
+
+namespace spin {
+namespace {
+
+// Pairwise coprime, in falling order; with signed residues |r| <= 128.
+__host__ __device__ constexpr int crt_modulus(int l) {
+    constexpr int p[kCrtMaxModuli] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227,
+                                      223, 217, 211, 199, 197, 193, 191, 181, 179, 173};
+    return p[l];
+}
+
+constexpr int kPiece = 14;  // bits of a balanced piece of the integer
+constexpr int kRunK = 1024;
+constexpr int kMaxRuns = 96;  // 96 runs of 2^24 fit int32
+
+// ----------------------------------------------------------------- split --
+
+// 2^(14 q) modulo p, balanced.
+__host__ __device__ constexpr int piece_weight(int l, int q) {
+    const int p = crt_modulus(l);
+    int v = 1;
+    for (int i = 0; i < q; i++) v = v * (1 << kPiece) % p;
+    return v > p / 2 ? v - p : v;
+}
+
+// round(x 2^(b - e)), |x| < 2^e (ties away from zero; integer arithmetic on
+// the IEEE fields), as PIECES balanced 14-bit pieces in FP32.
+template <int PIECES>
+__device__ __forceinline__ void fixed_pieces(double x, int e, int b, float (&f)[PIECES]) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    int fe = (int)(u >> 52) & 0x7FF;
+    unsigned long long m = u & ((1ull << 52) - 1);
+    if (fe == 0)
+        fe = 1;  // subnormal: no implicit bit
+    else
+        m |= 1ull << 52;
+    const int sh = fe - 1075 + b - e;  // <= b - 53
+    unsigned long long n;
+    if (sh >= 0)
+        n = m << sh;
+    else if (sh > -64)
+        n = (m + (1ull << (-sh - 1))) >> (-sh);
+    else
+        n = 0;
+    long long v = (u >> 63) ? -(long long)n : (long long)n;
+#pragma unroll
+    for (int q = 0; q < PIECES; q++) {
+        int d;
+        if (q + 1 < PIECES) {
+            d = (int)((unsigned)v << (32 - kPiece)) >> (32 - kPiece);  // low 14 bits, signed
+            v = (v - d) >> kPiece;
+        } else {
+            d = (int)v;
+        }
+        // d as FP32 without a conversion (16 per clock per SM): |d| < 2^22
+        f[q] = __uint_as_float(0x4B400000u + (unsigned)d) - 12582912.0f;
+    }
+}
+
+// The residue modulo modulus l, signed (|r| <= 128), as BF16 bits in the
+// high half of the returned word.
+template <int PIECES>
+__device__ __forceinline__ unsigned residue_bits(const float (&f)[PIECES], float p, float inv_p, const float (&w)[PIECES]) {
+    float t = f[0];
+#pragma unroll
+    for (int q = 1; q < PIECES; q++) t = fmaf(f[q], w[q], t);  // |t| < 2^23: exact
+    const float quot = fmaf(t, inv_p, 12582912.0f) - 12582912.0f;
+    return __float_as_uint(fmaf(-quot, p, t));
+}
+
+template <int PIECES>
+__device__ __forceinline__ void store_residues4(const float (&f)[4][PIECES], int moduli, uint16_t* dst, int64_t plane) {
+#pragma unroll
+    for (int l = 0; l < kCrtMaxModuli; l++) {
+        if (l >= moduli) break;
+        float w[PIECES];
+#pragma unroll
+        for (int q = 0; q < PIECES; q++) w[q] = (float)piece_weight(l, q);
+        const float p = (float)crt_modulus(l), inv_p = 1.0f / (float)crt_modulus(l);
+        unsigned r[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) r[u] = residue_bits<PIECES>(f[u], p, inv_p, w);
+        uint2 o;  // bytes 2, 3 of each word: the BF16 value (the rest is zero)
+        o.x = __byte_perm(r[0], r[1], 0x7632);
+        o.y = __byte_perm(r[2], r[3], 0x7632);
+        *reinterpret_cast<uint2*>(dst + l * plane) = o;
+    }
+}
+
+// Rows of a panel (rows row0 ..), K-major as they are: 4 consecutive columns
+// per thread (8-byte stores; planes are padded to a multiple of 8 columns).
+template <class Src, int PIECES>
+__global__ void __launch_bounds__(256)
+crt_rows_kernel(Src src, int row0, int rows, int cols, const int* __restrict__ ex, int64_t exs, int bits, int moduli,
+                uint16_t* __restrict__ dst, int64_t ld) {
+    const int z = blockIdx.z;
+    if (!src.on(z)) return;
+    const int64_t plane = (int64_t)rows * ld;
+    dst += (int64_t)z * moduli * plane;
+    ex += (int64_t)z * exs + row0;
+    const int groups = (cols + 3) / 4;
+    const int64_t total = (int64_t)rows * groups;
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        const int r = (int)(idx / groups), c = (int)(idx % groups) * 4;
+        const double* sr = src.row(z, row0 + r) + c;
+        const int e = ex[r];
+        float f[4][PIECES];
+#pragma unroll
+        for (int u = 0; u < 4; u++) fixed_pieces<PIECES>(c + u < cols ? sr[u] : 0.0, e, bits, f[u]);
+        store_residues4<PIECES>(f, moduli, dst + (int64_t)r * ld + c, plane);
+    }
+}
+
+// Columns of a panel (columns col0 ..) of a rows x cols operand, transposed:
+// 32 columns x 128 rows through shared memory, 4 consecutive rows (K) per
+// thread.
+constexpr int kTileK = 128;
+constexpr int kTileLd = kTileK + 2;  // even: 16-byte reads
+template <class Src, int PIECES>
+__global__ void __launch_bounds__(256)
+crt_cols_kernel(Src src, int col0, int rows, int cols, const int* __restrict__ ex, int64_t exs, int bits, int moduli,
+                uint16_t* __restrict__ dst, int64_t ld) {
+    __shared__ __align__(16) double tile[32][kTileLd];
+    const int z = blockIdx.z;
+    if (!src.on(z)) return;
+    const int64_t plane = (int64_t)cols * ld;
+    dst += (int64_t)z * moduli * plane;
+    ex += (int64_t)z * exs + col0;
+    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * kTileK;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 4
+    for (int i = warp; i < kTileK; i += 8) {
+        const int r = r0 + i, c = c0 + lane;
+        tile[lane][i] = (r < rows && c < cols) ? src.row(z, r)[col0 + c] : 0.0;
+    }
+    __syncthreads();
+    for (int i = warp; i < 32; i += 8) {
+        const int c = c0 + i, r = r0 + 4 * lane;
+        if (c >= cols || r >= rows) continue;
+        const int e = ex[c];
+        const double2 a = *reinterpret_cast<const double2*>(&tile[i][4 * lane]);
+        const double2 b = *reinterpret_cast<const double2*>(&tile[i][4 * lane + 2]);
+        float f[4][PIECES];
+        fixed_pieces<PIECES>(a.x, e, bits, f[0]);
+        fixed_pieces<PIECES>(a.y, e, bits, f[1]);
+        fixed_pieces<PIECES>(b.x, e, bits, f[2]);
+        fixed_pieces<PIECES>(b.y, e, bits, f[3]);
+        store_residues4<PIECES>(f, moduli, dst + (int64_t)c * ld + r, plane);
+    }
+}
+
+// --------------------------------------------------------------- product --
+
+struct CrtGemmParams {
+    int M, N, K;        // of the panel pair
+    int moduli, count;  // problems (>= 1)
+    uint8_t* res;       // [z][modulus][M][ldr]
+    int64_t ldr;        // a multiple of 16, >= N
+    const int* active;
+    int* err;
+    unsigned p[kCrtMaxModuli], magic[kCrtMaxModuli], shift[kCrtMaxModuli];  // x + shift >= 0, a multiple of p
+};
+
+constexpr int kCrtBN = 256;
+constexpr int kCrtEpiWarps = 16;
+constexpr int kCrtHalf = kCrtBN / (kCrtEpiWarps / 4);  // columns per epilogue warp
+
+// Persistent: one CTA per SM walks the items (problem, modulus, tile), the
+// drain of one overlapping the next one's MMAs in the other TMEM accumulator.
+// Warps as in tc_gemm_kernel: 0 TMA, 1 MMA, 2.. epilogue.
+__global__ void __maxnreg__(Epi<kCrtEpiWarps>::MAXREG)
+crt_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                const __grid_constant__ CrtGemmParams p) {
+    // a problem switched off: nothing to set up (every thread reads the same flag)
+    if (p.count == 1 && p.active != nullptr && p.active[0] == 0) return;
+    constexpr int BN = kCrtBN, HALF = kCrtHalf;
+    using C = Cfg<BN, 1>;
+    constexpr int STAGES = C::STAGES;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char* smA = base;
+    unsigned char* smB = base + STAGES * A_TILE_BYTES;
+    SmemCtl* ctl = reinterpret_cast<SmemCtl*>(base + STAGES * C::STAGE_BYTES);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int num_m = (p.M + BM - 1) / BM, num_n = (p.N + BN - 1) / BN;
+    const int tiles = num_m * num_n;
+    const int64_t items = (int64_t)p.count * p.moduli * tiles;
+    // item t: plane (problem and modulus) zl and the tile's origin; tiles in
+    // bands of GROUP_M row blocks, as in tc_gemm_kernel
+    auto item_of = [&](int64_t t, int& zl, int& m0, int& n0) -> bool {
+        zl = (int)(t / tiles);
+        const int pid = (int)(t - (int64_t)zl * tiles);
+        const int per_group = GROUP_M * num_n;
+        const int first_m = (pid / per_group) * GROUP_M;
+        const int gsize = min(num_m - first_m, GROUP_M);
+        const int in_group = pid % per_group;
+        m0 = (first_m + in_group % gsize) * BM;
+        n0 = (in_group / gsize) * BN;
+        return p.active == nullptr || p.active[zl / p.moduli] != 0;
+    };
+    const int KB = (p.K + BK - 1) / BK;
+    constexpr int run_kb = kRunK / BK;
+    const int runs = (KB + run_kb - 1) / run_kb;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; s++) {
+            mbar_init(&ctl->full[s], 1);
+            mbar_init(&ctl->empty[s], 1);
+        }
+        for (int b = 0; b < 2; b++) {
+            mbar_init(&ctl->tfull[b], 1);
+            mbar_init(&ctl->tempty[b], kCrtEpiWarps);
+        }
+        mbar_init(&ctl->final_bar, 1);
+        ctl->abort = 0;
+        fence_mbar_init();
+        prefetch_tensormap(&tmA);
+        prefetch_tensormap(&tmB);
+    }
+    if (warp == 1) {
+        tmem_alloc(&ctl->tmem_base, 2 * BN);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    volatile int* abort = &ctl->abort;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int it = 0;
+            bool ok = true;
+            int zl, m0, n0;
+            for (int64_t t = blockIdx.x; t < items && ok; t += gridDim.x) {
+                if (!item_of(t, zl, m0, n0)) continue;
+                const int ya = zl * p.M + m0, yb = zl * p.N + n0;
+                for (int kb = 0; kb < KB; kb++) {
+                    const int s = it % STAGES;
+                    ok = mbar_wait(&ctl->empty[s], (uint32_t)((it / STAGES) & 1) ^ 1u, abort, WAIT_LIMIT_NS);
+                    if (!ok) break;
+                    mbar_arrive_expect_tx(&ctl->full[s], C::STAGE_BYTES);
+                    tma_load_2d(smA + s * A_TILE_BYTES, &tmA, kb * BK, ya, &ctl->full[s]);
+                    tma_load_2d(smB + s * C::B_TILE_BYTES, &tmB, kb * BK, yb, &ctl->full[s]);
+                    it++;
+                }
+            }
+            if (!ok) raise_timeout(ctl, p.err);
+            // own copies still in flight: the last min(STAGES, it) loads
+            for (int j = max(0, it - STAGES); j < it; j++) {
+                volatile int never = 0;
+                mbar_wait(&ctl->full[j % STAGES], (uint32_t)((j / STAGES) & 1), &never, WAIT_LIMIT_NS);
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = idesc_bf16_f32(BM, BN);
+            int it = 0, run = 0;
+            bool ok = true;
+            int zl, m0, n0;
+            for (int64_t t = blockIdx.x; t < items && ok; t += gridDim.x) {
+                if (!item_of(t, zl, m0, n0)) continue;
+                for (int kb = 0; kb < KB && ok;) {
+                    const int buf = run & 1;
+                    ok = mbar_wait(&ctl->tempty[buf], (uint32_t)((run >> 1) & 1) ^ 1u, abort, WAIT_LIMIT_NS);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t d = tmem_base + (uint32_t)(buf * BN);
+                    const int kb0 = kb, kb1 = min(KB, kb + run_kb);
+                    for (; kb < kb1; kb++) {
+                        const int s = it % STAGES;
+                        ok = mbar_wait(&ctl->full[s], (uint32_t)((it / STAGES) & 1), abort, WAIT_LIMIT_NS);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint64_t ad = sdesc_kmajor_sw128(smem_u32(smA + s * A_TILE_BYTES));
+                        const uint64_t bd = sdesc_kmajor_sw128(smem_u32(smB + s * C::B_TILE_BYTES));
+#pragma unroll
+                        for (int k = 0; k < BK / 16; k++)
+                            mma_bf16(d, ad + ((k * 32) >> 4), bd + ((k * 32) >> 4), idesc, (kb == kb0 && k == 0) ? 0u : 1u);
+                        mma_commit(&ctl->empty[s]);
+                        it++;
+                    }
+                    if (ok) mma_commit(&ctl->tfull[buf]);
+                    run++;
+                }
+            }
+            if (!ok) raise_timeout(ctl, p.err);
+            // every MMA issued so far has completed once final_bar flips
+            mma_commit(&ctl->final_bar);
+            volatile int never = 0;
+            mbar_wait(&ctl->final_bar, 0u, &never, WAIT_LIMIT_NS);
+        }
+        __syncwarp();
+    } else {
+        const int quarter = warp & 3;       // TMEM lane quarter this warp may access
+        const int half = (warp - 2) >> 2;   // column group of the tile
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * HALF);
+        int run = 0;
+        int zl, m0, n0;
+        bool ok = true;
+        for (int64_t t = blockIdx.x; t < items && ok; t += gridDim.x) {
+            if (*abort) break;
+            if (!item_of(t, zl, m0, n0)) continue;
+            int acc[HALF];
+            for (int c = 0; c < runs && ok; c++) {
+                const int buf = run & 1;
+                ok = mbar_wait(&ctl->tfull[buf], (uint32_t)((run >> 1) & 1), abort, WAIT_LIMIT_NS);
+                if (!ok) {
+                    raise_timeout(ctl, p.err);
+                    break;
+                }
+                tc_fence_after();
+#pragma unroll
+                for (int c0 = 0; c0 < HALF; c0 += 16) {
+                    uint32_t v[16];
+                    tmem_ld_32x32b_x16(lane_addr + (uint32_t)(buf * BN + c0), v);
+                    tmem_ld_wait();
+                    if (c == 0) {
+#pragma unroll
+                        for (int j = 0; j < 16; j++) acc[c0 + j] = __float2int_rn(__uint_as_float(v[j]));
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; j++) acc[c0 + j] += __float2int_rn(__uint_as_float(v[j]));
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->tempty[buf]);
+                run++;
+            }
+            if (!ok) break;
+            const int row = m0 + quarter * 32 + lane, col0 = n0 + half * HALF;
+            if (row < p.M) {
+                const int l = zl % p.moduli;
+                const unsigned mod = p.p[l], magic = p.magic[l], shift = p.shift[l];
+                uint8_t* out = p.res + ((int64_t)zl * p.M + row) * p.ldr + col0;
+#pragma unroll
+                for (int c0 = 0; c0 < HALF; c0 += 16) {
+                    if (col0 + c0 >= p.ldr) break;
+                    uint32_t w[4];
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        uint32_t b[4];
+#pragma unroll
+                        for (int j = 0; j < 4; j++) {
+                            const unsigned u = (unsigned)acc[c0 + 4 * q + j] + shift;
+                            const unsigned r = u - __umulhi(u, magic) * mod;  // in [0, 2 mod)
+                            b[j] = min(r, r - mod);
+                        }
+                        w[q] = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
+                    }
+                    *reinterpret_cast<uint4*>(out + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 2 * BN);
+    }
+}
+
+// --------------------------------------------------------------- combine --
+
+struct CrtTable {
+    unsigned v[kCrtMaxModuli][4];  // u_l 2^128 / p_l modulo 2^128, low limb first
+    unsigned long long pm;         // the product of the moduli = pm 2^pe, 2^63 <= pm < 2^64
+    int pe;
+    int moduli, bits;
+};
+
+// The sum whose residue fraction (sum / P modulo 1, times 2^128) is f, times
+// 2^scale, rounded to FP64 (neg: times -1).
+__device__ __forceinline__ double crt_value(unsigned long long hi, unsigned long long lo, const CrtTable& t, int scale,
+                                            bool neg) {
+    if (hi >> 63) {  // the symmetric range: fractions of one half and more are negative
+        lo = 0ull - lo;
+        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
+        neg = !neg;
+    }
+    if ((hi | lo) == 0ull) return 0.0;
+    int lz;
+    unsigned long long h;
+    if (hi) {
+        lz = __clzll((long long)hi);
+        h = lz ? (hi << lz) | (lo >> (64 - lz)) : hi;
+    } else {
+        const int s = __clzll((long long)lo);
+        lz = 64 + s;
+        h = lo << s;
+    }
+    unsigned long long prod = __umul64hi(h, t.pm);  // the sum = prod 2^(pe - lz)
+    const int s = __clzll((long long)prod);         // 0 or 1
+    prod <<= s;
+    const unsigned long long m = (prod >> 11) + ((prod >> 10) & 1ull);  // 53 bits, or 2^53
+    const int e = 11 + t.pe - lz - s + scale;                          // value = m 2^e
+    const int be = e + 52 + 1023;
+    double v;
+    if (be >= 1 && be <= 2045)
+        v = __longlong_as_double((long long)(((unsigned long long)(be - 1) << 52) + m));
+    else
+        v = ldexp((double)m, e);
+    return neg ? -v : v;
+}
+
+// 4 columns of a row per thread.  p: the whole product (views, epilogue);
+// (row0, col0): the panel pair's origin; rows x cols its size.
+__global__ void __launch_bounds__(256)
+crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int cols, int row0, int col0,
+                   const __grid_constant__ CrtTable t, const __grid_constant__ TcGemmParams p) {
+    const int z = blockIdx.z;
+    if (p.active != nullptr && p.active[p.batch ? z : 0] == 0) return;
+    const int64_t plane = (int64_t)rows * ldr;
+    res += (int64_t)z * t.moduli * plane;
+    const int* row_exp = p.row_exp + (int64_t)z * p.M + row0;
+    const int* col_exp = p.col_exp + (int64_t)z * p.N + col0;
+    const int groups = (cols + 3) / 4;
+    const int64_t total = (int64_t)rows * groups;
+    const int so = p.sum_order ? p.sum_order[z] : 0x7fffffff;
+    double ss = 0.0;
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        const int r = (int)(idx / groups), c = (int)(idx % groups) * 4;
+        const uint8_t* src = res + (int64_t)r * ldr + c;
+        unsigned long long acc[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) acc[u][i] = 0ull;
+#pragma unroll 4
+        for (int l = 0; l < t.moduli; l++) {
+            const unsigned w = *reinterpret_cast<const unsigned*>(src + l * plane);
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const unsigned b = (w >> (8 * u)) & 255u;
+#pragma unroll
+                for (int i = 0; i < 4; i++) acc[u][i] += (unsigned long long)b * t.v[l][i];
+            }
+        }
+        const int er = row_exp[r], grow = row0 + r;
+        const double* crow = p.beta != 0.0 ? in_row(p, z, grow) : nullptr;
+        double* drow = out_row(p, z, grow);
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (c + u >= cols) break;
+            const int gcol = col0 + c + u, ec = col_exp[c + u];
+            const unsigned long long s1 = acc[u][1] + (acc[u][0] >> 32);
+            const unsigned long long s2 = acc[u][2] + (s1 >> 32);
+            const unsigned long long s3 = acc[u][3] + (s2 >> 32);
+            double val = crt_value((s3 << 32) | (s2 & 0xffffffffull), (s1 << 32) | (acc[u][0] & 0xffffffffull), t,
+                                   er + ec - 2 * t.bits, p.alpha < 0.0);
+            // an infinity or NaN in the row or column (no fixed point has it)
+            if (er > 1024 || ec > 1024) val = __longlong_as_double(0x7ff8000000000000ll);
+            if (p.beta != 0.0) val = fma(p.beta, crow[gcol], val);
+            if (p.add_identity && gcol == grow) val += 1.0;
+            drow[gcol] = val;
+            if (p.sumsq && grow < so && gcol < so) ss = fma(val, val, ss);
+        }
+    }
+    if (p.sumsq) {
+        __shared__ double part[8];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) ss += __shfl_down_sync(0xffffffffu, ss, off);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = ss;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int i = 1; i < 8; i++) ss += part[i];
+            if (ss != 0.0) atomicAdd(p.sumsq + (p.batch ? z : 0), ss);
+        }
+    }
+}
+
+// ------------------------------------------------------------------ host --
+
+// floor(2^128 u / p) with p, u < 2^9, rounded, as four limbs.
+void fraction_limbs(unsigned u, unsigned p, unsigned (&v)[4]) {
+    unsigned rem = u % p;
+    unsigned q[5];  // 32-bit digits of u / p behind the point, one more for the rounding
+    for (int i = 0; i < 5; i++) {
+        const unsigned long long t = (unsigned long long)rem << 32;
+        q[i] = (unsigned)(t / p);
+        rem = (unsigned)(t % p);
+    }
+    unsigned carry = q[4] >> 31;
+    for (int i = 3; i >= 0; i--) {
+        const unsigned long long t = (unsigned long long)q[i] + carry;
+        v[3 - i] = (unsigned)t;
+        carry = (unsigned)(t >> 32);
+    }
+}
+
+void crt_table(const CrtFormat& f, CrtTable* t) {
+    // P as a little-endian multi-limb integer (at most 160 bits)
+    unsigned limb[6] = {1, 0, 0, 0, 0, 0};
+    for (int l = 0; l < f.moduli; l++) {
+        unsigned long long carry = 0;
+        for (unsigned& x : limb) {
+            const unsigned long long s = (unsigned long long)x * (unsigned)crt_modulus(l) + carry;
+            x = (unsigned)s;
+            carry = s >> 32;
+        }
+    }
+    int top = 191;
+    while (top > 0 && !((limb[top / 32] >> (top % 32)) & 1u)) top--;
+    t->pm = 0;
+    for (int i = 0; i < 64; i++) {
+        const int bit = top - i;
+        t->pm = (t->pm << 1) | (bit >= 0 ? (limb[bit / 32] >> (bit % 32)) & 1u : 0u);
+    }
+    if (top >= 64 && ((limb[(top - 64) / 32] >> ((top - 64) % 32)) & 1u) && t->pm != ~0ull) t->pm++;
+    t->pe = top - 63;
+    for (int l = 0; l < f.moduli; l++) {
+        const unsigned p = (unsigned)crt_modulus(l);
+        unsigned rest = 1 % p;
+        for (int k = 0; k < f.moduli; k++)
+            if (k != l) rest = rest * (unsigned)crt_modulus(k) % p;
+        unsigned u = 1;
+        while (rest * u % p != 1 % p) u++;
+        fraction_limbs(u, p, t->v[l]);
+    }
+    t->moduli = f.moduli;
+    t->bits = f.bits;
+}
+
+constexpr int kMaxPanels = 64;
+size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+struct CrtPanels {
+    int64_t rows, cols;  // of a panel pair
+    int64_t ld, ldr;
+    size_t off_a, off_b, off_res, total;
+};
+
+CrtPanels panel_layout(int64_t m, int64_t n, int64_t k, int moduli, int64_t count, int64_t rows, int64_t cols) {
+    CrtPanels c;
+    c.rows = std::min(rows, m);
+    c.cols = std::min(cols, n);
+    c.ld = tc_ld(k);
+    c.ldr = (int64_t)round_up((size_t)c.cols, 16);
+    c.off_a = 256 + round_up((size_t)(count * (m + n)) * sizeof(int), 256);  // 256: alignment of the arena
+    c.off_b = c.off_a + round_up((size_t)(count * moduli * c.rows * c.ld) * 2, 256);
+    c.off_res = c.off_b + round_up((size_t)(count * moduli * c.cols * c.ld) * 2, 256);
+    c.total = c.off_res + round_up((size_t)(count * moduli * c.rows * c.ldr), 256);
+    return c;
+}
+
+// Panels that fit: A's rows once per row panel, B's columns once per row
+// panel and column panel.  The cheapest by the elements split (about 6 ps
+// each and modulus-proportional) and launches.
+bool choose_panels(int64_t m, int64_t n, int64_t k, int moduli, int64_t count, size_t bytes, CrtPanels* best) {
+    double least = 1e300;
+    for (int pa = 1; pa <= kMaxPanels; pa++) {
+        const int64_t rows = (int64_t)round_up((size_t)((m + pa - 1) / pa), BM);
+        if (pa > 1 && rows >= (int64_t)round_up((size_t)((m + pa - 2) / (pa - 1)), BM)) continue;
+        for (int pb = 1; pb <= kMaxPanels; pb++) {
+            const int64_t cols = (int64_t)round_up((size_t)((n + pb - 1) / pb), kCrtBN);
+            const CrtPanels c = panel_layout(m, n, k, moduli, count, rows, cols);
+            if (c.total > bytes) continue;
+            const double na = (double)((m + rows - 1) / rows), nb = (double)((n + cols - 1) / cols);
+            const double cost = na * (double)n * (double)k * (double)count * 6e-12 + na * nb * 15e-6;
+            if (cost < least) {
+                least = cost;
+                *best = c;
+            }
+            break;  // fewer columns only cost more
+        }
+    }
+    return least < 1e300;
+}
+
+template <class Src>
+int split_rows(Src src, int row0, int rows, int cols, const int* ex, int64_t exs, const CrtFormat& f, uint16_t* dst,
+               int64_t ld, int count, cudaStream_t s) {
+    const dim3 g = rows_grid((int64_t)rows * ((cols + 3) / 4), count);
+    if (f.bits <= 4 * kPiece - 1)
+        crt_rows_kernel<Src, 4><<<g, 256, 0, s>>>(src, row0, rows, cols, ex, exs, f.bits, f.moduli, dst, ld);
+    else
+        crt_rows_kernel<Src, 5><<<g, 256, 0, s>>>(src, row0, rows, cols, ex, exs, f.bits, f.moduli, dst, ld);
+    SPIN_CUDA_TRY(cudaGetLastError());
+    return SPIN_OK;
+}
+
+template <class Src>
+int split_cols(Src src, int col0, int rows, int cols, const int* ex, int64_t exs, const CrtFormat& f, uint16_t* dst,
+               int64_t ld, int count, cudaStream_t s) {
+    const dim3 g((unsigned)((cols + 31) / 32), (unsigned)((rows + kTileK - 1) / kTileK), (unsigned)count);
+    if (f.bits <= 4 * kPiece - 1)
+        crt_cols_kernel<Src, 4><<<g, 256, 0, s>>>(src, col0, rows, cols, ex, exs, f.bits, f.moduli, dst, ld);
+    else
+        crt_cols_kernel<Src, 5><<<g, 256, 0, s>>>(src, col0, rows, cols, ex, exs, f.bits, f.moduli, dst, ld);
+    SPIN_CUDA_TRY(cudaGetLastError());
+    return SPIN_OK;
+}
+
+template <class Src>
+int crt_run(const CrtProduct& p, Src sa, Src sb, const CrtFormat& f, const CrtPanels& c, unsigned char* arena,
+            cudaStream_t s, int* launches) {
+    const int count = p.count > 0 ? p.count : 1;
+    const int m = (int)p.m, n = (int)p.n, k = (int)p.k;
+    const int64_t sss = p.count > 0 ? 1 : 0;
+    int* ea = p.a_exps_out != nullptr ? p.a_exps_out : (int*)arena;
+    int* eb = (int*)arena + (size_t)count * (size_t)m;
+    uint16_t* pa = (uint16_t*)(arena + c.off_a - 256);
+    uint16_t* pb = (uint16_t*)(arena + c.off_b - 256);
+    uint8_t* res = arena + c.off_res - 256;
+    int nl = 0;
+    int rc = SPIN_OK;
+    if (p.a_exps == nullptr) {
+        if ((rc = operand_exponents(sa, m, k, false, ea, p.sumsq_a, sss, count, s))) return rc;
+        nl += 1;
+    } else {
+        ea = const_cast<int*>(p.a_exps);
+    }
+    if ((rc = operand_exponents(sb, k, n, true, eb, p.sumsq_b, sss, count, s))) return rc;
+    nl += 3;
+
+    CrtTable table;
+    crt_table(f, &table);
+    TcGemmParams q = {};
+    q.M = m;
+    q.N = n;
+    q.K = k;
+    q.alpha = p.alpha;
+    q.beta = p.beta;
+    q.C = p.C;
+    q.ldc = p.ldc;
+    q.D = p.D;
+    q.ldd = p.ldd;
+    q.row_exp = ea;
+    q.col_exp = eb;
+    q.add_identity = p.add_identity;
+    q.sumsq = p.sumsq_d;
+    q.active = p.active;
+    q.sum_order = p.valid;
+    if (p.count > 0) {
+        q.batch = p.count;
+        q.c_base = p.beta != 0.0 ? p.Cv.base : nullptr;
+        q.c_lds = p.Cv.lds;
+        q.c_ld = p.Cv.ld;
+        q.c_r0 = p.Cv.r0;
+        q.c_c0 = p.Cv.c0;
+        q.d_base = const_cast<double* const*>(p.Dv.base);
+        q.d_lds = p.Dv.lds;
+        q.d_ld = p.Dv.ld;
+        q.d_r0 = p.Dv.r0;
+        q.d_c0 = p.Dv.c0;
+    }
+    CrtGemmParams g = {};
+    g.K = k;
+    g.moduli = f.moduli;
+    g.count = count;
+    g.res = res;
+    g.active = p.active;
+    g.err = p.err;
+    for (int l = 0; l < f.moduli; l++) {
+        g.p[l] = (unsigned)crt_modulus(l);
+        g.magic[l] = (unsigned)((1ull << 32) / g.p[l]);
+        g.shift[l] = 0x80000000u / g.p[l] * g.p[l];
+    }
+    constexpr size_t smem = Cfg<kCrtBN, 1>::SMEM_BYTES;
+    static PerDeviceOnce attrs;
+    rc = attrs.run([&]() -> int {
+        SPIN_CUDA_TRY(cudaFuncSetAttribute(crt_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        return SPIN_OK;
+    });
+    if (rc) return rc;
+    const int sms = sm_count();
+    for (int row0 = 0; row0 < m; row0 += (int)c.rows) {
+        const int rows = std::min((int)c.rows, m - row0);
+        if ((rc = split_rows(sa, row0, rows, k, ea, m, f, pa, c.ld, count, s))) return rc;
+        CUtensorMap ta;
+        if ((rc = make_map(&ta, pa, k, (int64_t)count * f.moduli * rows, c.ld, BM))) return rc;
+        nl++;
+        for (int col0 = 0; col0 < n; col0 += (int)c.cols) {
+            const int cols = std::min((int)c.cols, n - col0);
+            if (row0 == 0 || c.cols < n) {  // one column panel: its planes are still there
+                if ((rc = split_cols(sb, col0, k, cols, eb, n, f, pb, c.ld, count, s))) return rc;
+                nl++;
+            }
+            CUtensorMap tb;
+            if ((rc = make_map(&tb, pb, k, (int64_t)count * f.moduli * cols, c.ld, kCrtBN))) return rc;
+            g.M = rows;
+            g.N = cols;
+            g.ldr = (int64_t)round_up((size_t)cols, 16);
+            const int64_t items =
+                (int64_t)((rows + BM - 1) / BM) * ((cols + kCrtBN - 1) / kCrtBN) * f.moduli * count;
+            crt_gemm_kernel<<<(unsigned)std::min<int64_t>(items, sms), Epi<kCrtEpiWarps>::THREADS, smem, s>>>(ta, tb, g);
+            SPIN_CUDA_TRY(cudaGetLastError());
+            const int64_t total = (int64_t)rows * ((cols + 3) / 4);
+            const int64_t per = std::max<int64_t>(1, (int64_t)sms * 8 / count);
+            const dim3 cg((unsigned)std::min<int64_t>((total + 255) / 256, per), 1, (unsigned)count);
+            crt_combine_kernel<<<cg, 256, 0, s>>>(res, g.ldr, rows, cols, row0, col0, table, q);
+            SPIN_CUDA_TRY(cudaGetLastError());
+            nl += 2;
+        }
+    }
+    if (launches) *launches += nl;
+    return SPIN_OK;
+}
+
+}  // namespace
+
+CrtFormat crt_format(int64_t k, int min_bits) {
+    CrtFormat f{0, 0};
+    if (k < 1 || k > (int64_t)kMaxRuns * kRunK) return f;
+    double log2p = 0.0;
+    for (int l = 0; l < kCrtMaxModuli; l++) {
+        log2p += std::log2((double)crt_modulus(l));
+        // P > 2 k 2^(2 bits); the margin covers the logarithms' rounding
+        const int bits = (int)std::floor((log2p - 1.0 - std::log2((double)k) - 1e-9) / 2.0);
+        if (bits >= min_bits) {
+            f.moduli = l + 1;
+            f.bits = std::min(bits, kCrtMaxBits);
+            return f;
+        }
+    }
+    return f;
+}
+
+size_t crt_full_bytes(int64_t m, int64_t n, int64_t k, int moduli, int count) {
+    return panel_layout(m, n, k, moduli, std::max(count, 1), m, n).total;
+}
+
+size_t crt_min_bytes(int64_t m, int64_t n, int64_t k, int moduli, int count) {
+    const int64_t rows = (int64_t)round_up((size_t)((m + kMaxPanels - 1) / kMaxPanels), BM);
+    const int64_t cols = (int64_t)round_up((size_t)((n + kMaxPanels - 1) / kMaxPanels), kCrtBN);
+    return panel_layout(m, n, k, moduli, std::max(count, 1), rows, cols).total;
+}
+
+int crt_product(const CrtProduct& p, void* arena, size_t bytes, cudaStream_t s, int* launches) {
+    if (p.m <= 0 || p.n <= 0) return SPIN_OK;
+    if (p.count < 0 || p.count > 65535) return SPIN_ERR_INVALID_ARG;
+    const CrtFormat f = crt_format(p.k, p.min_bits);
+    if (f.moduli == 0) return SPIN_ERR_INVALID_ARG;
+    const int64_t count = std::max(p.count, 1);
+    CrtPanels c;
+    if (!choose_panels(p.m, p.n, p.k, f.moduli, count, bytes, &c)) return SPIN_ERR_INVALID_ARG;
+    if (count * f.moduli * std::max(c.rows, c.cols) > INT32_MAX) return SPIN_ERR_INVALID_ARG;  // TMA row coordinate
+    unsigned char* base = (unsigned char*)round_up((size_t)(uintptr_t)arena, 256);
+    if (p.count > 0)
+        return crt_run(p, SrcMany{p.Av, p.active, p.valid}, SrcMany{p.Bv, p.active, p.valid}, f, c, base, s, launches);
+    return crt_run(p, SrcOne{p.A, p.lda, p.active}, SrcOne{p.B, p.ldb, p.active}, f, c, base, s, launches);
+}
+
+}  // namespace spin

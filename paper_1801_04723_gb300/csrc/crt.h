@@ -1,0 +1,72 @@
+// Exact integer products on the BF16 tensor cores by residues (crt.cu).
+#pragma once
+#include <cuda_runtime.h>
+#include <stddef.h>
+#include <stdint.h>
+
+#include "tc_gemm.h"
+
+namespace spin {
+
+constexpr int kCrtMaxModuli = 20;
+constexpr int kCrtMaxBits = 62;
+
+// Moduli and fixed-point bits per operand for an inner dimension k: the
+// fewest moduli whose product exceeds twice the largest |sum| at bits >=
+// min_bits, then every bit that they allow (at most kCrtMaxBits).  0 moduli:
+// none fits.
+struct CrtFormat {
+    int moduli;
+    int bits;
+};
+CrtFormat crt_format(int64_t k, int min_bits);
+
+// Bits that stand in for s 8-bit digit slices (pairs t + u < s): an FP64
+// simulation of the residual product (Householder SPD matrices of condition
+// 1e3 and Gram matrices, n = 512, s = 4, 5, 6) gives the residue form at 8 s
+// - 4 bits 0.32 to 0.44 of the digit form's error, which is mostly that of
+// the pairs it leaves out.
+inline int crt_bits_for_slices(int s) { return 8 * s - 4; }
+
+// One operand's or the whole product's device memory.
+//   exps       one int per row of A / column of B, for all of them
+//   planes     [panel of rows] x moduli BF16 planes, K-major
+//   residues   moduli bytes per output of a panel pair
+// crt_min_bytes: the least arena that crt_product accepts; crt_full_bytes:
+// the arena that holds everything in one panel pair (count problems).
+size_t crt_full_bytes(int64_t m, int64_t n, int64_t k, int moduli, int count = 1);
+size_t crt_min_bytes(int64_t m, int64_t n, int64_t k, int moduli, int count = 1);
+
+// D = beta*C + alpha*(A B) (+ I) for `count` problems (count = 0: one
+// problem given by plain pointers).  Views, sums of squares, active flags
+// and statuses as in TcGemmParams.
+struct CrtProduct {
+    int64_t m, n, k;
+    int min_bits;
+    double alpha, beta;
+    int add_identity;
+    // one problem
+    const double* A;
+    int64_t lda;
+    const double* B;
+    int64_t ldb;
+    const double* C;
+    int64_t ldc;
+    double* D;
+    int64_t ldd;
+    // count problems
+    int count;
+    BatchView Av, Bv, Cv, Dv;
+    const int* active;    // optional, device
+    const int* valid;     // optional, device: sums of squares cover the leading valid[z] x valid[z] block
+    double* sumsq_a;      // optional, device: += sum of squares of A (one entry per problem)
+    double* sumsq_b;
+    double* sumsq_d;
+    const int* a_exps;    // optional, device: row exponents of A from an earlier product with the same A
+    int* a_exps_out;      // optional, device: m ints per problem, where they are kept (else in the arena)
+    int* err;
+};
+// Launches, all on s; *launches (optional) counts them.
+int crt_product(const CrtProduct& p, void* arena, size_t bytes, cudaStream_t s, int* launches = nullptr);
+
+}  // namespace spin

@@ -2,8 +2,9 @@
 // and the two tensor-core product forms (see tc_gemm.cu):
 //
 //   bf16x3   D = beta*C + alpha*(A_hi B_hi + A_hi B_lo + A_lo B_hi)
-//   ozaki(s) D = beta*C + alpha*(A B) (+ I) with s fixed-point digit slices
-//            per operand, pairs (t, u) with t + u < s, exact partial sums.
+//   fp64_class(s)  D = beta*C + alpha*(A B) (+ I) as accurate as s fixed-point
+//            digit slices per operand: by residues (crt.cu) for s >= 4, by
+//            digits (pairs (t, u) with t + u < s, exact partial sums) below.
 //
 // The split planes live in a per-stream scratch arena owned by the caller
 // (struct MixScratch), reused across calls.
@@ -12,6 +13,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "crt.h"
 #include "mixed.h"
 #include "tc_gemm.h"
 
@@ -136,10 +138,6 @@ int split_a_bf16x3(const SplitPlan& sp, const double* A, int64_t lda, int64_t m,
 int split_b_bf16x3(const SplitPlan& sp, const double* B, int64_t ldb, int64_t k, int64_t n, cudaStream_t s) {
     return launch_split_bf16x2(B, ldb, (int)k, (int)n, true, sp.b, sp.ld, s);
 }
-int split_a_ozaki(const SplitPlan& sp, const double* A, int64_t lda, int64_t m, int64_t k, double* sumsq,
-                  cudaStream_t s) {
-    return launch_ozaki_split(A, lda, (int)m, (int)k, false, sp.slices, sp.ea, sp.a, sp.ld, sumsq, s);
-}
 int split_b_ozaki(const SplitPlan& sp, const double* B, int64_t ldb, int64_t k, int64_t n, double* sumsq,
                   cudaStream_t s, const int* active) {
     return launch_ozaki_split(B, ldb, (int)k, (int)n, true, sp.slices, sp.eb, sp.b, sp.ld, sumsq, s, active);
@@ -203,14 +201,13 @@ int product_bf16x6(const SplitPlan& sp, int64_t m, int64_t n, int64_t k, double 
 
 int product_ozaki(const SplitPlan& sp, int64_t m, int64_t n, int64_t k, double alpha, double beta, const double* C,
                   int64_t ldc, double* D, int64_t ldd, int add_identity, double* sumsq, int* err, cudaStream_t s,
-                  const int* active, int pair_slices) {
+                  const int* active) {
     const int slices = sp.slices;
-    if (pair_slices < 1 || pair_slices > slices) pair_slices = slices;
     TcGemmParams p = {};
     p.M = (int)m;
     p.N = (int)n;
     p.K = (int)k;
-    tc_pairs_ozaki(p, pair_slices);
+    tc_pairs_ozaki(p, slices);
     p.alpha = alpha;
     p.beta = beta;
     p.C = C;
@@ -240,29 +237,62 @@ int gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha, const double* A, 
     return product_bf16x3(sp, m, n, k, alpha, beta, C, ldc, D, ldd, err, s);
 }
 
-int gemm_ozaki(int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda, const double* B,
-               int64_t ldb, double beta, const double* C, int64_t ldc, double* D, int64_t ldd, int slices,
-               int add_identity, double* sumsq, double* sumsq_a, double* sumsq_b, void* scratch,
-               size_t scratch_bytes, int* err, cudaStream_t s, const OzakiCachedA* cached_a) {
+int fp64_class_moduli(int64_t k, int slices) {
+    const int n = crt_format(k, crt_bits_for_slices(slices)).moduli;
+    return n > 0 && n < slices * (slices + 1) / 2 ? n : 0;
+}
+
+size_t fp64_class_bytes(int64_t m, int64_t n, int64_t k, int slices) {
+    const int mods = fp64_class_moduli(k, slices);
+    return mods ? crt_full_bytes(m, n, k, mods) : ozaki_scratch_bytes(m, n, k, slices);
+}
+
+double fp64_class_products(int64_t k, int slices) {
+    const int mods = fp64_class_moduli(k, slices);
+    return mods ? mods : slices * (slices + 1) / 2;
+}
+
+int gemm_fp64_class(int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda, const double* B,
+                    int64_t ldb, double beta, const double* C, int64_t ldc, double* D, int64_t ldd, int slices,
+                    int add_identity, const Fp64ClassExtra& x, void* scratch, size_t scratch_bytes, int* err,
+                    cudaStream_t s) {
     if (m <= 0 || n <= 0) return SPIN_OK;
     if (k <= 0) return SPIN_ERR_INVALID_ARG;
+    const int mods = fp64_class_moduli(k, slices);
+    if (mods && scratch_bytes >= crt_min_bytes(m, n, k, mods)) {
+        CrtProduct p = {};
+        p.m = m;
+        p.n = n;
+        p.k = k;
+        p.min_bits = crt_bits_for_slices(slices);
+        p.alpha = alpha;
+        p.beta = beta;
+        p.add_identity = add_identity;
+        p.A = A;
+        p.lda = lda;
+        p.B = B;
+        p.ldb = ldb;
+        p.C = C;
+        p.ldc = ldc;
+        p.D = D;
+        p.ldd = ldd;
+        p.active = x.active;
+        p.sumsq_a = x.sumsq_a;
+        p.sumsq_b = x.sumsq_b;
+        p.sumsq_d = x.sumsq_d;
+        p.a_exps = x.a_known ? x.a_exps : nullptr;
+        p.a_exps_out = x.a_exps;
+        p.err = err;
+        return crt_product(p, scratch, scratch_bytes, s);
+    }
     SplitPlan sp;
     int rc = plan_ozaki(m, n, k, slices, scratch, scratch_bytes, &sp);
     if (rc) return rc;
-    if (cached_a != nullptr) {
-        sp.a = cached_a->planes;
-        sp.ea = cached_a->exps;
-    } else if ((rc = split_a_ozaki(sp, A, lda, m, k, sumsq_a, s))) {
+    if ((rc = launch_ozaki_split(A, lda, (int)m, (int)k, false, slices, sp.ea, sp.a, sp.ld,
+                                 x.a_known ? nullptr : x.sumsq_a, s, x.active)))
         return rc;
-    }
-    if ((rc = split_b_ozaki(sp, B, ldb, k, n, sumsq_b, s))) return rc;
-    return product_ozaki(sp, m, n, k, alpha, beta, C, ldc, D, ldd, add_identity, sumsq, err, s);
-}
-
-int ozaki_split_a(const double* A, int64_t lda, int64_t m, int64_t k, int slices, OzakiCachedA* out,
-                  double* sumsq, cudaStream_t s, const int* active) {
-    const int64_t ld = tc_ld(k);
-    return launch_ozaki_split(A, lda, (int)m, (int)k, false, slices, out->exps, out->planes, ld, sumsq, s, active);
+    if ((rc = split_b_ozaki(sp, B, ldb, k, n, x.sumsq_b, s, x.active))) return rc;
+    return product_ozaki(sp, m, n, k, alpha, beta, C, ldc, D, ldd, add_identity, x.sumsq_d, err, s, x.active);
 }
 
 }  // namespace spin
@@ -324,8 +354,14 @@ extern "C" int spin_gemm_ozaki(int64_t m, int64_t n, int64_t k, double alpha, co
     std::lock_guard<std::mutex> lk(g_mix_mu);
     int rc = ensure_test_err();
     if (rc) return rc;
-    rc = g_test_scratch.reserve(ozaki_scratch_bytes(m, n, k, slices));
+    // everything in one panel where the device has the memory, else in the
+    // panels that fit the digit form's arena
+    const size_t need = ozaki_scratch_bytes(m, n, k, slices);
+    rc = g_test_scratch.reserve(std::max(need, std::min(fp64_class_bytes(m, n, k, slices), kFp64ClassArena)));
+    if (rc == SPIN_ERR_OOM) rc = g_test_scratch.reserve(need);
     if (rc) return rc;
-    return gemm_ozaki(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, slices, add_identity, sumsq_dev, nullptr,
-                      nullptr, g_test_scratch.base, g_test_scratch.cap, g_test_err, (cudaStream_t)stream, nullptr);
+    Fp64ClassExtra x;
+    x.sumsq_d = sumsq_dev;
+    return gemm_fp64_class(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, slices, add_identity, x,
+                           g_test_scratch.base, g_test_scratch.cap, g_test_err, (cudaStream_t)stream);
 }

@@ -44,13 +44,6 @@ struct MixScratch {
     int reserve(size_t bytes);
 };
 
-// Digit planes and row exponents of an A operand split once and reused
-// (the refinement multiplies by the same A every iteration).
-struct OzakiCachedA {
-    uint16_t* planes;
-    int* exps;
-};
-
 size_t bf16x3_scratch_bytes(int64_t m, int64_t n, int64_t k);
 size_t bf16x6_scratch_bytes(int64_t m, int64_t n, int64_t k);
 size_t ozaki_scratch_bytes(int64_t m, int64_t n, int64_t k, int slices);
@@ -59,10 +52,32 @@ int gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha, const double* A, 
                 int64_t ldb, double beta, const double* C, int64_t ldc, double* D, int64_t ldd, void* scratch,
                 size_t scratch_bytes, int* err, cudaStream_t s);
 
-int gemm_ozaki(int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda, const double* B,
-               int64_t ldb, double beta, const double* C, int64_t ldc, double* D, int64_t ldd, int slices,
-               int add_identity, double* sumsq, double* sumsq_a, double* sumsq_b, void* scratch,
-               size_t scratch_bytes, int* err, cudaStream_t s, const OzakiCachedA* cached_a);
+// FP64-class product (the Schur complements, the refinement residual, the
+// level products of SPIN_MIXED_DIGITS): as accurate as s digit slices, by
+// residues (crt.cu) where those take fewer tensor-core products -- s >= 4: at
+// n = 2048, 9 instead of 10 for s = 4, 11 instead of 15, 13 instead of 21 and
+// 15 instead of 28 for s = 7 (n = 2048: 0.79 -> 0.40 ms at s = 7; the n = 16384
+// mixed inversion 380 -> 273 ms) -- else by digits (s <= 3, and k beyond 96
+// runs of 1024).
+int fp64_class_moduli(int64_t k, int slices);       // 0: digits
+size_t fp64_class_bytes(int64_t m, int64_t n, int64_t k, int slices);  // an arena that needs no panels
+double fp64_class_products(int64_t k, int slices);  // tensor-core products of m x n x k
+// The residue form runs in panels in any arena of at least the digit form's
+// size; library-owned arenas are made larger, up to this, to save the panels'
+// repeated splits and launches at small orders.
+constexpr size_t kFp64ClassArena = (size_t)2 << 30;
+struct Fp64ClassExtra {
+    const int* active = nullptr;  // optional, device int: runs only while nonzero
+    double* sumsq_a = nullptr;    // optional, device: += sums of squares of A, B and D
+    double* sumsq_b = nullptr;
+    double* sumsq_d = nullptr;
+    int* a_exps = nullptr;        // optional, device: m row exponents of A, kept between products
+    bool a_known = false;         // a_exps and *sumsq_a are there from an earlier product with this A
+};
+int gemm_fp64_class(int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda, const double* B,
+                    int64_t ldb, double beta, const double* C, int64_t ldc, double* D, int64_t ldd, int slices,
+                    int add_identity, const Fp64ClassExtra& x, void* scratch, size_t scratch_bytes, int* err,
+                    cudaStream_t s);
 
 // Split-then-multiply in two halves so callers can time them separately.
 struct SplitPlan {
@@ -78,8 +93,6 @@ int plan_ozaki(int64_t m, int64_t n, int64_t k, int slices, void* scratch, size_
 int split_a_bf16x3(const SplitPlan& sp, const double* A, int64_t lda, int64_t m, int64_t k, cudaStream_t s);
 int split_b_bf16x3(const SplitPlan& sp, const double* B, int64_t ldb, int64_t k, int64_t n, cudaStream_t s);
 // active (optional, device int): the split / product runs only while *active != 0.
-int split_a_ozaki(const SplitPlan& sp, const double* A, int64_t lda, int64_t m, int64_t k, double* sumsq,
-                  cudaStream_t s);
 int split_b_ozaki(const SplitPlan& sp, const double* B, int64_t ldb, int64_t k, int64_t n, double* sumsq,
                   cudaStream_t s, const int* active = nullptr);
 int product_bf16x3(const SplitPlan& sp, int64_t m, int64_t n, int64_t k, double alpha, double beta, const double* C,
@@ -92,14 +105,9 @@ int split_b_bf16x6(const SplitPlan& sp, const double* B, int64_t ldb, int64_t k,
                    const int* active = nullptr);
 int product_bf16x6(const SplitPlan& sp, int64_t m, int64_t n, int64_t k, double alpha, double beta, const double* C,
                    int64_t ldc, double* D, int64_t ldd, int* err, cudaStream_t s, const int* active = nullptr);
-// pair_slices (0: sp.slices): the pairs t + u < pair_slices of the first
-// pair_slices planes of each operand's stack.
 int product_ozaki(const SplitPlan& sp, int64_t m, int64_t n, int64_t k, double alpha, double beta, const double* C,
                   int64_t ldc, double* D, int64_t ldd, int add_identity, double* sumsq, int* err, cudaStream_t s,
-                  const int* active = nullptr, int pair_slices = 0);
-
-int ozaki_split_a(const double* A, int64_t lda, int64_t m, int64_t k, int slices, OzakiCachedA* out,
-                  double* sumsq, cudaStream_t s, const int* active = nullptr);
+                  const int* active = nullptr);
 
 // Device-side Newton-Schulz control (refine.cu) for `count` matrices whose
 // info records (INFO_WORDS int32 each) start at `records`:

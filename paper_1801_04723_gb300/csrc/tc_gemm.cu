@@ -44,24 +44,17 @@
 // MMAs, frees TMEM and returns.  tc_gemm_pair_kernel is the exact mode on
 // CTA pairs (tcgen05 cta_group::2, 256 x 128 tiles), selected by
 // SPIN_TC_PAIR=1.
-#include <cuda_bf16.h>
-#include <cudaTypedefs.h>
-
 #include <stdlib.h>
 
 #include <algorithm>
 
 #include "common.cuh"
 #include "tc_gemm.h"
-#include "tc_ptx.cuh"
+#include "tc_pipe.cuh"
 
 namespace spin {
 namespace {
 
-using namespace tc;
-
-constexpr int BM = 128, BK = 64;
-constexpr int GROUP_M = 8;  // row blocks per rasterisation band
 #ifndef SPIN_EXACT_BN
 #define SPIN_EXACT_BN 128
 #define SPIN_EXACT_EPI_WARPS 8
@@ -91,7 +84,6 @@ constexpr int kExactEpiWarps = SPIN_EXACT_EPI_WARPS;  // exact-mode epilogue war
 // power cap without raising the work per clock).
 constexpr int64_t kExactWideMinTiles = SPIN_EXACT_WIDE_MIN_TILES;
 constexpr int kExactWideMaxK = 16384;
-constexpr uint32_t A_TILE_BYTES = BM * BK * 2;  // 16 KB
 // 64-wide k-blocks per pipeline stage.  The MMA issuer's fixed cost per
 // stage (barrier wait, commit) is spread over 4 * KSUB MMAs: two k-blocks
 // for the 128-wide exact tiles (measured 1140 vs 970 TFLOP/s at n = 8192),
@@ -100,28 +92,6 @@ constexpr uint32_t A_TILE_BYTES = BM * BK * 2;  // 16 KB
 constexpr int KSUB_EXACT = SPIN_KSUB_EXACT;
 constexpr int KSUB_FLOAT = SPIN_KSUB_FLOAT;
 constexpr int FLUSH_LIMIT = 96;  // exact runs summed in int32 before an FP64 flush (96 * 2^24 < 2^31)
-constexpr uint64_t WAIT_LIMIT_NS = 10ull * 1000 * 1000 * 1000;
-
-template <int BN, int KS>
-struct Cfg {
-    static constexpr uint32_t B_TILE_BYTES = BN * BK * 2;
-    static constexpr uint32_t STAGE_BYTES = KS * (A_TILE_BYTES + B_TILE_BYTES);
-    static constexpr int STAGES = (196608 / STAGE_BYTES) > 6 ? 6 : (196608 / STAGE_BYTES);  // ~192 KB ring
-    static constexpr uint32_t TMEM_COLS = 2 * BN <= 256 ? 256 : 512;  // power of two >= 2 BN
-    static constexpr size_t SMEM_BYTES = 1024 /*align slack*/ + STAGES * STAGE_BYTES + 256 /*barriers etc.*/;
-};
-constexpr int STAGES_MAX = 8;
-
-struct SmemCtl {
-    uint64_t full[STAGES_MAX];
-    uint64_t empty[STAGES_MAX];
-    uint64_t tfull[2];
-    uint64_t tempty[2];
-    uint64_t final_bar;
-    uint32_t tmem_base;
-    int abort;
-    int issued;  // pair kernel: stage uses this CTA's producer issued
-};
 
 // x * 2^E exactly, for |x| < 2^31, from the bits: the leading one of |x|
 // becomes the implicit bit and the rest the fraction.  Integer operations
@@ -139,25 +109,6 @@ __device__ __forceinline__ double scaled_int(int x, int E) {
     return __longlong_as_double((long long)bits);
 }
 
-static_assert(sizeof(SmemCtl) <= 256, "control block");
-
-// Row grow of D (and of C, or null) for problem z.
-__device__ __forceinline__ double* out_row(const TcGemmParams& p, int z, int grow) {
-    if (!p.batch) return p.D + (int64_t)grow * p.ldd;
-    const int64_t ld = p.d_lds ? p.d_lds[z] : p.d_ld;
-    return p.d_base[z] + (p.d_r0 + grow) * ld + p.d_c0;
-}
-__device__ __forceinline__ const double* in_row(const TcGemmParams& p, int z, int grow) {
-    if (!p.batch) return p.C ? p.C + (int64_t)grow * p.ldc : nullptr;
-    if (!p.c_base) return nullptr;
-    const int64_t ld = p.c_lds ? p.c_lds[z] : p.c_ld;
-    return p.c_base[z] + (p.c_r0 + grow) * ld + p.c_c0;
-}
-
-__device__ __forceinline__ void raise_timeout(SmemCtl* ctl, int* err) {
-    ctl->abort = 1;
-    if (err) atomicCAS(err, 0, SPIN_ERR_TIMEOUT);
-}
 // CTA pair: stop both CTAs (the peer's waits read its own abort flag).
 __device__ __forceinline__ void raise_pair_error(SmemCtl* ctl, int* err, int code) {
     ctl->abort = 1;
@@ -167,14 +118,6 @@ __device__ __forceinline__ void raise_pair_error(SmemCtl* ctl, int* err, int cod
 __device__ __forceinline__ void raise_timeout_pair(SmemCtl* ctl, int* err) {
     raise_pair_error(ctl, err, SPIN_ERR_TIMEOUT);
 }
-
-template <int EPI_WARPS>
-struct Epi {
-    static constexpr int THREADS = 64 + 32 * EPI_WARPS;
-    // registers are granted per group of four warps: budget for the rounded-up count
-    static constexpr int ALLOC_THREADS = (THREADS + 127) / 128 * 128;
-    static constexpr int MAXREG = (65536 / ALLOC_THREADS) / 8 * 8 > 255 ? 248 : (65536 / ALLOC_THREADS) / 8 * 8;
-};
 
 // Exact-mode epilogue of one warp (HALF columns of one TMEM lane quarter):
 // drains every exact run from TMEM into int32 sums and, at the end of each
@@ -822,10 +765,6 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
 // ------------------------------------------------------------ splitting --
 
-__device__ __forceinline__ uint16_t bf16_bits(float f) {
-    return __bfloat16_as_ushort(__float2bfloat16_rn(f));
-}
-
 // hi = bf16(x), lo = bf16(x - hi), both computed from xf = fp32(x): one
 // FP64 operation per element (GB300's FP64 rate would otherwise bound this
 // memory-bound pass); xf differs from x by 2^-24 relative, far below what
@@ -847,30 +786,6 @@ __device__ __forceinline__ void split3(double a, uint16_t& hi, uint16_t& mid, ui
     mid = __bfloat16_as_ushort(m);
     lo = bf16_bits(r1 - __bfloat162float(m));  // exact in FP32
 }
-
-// Operand source of a split: one FP64 view, or problem z's view of a batch.
-// act (optional): problem z is split only while act[z] != 0.  nv
-// (optional): the sum of squares of problem z covers only its leading
-// nv[z] x nv[z] block (a matrix padded with the identity).
-struct SrcOne {
-    const double* p;
-    int64_t ld;
-    const int* act;
-    __device__ __forceinline__ const double* row(int, int r) const { return p + (int64_t)r * ld; }
-    __device__ __forceinline__ bool on(int) const { return act == nullptr || act[0] != 0; }
-    __device__ __forceinline__ int valid(int) const { return 0x7fffffff; }
-};
-struct SrcMany {
-    BatchView v;
-    const int* act;
-    const int* nv;
-    __device__ __forceinline__ const double* row(int z, int r) const {
-        const int64_t l = v.ld_of(z);
-        return v.base[z] + (v.r0 + r) * l + v.c0;
-    }
-    __device__ __forceinline__ bool on(int z) const { return act == nullptr || act[z] != 0; }
-    __device__ __forceinline__ int valid(int z) const { return nv ? nv[z] : 0x7fffffff; }
-};
 
 // Every split kernel handles problem z = blockIdx.z: its planes start at
 // dst + z * dzs, its exponents at ex + z * exs, its sum of squares at
@@ -964,94 +879,6 @@ __global__ void split_bf16x2_cols_kernel(Src src, int rows, int cols, uint16_t* 
     }
 }
 
-// Biased exponent field of x (0 for zero and subnormals).  The exponent e
-// with max|x| < 2^e (frexp convention) of a row is max(field) - 1022: the
-// largest magnitude has the largest field.  Integer work only.
-__device__ __forceinline__ int exp_field(double x) {
-    return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7FF;
-}
-
-// Per-row max exponent of an FP64 matrix (one warp per row) and optional
-// sum of squares of all entries.
-template <class Src>
-__global__ void row_exp_kernel(Src src, int rows, int cols, int* __restrict__ ex, int64_t exs, double* sumsq,
-                               int64_t sss) {
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    const int warps = blockDim.x >> 5;
-    const int r = blockIdx.x * warps + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (r >= rows) return;
-    const double* sr = src.row(z, r);
-    const int nv = src.valid(z);
-    const bool sum_row = sumsq != nullptr && r < nv;
-    int m = 0;
-    double ss = 0.0;
-    for (int c = lane; c < cols; c += 32) {
-        const double v = sr[c];
-        m = max(m, exp_field(v));
-        if (sum_row && c < nv) ss = fma(v, v, ss);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        m = max(m, __shfl_down_sync(0xffffffffu, m, off));
-        ss += __shfl_down_sync(0xffffffffu, ss, off);
-    }
-    if (lane == 0) {
-        ex[z * exs + r] = m - 1022;
-        if (sumsq) atomicAdd(sumsq + z * sss, ss);
-    }
-}
-
-// Per-column max exponent: atomicMax of exponent fields on a zero start,
-// converted to the frexp convention by col_exp_finish_kernel.
-template <class Src>
-__global__ void col_exp_kernel(Src src, int rows, int cols, int rows_per_block, int* __restrict__ ex, int64_t exs,
-                               double* sumsq, int64_t sss) {
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r0 = blockIdx.y * rows_per_block;
-    const int r1 = min(rows, r0 + rows_per_block);
-    int m = 0;
-    const int nv = src.valid(z);
-    const bool sum_col = sumsq != nullptr && c < nv;
-    double ss4[4] = {0.0, 0.0, 0.0, 0.0};  // four FMA chains: a dependent FP64 FMA takes 64+ cycles here
-    if (c < cols) {
-        int r = r0;
-        for (; r + 3 < r1; r += 4) {
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const double v = src.row(z, r + u)[c];
-                m = max(m, exp_field(v));
-                if (sum_col && r + u < nv) ss4[u] = fma(v, v, ss4[u]);
-            }
-        }
-        for (; r < r1; r++) {
-            const double v = src.row(z, r)[c];
-            m = max(m, exp_field(v));
-            if (sum_col && r < nv) ss4[0] = fma(v, v, ss4[0]);
-        }
-    }
-    double ss = (ss4[0] + ss4[1]) + (ss4[2] + ss4[3]);
-    if (c < cols && m > 0) atomicMax(&ex[z * exs + c], m);
-    if (sumsq) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) ss += __shfl_down_sync(0xffffffffu, ss, off);
-        if ((threadIdx.x & 31) == 0 && ss != 0.0) atomicAdd(sumsq + z * sss, ss);
-    }
-}
-
-__global__ void col_exp_finish_kernel(int* ex, int64_t n) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) ex[i] -= 1022;
-}
-
-__global__ void fill_int_kernel(int* p, int64_t n, int v) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
-}
-
 // Fixed-point digits of x relative to 2^e (|x| < 2^e): with t = x 2^(7-e)
 // (|t| < 128), N = round(|t| 2^(8(s-1))) is an integer below 2^(8s-1);
 // its balanced base-256 digits (low digits in [-128, 127], the top one in
@@ -1137,35 +964,6 @@ __global__ void ozaki_cols_kernel(Src src, int rows, int cols, const int* __rest
     }
 }
 
-// ----------------------------------------------------------- tensor maps --
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (fn == nullptr) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
-int make_map(CUtensorMap* m, const uint16_t* base, int64_t inner, int64_t outer, int64_t ld_elems, uint32_t box_rows) {
-    auto fn = encode_fn();
-    if (fn == nullptr) return SPIN_ERR_CUDA;
-    if (((uintptr_t)base & 15u) != 0 || (ld_elems * 2) % 16 != 0) return SPIN_ERR_INVALID_ARG;
-    cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
-    cuuint64_t strides[1] = {(cuuint64_t)(ld_elems * 2)};
-    cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
-    cuuint32_t es[2] = {1, 1};
-    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)base, dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? SPIN_OK : SPIN_ERR_CUDA;
-}
-
 // Float-mode products (bf16x3, bf16x6) run on persistent CTAs, one per SM
 // looping over the tiles: a float tile drains its one accumulator after its
 // last MMA, which the next tile's MMAs now overlap (n = 8192 bf16x3: 2.51
@@ -1188,15 +986,6 @@ int persistent_tiles_mode() {
 bool use_persistent_tiles(bool exact) {
     const int m = persistent_tiles_mode();
     return m == 2 || (m == 1 && !exact);
-}
-
-int sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return 152;
-    }
-    return n > 0 ? n : 152;
 }
 
 template <int BN, bool EXACT, int EPI_WARPS>
@@ -1323,13 +1112,6 @@ int launch_tc_gemm(const TcOperand& a, const TcOperand& b, const TcGemmParams& p
 
 namespace {
 
-// Grid of a row-wise split: blocks per problem so that the whole launch has
-// about 16 blocks per SM.
-dim3 rows_grid(int64_t total, int count) {
-    const int64_t per = std::max<int64_t>(1, (152 * 16) / std::max(1, count));
-    return dim3((unsigned)std::min<int64_t>((total + 255) / 256, per), 1, (unsigned)count);
-}
-
 template <class Src>
 int split_planes(Src src, int rows, int cols, bool transpose, int planes, uint16_t* dst, int64_t ldd, int count,
                  cudaStream_t s) {
@@ -1358,23 +1140,14 @@ int split_digits(Src src, int rows, int cols, bool transpose, int nslices, int* 
                  double* sumsq, int64_t sss, int count, cudaStream_t s) {
     if (rows <= 0 || cols <= 0 || count <= 0) return SPIN_OK;
     if (nslices < 1 || nslices > kMaxSlices) return SPIN_ERR_INVALID_ARG;
+    const int rc = operand_exponents(src, rows, cols, transpose, ex, sumsq, sss, count, s);
+    if (rc) return rc;
     if (!transpose) {
         const int64_t plane = (int64_t)rows * ldd, dzs = nslices * plane;
-        row_exp_kernel<Src><<<dim3((unsigned)((rows + 7) / 8), 1, (unsigned)count), 256, 0, s>>>(
-            src, rows, cols, ex, rows, sumsq, sss);
         ozaki_rows_kernel<Src><<<rows_grid((int64_t)rows * cols, count), 256, 0, s>>>(src, rows, cols, ex, rows,
                                                                                       nslices, dst, ldd, plane, dzs);
     } else {
-        const int64_t plane = (int64_t)cols * ldd, dzs = nslices * plane, nex = (int64_t)cols * count;
-        fill_int_kernel<<<(unsigned)((nex + 255) / 256), 256, 0, s>>>(ex, nex, 0);
-        // rows per block: enough blocks to cover the SMs at small orders,
-        // at most 256 (fewer atomics at large ones)
-        const int64_t col_blocks = (int64_t)((cols + 255) / 256) * count;
-        int rpb = (int)std::min<int64_t>(256, std::max<int64_t>(16, (int64_t)rows * col_blocks / 608));
-        rpb = (rpb + 7) & ~7;
-        const dim3 g1((unsigned)((cols + 255) / 256), (unsigned)((rows + rpb - 1) / rpb), (unsigned)count);
-        col_exp_kernel<Src><<<g1, 256, 0, s>>>(src, rows, cols, rpb, ex, cols, sumsq, sss);
-        col_exp_finish_kernel<<<(unsigned)((nex + 255) / 256), 256, 0, s>>>(ex, nex);
+        const int64_t plane = (int64_t)cols * ldd, dzs = nslices * plane;
         const dim3 g((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32), (unsigned)count);
         ozaki_cols_kernel<Src><<<g, dim3(32, 8), 0, s>>>(src, rows, cols, ex, cols, nslices, dst, ldd, plane, dzs);
     }
