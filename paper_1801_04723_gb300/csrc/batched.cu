@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "crt.h"
 #include "mixed.h"
 #include "persistent.h"
 #include "tc_gemm.h"
@@ -392,8 +393,19 @@ size_t mixed_cache_per(int64_t n, int sr) {
     return align256((size_t)sr * (size_t)n * (size_t)tc_ld(n) * 2 + (size_t)n * 4 + 512);
 }
 
+// Whether a bucket's residuals run by residues (crt.cu).  Up to order 128 a
+// residual is one mostly empty 128 x 256 tile per modulus, and the digit
+// form's 21 pairs, packed into a few exact runs, are cheaper: 256 matrices of
+// order 96 / 128 take 1.58 / 2.65 ms with digits, 1.74 / 2.87 ms with
+// residues; 192 of order 160 3.62 against 2.99 ms, 32 of order 1024 14.3
+// against 13.1 ms.  The Schur complements (28 pairs, 15 moduli) are cheaper by
+// residues at every order that reaches the tensor cores (128 matrices of
+// order 192, Schur order 32 at the second level: 2.84 -> 2.64 ms).
+bool residual_by_residues(int64_t n, int slices) { return n > 128 && fp64_class_moduli(n, slices) > 0; }
+
 struct BMix {
-    unsigned char* scratch;  // bucket's split planes: count * scratch_per bytes
+    unsigned char* scratch;  // bucket's split planes
+    size_t scratch_bytes;
     int count;
     int fp64_levels;
     int* err;
@@ -422,6 +434,22 @@ int bproduct(BMix& x, int depth, bool schur, int64_t m, int64_t n, int64_t k, do
     }
     const int64_t ld = tc_ld(k);
     const int64_t cnt = x.count;
+    if (schur && depth < x.fp64_levels) {
+        CrtProduct q = {};
+        q.m = m;
+        q.n = n;
+        q.k = k;
+        q.min_bits = crt_bits_for_slices(kSchurSlices);
+        q.alpha = alpha;
+        q.beta = beta;
+        q.count = x.count;
+        q.Av = A;
+        q.Bv = B;
+        q.Cv = C;
+        q.Dv = D;
+        q.err = x.err;
+        return crt_product(q, x.scratch, x.scratch_bytes, x.s, x.kernels);
+    }
     TcGemmParams p = {};
     p.M = (int)m;
     p.N = (int)n;
@@ -441,19 +469,6 @@ int bproduct(BMix& x, int depth, bool schur, int64_t m, int64_t n, int64_t k, do
     p.d_r0 = D.r0;
     p.d_c0 = D.c0;
     uint16_t* pa = (uint16_t*)x.scratch;
-    if (schur && depth < x.fp64_levels) {
-        const int sl = kSchurSlices;
-        uint16_t* pb = pa + cnt * sl * m * ld;
-        int* ea = after<int>(pb, (size_t)cnt * sl * n * ld * 2);
-        int* eb = ea + cnt * m;
-        *x.kernels += 2 * 3 + 1;
-        BRET(launch_ozaki_split_batched(A, (int)m, (int)k, false, sl, ea, pa, ld, nullptr, x.count, x.s));
-        BRET(launch_ozaki_split_batched(B, (int)k, (int)n, true, sl, eb, pb, ld, nullptr, x.count, x.s));
-        tc_pairs_ozaki(p, sl);
-        p.row_exp = ea;
-        p.col_exp = eb;
-        return launch_tc_gemm(TcOperand{pa, (int)m, sl, ld}, TcOperand{pb, (int)n, sl, ld}, p, x.s);
-    }
     uint16_t* pb = pa + cnt * 2 * m * ld;
     *x.kernels += 3;
     BRET(launch_split_planes_batched(A, (int)m, (int)k, false, 2, pa, ld, x.count, x.s));
@@ -511,7 +526,9 @@ int bucket_refine(BatchPlan& p, const Bucket& b, cudaStream_t s) {
     int32_t* rec = p.records + (int64_t)b.first * INFO_WORDS;
     const int64_t ld = tc_ld(b.n);
     unsigned char* scratch = p.arena + b.arena_offset;
+    const size_t scratch_bytes = (size_t)b.count * (b.scratch_per + b.cache_per);
     unsigned char* cache = scratch + (size_t)b.count * b.scratch_per;
+    const bool residues = residual_by_residues(b.n, b.s0) && residual_by_residues(b.n, sr);
     uint16_t* aplanes = (uint16_t*)cache;
     int* aex = after<int>(aplanes, (size_t)b.count * sr * b.n * ld * 2);
     uint16_t* xplanes = (uint16_t*)scratch;
@@ -520,34 +537,56 @@ int bucket_refine(BatchPlan& p, const Bucket& b, cudaStream_t s) {
     uint16_t* rp = xp + (int64_t)b.count * 3 * b.n * ld;
     BRET(launch_refine_init(rec, b.count, act, p.rel + b.first, p.iters + b.first, s));
     SPIN_CUDA_TRY(cudaMemsetAsync(nA, 0, b.count * sizeof(double), s));
-    p.kernels += 3;
+    p.kernels += residues ? 1 : 3;
     const int* nv = p.nvalid ? p.nvalid + b.first : nullptr;  // norms over the unpadded block
-    BRET(launch_ozaki_split_batched(Av, (int)b.n, (int)b.n, false, sr, aex, aplanes, ld, nA, b.count, s, act, nv));
+    if (!residues)
+        BRET(launch_ozaki_split_batched(Av, (int)b.n, (int)b.n, false, sr, aex, aplanes, ld, nA, b.count, s, act, nv));
     for (int it = 0; it <= p.max_refine; it++) {
         SPIN_CUDA_TRY(cudaMemsetAsync(nX, 0, b.count * sizeof(double), s));
         SPIN_CUDA_TRY(cudaMemsetAsync(nR, 0, b.count * sizeof(double), s));
-        BRET(launch_ozaki_split_batched(Xv, (int)b.n, (int)b.n, true, sr, xex, xplanes, ld, nX, b.count, s, act, nv));
-        // the first residual only feeds the update: fewer slice pairs
+        // the first residual only feeds the update: fewer slices
         const int s_it = it == 0 ? b.s0 : sr;
-        TcGemmParams q = {};
-        q.M = q.N = q.K = (int)b.n;
-        tc_pairs_ozaki(q, s_it);
-        q.alpha = -1.0;
-        q.beta = 0.0;
-        q.add_identity = 1;
-        q.sumsq = nR;
-        q.err = p.err;
-        q.active = act;
-        q.sum_order = nv;
-        q.row_exp = aex;
-        q.col_exp = xex;
-        q.batch = b.count;
-        q.d_base = p.w_base + b.first;
-        q.d_ld = b.n;
-        BRET(launch_tc_gemm(TcOperand{aplanes, (int)b.n, sr, ld}, TcOperand{xplanes, (int)b.n, sr, ld}, q, s));
+        if (residues) {
+            CrtProduct q = {};
+            q.m = q.n = q.k = b.n;
+            q.min_bits = crt_bits_for_slices(s_it);
+            q.alpha = -1.0;
+            q.add_identity = 1;
+            q.count = b.count;
+            q.Av = Av;
+            q.Bv = Xv;
+            q.Dv = Rv;
+            q.active = act;
+            q.valid = nv;
+            q.sumsq_a = it == 0 ? nA : nullptr;
+            q.sumsq_b = nX;
+            q.sumsq_d = nR;
+            q.err = p.err;
+            BRET(crt_product(q, scratch, scratch_bytes, s, &p.kernels));
+        } else {
+            BRET(launch_ozaki_split_batched(Xv, (int)b.n, (int)b.n, true, sr, xex, xplanes, ld, nX, b.count, s, act,
+                                            nv));
+            TcGemmParams q = {};
+            q.M = q.N = q.K = (int)b.n;
+            tc_pairs_ozaki(q, s_it);
+            q.alpha = -1.0;
+            q.beta = 0.0;
+            q.add_identity = 1;
+            q.sumsq = nR;
+            q.err = p.err;
+            q.active = act;
+            q.sum_order = nv;
+            q.row_exp = aex;
+            q.col_exp = xex;
+            q.batch = b.count;
+            q.d_base = p.w_base + b.first;
+            q.d_ld = b.n;
+            BRET(launch_tc_gemm(TcOperand{aplanes, (int)b.n, sr, ld}, TcOperand{xplanes, (int)b.n, sr, ld}, q, s));
+            p.kernels += 5;
+        }
         BRET(launch_refine_decide(nA, nX, nR, b.count, p.tol, residual_error_model(b.n, s_it), it, p.max_refine, act,
                                   p.rel + b.first, p.iters + b.first, rec, s));
-        p.kernels += 6;
+        p.kernels += 1;
         if (it == p.max_refine) break;
         BRET(launch_split_planes_batched(Xv, (int)b.n, (int)b.n, false, 3, xp, ld, b.count, s, act));
         BRET(launch_split_planes_batched(Rv, (int)b.n, (int)b.n, true, 3, rp, ld, b.count, s, act));
@@ -792,7 +831,8 @@ int build_plan(BatchPlan& p, const double* const* A, const int64_t* lda, double*
         BatchView Av{p.a_base + b.first, p.a_ld + b.first, 0, 0, 0};
         BatchView Xv{(const double* const*)(p.x_base + b.first), nullptr, b.n, 0, 0};
         if (mixed) {
-            BMix x{p.arena + b.arena_offset, b.count, p.fp64_levels, p.err, &p.kernels, p.streams[si]};
+            BMix x{p.arena + b.arena_offset, (size_t)b.count * (b.scratch_per + b.cache_per), b.count, p.fp64_levels,
+                   p.err, &p.kernels, p.streams[si]};
             rc = binv_mixed(r, x, 0, Av, Xv, (const double* const*)(p.w_base + b.first), 0, b.n);
             if (rc == SPIN_OK) rc = bucket_refine(p, b, p.streams[si]);
         } else {
@@ -990,7 +1030,7 @@ int run_bucket(const double* const* A, const int64_t* lda, double* const* X, con
     BatchView Xv{(const double* const*)p.x_base, nullptr, n, 0, 0};
     int rc;
     if (mixed) {
-        BMix x{p.arena, count, p.fp64_levels, p.err, &p.kernels, s};
+        BMix x{p.arena, (size_t)count * (b.scratch_per + b.cache_per), count, p.fp64_levels, p.err, &p.kernels, s};
         rc = binv_mixed(r, x, 0, Av, Xv, (const double* const*)p.w_base, 0, n);
         if (rc == SPIN_OK) rc = bucket_refine(p, b, s);
         if (rc == SPIN_OK) rc = launch_refine_finish(p.err, p.records, count, s);

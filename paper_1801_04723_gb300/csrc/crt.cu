@@ -344,6 +344,9 @@ crt_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         for (int64_t t = blockIdx.x; t < items && ok; t += gridDim.x) {
             if (*abort) break;
             if (!item_of(t, zl, m0, n0)) continue;
+            // columns (of this warp's HALF) and rows that exist
+            const int row = m0 + quarter * 32 + lane, col0 = n0 + half * HALF;
+            const int ncol = m0 + quarter * 32 < p.M ? min(HALF, p.N - col0) : 0;
             int acc[HALF];
             for (int c = 0; c < runs && ok; c++) {
                 const int buf = run & 1;
@@ -355,6 +358,7 @@ crt_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 tc_fence_after();
 #pragma unroll
                 for (int c0 = 0; c0 < HALF; c0 += 16) {
+                    if (c0 >= ncol) break;
                     uint32_t v[16];
                     tmem_ld_32x32b_x16(lane_addr + (uint32_t)(buf * BN + c0), v);
                     tmem_ld_wait();
@@ -372,14 +376,13 @@ crt_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 run++;
             }
             if (!ok) break;
-            const int row = m0 + quarter * 32 + lane, col0 = n0 + half * HALF;
             if (row < p.M) {
                 const int l = zl % p.moduli;
                 const unsigned mod = p.p[l], magic = p.magic[l], shift = p.shift[l];
                 uint8_t* out = p.res + ((int64_t)zl * p.M + row) * p.ldr + col0;
 #pragma unroll
                 for (int c0 = 0; c0 < HALF; c0 += 16) {
-                    if (col0 + c0 >= p.ldr) break;
+                    if (c0 >= ncol) break;
                     uint32_t w[4];
 #pragma unroll
                     for (int q = 0; q < 4; q++) {
@@ -590,16 +593,22 @@ CrtPanels panel_layout(int64_t m, int64_t n, int64_t k, int moduli, int64_t coun
     return c;
 }
 
+// A p-th of x, in whole tiles unless a panel is smaller than one.
+int64_t panel_size(int64_t x, int64_t p, int64_t tile) {
+    const size_t part = (size_t)((x + p - 1) / p);
+    return (int64_t)round_up(part, part > (size_t)tile ? (size_t)tile : 16);
+}
+
 // Panels that fit: A's rows once per row panel, B's columns once per row
 // panel and column panel.  The cheapest by the elements split (about 6 ps
 // each and modulus-proportional) and launches.
 bool choose_panels(int64_t m, int64_t n, int64_t k, int moduli, int64_t count, size_t bytes, CrtPanels* best) {
     double least = 1e300;
     for (int pa = 1; pa <= kMaxPanels; pa++) {
-        const int64_t rows = (int64_t)round_up((size_t)((m + pa - 1) / pa), BM);
-        if (pa > 1 && rows >= (int64_t)round_up((size_t)((m + pa - 2) / (pa - 1)), BM)) continue;
+        const int64_t rows = panel_size(m, pa, BM);
+        if (pa > 1 && rows >= panel_size(m, pa - 1, BM)) continue;
         for (int pb = 1; pb <= kMaxPanels; pb++) {
-            const int64_t cols = (int64_t)round_up((size_t)((n + pb - 1) / pb), kCrtBN);
+            const int64_t cols = panel_size(n, pb, kCrtBN);
             const CrtPanels c = panel_layout(m, n, k, moduli, count, rows, cols);
             if (c.total > bytes) continue;
             const double na = (double)((m + rows - 1) / rows), nb = (double)((n + cols - 1) / cols);
@@ -768,24 +777,72 @@ size_t crt_full_bytes(int64_t m, int64_t n, int64_t k, int moduli, int count) {
 }
 
 size_t crt_min_bytes(int64_t m, int64_t n, int64_t k, int moduli, int count) {
-    const int64_t rows = (int64_t)round_up((size_t)((m + kMaxPanels - 1) / kMaxPanels), BM);
-    const int64_t cols = (int64_t)round_up((size_t)((n + kMaxPanels - 1) / kMaxPanels), kCrtBN);
-    return panel_layout(m, n, k, moduli, std::max(count, 1), rows, cols).total;
+    return panel_layout(m, n, k, moduli, std::max(count, 1), panel_size(m, kMaxPanels, BM),
+                        panel_size(n, kMaxPanels, kCrtBN))
+        .total;
 }
+
+namespace {
+
+BatchView skip(BatchView v, int z) {
+    v.base += z;
+    if (v.lds) v.lds += z;
+    return v;
+}
+
+}  // namespace
 
 int crt_product(const CrtProduct& p, void* arena, size_t bytes, cudaStream_t s, int* launches) {
     if (p.m <= 0 || p.n <= 0) return SPIN_OK;
     if (p.count < 0 || p.count > 65535) return SPIN_ERR_INVALID_ARG;
     const CrtFormat f = crt_format(p.k, p.min_bits);
     if (f.moduli == 0) return SPIN_ERR_INVALID_ARG;
-    const int64_t count = std::max(p.count, 1);
-    CrtPanels c;
-    if (!choose_panels(p.m, p.n, p.k, f.moduli, count, bytes, &c)) return SPIN_ERR_INVALID_ARG;
-    if (count * f.moduli * std::max(c.rows, c.cols) > INT32_MAX) return SPIN_ERR_INVALID_ARG;  // TMA row coordinate
     unsigned char* base = (unsigned char*)round_up((size_t)(uintptr_t)arena, 256);
-    if (p.count > 0)
-        return crt_run(p, SrcMany{p.Av, p.active, p.valid}, SrcMany{p.Bv, p.active, p.valid}, f, c, base, s, launches);
-    return crt_run(p, SrcOne{p.A, p.lda, p.active}, SrcOne{p.B, p.ldb, p.active}, f, c, base, s, launches);
+    CrtPanels c;
+    if (p.count == 0) {
+        if (!choose_panels(p.m, p.n, p.k, f.moduli, 1, bytes, &c)) return SPIN_ERR_INVALID_ARG;
+        if (f.moduli * std::max(c.rows, c.cols) > INT32_MAX) return SPIN_ERR_INVALID_ARG;  // TMA row coordinate
+        return crt_run(p, SrcOne{p.A, p.lda, p.active}, SrcOne{p.B, p.ldb, p.active}, f, c, base, s, launches);
+    }
+    // as many problems at a time as the arena (and the TMA row coordinate)
+    // holds whole, the same number each time; in panels, one at a time, if none
+    const auto fits = [&](int64_t z) {
+        return crt_full_bytes(p.m, p.n, p.k, f.moduli, (int)z) <= bytes &&
+               z * f.moduli * std::max(p.m, p.n) <= INT32_MAX;
+    };
+    int most = p.count;
+    if (!fits(most)) {
+        int lo = 0;  // fits, or none
+        while (most - lo > 1) {
+            const int mid = lo + (most - lo) / 2;
+            if (fits(mid))
+                lo = mid;
+            else
+                most = mid;
+        }
+        most = std::max(lo, 1);
+    }
+    const int chunks = (p.count + most - 1) / most, step = (p.count + chunks - 1) / chunks;
+    for (int z = 0; z < p.count; z += step) {
+        CrtProduct q = p;
+        q.count = std::min(step, p.count - z);
+        q.Av = skip(p.Av, z);
+        q.Bv = skip(p.Bv, z);
+        if (p.beta != 0.0) q.Cv = skip(p.Cv, z);
+        q.Dv = skip(p.Dv, z);
+        if (p.active) q.active = p.active + z;
+        if (p.valid) q.valid = p.valid + z;
+        if (p.sumsq_a) q.sumsq_a = p.sumsq_a + z;
+        if (p.sumsq_b) q.sumsq_b = p.sumsq_b + z;
+        if (p.sumsq_d) q.sumsq_d = p.sumsq_d + z;
+        if (p.a_exps) q.a_exps = p.a_exps + (int64_t)z * p.m;
+        if (p.a_exps_out) q.a_exps_out = p.a_exps_out + (int64_t)z * p.m;
+        if (!choose_panels(q.m, q.n, q.k, f.moduli, q.count, bytes, &c)) return SPIN_ERR_INVALID_ARG;
+        const int rc = crt_run(q, SrcMany{q.Av, q.active, q.valid}, SrcMany{q.Bv, q.active, q.valid}, f, c, base, s,
+                               launches);
+        if (rc) return rc;
+    }
+    return SPIN_OK;
 }
 
 }  // namespace spin
