@@ -197,9 +197,9 @@ int spin_invert_ex(const double* A, int64_t lda, double* X, int64_t ldx, int64_t
  * Matrices of equal order form a bucket whose recursion runs in lockstep
  * (batched products, one leaf cluster per matrix); buckets run concurrently
  * on streams forked from `stream`.  The launch sequence is captured into a
- * CUDA graph on the first call and replayed while the arguments (pointers,
- * orders, leading dimensions, options) stay the same; the
- * workspace is library-owned.  The mixed form's refinement is part of the
+ * CUDA graph on the first call and replayed while the orders and options
+ * stay the same (other matrices of the same orders cost one small copy of
+ * their addresses); the workspace is library-owned.  The mixed form's refinement is part of the
  * graph: each matrix's stopping decision is taken on the device, so the
  * result of a matrix does not depend on the others in the batch, and the
  * call returns once the graph is enqueued (with opts->blocking, once it has

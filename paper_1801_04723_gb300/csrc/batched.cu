@@ -8,8 +8,9 @@
 // concurrently on a pool of streams forked from the caller's stream.
 //
 // The launch sequence (all buckets, fork and join) is captured once into a
-// CUDA graph and replayed while the caller passes the same arguments, so a
-// batch of thousands of matrices costs one graph launch on the host.
+// CUDA graph and replayed while the orders and options stay the same, so a
+// batch of thousands of matrices costs one graph launch on the host, and
+// other matrices of the same orders one copy of their addresses more.
 //
 // Mixed precision (SPIN_MIXED_BF16X3): the same lockstep recursion with the
 // level products on the tensor cores, batched over the bucket (one launch
@@ -61,8 +62,17 @@ void set_slices(Bucket& b, const spin_opts& o) {
     b.s0 = o.residual_slices > 0 ? o.residual_slices : first_residual_slices_for(b.n, o.tol, b.sr);
 }
 
+// What a call's shape decides (orders, options): buckets, device memory and
+// the captured graph.  The matrices' addresses and leading dimensions are
+// data of the plan, read by the kernels from one device block, so a call
+// with other matrices of the same orders replays the graph after one copy.
 struct BatchPlan {
     std::vector<uint64_t> key;
+    std::vector<uint64_t> operands;  // what the device block holds
+    std::vector<int> order;          // user's index of each sorted position
+    uint64_t* ptr_block = nullptr;   // device: a_base, a_ld, x_base
+    uint64_t* staging = nullptr;     // pinned copy of it, free again once `staged` has happened
+    cudaEvent_t staged = nullptr;
     std::vector<Bucket> buckets;
     // device arrays in sorted (bucket) order
     const double** a_base = nullptr;
@@ -121,10 +131,14 @@ void free_plan(BatchPlan& p) {
     p.rel = nullptr;
     p.iters = nullptr;
     p.err = nullptr;
-    cudaFree((void*)p.a_base);
-    cudaFree(p.a_ld);
-    cudaFree(p.x_base);
+    cudaFree(p.ptr_block);
     cudaFree(p.w_base);
+    if (p.staging) {
+        if (p.staged) cudaEventSynchronize(p.staged);
+        cudaFreeHost(p.staging);
+    }
+    p.ptr_block = p.staging = nullptr;
+    p.operands.clear();
     cudaFree(p.user_index);
     cudaFree(p.records);
     cudaFree(p.ws);
@@ -706,8 +720,28 @@ int capture_persistent(BatchPlan& p) {
     return SPIN_OK;
 }
 
-int build_plan(BatchPlan& p, const double* const* A, const int64_t* lda, double* const* X, const int64_t* n,
-               int count, const spin_opts& o, cudaStream_t s) {
+// The call's addresses and leading dimensions, in sorted order, into the
+// plan's device block on s (a launch queued before on s reads the old ones).
+int set_operands(BatchPlan& p, const double* const* A, const int64_t* lda, double* const* X, cudaStream_t s) {
+    const size_t c = (size_t)p.count;
+    std::vector<uint64_t> now(3 * c);
+    for (size_t pos = 0; pos < c; pos++) {
+        const int u = p.order[pos];
+        now[pos] = (uint64_t)(uintptr_t)A[u];
+        now[c + pos] = (uint64_t)lda[u];
+        now[2 * c + pos] = (uint64_t)(uintptr_t)X[u];
+    }
+    if (now == p.operands) return SPIN_OK;
+    SPIN_CUDA_TRY(cudaEventSynchronize(p.staged));  // the last copy from the staging block is done
+    p.operands.clear();                             // until the new copy is on its way
+    memcpy(p.staging, now.data(), now.size() * sizeof(uint64_t));
+    SPIN_CUDA_TRY(cudaMemcpyAsync(p.ptr_block, p.staging, now.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
+    SPIN_CUDA_TRY(cudaEventRecord(p.staged, s));
+    p.operands = std::move(now);
+    return SPIN_OK;
+}
+
+int build_plan(BatchPlan& p, const int64_t* n, int count, const spin_opts& o, cudaStream_t s) {
     free_plan(p);
     const int leaf_opt = o.leaf;
     const bool mixed = o.precision != SPIN_FP64;
@@ -718,7 +752,8 @@ int build_plan(BatchPlan& p, const double* const* A, const int64_t* lda, double*
     p.tol = o.tol;
     p.max_refine = o.max_refine;
     p.fp64_levels = o.fp64_levels;
-    std::vector<int> order(count);
+    std::vector<int>& order = p.order;
+    order.resize(count);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n[a] < n[b]; });
     p.buckets.clear();
@@ -748,10 +783,7 @@ int build_plan(BatchPlan& p, const double* const* A, const int64_t* lda, double*
         p.buckets.push_back(b);
         i = j;
     }
-    std::vector<const double*> ha(count);
-    std::vector<int64_t> hl(count);
-    std::vector<double*> hx(count), hw(count);
-    std::vector<int> hu(count);
+    std::vector<double*> hw(count);
     if (cudaMalloc(&p.ws, ws_total * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return SPIN_ERR_OOM;
@@ -770,24 +802,19 @@ int build_plan(BatchPlan& p, const double* const* A, const int64_t* lda, double*
     p.ws_bytes = ws_total * sizeof(double);
     for (const Bucket& b : p.buckets)
         for (int z = 0; z < b.count; z++) {
-            const int pos = b.first + z, u = order[pos];
-            ha[pos] = A[u];
-            hl[pos] = lda[u];
-            hx[pos] = X[u];
-            hw[pos] = p.ws + b.ws_offset + (size_t)z * b.ws_elems;
-            hu[pos] = u;
+            hw[b.first + z] = p.ws + b.ws_offset + (size_t)z * b.ws_elems;
         }
-    SPIN_CUDA_TRY(cudaMalloc((void**)&p.a_base, count * sizeof(double*)));
-    SPIN_CUDA_TRY(cudaMalloc(&p.a_ld, count * sizeof(int64_t)));
-    SPIN_CUDA_TRY(cudaMalloc(&p.x_base, count * sizeof(double*)));
+    SPIN_CUDA_TRY(cudaMalloc(&p.ptr_block, 3 * (size_t)count * sizeof(uint64_t)));
+    SPIN_CUDA_TRY(cudaMallocHost(&p.staging, 3 * (size_t)count * sizeof(uint64_t)));
+    if (!p.staged) SPIN_CUDA_TRY(cudaEventCreateWithFlags(&p.staged, cudaEventDisableTiming));
+    p.a_base = (const double**)p.ptr_block;
+    p.a_ld = (int64_t*)(p.ptr_block + count);
+    p.x_base = (double**)(p.ptr_block + 2 * (size_t)count);
     SPIN_CUDA_TRY(cudaMalloc(&p.w_base, count * sizeof(double*)));
     SPIN_CUDA_TRY(cudaMalloc(&p.user_index, count * sizeof(int)));
     SPIN_CUDA_TRY(cudaMalloc(&p.records, (size_t)count * INFO_WORDS * sizeof(int32_t)));
-    SPIN_CUDA_TRY(cudaMemcpy((void*)p.a_base, ha.data(), count * sizeof(double*), cudaMemcpyHostToDevice));
-    SPIN_CUDA_TRY(cudaMemcpy(p.a_ld, hl.data(), count * sizeof(int64_t), cudaMemcpyHostToDevice));
-    SPIN_CUDA_TRY(cudaMemcpy(p.x_base, hx.data(), count * sizeof(double*), cudaMemcpyHostToDevice));
     SPIN_CUDA_TRY(cudaMemcpy(p.w_base, hw.data(), count * sizeof(double*), cudaMemcpyHostToDevice));
-    SPIN_CUDA_TRY(cudaMemcpy(p.user_index, hu.data(), count * sizeof(int), cudaMemcpyHostToDevice));
+    SPIN_CUDA_TRY(cudaMemcpy(p.user_index, order.data(), count * sizeof(int), cudaMemcpyHostToDevice));
     for (int i = 0; i < kStreams; i++) {
         if (!p.streams[i]) SPIN_CUDA_TRY(cudaStreamCreateWithFlags(&p.streams[i], cudaStreamNonBlocking));
         if (!p.join[i]) SPIN_CUDA_TRY(cudaEventCreateWithFlags(&p.join[i], cudaEventDisableTiming));
@@ -864,10 +891,9 @@ int build_plan(BatchPlan& p, const double* const* A, const int64_t* lda, double*
     return SPIN_OK;
 }
 
-std::vector<uint64_t> make_key(const double* const* A, const int64_t* lda, double* const* X, const int64_t* n,
-                               int count, const spin_opts& o) {
+std::vector<uint64_t> make_key(const int64_t* n, int count, const spin_opts& o) {
     std::vector<uint64_t> k;
-    k.reserve((size_t)count * 4 + 8);
+    k.reserve((size_t)count + 16);
     k.push_back((uint64_t)count);
     k.push_back((uint64_t)(int64_t)o.leaf);
     k.push_back((uint64_t)(int64_t)o.precision);
@@ -885,12 +911,7 @@ std::vector<uint64_t> make_key(const double* const* A, const int64_t* lda, doubl
     int dev = 0;
     cudaGetDevice(&dev);
     k.push_back((uint64_t)dev);
-    for (int i = 0; i < count; i++) {
-        k.push_back((uint64_t)(uintptr_t)A[i]);
-        k.push_back((uint64_t)lda[i]);
-        k.push_back((uint64_t)(uintptr_t)X[i]);
-        k.push_back((uint64_t)n[i]);
-    }
+    for (int i = 0; i < count; i++) k.push_back((uint64_t)n[i]);
     return k;
 }
 
@@ -1274,15 +1295,19 @@ extern "C" int spin_invert_batched(const double* const* A, const int64_t* lda, d
     cudaStream_t s = (cudaStream_t)stream;
     std::lock_guard<std::mutex> lk(g_bmu);
     BatchPlan& p = g_plans[s];
-    std::vector<uint64_t> key = make_key(A, lda, X, n, count, o);
+    std::vector<uint64_t> key = make_key(n, count, o);
     if (p.exec == nullptr || key != p.key) {
-        int rc = build_plan(p, A, lda, X, n, count, o, s);
+        int rc = build_plan(p, n, count, o, s);
         if (rc != SPIN_OK) {
             free_plan(p);
             p.key.clear();
             return rc;
         }
         p.key = key;
+    }
+    {
+        const int rc = set_operands(p, A, lda, X, s);
+        if (rc != SPIN_OK) return rc;
     }
     SPIN_CUDA_TRY(cudaGraphLaunch(p.exec, s));
     p.kernels = p.graph_kernels;

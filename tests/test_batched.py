@@ -297,3 +297,33 @@ def test_batch_persistent_autotuner(spin):
             check(As[i], X0[i].cpu().numpy(), rec[orders[i]][0])
     finally:
         spin.autotune_batched_leaf(sorted(set(orders)), "fp64", candidates=())
+
+
+@pytest.mark.parametrize("precision", ["fp64", "bf16x3"])
+def test_batch_other_matrices_of_the_same_orders(spin, precision):
+    """Calls that alternate between two sets of matrices of the same orders,
+    with other addresses and leading dimensions, and do not wait in between:
+    each set's results are those of a call of its own."""
+    orders = [200, 96, 200, 33, 320]
+    big = torch.zeros((400, 700), dtype=torch.float64, device="cuda:0")
+    sets = []
+    for i in range(2):
+        As = [torch.from_numpy(inputs.sdd(n, seed=4000 + 10 * i + j)).cuda() for j, n in enumerate(orders)]
+        if i:
+            big[5:205, 9:209] = As[2]
+            As[2] = big[5:205, 9:209]
+        sets.append(As)
+    want = []
+    for As in sets:
+        Xs, info = spin.invert_batched(As, precision=precision)
+        spin.invert_batched([As[1]], precision=precision)  # other orders in between
+        want.append([x.clone() for x in Xs])
+        assert int(info.abs().sum()) == 0
+    outs = [[torch.zeros_like(x) for x in w] for w in want]
+    for _ in range(3):
+        for As, Xs in zip(sets, outs):
+            spin.invert_batched(As, outs=Xs, precision=precision, blocking=False)
+    torch.cuda.synchronize()
+    for w, Xs in zip(want, outs):
+        for a, b in zip(w, Xs):
+            assert torch.equal(a, b)
