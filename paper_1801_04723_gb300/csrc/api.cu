@@ -281,12 +281,8 @@ int level_gemm(Run& r, int depth, bool schur, int64_t m, int64_t n, int64_t k, d
     }
     RET(plan_bf16x3(m, n, k, r.scratch, r.scratch_bytes, &sp));
     {
-        ProfScope ps(r.prof, r.s, SPIN_KERNEL_SPLIT, depth, m, k, 0, 0.0, 12.0 * m * k);
-        RET(split_a_bf16x3(sp, A, lda, m, k, r.s));
-    }
-    {
-        ProfScope ps(r.prof, r.s, SPIN_KERNEL_SPLIT, depth, k, n, 0, 0.0, 12.0 * k * n);
-        RET(split_b_bf16x3(sp, B, ldb, k, n, r.s));
+        ProfScope ps(r.prof, r.s, SPIN_KERNEL_SPLIT, depth, m, n, k, 0.0, 12.0 * (m * k + k * n));
+        RET(split_bf16(sp, A, lda, B, ldb, m, n, k, r.s));
     }
     ProfScope ps(r.prof, r.s, SPIN_KERNEL_GEMM_TC, depth, m, n, k, 3.0 * f,
                  4.0 * (m * k + k * n) + 8.0 * m * n * (beta != 0.0 ? 2 : 1));
@@ -549,7 +545,6 @@ int refine(Run& r, StreamState* st, const double* A, int64_t lda, double* X, int
     for (int it = 0; it <= o.max_refine; it++) {
         // the first residual only feeds the update: fewer slices
         const int s_it = it == 0 ? L.s0 : L.sr;
-        if (it > 0) SPIN_CUDA_TRY(cudaMemsetAsync(norms + 1, 0, 2 * sizeof(double), s));
         {
             Fp64ClassExtra x;
             x.active = act;
@@ -573,8 +568,7 @@ int refine(Run& r, StreamState* st, const double* A, int64_t lda, double* X, int
         RET(plan_bf16x6(n, n, n, scratch, scratch_bytes, &up));
         {
             ProfScope ps(r.prof, s, SPIN_KERNEL_SPLIT, -1, n, n, 0, 0.0, 28.0 * n * n, act);
-            RET(split_a_bf16x6(up, X, ldx, n, n, s, act));
-            RET(split_b_bf16x6(up, R, n, n, n, s, act));
+            RET(split_bf16(up, X, ldx, R, n, n, n, n, s, act));
         }
         ProfScope ps(r.prof, s, SPIN_KERNEL_UPDATE, -1, n, n, n, 6.0 * f, 12.0 * n * n + 16.0 * n * n, act);
         RET(product_bf16x6(up, n, n, n, 1.0, 1.0, X, ldx, X, ldx, r.err, s, act));

@@ -34,6 +34,7 @@
 #include "crt.h"
 #include "mixed.h"
 #include "persistent.h"
+#include "split.h"
 #include "tc_gemm.h"
 
 namespace spin {
@@ -484,9 +485,15 @@ int bproduct(BMix& x, int depth, bool schur, int64_t m, int64_t n, int64_t k, do
     p.d_c0 = D.c0;
     uint16_t* pa = (uint16_t*)x.scratch;
     uint16_t* pb = pa + cnt * 2 * m * ld;
-    *x.kernels += 3;
-    BRET(launch_split_planes_batched(A, (int)m, (int)k, false, 2, pa, ld, x.count, x.s));
-    BRET(launch_split_planes_batched(B, (int)k, (int)n, true, 2, pb, ld, x.count, x.s));
+    *x.kernels += 2;
+    SplitSource src;
+    src.count = x.count;
+    src.Av = A;
+    src.Bv = B;
+    BRET(launch_split(src,
+                      SplitTarget{SPLIT_BF16, 2, 0, (int)m, (int)n, (int)k, 0, (int)m, 0, (int)n, nullptr, nullptr, pa, pb,
+                                  ld},
+                      x.s));
     tc_pairs_bf16x3(p);
     return launch_tc_gemm(TcOperand{pa, (int)m, 2, ld}, TcOperand{pb, (int)n, 2, ld}, p, x.s);
 }
@@ -550,14 +557,20 @@ int bucket_refine(BatchPlan& p, const Bucket& b, cudaStream_t s) {
     uint16_t* xp = (uint16_t*)scratch;  // update: three planes of X, then of R
     uint16_t* rp = xp + (int64_t)b.count * 3 * b.n * ld;
     BRET(launch_refine_init(rec, b.count, act, p.rel + b.first, p.iters + b.first, s));
-    SPIN_CUDA_TRY(cudaMemsetAsync(nA, 0, b.count * sizeof(double), s));
-    p.kernels += residues ? 1 : 3;
+    SPIN_CUDA_TRY(cudaMemset2DAsync(nA, count * sizeof(double), 0, b.count * sizeof(double), 3, s));  // nA, nX, nR
+    p.kernels += 1;
     const int* nv = p.nvalid ? p.nvalid + b.first : nullptr;  // norms over the unpadded block
-    if (!residues)
-        BRET(launch_ozaki_split_batched(Av, (int)b.n, (int)b.n, false, sr, aex, aplanes, ld, nA, b.count, s, act, nv));
+    SplitSource ax;  // A and X
+    ax.count = b.count;
+    ax.Av = Av;
+    ax.Bv = Xv;
+    ax.active = act;
+    ax.valid = nv;
+    SplitSource xr = ax;  // X and R
+    xr.Av = Xv;
+    xr.Bv = Rv;
+    const int nn = (int)b.n;
     for (int it = 0; it <= p.max_refine; it++) {
-        SPIN_CUDA_TRY(cudaMemsetAsync(nX, 0, b.count * sizeof(double), s));
-        SPIN_CUDA_TRY(cudaMemsetAsync(nR, 0, b.count * sizeof(double), s));
         // the first residual only feeds the update: fewer slices
         const int s_it = it == 0 ? b.s0 : sr;
         if (residues) {
@@ -578,8 +591,12 @@ int bucket_refine(BatchPlan& p, const Bucket& b, cudaStream_t s) {
             q.err = p.err;
             BRET(crt_product(q, scratch, scratch_bytes, s, &p.kernels));
         } else {
-            BRET(launch_ozaki_split_batched(Xv, (int)b.n, (int)b.n, true, sr, xex, xplanes, ld, nX, b.count, s, act,
-                                            nv));
+            // A's exponents and digits are kept over the rounds
+            BRET(launch_exponents(ax, nn, nn, nn, it == 0 ? aex : nullptr, xex, nA, nX, nullptr, s));
+            BRET(launch_split(ax,
+                              SplitTarget{SPLIT_DIGITS, sr, 0, nn, nn, nn, 0, it == 0 ? nn : 0, 0, nn, aex, xex, aplanes,
+                                          xplanes, ld},
+                              s));
             TcGemmParams q = {};
             q.M = q.N = q.K = (int)b.n;
             tc_pairs_ozaki(q, s_it);
@@ -596,14 +613,14 @@ int bucket_refine(BatchPlan& p, const Bucket& b, cudaStream_t s) {
             q.d_base = p.w_base + b.first;
             q.d_ld = b.n;
             BRET(launch_tc_gemm(TcOperand{aplanes, (int)b.n, sr, ld}, TcOperand{xplanes, (int)b.n, sr, ld}, q, s));
-            p.kernels += 5;
+            p.kernels += 3;
         }
         BRET(launch_refine_decide(nA, nX, nR, b.count, p.tol, residual_error_model(b.n, s_it), it, p.max_refine, act,
                                   p.rel + b.first, p.iters + b.first, rec, s));
         p.kernels += 1;
         if (it == p.max_refine) break;
-        BRET(launch_split_planes_batched(Xv, (int)b.n, (int)b.n, false, 3, xp, ld, b.count, s, act));
-        BRET(launch_split_planes_batched(Rv, (int)b.n, (int)b.n, true, 3, rp, ld, b.count, s, act));
+        BRET(launch_split(xr,
+                          SplitTarget{SPLIT_BF16, 3, 0, nn, nn, nn, 0, nn, 0, nn, nullptr, nullptr, xp, rp, ld}, s));
         TcGemmParams u = {};
         u.M = u.N = u.K = (int)b.n;
         tc_pairs_bf16x6(u);
@@ -616,7 +633,7 @@ int bucket_refine(BatchPlan& p, const Bucket& b, cudaStream_t s) {
         u.c_ld = b.n;
         u.d_base = p.x_base + b.first;
         u.d_ld = b.n;
-        p.kernels += 3;
+        p.kernels += 2;
         BRET(launch_tc_gemm(TcOperand{xp, (int)b.n, 3, ld}, TcOperand{rp, (int)b.n, 3, ld}, u, s));
     }
     return SPIN_OK;

@@ -13,11 +13,9 @@
 // products falls from 21 to 13 or 14 for s = 6, from 28 to 15 or 16 for s = 7.
 //
 // Three kernels:
-//   split    FP64 -> N BF16 planes of signed residues (|r| <= 128, exact):
-//            the integer is cut into balanced 14-bit pieces, and a residue is
-//            one FP32 dot product of 4 or 5 pieces with the powers of 2^14
-//            modulo p (every partial sum below 2^24, exact) and one rounded
-//            quotient: six FP32 operations per residue.
+//   split    (split.cu) FP64 -> N BF16 planes of signed residues (|r| <= 128,
+//            exact), six FP32 operations per residue, after a pass that takes
+//            the exponents.
 //   product  per modulus and 128 x 256 tile, exact FP32 runs of 1024 products
 //            (|r r'| <= 2^14, sums <= 2^24) drained into int32, reduced
 //            modulo p and written as one byte per output.  A tile of one
@@ -37,158 +35,14 @@
 #include <algorithm>
 
 #include "crt.h"
+#include "split.h"
 #include "tc_pipe.cuh"
 
 namespace spin {
 namespace {
 
-// Pairwise coprime, in falling order; with signed residues |r| <= 128.
-__host__ __device__ constexpr int crt_modulus(int l) {
-    constexpr int p[kCrtMaxModuli] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227,
-                                      223, 217, 211, 199, 197, 193, 191, 181, 179, 173};
-    return p[l];
-}
-
-constexpr int kPiece = 14;  // bits of a balanced piece of the integer
 constexpr int kRunK = 1024;
 constexpr int kMaxRuns = 96;  // 96 runs of 2^24 fit int32
-
-// ----------------------------------------------------------------- split --
-
-// 2^(14 q) modulo p, balanced.
-__host__ __device__ constexpr int piece_weight(int l, int q) {
-    const int p = crt_modulus(l);
-    int v = 1;
-    for (int i = 0; i < q; i++) v = v * (1 << kPiece) % p;
-    return v > p / 2 ? v - p : v;
-}
-
-// round(x 2^(b - e)), |x| < 2^e (ties away from zero; integer arithmetic on
-// the IEEE fields), as PIECES balanced 14-bit pieces in FP32.
-template <int PIECES>
-__device__ __forceinline__ void fixed_pieces(double x, int e, int b, float (&f)[PIECES]) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-    int fe = (int)(u >> 52) & 0x7FF;
-    unsigned long long m = u & ((1ull << 52) - 1);
-    if (fe == 0)
-        fe = 1;  // subnormal: no implicit bit
-    else
-        m |= 1ull << 52;
-    const int sh = fe - 1075 + b - e;  // <= b - 53
-    unsigned long long n;
-    if (sh >= 0)
-        n = m << sh;
-    else if (sh > -64)
-        n = (m + (1ull << (-sh - 1))) >> (-sh);
-    else
-        n = 0;
-    long long v = (u >> 63) ? -(long long)n : (long long)n;
-#pragma unroll
-    for (int q = 0; q < PIECES; q++) {
-        int d;
-        if (q + 1 < PIECES) {
-            d = (int)((unsigned)v << (32 - kPiece)) >> (32 - kPiece);  // low 14 bits, signed
-            v = (v - d) >> kPiece;
-        } else {
-            d = (int)v;
-        }
-        // d as FP32 without a conversion (16 per clock per SM): |d| < 2^22
-        f[q] = __uint_as_float(0x4B400000u + (unsigned)d) - 12582912.0f;
-    }
-}
-
-// The residue modulo modulus l, signed (|r| <= 128), as BF16 bits in the
-// high half of the returned word.
-template <int PIECES>
-__device__ __forceinline__ unsigned residue_bits(const float (&f)[PIECES], float p, float inv_p, const float (&w)[PIECES]) {
-    float t = f[0];
-#pragma unroll
-    for (int q = 1; q < PIECES; q++) t = fmaf(f[q], w[q], t);  // |t| < 2^23: exact
-    const float quot = fmaf(t, inv_p, 12582912.0f) - 12582912.0f;
-    return __float_as_uint(fmaf(-quot, p, t));
-}
-
-template <int PIECES>
-__device__ __forceinline__ void store_residues4(const float (&f)[4][PIECES], int moduli, uint16_t* dst, int64_t plane) {
-#pragma unroll
-    for (int l = 0; l < kCrtMaxModuli; l++) {
-        if (l >= moduli) break;
-        float w[PIECES];
-#pragma unroll
-        for (int q = 0; q < PIECES; q++) w[q] = (float)piece_weight(l, q);
-        const float p = (float)crt_modulus(l), inv_p = 1.0f / (float)crt_modulus(l);
-        unsigned r[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) r[u] = residue_bits<PIECES>(f[u], p, inv_p, w);
-        uint2 o;  // bytes 2, 3 of each word: the BF16 value (the rest is zero)
-        o.x = __byte_perm(r[0], r[1], 0x7632);
-        o.y = __byte_perm(r[2], r[3], 0x7632);
-        *reinterpret_cast<uint2*>(dst + l * plane) = o;
-    }
-}
-
-// Rows of a panel (rows row0 ..), K-major as they are: 4 consecutive columns
-// per thread (8-byte stores; planes are padded to a multiple of 8 columns).
-template <class Src, int PIECES>
-__global__ void __launch_bounds__(256)
-crt_rows_kernel(Src src, int row0, int rows, int cols, const int* __restrict__ ex, int64_t exs, int bits, int moduli,
-                uint16_t* __restrict__ dst, int64_t ld) {
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    const int64_t plane = (int64_t)rows * ld;
-    dst += (int64_t)z * moduli * plane;
-    ex += (int64_t)z * exs + row0;
-    const int groups = (cols + 3) / 4;
-    const int64_t total = (int64_t)rows * groups;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / groups), c = (int)(idx % groups) * 4;
-        const double* sr = src.row(z, row0 + r) + c;
-        const int e = ex[r];
-        float f[4][PIECES];
-#pragma unroll
-        for (int u = 0; u < 4; u++) fixed_pieces<PIECES>(c + u < cols ? sr[u] : 0.0, e, bits, f[u]);
-        store_residues4<PIECES>(f, moduli, dst + (int64_t)r * ld + c, plane);
-    }
-}
-
-// Columns of a panel (columns col0 ..) of a rows x cols operand, transposed:
-// 32 columns x 128 rows through shared memory, 4 consecutive rows (K) per
-// thread.
-constexpr int kTileK = 128;
-constexpr int kTileLd = kTileK + 2;  // even: 16-byte reads
-template <class Src, int PIECES>
-__global__ void __launch_bounds__(256)
-crt_cols_kernel(Src src, int col0, int rows, int cols, const int* __restrict__ ex, int64_t exs, int bits, int moduli,
-                uint16_t* __restrict__ dst, int64_t ld) {
-    __shared__ __align__(16) double tile[32][kTileLd];
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    const int64_t plane = (int64_t)cols * ld;
-    dst += (int64_t)z * moduli * plane;
-    ex += (int64_t)z * exs + col0;
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * kTileK;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll 4
-    for (int i = warp; i < kTileK; i += 8) {
-        const int r = r0 + i, c = c0 + lane;
-        tile[lane][i] = (r < rows && c < cols) ? src.row(z, r)[col0 + c] : 0.0;
-    }
-    __syncthreads();
-    for (int i = warp; i < 32; i += 8) {
-        const int c = c0 + i, r = r0 + 4 * lane;
-        if (c >= cols || r >= rows) continue;
-        const int e = ex[c];
-        const double2 a = *reinterpret_cast<const double2*>(&tile[i][4 * lane]);
-        const double2 b = *reinterpret_cast<const double2*>(&tile[i][4 * lane + 2]);
-        float f[4][PIECES];
-        fixed_pieces<PIECES>(a.x, e, bits, f[0]);
-        fixed_pieces<PIECES>(a.y, e, bits, f[1]);
-        fixed_pieces<PIECES>(b.x, e, bits, f[2]);
-        fixed_pieces<PIECES>(b.y, e, bits, f[3]);
-        store_residues4<PIECES>(f, moduli, dst + (int64_t)c * ld + r, plane);
-    }
-}
 
 // --------------------------------------------------------------- product --
 
@@ -623,51 +477,31 @@ bool choose_panels(int64_t m, int64_t n, int64_t k, int moduli, int64_t count, s
     return least < 1e300;
 }
 
-template <class Src>
-int split_rows(Src src, int row0, int rows, int cols, const int* ex, int64_t exs, const CrtFormat& f, uint16_t* dst,
-               int64_t ld, int count, cudaStream_t s) {
-    const dim3 g = rows_grid((int64_t)rows * ((cols + 3) / 4), count);
-    if (f.bits <= 4 * kPiece - 1)
-        crt_rows_kernel<Src, 4><<<g, 256, 0, s>>>(src, row0, rows, cols, ex, exs, f.bits, f.moduli, dst, ld);
-    else
-        crt_rows_kernel<Src, 5><<<g, 256, 0, s>>>(src, row0, rows, cols, ex, exs, f.bits, f.moduli, dst, ld);
-    SPIN_CUDA_TRY(cudaGetLastError());
-    return SPIN_OK;
-}
-
-template <class Src>
-int split_cols(Src src, int col0, int rows, int cols, const int* ex, int64_t exs, const CrtFormat& f, uint16_t* dst,
-               int64_t ld, int count, cudaStream_t s) {
-    const dim3 g((unsigned)((cols + 31) / 32), (unsigned)((rows + kTileK - 1) / kTileK), (unsigned)count);
-    if (f.bits <= 4 * kPiece - 1)
-        crt_cols_kernel<Src, 4><<<g, 256, 0, s>>>(src, col0, rows, cols, ex, exs, f.bits, f.moduli, dst, ld);
-    else
-        crt_cols_kernel<Src, 5><<<g, 256, 0, s>>>(src, col0, rows, cols, ex, exs, f.bits, f.moduli, dst, ld);
-    SPIN_CUDA_TRY(cudaGetLastError());
-    return SPIN_OK;
-}
-
-template <class Src>
-int crt_run(const CrtProduct& p, Src sa, Src sb, const CrtFormat& f, const CrtPanels& c, unsigned char* arena,
-            cudaStream_t s, int* launches) {
+int crt_run(const CrtProduct& p, const CrtFormat& f, const CrtPanels& c, unsigned char* arena, cudaStream_t s,
+            int* launches) {
     const int count = p.count > 0 ? p.count : 1;
     const int m = (int)p.m, n = (int)p.n, k = (int)p.k;
-    const int64_t sss = p.count > 0 ? 1 : 0;
     int* ea = p.a_exps_out != nullptr ? p.a_exps_out : (int*)arena;
     int* eb = (int*)arena + (size_t)count * (size_t)m;
     uint16_t* pa = (uint16_t*)(arena + c.off_a - 256);
     uint16_t* pb = (uint16_t*)(arena + c.off_b - 256);
     uint8_t* res = arena + c.off_res - 256;
     int nl = 0;
-    int rc = SPIN_OK;
-    if (p.a_exps == nullptr) {
-        if ((rc = operand_exponents(sa, m, k, false, ea, p.sumsq_a, sss, count, s))) return rc;
-        nl += 1;
-    } else {
-        ea = const_cast<int*>(p.a_exps);
-    }
-    if ((rc = operand_exponents(sb, k, n, true, eb, p.sumsq_b, sss, count, s))) return rc;
-    nl += 3;
+    SplitSource src;
+    src.count = p.count;
+    src.A = p.A;
+    src.lda = p.lda;
+    src.B = p.B;
+    src.ldb = p.ldb;
+    src.Av = p.Av;
+    src.Bv = p.Bv;
+    src.active = p.active;
+    src.valid = p.valid;
+    const bool known = p.a_exps != nullptr;
+    if (known) ea = const_cast<int*>(p.a_exps);
+    int rc = launch_exponents(src, m, n, k, known ? nullptr : ea, eb, p.sumsq_a, p.sumsq_b, nullptr, s);
+    if (rc) return rc;
+    nl++;
 
     CrtTable table;
     crt_table(f, &table);
@@ -722,16 +556,17 @@ int crt_run(const CrtProduct& p, Src sa, Src sb, const CrtFormat& f, const CrtPa
     const int sms = sm_count();
     for (int row0 = 0; row0 < m; row0 += (int)c.rows) {
         const int rows = std::min((int)c.rows, m - row0);
-        if ((rc = split_rows(sa, row0, rows, k, ea, m, f, pa, c.ld, count, s))) return rc;
         CUtensorMap ta;
         if ((rc = make_map(&ta, pa, k, (int64_t)count * f.moduli * rows, c.ld, BM))) return rc;
-        nl++;
         for (int col0 = 0; col0 < n; col0 += (int)c.cols) {
             const int cols = std::min((int)c.cols, n - col0);
-            if (row0 == 0 || c.cols < n) {  // one column panel: its planes are still there
-                if ((rc = split_cols(sb, col0, k, cols, eb, n, f, pb, c.ld, count, s))) return rc;
-                nl++;
-            }
+            // the row panel's planes with its first column panel; a lone
+            // column panel's planes are still there from the first row panel
+            SplitTarget t{SPLIT_RESIDUES, f.moduli, f.bits, m, n, k, row0, col0 == 0 ? rows : 0, col0, cols, ea, eb, pa,
+                          pb, c.ld};
+            if (row0 > 0 && c.cols >= n) t.cols = 0;
+            if ((rc = launch_split(src, t, s))) return rc;
+            nl++;
             CUtensorMap tb;
             if ((rc = make_map(&tb, pb, k, (int64_t)count * f.moduli * cols, c.ld, kCrtBN))) return rc;
             g.M = rows;
@@ -802,7 +637,7 @@ int crt_product(const CrtProduct& p, void* arena, size_t bytes, cudaStream_t s, 
     if (p.count == 0) {
         if (!choose_panels(p.m, p.n, p.k, f.moduli, 1, bytes, &c)) return SPIN_ERR_INVALID_ARG;
         if (f.moduli * std::max(c.rows, c.cols) > INT32_MAX) return SPIN_ERR_INVALID_ARG;  // TMA row coordinate
-        return crt_run(p, SrcOne{p.A, p.lda, p.active}, SrcOne{p.B, p.ldb, p.active}, f, c, base, s, launches);
+        return crt_run(p, f, c, base, s, launches);
     }
     // as many problems at a time as the arena (and the TMA row coordinate)
     // holds whole, the same number each time; in panels, one at a time, if none
@@ -838,8 +673,7 @@ int crt_product(const CrtProduct& p, void* arena, size_t bytes, cudaStream_t s, 
         if (p.a_exps) q.a_exps = p.a_exps + (int64_t)z * p.m;
         if (p.a_exps_out) q.a_exps_out = p.a_exps_out + (int64_t)z * p.m;
         if (!choose_panels(q.m, q.n, q.k, f.moduli, q.count, bytes, &c)) return SPIN_ERR_INVALID_ARG;
-        const int rc = crt_run(q, SrcMany{q.Av, q.active, q.valid}, SrcMany{q.Bv, q.active, q.valid}, f, c, base, s,
-                               launches);
+        const int rc = crt_run(q, f, c, base, s, launches);
         if (rc) return rc;
     }
     return SPIN_OK;

@@ -11,6 +11,13 @@ namespace spin {
 constexpr int kCrtMaxModuli = 20;
 constexpr int kCrtMaxBits = 62;
 
+// Pairwise coprime, in falling order; signed residues |r| <= 128.
+__host__ __device__ constexpr int crt_modulus(int l) {
+    constexpr int p[kCrtMaxModuli] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227,
+                                      223, 217, 211, 199, 197, 193, 191, 181, 179, 173};
+    return p[l];
+}
+
 // Moduli and fixed-point bits per operand for an inner dimension k: the
 // fewest moduli whose product exceeds twice the largest |sum| at bits >=
 // min_bits, then every bit that they allow (at most kCrtMaxBits).  0 moduli:

@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "crt.h"
 #include "mixed.h"
+#include "split.h"
 #include "tc_gemm.h"
 
 namespace spin {
@@ -132,15 +133,18 @@ int plan_ozaki(int64_t m, int64_t n, int64_t k, int slices, void* scratch, size_
     return SPIN_OK;
 }
 
-int split_a_bf16x3(const SplitPlan& sp, const double* A, int64_t lda, int64_t m, int64_t k, cudaStream_t s) {
-    return launch_split_bf16x2(A, lda, (int)m, (int)k, false, sp.a, sp.ld, s);
-}
-int split_b_bf16x3(const SplitPlan& sp, const double* B, int64_t ldb, int64_t k, int64_t n, cudaStream_t s) {
-    return launch_split_bf16x2(B, ldb, (int)k, (int)n, true, sp.b, sp.ld, s);
-}
-int split_b_ozaki(const SplitPlan& sp, const double* B, int64_t ldb, int64_t k, int64_t n, double* sumsq,
-                  cudaStream_t s, const int* active) {
-    return launch_ozaki_split(B, ldb, (int)k, (int)n, true, sp.slices, sp.eb, sp.b, sp.ld, sumsq, s, active);
+int split_bf16(const SplitPlan& sp, const double* A, int64_t lda, const double* B, int64_t ldb, int64_t m, int64_t n,
+               int64_t k, cudaStream_t s, const int* active) {
+    SplitSource src;
+    src.A = A;
+    src.lda = lda;
+    src.B = B;
+    src.ldb = ldb;
+    src.active = active;
+    return launch_split(src,
+                        SplitTarget{SPLIT_BF16, sp.slices, 0, (int)m, (int)n, (int)k, 0, (int)m, 0, (int)n, nullptr,
+                                    nullptr, sp.a, sp.b, sp.ld},
+                        s);
 }
 
 int product_bf16x3(const SplitPlan& sp, int64_t m, int64_t n, int64_t k, double alpha, double beta, const double* C,
@@ -169,15 +173,6 @@ int plan_bf16x6(int64_t m, int64_t n, int64_t k, void* scratch, size_t bytes, Sp
     sp->ea = sp->eb = nullptr;
     sp->slices = 3;
     return SPIN_OK;
-}
-
-int split_a_bf16x6(const SplitPlan& sp, const double* A, int64_t lda, int64_t m, int64_t k, cudaStream_t s,
-                   const int* active) {
-    return launch_split_bf16x3p(A, lda, (int)m, (int)k, false, sp.a, sp.ld, s, active);
-}
-int split_b_bf16x6(const SplitPlan& sp, const double* B, int64_t ldb, int64_t k, int64_t n, cudaStream_t s,
-                   const int* active) {
-    return launch_split_bf16x3p(B, ldb, (int)k, (int)n, true, sp.b, sp.ld, s, active);
 }
 
 int product_bf16x6(const SplitPlan& sp, int64_t m, int64_t n, int64_t k, double alpha, double beta, const double* C,
@@ -232,8 +227,7 @@ int gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha, const double* A, 
     SplitPlan sp;
     int rc = plan_bf16x3(m, n, k, scratch, scratch_bytes, &sp);
     if (rc) return rc;
-    if ((rc = split_a_bf16x3(sp, A, lda, m, k, s))) return rc;
-    if ((rc = split_b_bf16x3(sp, B, ldb, k, n, s))) return rc;
+    if ((rc = split_bf16(sp, A, lda, B, ldb, m, n, k, s))) return rc;
     return product_bf16x3(sp, m, n, k, alpha, beta, C, ldc, D, ldd, err, s);
 }
 
@@ -288,10 +282,20 @@ int gemm_fp64_class(int64_t m, int64_t n, int64_t k, double alpha, const double*
     SplitPlan sp;
     int rc = plan_ozaki(m, n, k, slices, scratch, scratch_bytes, &sp);
     if (rc) return rc;
-    if ((rc = launch_ozaki_split(A, lda, (int)m, (int)k, false, slices, sp.ea, sp.a, sp.ld,
-                                 x.a_known ? nullptr : x.sumsq_a, s, x.active)))
+    SplitSource src;
+    src.A = A;
+    src.lda = lda;
+    src.B = B;
+    src.ldb = ldb;
+    src.active = x.active;
+    if ((rc = launch_exponents(src, (int)m, (int)n, (int)k, sp.ea, sp.eb, x.a_known ? nullptr : x.sumsq_a, x.sumsq_b,
+                               nullptr, s)))
         return rc;
-    if ((rc = split_b_ozaki(sp, B, ldb, k, n, x.sumsq_b, s, x.active))) return rc;
+    if ((rc = launch_split(src,
+                           SplitTarget{SPLIT_DIGITS, slices, 0, (int)m, (int)n, (int)k, 0, (int)m, 0, (int)n, sp.ea,
+                                       sp.eb, sp.a, sp.b, sp.ld},
+                           s)))
+        return rc;
     return product_ozaki(sp, m, n, k, alpha, beta, C, ldc, D, ldd, add_identity, x.sumsq_d, err, s, x.active);
 }
 

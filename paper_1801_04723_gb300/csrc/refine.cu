@@ -3,7 +3,7 @@
 // Sec. 2.1), for one matrix or for every matrix of a batch.
 //
 // Each matrix z has an active flag.  Every refinement round enqueues the same
-// launches (split X, residual R = I - A X, decision, split X and R, update);
+// launches (residual R = I - A X, decision, split X and R, update);
 // the tensor-core products and the splits of a matrix whose flag is 0 return
 // at once, so a round costs a matrix nothing once it has converged.  The
 // decision kernel reads the round's sums of squares, computes
@@ -32,12 +32,13 @@ __global__ void refine_init_kernel(const int32_t* records, int count, int* activ
     iters[z] = 0;
 }
 
-__global__ void refine_decide_kernel(const double* nA, const double* nX, const double* nR, int count, double tol,
+__global__ void refine_decide_kernel(const double* nA, double* nX, double* nR, int count, double tol,
                                      double margin, int it, int max_refine, int* active, double* rel, int* iters,
                                      int32_t* records) {
     const int z = blockIdx.x * blockDim.x + threadIdx.x;
     if (z >= count || active[z] == 0) return;
     const double r = sqrt(nR[z]) / (sqrt(nA[z]) * sqrt(nX[z]));
+    nX[z] = nR[z] = 0.0;  // the next round's sums
     rel[z] = r;
     iters[z] = it;
     if (r + margin <= tol) {
@@ -68,7 +69,7 @@ int launch_refine_init(const int32_t* records, int count, int* active, double* r
     return SPIN_OK;
 }
 
-int launch_refine_decide(const double* nA, const double* nX, const double* nR, int count, double tol, double margin,
+int launch_refine_decide(const double* nA, double* nX, double* nR, int count, double tol, double margin,
                          int it, int max_refine, int* active, double* rel, int* iters, int32_t* records,
                          cudaStream_t s) {
     if (count <= 0) return SPIN_OK;

@@ -1,0 +1,440 @@
+// Operand splits of the tensor-core products.
+//
+// Both operands of a product in one launch: the products of a recursion at
+// small orders are bound by launches, and two half-empty launches cost more
+// than one.  A thread block takes a tile of one operand:
+//   A   32 rows x 128 columns, a warp per row, 4 consecutive columns per lane;
+//   B   128 rows x 32 columns, transposed through shared memory, a warp per
+//       column, 4 consecutive rows per lane;
+// so that every plane is written in 8-byte pieces, 256 bytes per warp.  Bound
+// by HBM (8 bytes read, 2 written per plane and entry) for the BF16 and digit
+// planes, by FP32 arithmetic (6 operations per residue) for the residues.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "crt.h"
+#include "split.h"
+
+namespace spin {
+namespace {
+
+// ------------------------------------------------------------- sources --
+
+struct SideOne {
+    const double* p;
+    int64_t ld;
+    __device__ __forceinline__ const double* row(int, int r) const { return p + (int64_t)r * ld; }
+};
+struct SideMany {
+    BatchView v;
+    __device__ __forceinline__ const double* row(int z, int r) const {
+        const int64_t l = v.ld_of(z);
+        return v.base[z] + (v.r0 + r) * l + v.c0;
+    }
+};
+
+__device__ __forceinline__ bool problem_on(const int* active, int z) { return active == nullptr || active[z] != 0; }
+
+// ----------------------------------------------------------- exponents --
+
+// Biased exponent field of x (0 for zero and subnormals).  The exponent e
+// with max|x| < 2^e (frexp convention) of a row is max(field) - 1022: the
+// largest magnitude has the largest field.  Integer work only.
+__device__ __forceinline__ int exp_field(double x) {
+    return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7FF;
+}
+
+constexpr int kSpreadSteps = 13;  // t = 0, 2, ..., 24
+constexpr int kNoSpread = 1000;
+
+// Least t of 0, 2, ... 24 with count[t] >= 3/4 k (count: entries whose
+// exponent is at least the largest - t).
+__device__ __forceinline__ int spread_of(const int (&count)[kSpreadSteps], int k, int top) {
+    if (top == 0x7FF) return kNoSpread;  // an infinity or NaN
+    int t = kNoSpread;
+#pragma unroll
+    for (int i = kSpreadSteps - 1; i >= 0; i--)
+        if (4ll * count[i] >= 3ll * k) t = 2 * i;
+    return t;
+}
+__device__ __forceinline__ void count_entry(int (&count)[kSpreadSteps], double v, int top) {
+    const int f = exp_field(v), d = f == 0 ? 1 << 20 : top - f;
+#pragma unroll
+    for (int i = 0; i < kSpreadSteps; i++) count[i] += d <= 2 * i;
+}
+
+constexpr int kExpWarps = 16;
+
+// Blocks [0, blocks_a): kExpWarps rows of A, a warp each; the others: 32
+// columns of B, all warps over the rows.
+template <class Side>
+__global__ void __launch_bounds__(32 * kExpWarps)
+exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restrict__ ea, int* __restrict__ eb,
+                 double* sumsq_a, double* sumsq_b, int64_t sss, int* spread, const int* active, const int* valid) {
+    const int z = blockIdx.y;
+    if (!problem_on(active, z)) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nv = valid ? valid[z] : 0x7fffffff;
+    __shared__ int smax[kExpWarps][32];
+    __shared__ int scount[32][kSpreadSteps + 1];
+    __shared__ double ssum[kExpWarps];
+    double ss = 0.0;
+    double* sum;
+    if ((int)blockIdx.x < blocks_a) {
+        sum = sumsq_a;
+        const int r = (int)blockIdx.x * kExpWarps + warp;
+        if (r < m) {
+            const double* p = A.row(z, r);
+            const bool sum_row = sum != nullptr && r < nv;
+            int top = 0;
+            for (int c = lane; c < k; c += 32) {
+                const double v = p[c];
+                top = max(top, exp_field(v));
+                if (sum_row && c < nv) ss = fma(v, v, ss);
+            }
+            top = __reduce_max_sync(0xffffffffu, top);
+            if (lane == 0) ea[(int64_t)z * m + r] = top - 1022;
+            if (spread != nullptr) {
+                int count[kSpreadSteps] = {};
+                bool nonzero = false;
+                for (int c = lane; c < k; c += 32) {
+                    const double v = p[c];
+                    nonzero |= v != 0.0;
+                    count_entry(count, v, top);
+                }
+#pragma unroll
+                for (int i = 0; i < kSpreadSteps; i++) count[i] = __reduce_add_sync(0xffffffffu, count[i]);
+                const bool any = __any_sync(0xffffffffu, nonzero);
+                if (lane == 0 && any) atomicMax(&spread[0], spread_of(count, k, top));
+            }
+        }
+    } else {
+        sum = sumsq_b;
+        const int c = ((int)blockIdx.x - blocks_a) * 32 + lane;
+        const bool col_ok = c < n;
+        const bool sum_col = sum != nullptr && c < nv;
+        int top = 0;
+        double ss4[4] = {0.0, 0.0, 0.0, 0.0};  // a dependent FP64 FMA takes 64 cycles and more here
+        if (col_ok) {
+            int r = warp;
+            for (; r + 3 * kExpWarps < k; r += 4 * kExpWarps) {
+                double v[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) v[u] = B.row(z, r + u * kExpWarps)[c];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    top = max(top, exp_field(v[u]));
+                    if (sum_col && r + u * kExpWarps < nv) ss4[u] = fma(v[u], v[u], ss4[u]);
+                }
+            }
+            for (; r < k; r += kExpWarps) {
+                const double v = B.row(z, r)[c];
+                top = max(top, exp_field(v));
+                if (sum_col && r < nv) ss4[0] = fma(v, v, ss4[0]);
+            }
+        }
+        ss = (ss4[0] + ss4[1]) + (ss4[2] + ss4[3]);
+        smax[warp][lane] = top;
+        if (spread != nullptr)
+            for (int i = threadIdx.x; i < 32 * (kSpreadSteps + 1); i += blockDim.x) (&scount[0][0])[i] = 0;
+        __syncthreads();
+        top = 0;
+#pragma unroll
+        for (int w = 0; w < kExpWarps; w++) top = max(top, smax[w][lane]);
+        if (warp == 0 && col_ok) eb[(int64_t)z * n + c] = top - 1022;
+        if (spread != nullptr) {
+            int count[kSpreadSteps] = {};
+            int nonzero = 0;
+            if (col_ok)
+                for (int r = warp; r < k; r += kExpWarps) {
+                    const double v = B.row(z, r)[c];
+                    nonzero |= v != 0.0;
+                    count_entry(count, v, top);
+                }
+#pragma unroll
+            for (int i = 0; i < kSpreadSteps; i++)
+                if (count[i]) atomicAdd(&scount[lane][i], count[i]);
+            if (nonzero) scount[lane][kSpreadSteps] = 1;
+            __syncthreads();
+            if (warp == 0 && col_ok && scount[lane][kSpreadSteps]) {
+#pragma unroll
+                for (int i = 0; i < kSpreadSteps; i++) count[i] = scount[lane][i];
+                atomicMax(&spread[1], spread_of(count, k, top));
+            }
+        }
+    }
+    if (sum != nullptr) {  // the same for the whole block
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) ss += __shfl_down_sync(0xffffffffu, ss, off);
+        if (lane == 0) ssum[warp] = ss;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kExpWarps; w++) ss += ssum[w];
+            if (ss != 0.0) atomicAdd(sum + (int64_t)z * sss, ss);
+        }
+    }
+}
+
+// --------------------------------------------------------- conversions --
+// Each writes the planes' entries of 4 consecutive K positions.
+
+__device__ __forceinline__ unsigned bf16_bits(float f) { return __bfloat16_as_ushort(__float2bfloat16_rn(f)); }
+
+__device__ __forceinline__ void store4(uint16_t* dst, unsigned a, unsigned b, unsigned c, unsigned d) {
+    *reinterpret_cast<uint2*>(dst) = make_uint2(a | (b << 16), c | (d << 16));
+}
+
+// hi = bf16(x), lo = bf16(x - hi) (three planes: hi, mid, lo), computed from
+// xf = fp32(x): one FP64 operation per element (GB300's FP64 rate would
+// otherwise bound this memory-bound pass); xf differs from x by 2^-24
+// relative, far below what the three-product form keeps (~2^-16).
+template <int PLANES>
+struct ToBf16 {
+    __device__ __forceinline__ void operator()(const double (&x)[4], int, uint16_t* dst, int64_t plane) const {
+        float r[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) r[u] = __double2float_rn(x[u]);
+#pragma unroll
+        for (int q = 0; q < PLANES; q++) {
+            __nv_bfloat16 h[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                h[u] = __float2bfloat16_rn(r[u]);
+                r[u] -= __bfloat162float(h[u]);  // exact in FP32
+            }
+            store4(dst + q * plane, __bfloat16_as_ushort(h[0]), __bfloat16_as_ushort(h[1]), __bfloat16_as_ushort(h[2]),
+                   __bfloat16_as_ushort(h[3]));
+        }
+    }
+};
+
+// round(|x| 2^(b - e)), |x| < 2^e, ties away from zero: integer arithmetic on
+// the IEEE fields.
+__device__ __forceinline__ unsigned long long fixed_point(double x, int e, int b) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    int fe = (int)(u >> 52) & 0x7FF;
+    unsigned long long m = u & ((1ull << 52) - 1);
+    if (fe == 0)
+        fe = 1;  // subnormal: no implicit bit
+    else
+        m |= 1ull << 52;
+    const int sh = fe - 1075 + b - e;  // <= b - 53
+    if (sh >= 0) return m << sh;
+    return sh > -64 ? (m + (1ull << (-sh - 1))) >> (-sh) : 0ull;
+}
+
+// Fixed-point digits of x relative to 2^e (|x| < 2^e): N = round(|x| 2^(8s -
+// 1 - e)) in balanced base 256 (low digits in [-128, 127], the top one in
+// [-128, 128]), so x = 2^(e-7) sum_i d_i 2^(-8 i) to within half a unit of the
+// last slice.
+struct ToDigits {
+    int planes;
+    __device__ __forceinline__ void operator()(const double (&x)[4], int e, uint16_t* dst, int64_t plane) const {
+        unsigned long long n[4];
+        bool neg[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            n[u] = fixed_point(x[u], e, 8 * planes - 1);
+            neg[u] = __double2hiint(x[u]) < 0;
+        }
+        for (int q = planes - 1; q >= 0; q--) {
+            unsigned d[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                int v = q > 0 ? (int)(n[u] & 255u) : (int)n[u];
+                if (q > 0) {
+                    n[u] >>= 8;
+                    if (v >= 128) {
+                        v -= 256;
+                        n[u] += 1;
+                    }
+                }
+                d[u] = bf16_bits((float)(neg[u] ? -v : v));  // |d| <= 128: exact
+            }
+            store4(dst + q * plane, d[0], d[1], d[2], d[3]);
+        }
+    }
+};
+
+// Residues of the signed fixed-point integer: cut into PIECES balanced 14-bit
+// pieces, each residue is one FP32 dot product of the pieces with the powers
+// of 2^14 modulo p (every partial sum below 2^23, exact) minus p times the
+// rounded quotient; |r| <= 128, exact in BF16.
+constexpr int kPiece = 14;
+
+__host__ __device__ constexpr int piece_weight(int l, int q) {  // 2^(14 q) modulo p, balanced
+    const int p = crt_modulus(l);
+    int v = 1;
+    for (int i = 0; i < q; i++) v = v * (1 << kPiece) % p;
+    return v > p / 2 ? v - p : v;
+}
+
+template <int PIECES>
+struct ToResidues {
+    int bits, moduli;
+    __device__ __forceinline__ void operator()(const double (&x)[4], int e, uint16_t* dst, int64_t plane) const {
+        float f[4][PIECES];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const unsigned long long n = fixed_point(x[u], e, bits);
+            long long v = __double2hiint(x[u]) < 0 ? -(long long)n : (long long)n;
+#pragma unroll
+            for (int q = 0; q < PIECES; q++) {
+                int d;
+                if (q + 1 < PIECES) {
+                    d = (int)((unsigned)v << (32 - kPiece)) >> (32 - kPiece);  // low 14 bits, signed
+                    v = (v - d) >> kPiece;
+                } else {
+                    d = (int)v;
+                }
+                // d as FP32 without a conversion (16 per clock per SM): |d| < 2^22
+                f[u][q] = __uint_as_float(0x4B400000u + (unsigned)d) - 12582912.0f;
+            }
+        }
+#pragma unroll
+        for (int l = 0; l < kCrtMaxModuli; l++) {
+            if (l >= moduli) break;
+            const float p = (float)crt_modulus(l), inv_p = 1.0f / (float)crt_modulus(l);
+            unsigned r[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                float t = f[u][0];
+#pragma unroll
+                for (int q = 1; q < PIECES; q++) t = fmaf(f[u][q], (float)piece_weight(l, q), t);
+                const float quot = fmaf(t, inv_p, 12582912.0f) - 12582912.0f;
+                r[u] = __float_as_uint(fmaf(-quot, p, t));
+            }
+            // the high halves: the BF16 values (the rest of the words is zero)
+            *reinterpret_cast<uint2*>(dst + l * plane) =
+                make_uint2(__byte_perm(r[0], r[1], 0x7632), __byte_perm(r[2], r[3], 0x7632));
+        }
+    }
+};
+
+// --------------------------------------------------------------- kernel --
+
+constexpr int kTileRows = 32, kTileK = 128;
+constexpr int kTileLd = kTileK + 2;  // even: 16-byte reads
+
+template <class Side, class Convert>
+__global__ void __launch_bounds__(256)
+split_kernel(Side A, Side B, const __grid_constant__ SplitTarget t, int64_t tiles_a, Convert convert,
+             const int* active) {
+    __shared__ __align__(16) double tile[kTileRows][kTileLd];
+    const int z = blockIdx.y;
+    if (!problem_on(active, z)) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ktiles = (t.k + kTileK - 1) / kTileK;
+    if ((int64_t)blockIdx.x < tiles_a) {
+        const int64_t plane = (int64_t)t.rows * t.ld;
+        uint16_t* dst = t.a + (int64_t)z * t.planes * plane;
+        const int r0 = (int)(blockIdx.x / ktiles) * kTileRows, c = (int)(blockIdx.x % ktiles) * kTileK + 4 * lane;
+        if (c >= t.k) return;
+#pragma unroll
+        for (int i = warp; i < kTileRows; i += 8) {
+            const int r = r0 + i;
+            if (r >= t.rows) break;
+            const double* p = A.row(z, t.row0 + r) + c;
+            double x[4];
+            if (c + 3 < t.k && ((uintptr_t)p & 15u) == 0) {
+                const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
+                x[0] = a.x;
+                x[1] = a.y;
+                x[2] = b.x;
+                x[3] = b.y;
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; u++) x[u] = c + u < t.k ? p[u] : 0.0;
+            }
+            const int e = t.ea ? t.ea[(int64_t)z * t.m + t.row0 + r] : 0;
+            convert(x, e, dst + (int64_t)r * t.ld + c, plane);
+        }
+        return;
+    }
+    const int64_t id = (int64_t)blockIdx.x - tiles_a;
+    const int64_t plane = (int64_t)t.cols * t.ld;
+    uint16_t* dst = t.b + (int64_t)z * t.planes * plane;
+    // neighbouring blocks take neighbouring columns: whole lines of B
+    const int ctiles = (t.cols + kTileRows - 1) / kTileRows;
+    const int c0 = (int)(id % ctiles) * kTileRows, r0 = (int)(id / ctiles) * kTileK;
+#pragma unroll 4
+    for (int i = warp; i < kTileK; i += 8) {
+        const int r = r0 + i, c = c0 + lane;
+        tile[lane][i] = (r < t.k && c < t.cols) ? B.row(z, r)[t.col0 + c] : 0.0;
+    }
+    __syncthreads();
+    const int r = r0 + 4 * lane;
+    if (r >= t.k) return;
+#pragma unroll
+    for (int i = warp; i < kTileRows; i += 8) {
+        const int c = c0 + i;
+        if (c >= t.cols) break;
+        const double2 a = *reinterpret_cast<const double2*>(&tile[i][4 * lane]);
+        const double2 b = *reinterpret_cast<const double2*>(&tile[i][4 * lane + 2]);
+        const double x[4] = {a.x, a.y, b.x, b.y};
+        const int e = t.eb ? t.eb[(int64_t)z * t.n + t.col0 + c] : 0;
+        convert(x, e, dst + (int64_t)c * t.ld + r, plane);
+    }
+}
+
+template <class Side, class Convert>
+int split_with(Side A, Side B, const SplitTarget& t, Convert c, int count, const int* active, cudaStream_t s) {
+    const int64_t ktiles = (t.k + kTileK - 1) / kTileK;
+    const int64_t ta = ktiles * ((t.rows + kTileRows - 1) / kTileRows), tb = ktiles * ((t.cols + kTileRows - 1) / kTileRows);
+    if (ta + tb <= 0) return SPIN_OK;
+    if (ta + tb > INT32_MAX) return SPIN_ERR_INVALID_ARG;
+    split_kernel<Side, Convert><<<dim3((unsigned)(ta + tb), (unsigned)count), 256, 0, s>>>(A, B, t, ta, c, active);
+    SPIN_CUDA_TRY(cudaGetLastError());
+    return SPIN_OK;
+}
+
+template <class Side>
+int split_sides(Side A, Side B, const SplitTarget& t, int count, const int* active, cudaStream_t s) {
+    switch (t.kind) {
+        case SPLIT_BF16:
+            if (t.planes == 2) return split_with(A, B, t, ToBf16<2>(), count, active, s);
+            if (t.planes == 3) return split_with(A, B, t, ToBf16<3>(), count, active, s);
+            return SPIN_ERR_INVALID_ARG;
+        case SPLIT_DIGITS:
+            if (t.planes < 1 || t.planes > 7) return SPIN_ERR_INVALID_ARG;
+            return split_with(A, B, t, ToDigits{t.planes}, count, active, s);
+        default:
+            if (t.planes < 1 || t.planes > kCrtMaxModuli || t.bits < 1 || t.bits > kCrtMaxBits)
+                return SPIN_ERR_INVALID_ARG;
+            if (t.bits <= 4 * kPiece - 1)
+                return split_with(A, B, t, ToResidues<4>{t.bits, t.planes}, count, active, s);
+            return split_with(A, B, t, ToResidues<5>{t.bits, t.planes}, count, active, s);
+    }
+}
+
+template <class Side>
+int exponents_sides(Side A, Side B, const SplitSource& src, int m, int n, int k, int* ea, int* eb, double* sa,
+                    double* sb, int* spread, int count, int64_t sss, cudaStream_t s) {
+    const int ba = ea ? (m + kExpWarps - 1) / kExpWarps : 0, bb = eb ? (n + 31) / 32 : 0;
+    if (ba + bb == 0) return SPIN_OK;
+    exponents_kernel<Side><<<dim3((unsigned)(ba + bb), (unsigned)count), 32 * kExpWarps, 0, s>>>(
+        A, B, m, n, k, ba, ea, eb, sa, sb, sss, spread, src.active, src.valid);
+    SPIN_CUDA_TRY(cudaGetLastError());
+    return SPIN_OK;
+}
+
+}  // namespace
+
+int launch_exponents(const SplitSource& src, int m, int n, int k, int* ea, int* eb, double* sumsq_a, double* sumsq_b,
+                     int* spread, cudaStream_t s) {
+    if (src.count > 65535 || (spread != nullptr && src.count > 0)) return SPIN_ERR_INVALID_ARG;
+    if (src.count > 0)
+        return exponents_sides(SideMany{src.Av}, SideMany{src.Bv}, src, m, n, k, ea, eb, sumsq_a, sumsq_b, spread,
+                               src.count, 1, s);
+    return exponents_sides(SideOne{src.A, src.lda}, SideOne{src.B, src.ldb}, src, m, n, k, ea, eb, sumsq_a, sumsq_b,
+                           spread, 1, 0, s);
+}
+
+int launch_split(const SplitSource& src, const SplitTarget& t, cudaStream_t s) {
+    if (src.count > 65535) return SPIN_ERR_INVALID_ARG;
+    if (src.count > 0) return split_sides(SideMany{src.Av}, SideMany{src.Bv}, t, src.count, src.active, s);
+    return split_sides(SideOne{src.A, src.lda}, SideOne{src.B, src.ldb}, t, 1, src.active, s);
+}
+
+}  // namespace spin

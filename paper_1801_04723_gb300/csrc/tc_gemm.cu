@@ -763,207 +763,6 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
 }
 
-// ------------------------------------------------------------ splitting --
-
-// hi = bf16(x), lo = bf16(x - hi), both computed from xf = fp32(x): one
-// FP64 operation per element (GB300's FP64 rate would otherwise bound this
-// memory-bound pass); xf differs from x by 2^-24 relative, far below what
-// the three-product form keeps (~2^-16).
-__device__ __forceinline__ void split2(double a, uint16_t& hi, uint16_t& lo) {
-    const float xf = __double2float_rn(a);
-    const __nv_bfloat16 h = __float2bfloat16_rn(xf);
-    hi = __bfloat16_as_ushort(h);
-    lo = bf16_bits(xf - __bfloat162float(h));  // exact in FP32
-}
-
-// hi, mid, lo planes: the same from xf with one more level.
-__device__ __forceinline__ void split3(double a, uint16_t& hi, uint16_t& mid, uint16_t& lo) {
-    const float xf = __double2float_rn(a);
-    const __nv_bfloat16 h = __float2bfloat16_rn(xf);
-    const float r1 = xf - __bfloat162float(h);  // exact in FP32
-    const __nv_bfloat16 m = __float2bfloat16_rn(r1);
-    hi = __bfloat16_as_ushort(h);
-    mid = __bfloat16_as_ushort(m);
-    lo = bf16_bits(r1 - __bfloat162float(m));  // exact in FP32
-}
-
-// Every split kernel handles problem z = blockIdx.z: its planes start at
-// dst + z * dzs, its exponents at ex + z * exs, its sum of squares at
-// sumsq[z * sss] (sss = 0: one shared sum).
-
-template <class Src>
-__global__ void split_bf16x3p_rows_kernel(Src src, int rows, int cols, uint16_t* __restrict__ dst, int64_t ldd,
-                                          int64_t plane, int64_t dzs) {
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    dst += z * dzs;
-    const int64_t total = (int64_t)rows * cols;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / cols), c = (int)(idx % cols);
-        uint16_t hi, mid, lo;
-        split3(src.row(z, r)[c], hi, mid, lo);
-        const int64_t o = (int64_t)r * ldd + c;
-        dst[o] = hi;
-        dst[plane + o] = mid;
-        dst[2 * plane + o] = lo;
-    }
-}
-
-template <class Src>
-__global__ void split_bf16x3p_cols_kernel(Src src, int rows, int cols, uint16_t* __restrict__ dst, int64_t ldd,
-                                          int64_t plane, int64_t dzs) {
-    __shared__ double tile[32][33];
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    dst += z * dzs;
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        tile[i][threadIdx.x] = (r < rows && c < cols) ? src.row(z, r)[c] : 0.0;
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (c < cols && r < rows) {
-            uint16_t hi, mid, lo;
-            split3(tile[threadIdx.x][i], hi, mid, lo);
-            const int64_t o = (int64_t)c * ldd + r;
-            dst[o] = hi;
-            dst[plane + o] = mid;
-            dst[2 * plane + o] = lo;
-        }
-    }
-}
-
-// Row-major FP64 (rows x cols) -> two BF16 planes [2][rows][ldd].
-template <class Src>
-__global__ void split_bf16x2_rows_kernel(Src src, int rows, int cols, uint16_t* __restrict__ dst, int64_t ldd,
-                                         int64_t plane, int64_t dzs) {
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    dst += z * dzs;
-    const int64_t total = (int64_t)rows * cols;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / cols), c = (int)(idx % cols);
-        uint16_t hi, lo;
-        split2(src.row(z, r)[c], hi, lo);
-        dst[(int64_t)r * ldd + c] = hi;
-        dst[plane + (int64_t)r * ldd + c] = lo;
-    }
-}
-
-// FP64 (rows=K x cols=N) -> transposed BF16 planes [2][N][ldd] (N x K).
-template <class Src>
-__global__ void split_bf16x2_cols_kernel(Src src, int rows, int cols, uint16_t* __restrict__ dst, int64_t ldd,
-                                         int64_t plane, int64_t dzs) {
-    __shared__ double tile[32][33];
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    dst += z * dzs;
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        tile[i][threadIdx.x] = (r < rows && c < cols) ? src.row(z, r)[c] : 0.0;
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;  // output row c (a column of src), output col r
-        if (c < cols && r < rows) {
-            uint16_t hi, lo;
-            split2(tile[threadIdx.x][i], hi, lo);
-            dst[(int64_t)c * ldd + r] = hi;
-            dst[plane + (int64_t)c * ldd + r] = lo;
-        }
-    }
-}
-
-// Fixed-point digits of x relative to 2^e (|x| < 2^e): with t = x 2^(7-e)
-// (|t| < 128), N = round(|t| 2^(8(s-1))) is an integer below 2^(8s-1);
-// its balanced base-256 digits (low digits in [-128, 127], the top one in
-// [-128, 128]) are the slices, so x = 2^(e-7) sum_i d_i 2^(-8 i) to within
-// half a unit of the last slice.  Integer arithmetic on the IEEE fields.
-template <int MAXS>
-__device__ __forceinline__ void digits(double x, int e, int nslices, uint16_t (&d)[MAXS]) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const bool neg = (b >> 63) != 0;
-    int fe = (int)(b >> 52) & 0x7FF;
-    unsigned long long m = b & ((1ull << 52) - 1);
-    if (fe == 0)
-        fe = 1;  // subnormal: no implicit bit
-    else
-        m |= 1ull << 52;
-    const int sh = fe - 1075 + 7 - e + 8 * (nslices - 1);  // |x| 2^(7-e+8(s-1)) = m 2^sh
-    unsigned long long N;
-    if (sh >= 0)
-        N = m << sh;  // < 2^(8 s - 1) because |t| < 128
-    else if (sh > -64)
-        N = (m + (1ull << (-sh - 1))) >> (-sh);
-    else
-        N = 0;
-    int dig[MAXS];
-#pragma unroll
-    for (int i = MAXS - 1; i >= 1; i--) {
-        if (i < nslices) {
-            int v = (int)(N & 255u);
-            N >>= 8;
-            if (v >= 128) {
-                v -= 256;
-                N += 1;
-            }
-            dig[i] = v;
-        }
-    }
-    dig[0] = (int)N;
-#pragma unroll
-    for (int i = 0; i < MAXS; i++)
-        if (i < nslices) d[i] = bf16_bits((float)(neg ? -dig[i] : dig[i]));  // |d| <= 128: exact
-}
-
-constexpr int kMaxSlices = 8;
-
-template <class Src>
-__global__ void ozaki_rows_kernel(Src src, int rows, int cols, const int* __restrict__ ex, int64_t exs, int nslices,
-                                  uint16_t* __restrict__ dst, int64_t ldd, int64_t plane, int64_t dzs) {
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    dst += z * dzs;
-    ex += z * exs;
-    const int64_t total = (int64_t)rows * cols;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / cols), c = (int)(idx % cols);
-        uint16_t d[kMaxSlices];
-        digits<kMaxSlices>(src.row(z, r)[c], ex[r], nslices, d);
-        for (int q = 0; q < nslices; q++) dst[q * plane + (int64_t)r * ldd + c] = d[q];
-    }
-}
-
-template <class Src>
-__global__ void ozaki_cols_kernel(Src src, int rows, int cols, const int* __restrict__ ex, int64_t exs, int nslices,
-                                  uint16_t* __restrict__ dst, int64_t ldd, int64_t plane, int64_t dzs) {
-    __shared__ double tile[32][33];
-    const int z = blockIdx.z;
-    if (!src.on(z)) return;
-    dst += z * dzs;
-    ex += z * exs;
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        tile[i][threadIdx.x] = (r < rows && c < cols) ? src.row(z, r)[c] : 0.0;
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (c < cols && r < rows) {
-            uint16_t d[kMaxSlices];
-            digits<kMaxSlices>(tile[threadIdx.x][i], ex[c], nslices, d);
-            for (int q = 0; q < nslices; q++) dst[q * plane + (int64_t)c * ldd + r] = d[q];
-        }
-    }
-}
-
 // Float-mode products (bf16x3, bf16x6) run on persistent CTAs, one per SM
 // looping over the tiles: a float tile drains its one accumulator after its
 // last MMA, which the next tile's MMAs now overlap (n = 8192 bf16x3: 2.51
@@ -1108,81 +907,6 @@ int launch_tc_gemm(const TcOperand& a, const TcOperand& b, const TcGemmParams& p
         return launch_impl<kExactBN, true, kExactEpiWarps>(a, b, p, s);
     }
     return launch_impl<kFloatBN, false, 8>(a, b, p, s);
-}
-
-namespace {
-
-template <class Src>
-int split_planes(Src src, int rows, int cols, bool transpose, int planes, uint16_t* dst, int64_t ldd, int count,
-                 cudaStream_t s) {
-    if (rows <= 0 || cols <= 0 || count <= 0) return SPIN_OK;
-    const int64_t plane = (int64_t)(transpose ? cols : rows) * ldd;
-    const int64_t dzs = planes * plane;
-    if (!transpose) {
-        const dim3 g = rows_grid((int64_t)rows * cols, count);
-        if (planes == 2)
-            split_bf16x2_rows_kernel<Src><<<g, 256, 0, s>>>(src, rows, cols, dst, ldd, plane, dzs);
-        else
-            split_bf16x3p_rows_kernel<Src><<<g, 256, 0, s>>>(src, rows, cols, dst, ldd, plane, dzs);
-    } else {
-        const dim3 g((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32), (unsigned)count);
-        if (planes == 2)
-            split_bf16x2_cols_kernel<Src><<<g, dim3(32, 8), 0, s>>>(src, rows, cols, dst, ldd, plane, dzs);
-        else
-            split_bf16x3p_cols_kernel<Src><<<g, dim3(32, 8), 0, s>>>(src, rows, cols, dst, ldd, plane, dzs);
-    }
-    SPIN_CUDA_TRY(cudaGetLastError());
-    return SPIN_OK;
-}
-
-template <class Src>
-int split_digits(Src src, int rows, int cols, bool transpose, int nslices, int* ex, uint16_t* dst, int64_t ldd,
-                 double* sumsq, int64_t sss, int count, cudaStream_t s) {
-    if (rows <= 0 || cols <= 0 || count <= 0) return SPIN_OK;
-    if (nslices < 1 || nslices > kMaxSlices) return SPIN_ERR_INVALID_ARG;
-    const int rc = operand_exponents(src, rows, cols, transpose, ex, sumsq, sss, count, s);
-    if (rc) return rc;
-    if (!transpose) {
-        const int64_t plane = (int64_t)rows * ldd, dzs = nslices * plane;
-        ozaki_rows_kernel<Src><<<rows_grid((int64_t)rows * cols, count), 256, 0, s>>>(src, rows, cols, ex, rows,
-                                                                                      nslices, dst, ldd, plane, dzs);
-    } else {
-        const int64_t plane = (int64_t)cols * ldd, dzs = nslices * plane;
-        const dim3 g((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32), (unsigned)count);
-        ozaki_cols_kernel<Src><<<g, dim3(32, 8), 0, s>>>(src, rows, cols, ex, cols, nslices, dst, ldd, plane, dzs);
-    }
-    SPIN_CUDA_TRY(cudaGetLastError());
-    return SPIN_OK;
-}
-
-}  // namespace
-
-int launch_split_bf16x2(const double* src, int64_t lds, int rows, int cols, bool transpose, uint16_t* dst,
-                        int64_t ldd, cudaStream_t s) {
-    return split_planes(SrcOne{src, lds, nullptr}, rows, cols, transpose, 2, dst, ldd, 1, s);
-}
-
-int launch_split_bf16x3p(const double* src, int64_t lds, int rows, int cols, bool transpose, uint16_t* dst,
-                         int64_t ldd, cudaStream_t s, const int* active) {
-    return split_planes(SrcOne{src, lds, active}, rows, cols, transpose, 3, dst, ldd, 1, s);
-}
-
-int launch_ozaki_split(const double* src, int64_t lds, int rows, int cols, bool transpose, int nslices, int* ex,
-                       uint16_t* dst, int64_t ldd, double* sumsq, cudaStream_t s, const int* active) {
-    return split_digits(SrcOne{src, lds, active}, rows, cols, transpose, nslices, ex, dst, ldd, sumsq, 0, 1, s);
-}
-
-int launch_split_planes_batched(const BatchView& src, int rows, int cols, bool transpose, int planes,
-                                uint16_t* dst, int64_t ldd, int count, cudaStream_t s, const int* active) {
-    if (planes != 2 && planes != 3) return SPIN_ERR_INVALID_ARG;
-    return split_planes(SrcMany{src, active, nullptr}, rows, cols, transpose, planes, dst, ldd, count, s);
-}
-
-int launch_ozaki_split_batched(const BatchView& src, int rows, int cols, bool transpose, int nslices, int* ex,
-                               uint16_t* dst, int64_t ldd, double* sumsq, int count, cudaStream_t s,
-                               const int* active, const int* valid) {
-    return split_digits(SrcMany{src, active, valid}, rows, cols, transpose, nslices, ex, dst, ldd, sumsq, 1, count,
-                        s);
 }
 
 }  // namespace spin

@@ -61,28 +61,5 @@ struct TcGemmParams {
 
 int64_t tc_ld(int64_t k);
 int launch_tc_gemm(const TcOperand& a, const TcOperand& b, const TcGemmParams& p, cudaStream_t s);
-// FP64 view -> (hi, mid, lo) BF16 planes; transpose=true writes the cols x rows transpose.
-// active (optional, device): split only while *active != 0.
-int launch_split_bf16x3p(const double* src, int64_t lds, int rows, int cols, bool transpose, uint16_t* dst,
-                         int64_t ldd, cudaStream_t s, const int* active = nullptr);
-// FP64 view -> (hi, lo) BF16 planes; transpose=true writes the cols x rows transpose.
-int launch_split_bf16x2(const double* src, int64_t lds, int rows, int cols, bool transpose, uint16_t* dst,
-                        int64_t ldd, cudaStream_t s);
-// FP64 view -> nslices fixed-point digit planes plus per-row (or, transposed,
-// per-column) exponents in ex; sumsq (optional) += sum of squares of src.
-int launch_ozaki_split(const double* src, int64_t lds, int rows, int cols, bool transpose, int nslices, int* ex,
-                       uint16_t* dst, int64_t ldd, double* sumsq, cudaStream_t s, const int* active = nullptr);
-
-// Batched forms: problem z's FP64 view is src(z); its planes start at
-// dst + z * planes * (transpose ? cols : rows) * ldd (the slice stack a
-// batched product expects), its exponents at ex + z * (rows or cols) and its
-// sum of squares at sumsq[z] (sumsq optional); problem z is split only while
-// active[z] != 0 (active optional, device); with valid (optional, device) the
-// sum of squares of problem z covers its leading valid[z] x valid[z] block.
-int launch_split_planes_batched(const BatchView& src, int rows, int cols, bool transpose, int planes,
-                                uint16_t* dst, int64_t ldd, int count, cudaStream_t s, const int* active = nullptr);
-int launch_ozaki_split_batched(const BatchView& src, int rows, int cols, bool transpose, int nslices, int* ex,
-                               uint16_t* dst, int64_t ldd, double* sumsq, int count, cudaStream_t s,
-                               const int* active = nullptr, const int* valid = nullptr);
 
 }  // namespace spin
