@@ -61,6 +61,36 @@ __device__ __forceinline__ void record_failure(int32_t* info, int code, int leaf
     }
 }
 
+// Conversions between FP32 and FP64 on the integer units, with the results of
+// the hardware's.  Those run on the FP64 pipe, one warp instruction per 16
+// clocks and SM, and bounded the passes that did little else: the float-mode
+// products' drain and the BF16 splits.
+__device__ __forceinline__ double f32_to_f64(unsigned bits) {
+    const unsigned u = bits & 0x7fffffffu;
+    if (u - 0x00800000u >= 0x7f000000u && u != 0u) return (double)__uint_as_float(bits);  // subnormal, infinity, NaN
+    const unsigned hi = (bits & 0x80000000u) | (u ? (u >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ float f64_to_f32_rn(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u < 253u) {  // a normal FP32 value, rounded up or not
+        const unsigned m = ((hi & 0x7fffffffu) << 3 | lo >> 29) - 0xC0000000u;  // exponent re-biased, 23 bits
+        const unsigned rest = lo << 3;
+        return __uint_as_float((hi & 0x80000000u) |
+                               (m + (rest > 0x80000000u || (rest == 0x80000000u && (m & 1u)) ? 1u : 0u)));
+    }
+    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
+    return __double2float_rn(x);
+}
+
+// a + b where it stands: an FP64 operation under a condition that the compiler
+// must not compute for everyone and select afterwards.
+__device__ __forceinline__ double add_now(double a, double b) {
+    double r;
+    asm volatile("add.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
+}
 // A strided view inside each matrix of a batch: problem z's view starts at
 // base[z] + r0 * ld + c0, with ld = lds[z] when lds is given, else ld.
 struct BatchView {

@@ -22,9 +22,9 @@
 //            modulus is a work item of its own, so small products still fill
 //            the SMs, and the drain is a conversion and an add per run.
 //   combine  sum / P = frac(sum_l c_l u_l / p_l) with u_l the inverse of P /
-//            p_l modulo p_l: one 128-bit fixed-point accumulation per output
-//            with the constants u_l 2^128 / p_l (four 32-bit limbs, no carries
-//            between moduli), then times P 2^(e + f - 2 b), rounded once to
+//            p_l modulo p_l: one 96- or 128-bit fixed-point accumulation per
+//            output with the constants u_l 2^128 / p_l (32-bit limbs, no
+//            carries between moduli), then times P 2^(e + f - 2 b), rounded once to
 //            FP64, and the product's epilogue (alpha, beta C, identity, sum of
 //            squares).
 // The integers are exact and every output depends on its row and column
@@ -307,7 +307,10 @@ __device__ __forceinline__ double crt_value(unsigned long long hi, unsigned long
 }
 
 // 4 columns of a row per thread.  p: the whole product (views, epilogue);
-// (row0, col0): the panel pair's origin; rows x cols its size.
+// (row0, col0): the panel pair's origin; rows x cols its size.  LIMBS 32-bit
+// limbs of the fraction: 3 leave an error of 2^-84 P, i.e. below 2^-60 of the
+// largest entries' product for the formats that use it (bits <= 55).
+template <int LIMBS>
 __global__ void __launch_bounds__(256)
 crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int cols, int row0, int col0,
                    const __grid_constant__ CrtTable t, const __grid_constant__ TcGemmParams p) {
@@ -320,16 +323,17 @@ crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int c
     const int groups = (cols + 3) / 4;
     const int64_t total = (int64_t)rows * groups;
     const int so = p.sum_order ? p.sum_order[z] : 0x7fffffff;
-    double ss = 0.0;
+    const bool add = p.beta != 0.0;
+    double ss = 0.0, ss2 = 0.0;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(idx / groups), c = (int)(idx % groups) * 4;
         const uint8_t* src = res + (int64_t)r * ldr + c;
-        unsigned long long acc[4][4];
+        unsigned long long acc[4][LIMBS];
 #pragma unroll
         for (int u = 0; u < 4; u++)
 #pragma unroll
-            for (int i = 0; i < 4; i++) acc[u][i] = 0ull;
+            for (int i = 0; i < LIMBS; i++) acc[u][i] = 0ull;
 #pragma unroll 4
         for (int l = 0; l < t.moduli; l++) {
             const unsigned w = *reinterpret_cast<const unsigned*>(src + l * plane);
@@ -337,31 +341,72 @@ crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int c
             for (int u = 0; u < 4; u++) {
                 const unsigned b = (w >> (8 * u)) & 255u;
 #pragma unroll
-                for (int i = 0; i < 4; i++) acc[u][i] += (unsigned long long)b * t.v[l][i];
+                for (int i = 0; i < LIMBS; i++) acc[u][i] += (unsigned long long)b * t.v[l][4 - LIMBS + i];
             }
         }
         const int er = row_exp[r], grow = row0 + r;
-        const double* crow = p.beta != 0.0 ? in_row(p, z, grow) : nullptr;
-        double* drow = out_row(p, z, grow);
+        const double* crow = add ? in_row(p, z, grow) + col0 + c : nullptr;
+        double* drow = out_row(p, z, grow) + col0 + c;
+        double val[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            if (c + u >= cols) break;
-            const int gcol = col0 + c + u, ec = col_exp[c + u];
-            const unsigned long long s1 = acc[u][1] + (acc[u][0] >> 32);
-            const unsigned long long s2 = acc[u][2] + (s1 >> 32);
-            const unsigned long long s3 = acc[u][3] + (s2 >> 32);
-            double val = crt_value((s3 << 32) | (s2 & 0xffffffffull), (s1 << 32) | (acc[u][0] & 0xffffffffull), t,
-                                   er + ec - 2 * t.bits, p.alpha < 0.0);
+            const int ec = c + u < cols ? col_exp[c + u] : 0;
+            unsigned w[LIMBS];  // the limbs, carried
+            unsigned long long carry = 0ull;
+#pragma unroll
+            for (int i = 0; i < LIMBS; i++) {
+                carry += acc[u][i];
+                w[i] = (unsigned)carry;
+                carry >>= 32;
+            }
+            const unsigned long long hi = (unsigned long long)w[LIMBS - 1] << 32 | w[LIMBS - 2];
+            const unsigned long long lo = LIMBS == 4 ? (unsigned long long)w[1] << 32 | w[0] : (unsigned long long)w[0] << 32;
+            val[u] = crt_value(hi, lo, t, er + ec - 2 * t.bits, p.alpha < 0.0);
             // an infinity or NaN in the row or column (no fixed point has it)
-            if (er > 1024 || ec > 1024) val = __longlong_as_double(0x7ff8000000000000ll);
-            if (p.beta != 0.0) val = fma(p.beta, crow[gcol], val);
-            if (p.add_identity && gcol == grow) val += 1.0;
-            drow[gcol] = val;
-            if (p.sumsq && grow < so && gcol < so) ss = fma(val, val, ss);
+            if (er > 1024 || ec > 1024) val[u] = __longlong_as_double(0x7ff8000000000000ll);
+        }
+        const int gcol = col0 + c;
+        // whole 32-byte sectors where the views allow it
+        const bool quad = c + 3 < cols && aligned32(drow) && (!add || aligned32(crow));
+        if (add) {  // beta = 1
+            double old[4];
+            if (quad) {
+                ld_global_v4(crow, old);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; u++) old[u] = c + u < cols ? crow[u] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) val[u] = old[u] + val[u];
+        }
+        if (p.add_identity && (unsigned)(grow - gcol) < 4u) {
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (gcol + u == grow) val[u] = add_now(val[u], 1.0);
+        }
+        if (p.sumsq && grow < so) {
+            if (c + 3 < cols && gcol + 3 < so) {
+                ss = fma(val[0], val[0], ss);
+                ss2 = fma(val[1], val[1], ss2);
+                ss = fma(val[2], val[2], ss);
+                ss2 = fma(val[3], val[3], ss2);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    if (gcol + u < so && c + u < cols) ss = fma(val[u], val[u], ss);
+            }
+        }
+        if (quad) {
+            st_global_v4(drow, val);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (c + u < cols) drow[u] = val[u];
         }
     }
     if (p.sumsq) {
         __shared__ double part[8];
+        ss += ss2;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) ss += __shfl_down_sync(0xffffffffu, ss, off);
         if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = ss;
@@ -579,7 +624,10 @@ int crt_run(const CrtProduct& p, const CrtFormat& f, const CrtPanels& c, unsigne
             const int64_t total = (int64_t)rows * ((cols + 3) / 4);
             const int64_t per = std::max<int64_t>(1, (int64_t)sms * 8 / count);
             const dim3 cg((unsigned)std::min<int64_t>((total + 255) / 256, per), 1, (unsigned)count);
-            crt_combine_kernel<<<cg, 256, 0, s>>>(res, g.ldr, rows, cols, row0, col0, table, q);
+            if (f.bits <= 55)
+                crt_combine_kernel<3><<<cg, 256, 0, s>>>(res, g.ldr, rows, cols, row0, col0, table, q);
+            else
+                crt_combine_kernel<4><<<cg, 256, 0, s>>>(res, g.ldr, rows, cols, row0, col0, table, q);
             SPIN_CUDA_TRY(cudaGetLastError());
             nl += 2;
         }
@@ -630,6 +678,7 @@ BatchView skip(BatchView v, int z) {
 int crt_product(const CrtProduct& p, void* arena, size_t bytes, cudaStream_t s, int* launches) {
     if (p.m <= 0 || p.n <= 0) return SPIN_OK;
     if (p.count < 0 || p.count > 65535) return SPIN_ERR_INVALID_ARG;
+    if (!(p.alpha == 1.0 || p.alpha == -1.0) || !(p.beta == 0.0 || p.beta == 1.0)) return SPIN_ERR_INVALID_ARG;
     const CrtFormat f = crt_format(p.k, p.min_bits);
     if (f.moduli == 0) return SPIN_ERR_INVALID_ARG;
     unsigned char* base = (unsigned char*)round_up((size_t)(uintptr_t)arena, 256);

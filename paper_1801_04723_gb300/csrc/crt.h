@@ -44,8 +44,8 @@ inline int crt_bits_for_slices(int s) { return 8 * s - 4; }
 size_t crt_full_bytes(int64_t m, int64_t n, int64_t k, int moduli, int count = 1);
 size_t crt_min_bytes(int64_t m, int64_t n, int64_t k, int moduli, int count = 1);
 
-// D = beta*C + alpha*(A B) (+ I) for `count` problems (count = 0: one
-// problem given by plain pointers).  Views, sums of squares, active flags
+// D = beta*C + alpha*(A B) (+ I), alpha = +-1, beta = 0 or 1, for `count`
+// problems (count = 0: one problem given by plain pointers).  Views, sums of squares, active flags
 // and statuses as in TcGemmParams.
 struct CrtProduct {
     int64_t m, n, k;

@@ -186,15 +186,15 @@ __device__ __forceinline__ void store4(uint16_t* dst, unsigned a, unsigned b, un
 }
 
 // hi = bf16(x), lo = bf16(x - hi) (three planes: hi, mid, lo), computed from
-// xf = fp32(x): one FP64 operation per element (GB300's FP64 rate would
-// otherwise bound this memory-bound pass); xf differs from x by 2^-24
+// xf = fp32(x), no FP64 operation (GB300's FP64 rate would bound this
+// memory-bound pass); xf differs from x by 2^-24
 // relative, far below what the three-product form keeps (~2^-16).
 template <int PLANES>
 struct ToBf16 {
     __device__ __forceinline__ void operator()(const double (&x)[4], int, uint16_t* dst, int64_t plane) const {
         float r[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) r[u] = __double2float_rn(x[u]);
+        for (int u = 0; u < 4; u++) r[u] = f64_to_f32_rn(x[u]);
 #pragma unroll
         for (int q = 0; q < PLANES; q++) {
             __nv_bfloat16 h[4];

@@ -502,30 +502,51 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const int col0 = n0 + half * HALF;
             double sumsq = 0.0;
             if (!EXACT) {
-                const int so = p.sum_order ? p.sum_order[z] : 0x7fffffff;
+                // D = beta C + alpha (the FP32 sum), alpha = +-1 (the sign bit),
+                // beta = 0 or 1: no FP64 operation without C, one addition
+                // per output with it.  The FP64 pipe takes a warp instruction
+                // per 16 to 20 clocks and SM, so the 32768 outputs of a tile
+                // cost 8 us per operation and output: a conversion, a product
+                // with alpha and a fused multiply-add with beta made a 512^3
+                // product of 8 tiles 50 us long, its MMAs 6.
+                const uint32_t sign = p.alpha < 0.0 ? 0x80000000u : 0u;
+                const bool add = p.beta != 0.0;
                 const int buf = chunk & 1;
                 bool ok = mbar_wait(&ctl->tfull[buf], (uint32_t)((chunk >> 1) & 1), abort, WAIT_LIMIT_NS);
                 if (!ok) raise_timeout(ctl, p.err);
                 tc_fence_after();
-                if (ok) {
+                if (ok && m0 + quarter * 32 < p.M) {
+                    const double* crow = row_ok ? in_row(p, z, grow) : nullptr;
+                    double* drow = row_ok ? out_row(p, z, grow) : nullptr;
 #pragma unroll 1
-                    for (int cc = 0; cc < HALF; cc += 16) {
+                    for (int cc = 0; cc < HALF && col0 + cc < p.N; cc += 16) {
                         uint32_t v[16];
                         tmem_ld_32x32b_x16(lane_addr + (uint32_t)(buf * BN + half * HALF + cc), v);
                         tmem_ld_wait();
-                        if (row_ok) {
-                            const double* crow = in_row(p, z, grow);
-                            double* drow = out_row(p, z, grow);
+                        if (!row_ok) continue;
 #pragma unroll
-                            for (int j = 0; j < 16; j++) {
-                                const int gcol = col0 + cc + j;
-                                if (gcol < p.N) {
-                                    double val = p.alpha * (double)__uint_as_float(v[j]);
-                                    if (p.beta != 0.0) val = fma(p.beta, crow[gcol], val);
-                                    if (p.add_identity && gcol == grow) val += 1.0;
-                                    drow[gcol] = val;
-                                    if (grow < so && gcol < so) sumsq = fma(val, val, sumsq);
+                        for (int j4 = 0; j4 < 16; j4 += 4) {
+                            const int gcol = col0 + cc + j4;
+                            if (gcol >= p.N) break;
+                            double val[4];
+#pragma unroll
+                            for (int u = 0; u < 4; u++) val[u] = f32_to_f64(v[j4 + u] ^ sign);
+                            // whole 32-byte sectors where the views allow it
+                            if (gcol + 3 < p.N && aligned32(drow + gcol) && (!add || aligned32(crow + gcol))) {
+                                if (add) {
+                                    double old[4];
+                                    ld_global_v4(crow + gcol, old);
+#pragma unroll
+                                    for (int u = 0; u < 4; u++) val[u] = add_now(old[u], val[u]);
                                 }
+                                st_global_v4(drow + gcol, val);
+                            } else {
+#pragma unroll
+                                for (int u = 0; u < 4; u++)
+                                    if (gcol + u < p.N) {
+                                        if (add) val[u] = add_now(crow[gcol + u], val[u]);
+                                        drow[gcol + u] = val[u];
+                                    }
                             }
                         }
                     }
@@ -886,6 +907,10 @@ int launch_tc_gemm(const TcOperand& a, const TcOperand& b, const TcGemmParams& p
     if (prm.K <= 0 || prm.num_pairs <= 0 || prm.num_pairs > kTcMaxPairs) return SPIN_ERR_INVALID_ARG;
     // runs <= 1024 k (exactness: 1024 products of at most 2^14) made of whole pipeline stages
     if (prm.exact && (prm.chunk_kb < 1 || prm.chunk_kb > 16 || prm.chunk_kb % KSUB_EXACT != 0)) return SPIN_ERR_INVALID_ARG;
+    // the float mode's epilogue: alpha = +-1, beta = 0 or 1, nothing else
+    if (!prm.exact && (!(prm.alpha == 1.0 || prm.alpha == -1.0) || !(prm.beta == 0.0 || prm.beta == 1.0) ||
+                       prm.add_identity || prm.sumsq))
+        return SPIN_ERR_INVALID_ARG;
     if (prm.batch < 0 || prm.batch > 65535) return SPIN_ERR_INVALID_ARG;
     if (prm.batch && (int64_t)prm.batch * a.rows * a.slices > INT32_MAX) return SPIN_ERR_INVALID_ARG;
     if (prm.batch && (int64_t)prm.batch * b.rows * b.slices > INT32_MAX) return SPIN_ERR_INVALID_ARG;

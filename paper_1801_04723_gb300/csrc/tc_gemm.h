@@ -27,7 +27,8 @@ struct TcGemmParams {
     int8_t pa[kTcMaxPairs];  // A slice of each pair
     int8_t pb[kTcMaxPairs];  // B slice of each pair
     int8_t pg[kTcMaxPairs];  // group of each pair (pairs sorted by group)
-    int exact;               // 0: one FP32 accumulation of all pairs; 1: exact integer runs
+    int exact;               // 0: one FP32 accumulation of all pairs (alpha = +-1, beta = 0 or 1, no
+                             // identity, no sum of squares); 1: exact integer runs
     int chunk_kb;            // exact mode: 64-wide k-blocks per exact run
     int group_shift[kTcMaxGroups];  // exact mode: power-of-two weight of each group
     double alpha, beta;

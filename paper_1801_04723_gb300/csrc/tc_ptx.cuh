@@ -311,6 +311,20 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar, uint16_t cta_mask
         : "memory");
 }
 
+// 32-byte global loads and stores (32-byte aligned): a whole sector per
+// thread, where a thread per row writes or reads runs of its row.
+__device__ __forceinline__ void ld_global_v4(const double* p, double (&v)[4]) {
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void st_global_v4(double* p, const double (&v)[4]) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+                 : "memory");
+}
+__device__ __forceinline__ bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
+
 // Shared-memory matrix descriptor: K-major operand tile written by TMA with
 // 128-byte swizzling (rows of 64 bf16 = 128 B, 8-row swizzle atoms of 1 KB).
 //   bits  0-13 start address >> 4
