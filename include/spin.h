@@ -60,7 +60,9 @@ typedef enum {
 } spin_status;
 
 typedef enum {
-    SPIN_FP64 = 0,         /* every product in FP64 (plain method)                           */
+    SPIN_FP64 = 0,         /* every product in FP64 (plain method); those above 2048 in every
+                              dimension on the tensor cores, 63 bits per operand and the sum
+                              exact, where that has no larger error bound for these operands */
     SPIN_MIXED_BF16X3 = 1, /* products on BF16 tensor cores with 3-term splits, FP32 accumulate,
                               then Newton-Schulz refinement to opts.tol                       */
     /* 2 is not a precision (a call passing it gets SPIN_ERR_INVALID_ARG)                     */
@@ -165,6 +167,11 @@ int spin_invert(const double* A, double* X, int64_t n, int64_t lda, int leaf, sp
  * unless blocking or info asks for it; pretransform = 2 waits once for the
  * first attempt's status.  The caller-provided workspace (opts->workspace)
  * must be 256-byte aligned.
+ * A workspace larger than spin_workspace_bytes is put to use: the mixed forms
+ * then need fewer panels, and FP64 inversions above order 4096 have room for
+ * the tensor-core form of their large products (with exactly that size they
+ * run on the FP64 pipe; without a caller's workspace the library keeps an
+ * arena of at most 8 GB per stream for them).
  * Schedule: the recursion (Algorithm 2's driver) is a DAG of product and
  * leaf launches over views of X, A and the workspace, on the stream and, up
  * to order 8192 in FP64, a second library stream (II, then C21, beside the
@@ -449,7 +456,9 @@ int spin_default_leaf(int64_t n, int precision);
  * given leaf on one GB300: the paper's cost analysis (Sec. 4, Table 2)
  * restated for this GPU -- six products per node priced by tile waves over
  * 152 SMs at the FP64 rate, leaves priced per pivot step on one thread-block
- * cluster.  spin_default_leaf uses its optimum for untuned FP64 orders.
+ * cluster.  Above order 4096 it is an upper bound: the top levels' products
+ * leave the FP64 pipe there (the leaf's optimum is set by the lower levels).
+ * spin_default_leaf uses its optimum for untuned FP64 orders.
  * -1 for other precisions or bad arguments. */
 double spin_model_seconds(int64_t n, int leaf, int precision);
 

@@ -38,6 +38,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "f64_residues.h"
 #include "mixed.h"
 #include "tc_gemm.h"
 
@@ -128,6 +129,8 @@ struct StreamState {
     double* hostX = nullptr;
     size_t host_elems = 0;
     int* err_dev = nullptr;        // device: tensor-core bounded-wait failures
+    unsigned char* f64_arena = nullptr;  // large FP64 products by residues (two halves on two streams)
+    size_t f64_arena_bytes = 0;
     int last_mixed = 0;            // host: the latest call refined (mixed precision)
     int last_pretransformed = 0;   // host: the latest call went through the butterfly transform
     // The schedule as a CUDA graph: the previous call's arguments, and the
@@ -178,6 +181,34 @@ int ensure_ws(StreamState* st, size_t bytes) {
     return SPIN_OK;
 }
 
+// The arena of large FP64 products for inversions of order n on this stream:
+// what the top level needs at once, up to a bound, less when the device has
+// less (panels), none when it has too little or no product is large enough
+// (the FP64 kernel runs).  Kept for later calls, as the workspace is.
+size_t ensure_f64_arena(StreamState* st, int64_t n, int64_t leaf, bool two_streams) {
+    const int64_t n1 = split_order(n), n2 = n - n1;
+    if (n <= leaf || n2 <= kF64ResidueMin || f64_residue_moduli(n1) == 0) return 0;
+    const size_t parts = two_streams ? 2 : 1;
+    const size_t least = f64_residue_bytes(n1, n1, n1, true);
+    size_t want = std::max(least, std::min(f64_residue_bytes(n1, n1, n1, false), kF64ResidueArena / parts));
+    if (st->f64_arena_bytes >= parts * want) return st->f64_arena_bytes / parts / 256 * 256;
+    if (st->f64_arena) {
+        cudaFree(st->f64_arena);
+        st->f64_arena = nullptr;
+        st->f64_arena_bytes = 0;
+    }
+    for (; want >= least; want /= 2) {
+        want = (want + 255) / 256 * 256;
+        if (cudaMalloc(&st->f64_arena, parts * want) == cudaSuccess) {
+            st->f64_arena_bytes = parts * want;
+            return want;
+        }
+        cudaGetLastError();
+        st->f64_arena = nullptr;
+    }
+    return 0;
+}
+
 struct Run {
     cudaStream_t s;
     int32_t* info;
@@ -188,9 +219,9 @@ struct Run {
     cudaStream_t side = nullptr;
     std::vector<cudaEvent_t>* events = nullptr;
     size_t next_event = 0;
-    // mixed precision only
     int precision = SPIN_FP64;
     int fp64_levels = 0;
+    // split arena: the mixed forms' products, large FP64 products by residues
     void* scratch = nullptr;
     size_t scratch_bytes = 0;
     void* side_scratch = nullptr;  // split arena of the side stream's products
@@ -237,6 +268,25 @@ int gemm_f64_prof(Run& r, int depth, int64_t m, int64_t n, int64_t k, double alp
     return launch_gemm_f64(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, r.s);
 }
 
+// A large FP64 product: by residues or, where those would be less accurate
+// for these operands (decided on the device), by the FP64 kernel.
+int large_gemm_f64(Run& r, int depth, const F64Product& p) {
+    const double f = 2.0 * (double)p.m * (double)p.n * (double)p.k;
+    const double bytes = 8.0 * ((double)p.m * p.k + (double)p.k * p.n + (double)p.m * p.n * (p.beta != 0.0 ? 2.0 : 1.0));
+    F64Plan plan;
+    int rc = f64_residue_decide(p, r.scratch, &plan, r.s);
+    if (rc) return rc;
+    {
+        ProfScope ps(r.prof, r.s, SPIN_KERNEL_GEMM_TC, depth, p.m, p.n, p.k, f64_residue_moduli(p.k) * f, bytes,
+                     plan.use_residues);
+        rc = f64_residue_product(p, plan, r.scratch_bytes, r.scratch, r.err, r.s);
+        if (rc) return rc;
+    }
+    ProfScope ps(r.prof, r.s, SPIN_KERNEL_GEMM_F64, depth, p.m, p.n, p.k, f, bytes, plan.use_fp64);
+    return launch_gemm_f64(p.m, p.n, p.k, p.alpha, p.A, p.lda, p.B, p.ldb, p.beta, p.C, p.ldc, p.D, p.ldd, r.s,
+                           plan.use_fp64);
+}
+
 int leaf_prof(Run& r, int depth, const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, double* W) {
     ProfScope ps(r.prof, r.s, SPIN_KERNEL_LEAF, depth, n, n, 0, 2.0 * (double)n * n * n, 16.0 * (double)n * n);
     return launch_leaf_gj(A, lda, X, ldx, n, W, r.info, r.leaf_counter++, r.s);
@@ -267,6 +317,9 @@ int64_t tc_min() {
 int level_gemm(Run& r, int depth, bool schur, int64_t m, int64_t n, int64_t k, double alpha, const double* A,
                int64_t lda, const double* B, int64_t ldb, double beta, const double* C, int64_t ldc, double* D,
                int64_t ldd) {
+    if (r.precision == SPIN_FP64 && r.scratch_bytes > 0 && std::min({m, n, k}) > kF64ResidueMin &&
+        r.scratch_bytes >= f64_residue_bytes(m, n, k, true))
+        return large_gemm_f64(r, depth, F64Product{m, n, k, alpha, beta, A, lda, B, ldb, C, ldc, D, ldd});
     if (r.precision == SPIN_FP64 || m < tc_min() || n < tc_min() || k < 64)
         return gemm_f64_prof(r, depth, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd);
     const double f = 2.0 * (double)m * (double)n * (double)k;
@@ -580,7 +633,8 @@ int refine(Run& r, StreamState* st, const double* A, int64_t lda, double* X, int
 // transform undone afterwards (pretransform 1); mixed modes then refine
 // X against A itself.
 int enqueue_once(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, int64_t leaf, const spin_opts& o,
-                 bool rbt, StreamState* st, cudaStream_t s, unsigned char* ws, size_t ws_bytes) {
+                 bool rbt, StreamState* st, cudaStream_t s, unsigned char* ws, size_t ws_bytes, void* f64_arena,
+                 size_t f64_bytes) {
     const bool mixed = o.precision != SPIN_FP64;
     st->last_mixed = mixed ? 1 : 0;
     st->last_pretransformed = rbt ? 1 : 0;
@@ -612,7 +666,18 @@ int enqueue_once(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n
             r.side = st->side;
             r.events = &st->events;
         }
+        if (f64_bytes > 0) {
+            r.scratch = f64_arena;
+            r.scratch_bytes = f64_bytes;
+            if (r.side != nullptr) {
+                r.side_scratch = (unsigned char*)f64_arena + f64_bytes;
+                r.side_scratch_bytes = f64_bytes;
+            }
+            r.err = st->err_dev;
+            SPIN_CUDA_TRY(cudaMemsetAsync(st->err_dev, 0, sizeof(int), s));
+        }
         RET(inv_rec(r, 0, Ain, lda_in, Xout, ldx_out, n_in, (double*)inner));
+        if (f64_bytes > 0) RET(launch_refine_finish(r.err, st->info_dev, 1, s));
         if (rbt) RET(launch_rbt_backward(Xout, R.np, kRbtDepth, (const double*)ws, X, ldx, n, s));
         return SPIN_OK;
     }
@@ -655,18 +720,20 @@ uint64_t bits_of(double x) {
 
 // Every argument that shapes the launch sequence or its operands.
 std::vector<uint64_t> call_key(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, int64_t leaf,
-                               const spin_opts& o, const void* ws, size_t ws_bytes) {
+                               const spin_opts& o, const void* ws, size_t ws_bytes, const void* f64_arena,
+                               size_t f64_bytes) {
     return {(uint64_t)(uintptr_t)A, (uint64_t)lda, (uint64_t)(uintptr_t)X, (uint64_t)ldx, (uint64_t)n,
             (uint64_t)leaf, (uint64_t)o.precision, bits_of(o.tol), (uint64_t)o.max_refine,
             (uint64_t)o.fp64_levels, (uint64_t)o.residual_slices, (uint64_t)o.pretransform, o.rbt_seed,
             (uint64_t)(int64_t)o.schedule,
-            (uint64_t)(uintptr_t)ws, (uint64_t)ws_bytes};
+            (uint64_t)(uintptr_t)ws, (uint64_t)ws_bytes, (uint64_t)(uintptr_t)f64_arena, (uint64_t)f64_bytes};
 }
 
 // Capture the whole schedule of one call (every launch enqueue_once makes,
 // on this stream and on the side stream) into a graph on a private stream.
 int capture_schedule(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, int64_t leaf,
-                     const spin_opts& o, StreamState* st, unsigned char* ws, size_t ws_bytes) {
+                     const spin_opts& o, StreamState* st, unsigned char* ws, size_t ws_bytes, void* f64_arena,
+                     size_t f64_bytes) {
     if (st->cap == nullptr) SPIN_CUDA_TRY(cudaStreamCreateWithFlags(&st->cap, cudaStreamNonBlocking));
     if (st->exec) {
         cudaGraphExecDestroy(st->exec);
@@ -674,7 +741,8 @@ int capture_schedule(const double* A, int64_t lda, double* X, int64_t ldx, int64
         st->graph_key.clear();
     }
     SPIN_CUDA_TRY(cudaStreamBeginCapture(st->cap, cudaStreamCaptureModeThreadLocal));
-    const int rc = enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, st->cap, ws, ws_bytes);
+    const int rc = enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, st->cap, ws, ws_bytes,
+                                f64_arena, f64_bytes);
     cudaGraph_t graph = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(st->cap, &graph);
     if (rc != SPIN_OK) {
@@ -716,18 +784,37 @@ int enqueue(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, con
         ws = (unsigned char*)st->ws;
         ws_bytes = std::min(st->ws_bytes, want);
     }
+    // FP64: the residue arena of large products, the library's or what the
+    // caller's workspace holds beyond `need`
+    void* f64_arena = nullptr;
+    size_t f64_bytes = 0;  // per stream
+    if (!mixed) {
+        const int64_t top = o.pretransform != 0 ? rbt_padded_order(n, kRbtDepth) : n;
+        const bool two = overlap_schedule(top, o.precision, o.schedule);
+        if (o.workspace == nullptr) {
+            f64_bytes = ensure_f64_arena(st, top, leaf, two);
+            f64_arena = st->f64_arena;
+        } else if (top > leaf && top - split_order(top) > kF64ResidueMin) {
+            const size_t used = round256(need);
+            if (o.workspace_bytes > used) f64_bytes = (o.workspace_bytes - used) / (two ? 2 : 1) / 256 * 256;
+            f64_arena = ws + used;
+        }
+    }
     if (o.pretransform != 2) {
-        if (!graph_mode() || st->prof.on) return enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, s, ws, ws_bytes);
+        if (!graph_mode() || st->prof.on)
+            return enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, s, ws, ws_bytes, f64_arena,
+                                f64_bytes);
         // The second call with the same arguments captures the schedule;
         // later ones replay it (one graph launch, dependencies resolved on
         // the device); any other call runs the launches directly.
-        std::vector<uint64_t> key = call_key(A, lda, X, ldx, n, leaf, o, ws, ws_bytes);
+        std::vector<uint64_t> key = call_key(A, lda, X, ldx, n, leaf, o, ws, ws_bytes, f64_arena, f64_bytes);
         if (st->exec == nullptr || key != st->graph_key) {
             if (key != st->prev_key) {
                 st->prev_key = key;
-                return enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, s, ws, ws_bytes);
+                return enqueue_once(A, lda, X, ldx, n, leaf, o, o.pretransform == 1, st, s, ws, ws_bytes, f64_arena,
+                                    f64_bytes);
             }
-            RET(capture_schedule(A, lda, X, ldx, n, leaf, o, st, ws, ws_bytes));
+            RET(capture_schedule(A, lda, X, ldx, n, leaf, o, st, ws, ws_bytes, f64_arena, f64_bytes));
             st->graph_key = key;
         }
         st->last_mixed = st->graph_mixed;
@@ -738,12 +825,12 @@ int enqueue(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, con
     }
     // plain first; a zero or non-finite pivot (A11 or a Schur complement
     // singular in working precision) sends the call through the transform
-    RET(enqueue_once(A, lda, X, ldx, n, leaf, o, false, st, s, ws, ws_bytes));
+    RET(enqueue_once(A, lda, X, ldx, n, leaf, o, false, st, s, ws, ws_bytes, f64_arena, f64_bytes));
     SPIN_CUDA_TRY(cudaMemcpyAsync(st->info_host, st->info_dev, INFO_WORDS * sizeof(int32_t),
                                   cudaMemcpyDeviceToHost, s));
     SPIN_CUDA_TRY(cudaStreamSynchronize(s));
     if (st->info_host[INFO_STATUS] != SPIN_ERR_SINGULAR) return SPIN_OK;
-    return enqueue_once(A, lda, X, ldx, n, leaf, o, true, st, s, ws, ws_bytes);
+    return enqueue_once(A, lda, X, ldx, n, leaf, o, true, st, s, ws, ws_bytes, f64_arena, f64_bytes);
 }
 
 // ---- leaf autotuning ----
@@ -771,6 +858,10 @@ __global__ void synth_sdd_kernel(double* A, int64_t n, uint64_t seed) {
 
 // ---- cost model of the plain FP64 path (Sec. 4's cost analysis restated
 // for one GB300) ----
+//
+// Every product is priced on the FP64 kernel: above order 4096, whose top
+// levels leave it (f64_residues.cu), the model is an upper bound.  The leaf
+// choice it serves does not depend on those levels.
 //
 // The paper prices each step of Algorithm 1 on a Spark cluster (Table 2,
 // Eq. (SPIN-cost)) and finds a U-shaped dependence on the partition size

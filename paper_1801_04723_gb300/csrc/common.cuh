@@ -107,9 +107,10 @@ struct BatchView {
 int gemm_f64_tile_size(int64_t m, int64_t n, int64_t count);
 // The tile SPIN_F64_TILE forces (64, 32 or 16; for measurement), else 0.
 int forced_f64_tile();
+// gate (optional, device int): the product runs only while *gate != 0.
 int launch_gemm_f64(int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda,
                     const double* B, int64_t ldb, double beta, const double* C, int64_t ldc, double* D,
-                    int64_t ldd, cudaStream_t s);
+                    int64_t ldd, cudaStream_t s, const int* gate = nullptr);
 
 int launch_gemm_f64_batched(int64_t m, int64_t n, int64_t k, double alpha, const BatchView& a, const BatchView& b,
                             double beta, const BatchView& c, const BatchView& d, int count, cudaStream_t s);

@@ -544,9 +544,13 @@ int crt_run(const CrtProduct& p, const CrtFormat& f, const CrtPanels& c, unsigne
     src.valid = p.valid;
     const bool known = p.a_exps != nullptr;
     if (known) ea = const_cast<int*>(p.a_exps);
-    int rc = launch_exponents(src, m, n, k, known ? nullptr : ea, eb, p.sumsq_a, p.sumsq_b, nullptr, s);
-    if (rc) return rc;
-    nl++;
+    if (p.b_exps != nullptr) eb = const_cast<int*>(p.b_exps);
+    int rc = SPIN_OK;
+    if (!known || p.b_exps == nullptr) {
+        rc = launch_exponents(src, m, n, k, known ? nullptr : ea, eb, p.sumsq_a, p.sumsq_b, nullptr, s);
+        if (rc) return rc;
+        nl++;
+    }
 
     CrtTable table;
     crt_table(f, &table);

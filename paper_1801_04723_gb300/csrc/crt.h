@@ -9,7 +9,7 @@
 namespace spin {
 
 constexpr int kCrtMaxModuli = 20;
-constexpr int kCrtMaxBits = 62;
+constexpr int kCrtMaxBits = 63;  // signed in 64 bits
 
 // Pairwise coprime, in falling order; signed residues |r| <= 128.
 __host__ __device__ constexpr int crt_modulus(int l) {
@@ -70,6 +70,7 @@ struct CrtProduct {
     double* sumsq_b;
     double* sumsq_d;
     const int* a_exps;    // optional, device: row exponents of A from an earlier product with the same A
+    const int* b_exps;    // optional, device (with a_exps): column exponents of B
     int* a_exps_out;      // optional, device: m ints per problem, where they are kept (else in the arena)
     int* err;
 };

@@ -1,0 +1,51 @@
+// Large FP64 products by residues on the tensor cores (f64_residues.cu).
+#pragma once
+#include <cuda_runtime.h>
+#include <stddef.h>
+#include <stdint.h>
+
+#include "common.cuh"
+
+namespace spin {
+
+// Products whose m, n and k are all above this take the residue form when an
+// arena is there, i.e. the top levels of inversions above order 4096.  A 2048^3
+// product takes 14 ms on the FP64 pipe and 0.6 ms by residues, so the line is
+// not where the residues stop paying; it lies there because orders up to 4096
+// are held to the FP64 kernel elsewhere: spin_model_seconds prices it (within
+// 25 % of the measured inversion at n = 4096), and up to 1024 the batched, the
+// persistent and the no-allocation forms, which have no residue arena, give
+// the single inversion's bits.
+constexpr int64_t kF64ResidueMin = 2048;
+// Most device memory of one product's arena: a 16384^3 product then runs in
+// panels (its planes and residues take 24 GB at once).
+constexpr size_t kF64ResidueArena = (size_t)8 << 30;
+
+struct F64Product {
+    int64_t m, n, k;
+    double alpha, beta;
+    const double* A;
+    int64_t lda;
+    const double* B;
+    int64_t ldb;
+    const double* C;
+    int64_t ldc;
+    double* D;
+    int64_t ldd;
+};
+struct F64Plan {
+    const int* use_residues;  // device flags, one of them set
+    const int* use_fp64;
+    int *ea, *eb;
+    void* rest;
+};
+int f64_residue_moduli(int64_t k);  // 0: no such form for this k
+// Arena of one product: the least, or the one that needs no panels.
+size_t f64_residue_bytes(int64_t m, int64_t n, int64_t k, bool least);
+// Exponents, and which form runs; then the residue product (a no-op on the
+// device when the FP64 kernel, gated by use_fp64, is to run).
+int f64_residue_decide(const F64Product& p, void* arena, F64Plan* plan, cudaStream_t s);
+int f64_residue_product(const F64Product& p, const F64Plan& plan, size_t arena_bytes, const void* arena, int* err,
+                        cudaStream_t s);
+
+}  // namespace spin

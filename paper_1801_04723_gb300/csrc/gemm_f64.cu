@@ -144,7 +144,8 @@ template <int TM>
 __global__ void __launch_bounds__(NT, 2)
 gemm_f64_kernel(int64_t m, int64_t n, int64_t k, double alpha, const double* __restrict__ A, int64_t lda,
                 const double* __restrict__ B, int64_t ldb, double beta, const double* C, int64_t ldc,
-                double* D, int64_t ldd, int group) {
+                double* D, int64_t ldd, int group, const int* gate) {
+    if (gate != nullptr && *gate == 0) return;
     int64_t tile_m, tile_n;
     tile_of(group, tile_m, tile_n);
     gemm_f64_tile<TM>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_m, tile_n);
@@ -235,17 +236,17 @@ int launch_gemm_f64_batched(int64_t m, int64_t n, int64_t k, double alpha, const
 
 int launch_gemm_f64(int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda,
                     const double* B, int64_t ldb, double beta, const double* C, int64_t ldc, double* D,
-                    int64_t ldd, cudaStream_t s) {
+                    int64_t ldd, cudaStream_t s, const int* gate) {
     if (m <= 0 || n <= 0) return SPIN_OK;
     const int tm = gemm_f64_tile_size(m, n, 1);
     dim3 grid((unsigned)((n + tm - 1) / tm), (unsigned)((m + tm - 1) / tm));
     if (grid.y > 65535u) return SPIN_ERR_INVALID_ARG;
     if (tm == 64)
-        gemm_f64_kernel<64><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group());
+        gemm_f64_kernel<64><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group(), gate);
     else if (tm == 32)
-        gemm_f64_kernel<32><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group());
+        gemm_f64_kernel<32><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group(), gate);
     else
-        gemm_f64_kernel<16><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group());
+        gemm_f64_kernel<16><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group(), gate);
     SPIN_CUDA_TRY(cudaGetLastError());
     return SPIN_OK;
 }

@@ -45,23 +45,23 @@ __device__ __forceinline__ int exp_field(double x) {
     return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7FF;
 }
 
-constexpr int kSpreadSteps = 13;  // t = 0, 2, ..., 24
+constexpr int kSpreadSteps = 26;  // t = 0, 1, ..., 25
 constexpr int kNoSpread = 1000;
 
-// Least t of 0, 2, ... 24 with count[t] >= 3/4 k (count: entries whose
+// Least t of 0 .. 25 with count[t] >= (8 - g) / 8 k (count: entries whose
 // exponent is at least the largest - t).
-__device__ __forceinline__ int spread_of(const int (&count)[kSpreadSteps], int k, int top) {
+__device__ __forceinline__ int spread_of(const int (&count)[kSpreadSteps], int k, int top, int g) {
     if (top == 0x7FF) return kNoSpread;  // an infinity or NaN
     int t = kNoSpread;
 #pragma unroll
     for (int i = kSpreadSteps - 1; i >= 0; i--)
-        if (4ll * count[i] >= 3ll * k) t = 2 * i;
+        if (8ll * count[i] >= (long long)(8 - g) * k) t = i;
     return t;
 }
 __device__ __forceinline__ void count_entry(int (&count)[kSpreadSteps], double v, int top) {
     const int f = exp_field(v), d = f == 0 ? 1 << 20 : top - f;
 #pragma unroll
-    for (int i = 0; i < kSpreadSteps; i++) count[i] += d <= 2 * i;
+    for (int i = 0; i < kSpreadSteps; i++) count[i] += d <= i;
 }
 
 constexpr int kExpWarps = 16;
@@ -106,7 +106,7 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
 #pragma unroll
                 for (int i = 0; i < kSpreadSteps; i++) count[i] = __reduce_add_sync(0xffffffffu, count[i]);
                 const bool any = __any_sync(0xffffffffu, nonzero);
-                if (lane == 0 && any) atomicMax(&spread[0], spread_of(count, k, top));
+                if (lane >= 1 && lane <= kSpreadLevels && any) atomicMax(&spread[lane - 1], spread_of(count, k, top, lane));
             }
         }
     } else {
@@ -157,10 +157,12 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
                 if (count[i]) atomicAdd(&scount[lane][i], count[i]);
             if (nonzero) scount[lane][kSpreadSteps] = 1;
             __syncthreads();
-            if (warp == 0 && col_ok && scount[lane][kSpreadSteps]) {
+            if (warp >= 1 && warp <= kSpreadLevels) {  // a level per warp, a column per lane
 #pragma unroll
                 for (int i = 0; i < kSpreadSteps; i++) count[i] = scount[lane][i];
-                atomicMax(&spread[1], spread_of(count, k, top));
+                const bool wanted = col_ok && scount[lane][kSpreadSteps];
+                const int t = __reduce_max_sync(0xffffffffu, wanted ? spread_of(count, k, top, warp) : 0);
+                if (lane == 0) atomicMax(&spread[kSpreadLevels + warp - 1], t);
             }
         }
     }

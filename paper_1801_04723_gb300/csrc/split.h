@@ -25,10 +25,12 @@ struct SplitSource {
 // Exponents e with |a_ik| < 2^e for every row i of A (k entries) and every
 // column j of B: ea (m per problem, or null: not wanted), eb (n per problem,
 // or null), += sums of squares (optional, one entry per problem).  spread
-// (optional, device int[2], count = 0 only): raised to the largest over the
-// rows (spread[0]; columns: spread[1]) of the least t of 0, 2, 4, ... 24 such
-// that three quarters of the row's entries are at least 2^-t of its largest
-// (by exponents), 1000 where none is or an entry is not finite.
+// (optional, device int[2 * kSpreadLevels], count = 0 only): entry g - 1 of A's
+// half is raised to the largest over the rows (of B's half: over the columns)
+// of the least t of 0 .. 25 such that 8 - g eighths of the row's exponents are
+// at least its largest - t; 1000 where none is or an entry is not finite; rows
+// of zeros do not count.
+constexpr int kSpreadLevels = 7;
 int launch_exponents(const SplitSource& src, int m, int n, int k, int* ea, int* eb, double* sumsq_a, double* sumsq_b,
                      int* spread, cudaStream_t s);
 

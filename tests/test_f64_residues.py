@@ -1,0 +1,92 @@
+"""Plain inversions above order 4096, whose large products run by residues on
+the tensor cores where that is at least as accurate as the FP64 kernel, decided
+on the device from the operands' exponents.  An inversion in a caller's
+workspace of exactly spin_workspace_bytes has no room for the residues: it is
+the FP64 kernel's result, to compare with."""
+import numpy as np
+import pytest
+
+import bounds
+import oracle
+from paper_1801_04723_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+N = 4161  # split 2112 + 2049: every product of the top level is above the line, none below it
+LEAF = 128
+
+
+@pytest.fixture(scope="module")
+def spin():
+    import paper_1801_04723_gb300 as s
+
+    s.build()
+    s.lib()
+    return s
+
+
+def fp64_kernel_inverse(spin, A, schedule="default", check=True):
+    n = A.shape[0]
+    size = spin.workspace_bytes(n, leaf=LEAF, schedule=schedule)
+    ws = torch.empty(size, dtype=torch.uint8, device="cuda:0")
+    X, info = spin.invert(A, leaf=LEAF, workspace=ws, schedule=schedule, check=check)
+    torch.cuda.synchronize()
+    return X, info
+
+
+def products_by_residues(spin, A, **kw):
+    spin.profile_start()
+    X, info = spin.invert(A, leaf=LEAF, **kw)
+    rec = spin.profile_collect()
+    torch.cuda.synchronize()
+    return X, info, sum(r["kind"] == "gemm_tc" for r in rec)
+
+
+@pytest.mark.parametrize("family", ["spd", "sdd"])
+def test_as_accurate_as_the_fp64_kernel(spin, family):
+    A = (inputs.spd_gram_device(N, 5, "cuda:0", alpha=0.3) if family == "spd" else inputs.sdd_device(N, 6, "cuda:0"))
+    X, info, count = products_by_residues(spin, A)
+    assert info["status"] == 0 and count == 6
+    Y, _ = fp64_kernel_inverse(spin, A)
+    assert not torch.equal(X, Y)  # another rounding, so the other form did run
+    Ah, Xh, Yh = A.cpu().numpy(), X.cpu().numpy(), Y.cpu().numpy()
+    ref, _ = oracle.strassen_inv(Ah, LEAF)
+    assert bounds.elementwise_ok(Xh, ref, Ah)
+    rx, ry = oracle.residual(Ah, Xh)[0], oracle.residual(Ah, Yh)[0]
+    assert rx <= 1e-13 and rx <= 1.5 * ry
+
+
+def test_same_bits_on_one_stream_and_in_panels(spin):
+    """The same products on one or two streams, and in an arena a caller's
+    workspace leaves (several panels)."""
+    A = inputs.spd_gram_device(N, 7, "cuda:0", alpha=0.5)
+    X, _, _ = products_by_residues(spin, A)
+    Y, _, _ = products_by_residues(spin, A, schedule="lockstep")
+    assert torch.equal(X, Y)
+    ws = torch.empty(spin.workspace_bytes(N, leaf=LEAF) + (400 << 20), dtype=torch.uint8, device="cuda:0")
+    Z, _, count = products_by_residues(spin, A, workspace=ws)
+    assert count == 6 and torch.equal(X, Z)
+
+
+def test_widely_spread_operands_keep_the_fp64_kernel(spin):
+    """Rows and columns scaled by powers of two over a range of 2^80: fixed
+    point relative to the largest entry would lose the small ones."""
+    A = inputs.spd_gram_device(N, 8, "cuda:0", alpha=0.5)
+    g = torch.Generator(device="cuda:0").manual_seed(3)
+    d = torch.exp2(torch.randint(-40, 41, (N,), generator=g, device="cuda:0").double())
+    A = (A * d[:, None]) * d[None, :]
+    X, info, count = products_by_residues(spin, A)
+    assert info["status"] == 0 and count == 0
+    Y, _ = fp64_kernel_inverse(spin, A)
+    assert torch.equal(X, Y)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_non_finite_entries(spin, bad):
+    A = inputs.spd_gram_device(N, 9, "cuda:0", alpha=0.5)
+    A[17, N - 5] = bad
+    X, info, _ = products_by_residues(spin, A, check=False)
+    Y, info2 = fp64_kernel_inverse(spin, A, check=False)
+    assert info["status"] == info2["status"] == 2
+    assert (info["fail_leaf"], info["fail_col"]) == (info2["fail_leaf"], info2["fail_col"])
