@@ -60,18 +60,21 @@ struct LeafWait {
 
 // One lane's wait (the clock is read only after some polls: reading it takes
 // longer than a poll).
-__device__ __forceinline__ bool slot_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
+__device__ __forceinline__ bool slot_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
+                                          const volatile int* quit = nullptr) {
     for (int i = 0; i < 32; i++)
         if (tc::mbar_try_wait_cluster(bar, parity)) return true;
     const uint64_t t0 = tc::globaltimer_ns();
     for (uint32_t spins = 1;; spins++) {
         if (tc::mbar_try_wait_cluster(bar, parity)) return true;
+        if (quit != nullptr && *quit) return false;
         if ((spins & 63u) == 0 && tc::globaltimer_ns() - t0 > limit_ns) return false;
     }
 }
 // A warp's wait: the same answer in every lane.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
-    return __all_sync(FULL, slot_wait(bar, parity, limit_ns));
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
+                                          const volatile int* quit = nullptr) {
+    return __all_sync(FULL, slot_wait(bar, parity, limit_ns, quit));
 }
 
 struct ColSmemLayout {
@@ -169,7 +172,7 @@ __host__ __device__ inline int col_panel(int L, int cmax) {
     return w > kColMinPanel ? w : kColMinPanel;
 }
 template <int T>
-constexpr int kColMaxWarps = 2 * T > kColMinPanel ? 2 * T : kColMinPanel;  // 32 T columns on 16 CTAs
+constexpr int kColMaxWarps = T == 1 ? 8 : 16;
 
 // One bulk copy of a slot to the same place in CTA `peer`, completing on its
 // barrier there.
@@ -181,9 +184,9 @@ __device__ __forceinline__ void send_slot(double* slot, uint64_t* bar, uint32_t 
 // T rows per lane: row lane + 32 t.  One warp per column, w warps per CTA,
 // and the sender.
 template <int T>
-__global__ void __launch_bounds__(32 * (kColMaxWarps<T> + 1), 1)
-leaf_gj_col_kernel(const double* __restrict__ src, int64_t lds, double* __restrict__ dst, int64_t ldd, int L, int w,
-                   int32_t* info, int leaf_index, LeafWait lw) {
+__device__ __forceinline__ void leaf_gj_col_body(const double* __restrict__ src, int64_t lds, double* __restrict__ dst,
+                                                 int64_t ldd, int L, int w, int32_t* info, int leaf_index,
+                                                 const LeafWait& lw) {
     constexpr int P = kColPanelsInRing;
     const int rank = (int)tc::cluster_ctarank();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -191,6 +194,7 @@ leaf_gj_col_kernel(const double* __restrict__ src, int64_t lds, double* __restri
     const int col = rank * w + warp;
     const bool own = warp < w && col < L;
 
+    __shared__ int quit;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const ColSmemLayout lay = col_layout(L, w);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + lay.full_off);  // [P][w]
@@ -208,7 +212,10 @@ leaf_gj_col_kernel(const double* __restrict__ src, int64_t lds, double* __restri
     // below, which also expects the copy's bytes).  The credit barrier takes
     // one arrival from every warp that owns a column.
     for (int i = tid; i < P * w; i += blockDim.x) tc::mbar_init(&full[i], 1);
-    if (tid == 0) tc::mbar_init(credit, (uint32_t)L);
+    if (tid == 0) {
+        tc::mbar_init(credit, (uint32_t)L);
+        quit = 0;
+    }
     if (tid < w) tc::mbar_init(&send[tid], 1);
     for (int i = tid; i < 2 * w * w; i += blockDim.x) tc::mbar_init(&go[i], 1);
     tc::fence_mbar_init();
@@ -300,6 +307,9 @@ leaf_gj_col_kernel(const double* __restrict__ src, int64_t lds, double* __restri
                 for (int t = 0; t < T; t++) f[t] = slot[2 + lane + 32 * t];
                 const int p = __double2loint(head.y), ppos = __double2hiint(head.y);
                 if (p < 0) {  // a bad pivot: every warp of the cluster leaves at this step
+                    // (a sender whose panel never comes, too; this panel's
+                    // own finds the bad slot itself and sends it first)
+                    if (tid == 0 && q != rank) *(volatile int*)&quit = 1;
                     if (mine != nullptr && lane == 0) tc::mbar_arrive(mine);
                     return false;
                 }
@@ -427,7 +437,7 @@ leaf_gj_col_kernel(const double* __restrict__ src, int64_t lds, double* __restri
     } else if (warp == w && nact > 2) {
         // the sender: this CTA's slots to every CTA but the next one
         for (int s = 0; s < w && rank * w + s < L; s++) {
-            if (!warp_wait(&send[s], 0, lw.limit_ns)) break;
+            if (!warp_wait(&send[s], 0, lw.limit_ns, &quit)) break;
             double* slot = slots + (size_t)((rank % P) * w + s) * SD;
             if (lane < nact - 2 && rank != lw.mute_rank)
                 send_slot(slot, &full[(rank % P) * w + s], slot_bytes, (rank + 2 + lane) % nact);
@@ -469,6 +479,23 @@ leaf_gj_col_kernel(const double* __restrict__ src, int64_t lds, double* __restri
             const int r = idx / nc, c = idx % nc;
             dst[(size_t)step_of[r] * ldd + prow_of[c0 + c]] = stage[(size_t)c * lay.stage_ld + r];
         }
+}
+
+template <int T>
+__global__ void __launch_bounds__(32 * (kColMaxWarps<T> + 1), 1)
+leaf_gj_col_kernel(const double* __restrict__ src, int64_t lds, double* __restrict__ dst, int64_t ldd, int L, int w,
+                   int32_t* info, int leaf_index, LeafWait lw) {
+    leaf_gj_col_body<T>(src, lds, dst, ldd, L, w, info, leaf_index, lw);
+}
+
+// Problem blockIdx.y of a batch, on a cluster of its own.
+template <int T>
+__global__ void __launch_bounds__(32 * (kColMaxWarps<T> + 1), 1)
+leaf_gj_col_batched_kernel(BatchView src, BatchView dst, int L, int w, int32_t* info_base, int leaf_index) {
+    const int z = blockIdx.y;
+    const int64_t lds = src.ld_of(z), ldd = dst.ld_of(z);
+    leaf_gj_col_body<T>(src.ptr(z, lds), lds, const_cast<double*>(dst.ptr(z, ldd)), ldd, L, w,
+                        info_base + (int64_t)z * INFO_WORDS, leaf_index, LeafWait());
 }
 
 }  // namespace

@@ -628,11 +628,11 @@ int prepare_leaf_kernel(K kern) {
     return SPIN_OK;
 }
 
-// Launch kern on one cluster of C CTAs.
+// Launch kern on `count` clusters of C CTAs.
 template <typename K, typename... Args>
-int launch_cluster(K kern, int C, int threads, size_t smem, cudaStream_t s, Args... args) {
+int launch_clusters(K kern, int C, int count, int threads, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)C, 1, 1);
+    cfg.gridDim = dim3((unsigned)C, (unsigned)count, 1);
     cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -654,7 +654,7 @@ int launch_leaf_pull(const double* A, int64_t lda, double* X, int64_t ldx, const
     auto kern = leaf_gj_kernel<S>;
     const int rc = attrs.run([&] { return prepare_leaf_kernel(kern); });
     if (rc != SPIN_OK) return rc;
-    return launch_cluster(kern, c.C, NT, c.smem, s, A, lda, X, ldx, scratch, (int)L, c.R, info, leaf_index);
+    return launch_clusters(kern, c.C, 1, NT, c.smem, s, A, lda, X, ldx, scratch, (int)L, c.R, info, leaf_index);
 }
 
 // The column form's cluster for order L: w columns per CTA, and the CTAs (a
@@ -664,12 +664,12 @@ int launch_leaf_pull(const double* A, int64_t lda, double* X, int64_t ldx, const
 struct ColConfig {
     int T, w, C;
 };
-bool col_config(int64_t L, ColConfig* c) {
+bool col_config(int64_t L, ColConfig* c, int cmax = kColMaxCtas) {
     if (L < 1 || L > kColMaxL) return false;
-    const int cmax = std::min({max_cluster_size(), leaf_cluster_cap(), kColMaxCtas});
+    cmax = std::min({max_cluster_size(), leaf_cluster_cap(), cmax});
     c->T = col_rows((int)L);
     c->w = col_panel((int)L, cmax);
-    if (c->w > std::max(2 * c->T, kColMinPanel)) return false;
+    if (c->w > (c->T == 1 ? 8 : 16)) return false;  // kColMaxWarps
     const int nact = (int)((L + c->w - 1) / c->w);
     c->C = 1;
     while (c->C < nact) c->C <<= 1;
@@ -683,7 +683,7 @@ int launch_leaf_col_t(const double* A, int64_t lda, double* X, int64_t ldx, cons
     auto kern = leaf_gj_col_kernel<T>;
     const int rc = attrs.run([&] { return prepare_leaf_kernel(kern); });
     if (rc != SPIN_OK) return rc;
-    return launch_cluster(kern, c.C, 32 * (c.w + 1), col_layout((int)L, c.w).total, s, A, lda, X, ldx, (int)L, c.w, info,
+    return launch_clusters(kern, c.C, 1, 32 * (c.w + 1), col_layout((int)L, c.w).total, s, A, lda, X, ldx, (int)L, c.w, info,
                           leaf_index, lw);
 }
 
@@ -695,6 +695,45 @@ int launch_leaf_col(const double* A, int64_t lda, double* X, int64_t ldx, const 
         case 4: return launch_leaf_col_t<4>(A, lda, X, ldx, c, L, info, leaf_index, s, lw);
         default: return launch_leaf_col_t<8>(A, lda, X, ldx, c, L, info, leaf_index, s, lw);
     }
+}
+
+// Batches of few leaves: a cluster per leaf while all of them fit the GPU at
+// once (one CTA per SM), on as many CTAs as that leaves each; else one CTA
+// per leaf, which takes a fifth of the SM time.  One leaf of order 64 takes
+// 165 us on one CTA; 8 of them 39 us on 16 CTAs each.  (SPIN_LEAF_COL_SMS: the
+// SMs to fill, for measurement; read once.)
+constexpr int kColBatchSms = 152;
+int col_batch_sms() {
+    static const int v = [] {
+        const char* e = getenv("SPIN_LEAF_COL_SMS");
+        return e && e[0] ? atoi(e) : kColBatchSms;
+    }();
+    return v;
+}
+template <int T>
+int launch_leaf_col_batched_t(const BatchView& src, const BatchView& dst, const ColConfig& c, int64_t L, int32_t* info,
+                              int leaf_index, int count, cudaStream_t s) {
+    static PerDeviceOnce attrs;
+    auto kern = leaf_gj_col_batched_kernel<T>;
+    const int rc = attrs.run([&] { return prepare_leaf_kernel(kern); });
+    if (rc != SPIN_OK) return rc;
+    return launch_clusters(kern, c.C, count, 32 * (c.w + 1), col_layout((int)L, c.w).total, s, src, dst, (int)L, c.w,
+                           info, leaf_index);
+}
+// false: not for this batch (*rc untouched)
+bool launch_leaf_col_batched(const BatchView& src, const BatchView& dst, int64_t L, int32_t* info, int leaf_index,
+                             int count, cudaStream_t s, int* rc) {
+    ColConfig c;
+    int cmax = kColMaxCtas;
+    while (cmax > 1 && (!col_config(L, &c, cmax) || (int64_t)c.C * count > col_batch_sms())) cmax /= 2;
+    if (cmax <= 1 || L < 16) return false;  // a leaf below 16 is a handful of steps either way
+    switch (c.T) {
+        case 1: *rc = launch_leaf_col_batched_t<1>(src, dst, c, L, info, leaf_index, count, s); break;
+        case 2: *rc = launch_leaf_col_batched_t<2>(src, dst, c, L, info, leaf_index, count, s); break;
+        case 4: *rc = launch_leaf_col_batched_t<4>(src, dst, c, L, info, leaf_index, count, s); break;
+        default: *rc = launch_leaf_col_batched_t<8>(src, dst, c, L, info, leaf_index, count, s); break;
+    }
+    return true;
 }
 
 template <bool S, bool P>
@@ -729,6 +768,10 @@ int launch_leaf_gj_batched(const BatchView& src, const BatchView& dst, int64_t L
                            int64_t scratch_stride, int32_t* info, int leaf_index, int count, cudaStream_t s) {
     if (L <= 0 || count <= 0) return SPIN_OK;
     if (L > kMaxLeaf || count > 65535) return SPIN_ERR_INVALID_ARG;
+    {
+        int rc = SPIN_OK;
+        if (launch_leaf_col_batched(src, dst, L, info, leaf_index, count, s, &rc)) return rc;
+    }
     if (L <= kCtaMaxL && !use_cluster_leaf_for_batches()) {
         static PerDeviceOnce attrs;
         const size_t smem = cta_leaf_smem((int)L);

@@ -3,6 +3,8 @@
 slot ring) and of its pivot search and reciprocal: bit for bit the batched
 paths' leaf, which shares none of that code (rows in one CTA up to 128, rows
 over a cluster above), with the same status."""
+import time
+
 import numpy as np
 import pytest
 
@@ -45,9 +47,17 @@ def matrix(kind, L, rng):
 def test_same_bits_as_the_batched_leaf(spin, L, kind):
     A = torch.from_numpy(np.ascontiguousarray(matrix(kind, L, np.random.default_rng(1000 * L + len(kind))))).cuda()
     info = torch.zeros(4, dtype=torch.int32, device="cuda:0")
+    torch.cuda.synchronize()
+    start = time.perf_counter()
     X = spin.leaf_inverse(A, info_dev=info)
-    Y, status = spin.invert_batched([A], leaf=L, schedule="lockstep")
+    torch.cuda.synchronize()
+    assert time.perf_counter() - start < 2.0  # a bad pivot ends every warp, none waits for its limit (4 s)
+    # enough leaves that the batch does not take clusters of columns as well
+    Y, status = spin.invert_batched([A] * 80, leaf=L, schedule="lockstep")
     torch.cuda.synchronize()
     assert info[0].item() == status[0].item()
+    Z, few = spin.invert_batched([A] * 3, leaf=L, schedule="lockstep")  # clusters of columns, up to 152 CTAs
+    torch.cuda.synchronize()
+    assert few[2].item() == status[0].item()
     if info[0].item() == 0:
-        assert torch.equal(X, Y[0])
+        assert torch.equal(X, Y[0]) and torch.equal(X, Z[2])
