@@ -31,9 +31,9 @@ CrtFormat crt_format(int64_t k, int min_bits);
 // Bits that stand in for s 8-bit digit slices (pairs t + u < s): an FP64
 // simulation of the residual product (Householder SPD matrices of condition
 // 1e3 and Gram matrices, n = 512, s = 4, 5, 6) gives the residue form at 8 s
-// - 4 bits 0.32 to 0.44 of the digit form's error, which is mostly that of
+// - 5 bits 0.65 to 0.88 of the digit form's error, which is mostly that of
 // the pairs it leaves out.
-inline int crt_bits_for_slices(int s) { return 8 * s - 4; }
+inline int crt_bits_for_slices(int s) { return 8 * s - 5; }
 
 // One operand's or the whole product's device memory.
 //   exps       one int per row of A / column of B, for all of them
