@@ -272,8 +272,10 @@ int spin_batch_schedule_info(const int64_t* n, int count, int leaf, int64_t* sta
  * task to its bucket's counter (two counted runs, the smaller count kept),
  * and each bucket is given the pair under which its tasks took the fewest
  * clocks -- its share of the whole launch, measured beside the other
- * buckets -- when that beats the library's own pair (leaf 64, tile 64, or
- * the first candidate pair if that one is not among them) by 2 %.  The pairs are recorded per order:
+ * buckets -- when that beats the library's own pair (leaf 64 and the tile the
+ * batch gets without a record: 16, 32 or 64 by its total work in units of its
+ * largest matrix; or the first candidate pair if that one is not among them)
+ * by 2 %.  The pairs are recorded per order:
  * plain spin_invert_batched calls with opts.leaf = 0 on the persistent
  * schedule use them (plans captured before are rebuilt).  leaf_out,
  * tile_out (host, count): the chosen pair per entry of orders; ms_out

@@ -656,14 +656,42 @@ int64_t batched_leaf(int64_t n, int leaf_opt, int precision) {
     return std::min<int64_t>(L, n);
 }
 
-// Largest product tile of a bucket of order n in the persistent schedule:
-// the one spin_autotune_batched_persistent recorded, else 64.
+// Largest product tile of the buckets of a plain batch where the autotuner
+// recorded none.  A wide tile reads its operands less often (a 16x16 one keeps
+// the FP64 pipe 15 % less busy than a 32x32 or 64x64 one once every SM has
+// work); a narrow one spreads a product over more SMs, which is what counts
+// while the chain of the largest matrix's products is longer than the rest of
+// the batch can hide.  So the line is the batch's work in units of its largest
+// matrix, sum n^3 / max n^3.  Milliseconds with caps 64, 32 and 16, orders
+// equal (or drawn from 64 to the order given):
+//   1 x 1024: 22.9, 8.95, 6.00       1 x 4096: 207, 138, 133
+//   4 x 2048: 91.7, 66.9, 65.3       4 x 4096: 512, 464, 466
+//   16 to 1024 (3.5): 17.4, 9.79, 8.47    64 to 1024 (9.3): 32.1, 22.0, 21.8
+//   16 x 2048: 247, 231, 239         64 x 700: 39.4, 38.9, 43.2
+//   256 to 512 (35): 11.9, 9.63, 11.1     512 to 1024 (50): 93.0, 90.0, 100.7
+//   1024 to 1024 (92): 165.8, 165.4, 187  2048 to 1024 (194): 346.1, 347.5, 393
+//   256 x 700: 148.1, 148.0, 168     1024 x 128: 6.22, 6.30, 7.55
+int default_tile_cap(const std::vector<Bucket>& buckets) {
+    double work = 0.0, largest = 0.0;
+    for (const Bucket& b : buckets) {
+        const double c = (double)b.n * (double)b.n * (double)b.n;
+        work += c * b.count;
+        largest = std::max(largest, c);
+    }
+    return work < 8.0 * largest ? 16 : work < 100.0 * largest ? 32 : 64;
+}
+
+// Largest product tile per bucket in the persistent schedule: the one
+// spin_autotune_batched_persistent recorded for its order, else the batch's.
 std::map<int64_t, int> g_btile;  // order -> tile cap (guarded by g_bleaf_mu)
 
-int persist_tile_cap(int64_t n) {
+void set_tile_caps(std::vector<Bucket>& buckets) {
+    const int cap = default_tile_cap(buckets);
     std::lock_guard<std::mutex> lk(g_bleaf_mu);
-    auto it = g_btile.find(n);
-    return it == g_btile.end() ? 64 : it->second;
+    for (Bucket& b : buckets) {
+        auto it = g_btile.find(b.n);
+        b.tile_cap = it == g_btile.end() ? cap : it->second;
+    }
 }
 
 // Plain batches run on the persistent kernel unless the caller asks for the
@@ -781,10 +809,7 @@ int build_plan(BatchPlan& p, const int64_t* n, int count, const spin_opts& o, cu
         Bucket b;
         b.n = n[order[i]];
         b.leaf = batched_leaf(b.n, leaf_opt, o.precision);
-        if (p.persistent) {
-            b.leaf = std::min(b.leaf, kPersistMaxLeaf);
-            b.tile_cap = persist_tile_cap(b.n);
-        }
+        if (p.persistent) b.leaf = std::min(b.leaf, kPersistMaxLeaf);
         b.count = j - i;
         b.first = i;
         b.ws_elems = std::max<size_t>(fp64_workspace_elems(b.n, b.leaf), 1);
@@ -800,6 +825,7 @@ int build_plan(BatchPlan& p, const int64_t* n, int count, const spin_opts& o, cu
         p.buckets.push_back(b);
         i = j;
     }
+    if (p.persistent) set_tile_caps(p.buckets);
     std::vector<double*> hw(count);
     if (cudaMalloc(&p.ws, ws_total * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
@@ -1212,12 +1238,12 @@ extern "C" int spin_batch_schedule_info(const int64_t* n, int count, int leaf, i
         Bucket b;
         b.n = sorted[i];
         b.leaf = std::min(batched_leaf(b.n, leaf, SPIN_FP64), kPersistMaxLeaf);
-        b.tile_cap = persist_tile_cap(b.n);
         b.count = j - i;
         b.first = i;
         buckets.push_back(b);
         i = j;
     }
+    set_tile_caps(buckets);
     std::vector<PStage> st;
     std::vector<int64_t> start;
     order_stages(buckets, st, start);
@@ -1269,12 +1295,12 @@ extern "C" int spin_batch_schedule_stages(const int64_t* n, int count, int leaf,
         Bucket b;
         b.n = sorted[i];
         b.leaf = std::min(batched_leaf(b.n, leaf, SPIN_FP64), kPersistMaxLeaf);
-        b.tile_cap = persist_tile_cap(b.n);
         b.count = j - i;
         b.first = i;
         buckets.push_back(b);
         i = j;
     }
+    set_tile_caps(buckets);
     std::vector<PStage> st;
     std::vector<int64_t> start;
     order_stages(buckets, st, start);
@@ -1552,6 +1578,7 @@ extern "C" int spin_autotune_batched_persistent(const int64_t* orders, int count
     std::vector<int64_t> best_leaf(nb, 0), ref_leaf(nb, 0);
     std::vector<int> best_tile(nb, 0), ref_tile(nb, 0);
     std::vector<std::pair<int, int>> tried;
+    const int own_tile = default_tile_cap(buckets);
     PersistBatchRun runner;
     for (int li = 0; li < nleaf && rc == SPIN_OK; li++)
         for (int ti = 0; ti < ntile && rc == SPIN_OK; ti++) {
@@ -1576,10 +1603,10 @@ extern "C" int spin_autotune_batched_persistent(const int64_t* orders, int count
                 }
             }
             if (rc != SPIN_OK) break;
-            // the library's own pair (leaf 64, tile 64), or else the first one, is the
+            // the library's own pair (leaf 64, the batch's tile), or else the first one, is the
             // reference; another pair must beat it by 2 % (task clocks vary by about
             // 1 % between runs, as the buckets share the SMs)
-            const bool is_ref = tried.size() == 1 || (leaves[li] == kPersistMaxLeaf && tiles[ti] == 64);
+            const bool is_ref = tried.size() == 1 || (leaves[li] == kPersistMaxLeaf && tiles[ti] == own_tile);
             for (size_t i = 0; i < nb; i++) {
                 if (is_ref) {
                     ref_clk[i] = m[i];

@@ -188,3 +188,23 @@ def test_protocol_simulation_catches_a_bad_order(L):
     bad[[i0, i1]] = bad[[i1, i0]]
     with pytest.raises(AssertionError, match="deadlock"):
         simulate(bad, 1, seed=0)
+
+
+@pytest.mark.parametrize("count,per_matrix", [(1, 580), (7, 580), (8, 148), (99, 148), (100, 40), (300, 40)])
+def test_product_tile_follows_the_batch_s_work(L, count, per_matrix):
+    """Equal matrices of order 256 (leaf 64: six products of order 128, twelve
+    of order 64, four leaves): tiles of 16 while the batch's work is under 8
+    of its largest matrices, of 32 under 100, of 64 from there on."""
+    rc, got = info(L, [256] * count, 64)
+    assert rc == 0
+    assert got["tasks"] == count * per_matrix
+
+
+def test_product_tile_counts_the_smaller_matrices(L):
+    """Small matrices add their share of work, not their number: beside one
+    matrix of order 256, 448 of order 64 (one leaf each, 1/64 of its work) make
+    the batch 8 matrices of order 256."""
+    for count, per_matrix in ((447, 580), (448, 148)):
+        rc, got = info(L, [256] + [64] * count, 64)
+        assert rc == 0
+        assert got["tasks"] == count + per_matrix
