@@ -60,9 +60,10 @@ typedef enum {
 } spin_status;
 
 typedef enum {
-    SPIN_FP64 = 0,         /* every product in FP64 (plain method); those above 2048 in every
-                              dimension on the tensor cores, 63 bits per operand and the sum
-                              exact, where that has no larger error bound for these operands */
+    SPIN_FP64 = 0,         /* every product in FP64 (plain method); in inversions above order
+                              4096 those above 256 in every dimension on the tensor cores, 63
+                              bits per operand and the sum exact, where that has no larger
+                              error bound for these operands                                 */
     SPIN_MIXED_BF16X3 = 1, /* products on BF16 tensor cores with 3-term splits, FP32 accumulate,
                               then Newton-Schulz refinement to opts.tol                       */
     /* 2 is not a precision (a call passing it gets SPIN_ERR_INVALID_ARG)                     */
@@ -458,8 +459,8 @@ int spin_default_leaf(int64_t n, int precision);
  * given leaf on one GB300: the paper's cost analysis (Sec. 4, Table 2)
  * restated for this GPU -- six products per node priced by tile waves over
  * 152 SMs at the FP64 rate, leaves priced per pivot step on one thread-block
- * cluster.  Above order 4096 it is an upper bound: the top levels' products
- * leave the FP64 pipe there (the leaf's optimum is set by the lower levels).
+ * cluster.  Above order 4096 it is an upper bound: the products above 256
+ * leave the FP64 pipe there (the leaf's optimum is set by those below).
  * spin_default_leaf uses its optimum for untuned FP64 orders.
  * -1 for other precisions or bad arguments. */
 double spin_model_seconds(int64_t n, int leaf, int precision);

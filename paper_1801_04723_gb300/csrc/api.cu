@@ -187,7 +187,7 @@ int ensure_ws(StreamState* st, size_t bytes) {
 // (the FP64 kernel runs).  Kept for later calls, as the workspace is.
 size_t ensure_f64_arena(StreamState* st, int64_t n, int64_t leaf, bool two_streams) {
     const int64_t n1 = split_order(n), n2 = n - n1;
-    if (n <= leaf || n2 <= kF64ResidueMin || f64_residue_moduli(n1) == 0) return 0;
+    if (n <= leaf || n2 <= kF64ResidueTop || f64_residue_moduli(n1) == 0) return 0;
     const size_t parts = two_streams ? 2 : 1;
     const size_t least = f64_residue_bytes(n1, n1, n1, true);
     size_t want = std::max(least, std::min(f64_residue_bytes(n1, n1, n1, false), kF64ResidueArena / parts));
@@ -794,7 +794,7 @@ int enqueue(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, con
         if (o.workspace == nullptr) {
             f64_bytes = ensure_f64_arena(st, top, leaf, two);
             f64_arena = st->f64_arena;
-        } else if (top > leaf && top - split_order(top) > kF64ResidueMin) {
+        } else if (top > leaf && top - split_order(top) > kF64ResidueTop) {
             const size_t used = round256(need);
             if (o.workspace_bytes > used) f64_bytes = (o.workspace_bytes - used) / (two ? 2 : 1) / 256 * 256;
             f64_arena = ws + used;
@@ -859,9 +859,9 @@ __global__ void synth_sdd_kernel(double* A, int64_t n, uint64_t seed) {
 // ---- cost model of the plain FP64 path (Sec. 4's cost analysis restated
 // for one GB300) ----
 //
-// Every product is priced on the FP64 kernel: above order 4096, whose top
-// levels leave it (f64_residues.cu), the model is an upper bound.  The leaf
-// choice it serves does not depend on those levels.
+// Every product is priced on the FP64 kernel: above order 4096, where those
+// above 256 leave it (f64_residues.cu), the model is an upper bound.  The leaf
+// choice it serves is made by the levels below.
 //
 // The paper prices each step of Algorithm 1 on a Spark cluster (Table 2,
 // Eq. (SPIN-cost)) and finds a U-shaped dependence on the partition size

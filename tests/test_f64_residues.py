@@ -13,8 +13,9 @@ from paper_1801_04723_gb300 import inputs
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-N = 4161  # split 2112 + 2049: every product of the top level is above the line, none below it
+N = 4161  # split 2112 + 2049: every product of the top level is above 2048
 LEAF = 128
+LINE = 256  # products above it in every dimension, in inversions whose top products are above 2048
 
 
 @pytest.fixture(scope="module")
@@ -40,14 +41,20 @@ def products_by_residues(spin, A, **kw):
     X, info = spin.invert(A, leaf=LEAF, **kw)
     rec = spin.profile_collect()
     torch.cuda.synchronize()
-    return X, info, sum(r["kind"] == "gemm_tc" for r in rec)
+    small = [r for r in rec if r["kind"] in ("gemm_tc", "gemm_f64") and min(r["m"], r["n"], r["k"]) <= LINE]
+    assert small and all(r["kind"] == "gemm_f64" for r in small)
+    large = [r for r in rec if r["kind"] in ("gemm_tc", "gemm_f64") and r not in small]
+    assert sum(r["depth"] == 0 for r in large) == 6
+    return X, info, [sum(r["kind"] == "gemm_tc" and (r["depth"] == 0 or not top) for r in large)
+                     for top in (True, False)], len(large)
 
 
 @pytest.mark.parametrize("family", ["spd", "sdd"])
 def test_as_accurate_as_the_fp64_kernel(spin, family):
     A = (inputs.spd_gram_device(N, 5, "cuda:0", alpha=0.3) if family == "spd" else inputs.sdd_device(N, 6, "cuda:0"))
-    X, info, count = products_by_residues(spin, A)
-    assert info["status"] == 0 and count == 6
+    X, info, (top, count), large = products_by_residues(spin, A)
+    assert info["status"] == 0 and top == 6
+    assert count == large or family == "sdd"  # a diagonally dominant inverse's short products are refused
     Y, _ = fp64_kernel_inverse(spin, A)
     assert not torch.equal(X, Y)  # another rounding, so the other form did run
     Ah, Xh, Yh = A.cpu().numpy(), X.cpu().numpy(), Y.cpu().numpy()
@@ -61,12 +68,12 @@ def test_same_bits_on_one_stream_and_in_panels(spin):
     """The same products on one or two streams, and in an arena a caller's
     workspace leaves (several panels)."""
     A = inputs.spd_gram_device(N, 7, "cuda:0", alpha=0.5)
-    X, _, _ = products_by_residues(spin, A)
-    Y, _, _ = products_by_residues(spin, A, schedule="lockstep")
+    X, _, _, large = products_by_residues(spin, A)
+    Y, _, _, _ = products_by_residues(spin, A, schedule="lockstep")
     assert torch.equal(X, Y)
     ws = torch.empty(spin.workspace_bytes(N, leaf=LEAF) + (400 << 20), dtype=torch.uint8, device="cuda:0")
-    Z, _, count = products_by_residues(spin, A, workspace=ws)
-    assert count == 6 and torch.equal(X, Z)
+    Z, _, (_, count), _ = products_by_residues(spin, A, workspace=ws)
+    assert count == large and torch.equal(X, Z)
 
 
 def test_widely_spread_operands_keep_the_fp64_kernel(spin):
@@ -76,7 +83,7 @@ def test_widely_spread_operands_keep_the_fp64_kernel(spin):
     g = torch.Generator(device="cuda:0").manual_seed(3)
     d = torch.exp2(torch.randint(-40, 41, (N,), generator=g, device="cuda:0").double())
     A = (A * d[:, None]) * d[None, :]
-    X, info, count = products_by_residues(spin, A)
+    X, info, (_, count), _ = products_by_residues(spin, A)
     assert info["status"] == 0 and count == 0
     Y, _ = fp64_kernel_inverse(spin, A)
     assert torch.equal(X, Y)
@@ -86,7 +93,7 @@ def test_widely_spread_operands_keep_the_fp64_kernel(spin):
 def test_non_finite_entries(spin, bad):
     A = inputs.spd_gram_device(N, 9, "cuda:0", alpha=0.5)
     A[17, N - 5] = bad
-    X, info, _ = products_by_residues(spin, A, check=False)
+    X, info, _, _ = products_by_residues(spin, A, check=False)
     Y, info2 = fp64_kernel_inverse(spin, A, check=False)
     assert info["status"] == info2["status"] == 2
     assert (info["fail_leaf"], info["fail_col"]) == (info2["fail_leaf"], info2["fail_col"])
