@@ -32,6 +32,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <utility>
+
 #include <algorithm>
 
 #include "crt.h"
@@ -272,110 +274,122 @@ struct CrtTable {
     int moduli, bits;
 };
 
-// The sum whose residue fraction (sum / P modulo 1, times 2^128) is f, times
-// 2^scale, rounded to FP64 (neg: times -1).
-__device__ __forceinline__ double crt_value(unsigned long long hi, unsigned long long lo, const CrtTable& t, int scale,
-                                            bool neg) {
-    if (hi >> 63) {  // the symmetric range: fractions of one half and more are negative
-        lo = 0ull - lo;
-        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
-        neg = !neg;
+// The sum whose residue fraction (sum / P modulo 1) has the limbs w, lowest
+// first, times 2^scale, rounded to FP64 (neg: times -1).
+template <int LIMBS>
+__device__ __forceinline__ double crt_value(unsigned (&w)[LIMBS], const CrtTable& t, int scale, bool neg) {
+    const unsigned flip = (unsigned)((int)w[LIMBS - 1] >> 31);  // the symmetric range: fractions of
+    unsigned carry = flip & 1u;                                 // one half and more are negative
+    unsigned any = 0u;
+#pragma unroll
+    for (int i = 0; i < LIMBS; i++) {
+        const unsigned x = (w[i] ^ flip) + carry;
+        carry = x < carry ? 1u : 0u;
+        w[i] = x;
+        any |= x;
     }
-    if ((hi | lo) == 0ull) return 0.0;
-    int lz;
-    unsigned long long h;
-    if (hi) {
-        lz = __clzll((long long)hi);
-        h = lz ? (hi << lz) | (lo >> (64 - lz)) : hi;
-    } else {
-        const int s = __clzll((long long)lo);
-        lz = 64 + s;
-        h = lo << s;
+    if (any == 0u) return 0.0;
+    int lz = 0;  // bits before the first set one, below 32 but for sums of under 2^-32 P
+    while (w[LIMBS - 1] == 0u) {
+#pragma unroll
+        for (int i = LIMBS - 1; i > 0; i--) w[i] = w[i - 1];
+        w[0] = 0u;
+        lz += 32;
     }
-    unsigned long long prod = __umul64hi(h, t.pm);  // the sum = prod 2^(pe - lz)
-    const int s = __clzll((long long)prod);         // 0 or 1
-    prod <<= s;
+    const int s = __clz((int)w[LIMBS - 1]);
+    lz += s;
+    const unsigned h1 = __funnelshift_l(w[LIMBS - 2], w[LIMBS - 1], s), h0 = __funnelshift_l(w[LIMBS - 3], w[LIMBS - 2], s);
+    unsigned long long prod = __umul64hi((unsigned long long)h1 << 32 | h0, t.pm);  // the sum = prod 2^(pe - lz)
+    const int one = (int)(~prod >> 63);                                             // prod >= 2^62
+    if (one) prod += prod;
     const unsigned long long m = (prod >> 11) + ((prod >> 10) & 1ull);  // 53 bits, or 2^53
-    const int e = 11 + t.pe - lz - s + scale;                          // value = m 2^e
+    const int e = 11 + t.pe - lz - one + scale;                         // value = m 2^e
     const int be = e + 52 + 1023;
     double v;
     if (be >= 1 && be <= 2045)
         v = __longlong_as_double((long long)(((unsigned long long)(be - 1) << 52) + m));
     else
         v = ldexp((double)m, e);
-    return neg ? -v : v;
+    return neg != (flip != 0u) ? -v : v;
 }
 
 // 4 columns of a row per thread.  p: the whole product (views, epilogue);
 // (row0, col0): the panel pair's origin; rows x cols its size.  LIMBS 32-bit
 // limbs of the fraction: 3 leave an error of 2^-84 P, i.e. below 2^-60 of the
 // largest entries' product for the formats that use it (bits <= 55).
-template <int LIMBS>
-__global__ void __launch_bounds__(256)
+// Bound by instructions (about 200 per output, 39 to 80 of them 32 x 32 + 64
+// bit multiply-adds): the number of moduli is a template argument, so the words
+// of a thread's four outputs (and of C) are all requested before the first is
+// used and the constants are immediate.  4096^2 outputs of 15 moduli with C:
+// 187 us, 344 with four words in flight in a run-time loop and the indices by a
+// division each (540 MB: 80 us).  Four blocks an SM spill: 64 registers.
+template <int LIMBS, int MODULI>
+__global__ void __launch_bounds__(256, 2)
 crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int cols, int row0, int col0,
                    const __grid_constant__ CrtTable t, const __grid_constant__ TcGemmParams p) {
     const int z = blockIdx.z;
     if (p.active != nullptr && p.active[p.batch ? z : 0] == 0) return;
     const int64_t plane = (int64_t)rows * ldr;
-    res += (int64_t)z * t.moduli * plane;
+    res += (int64_t)z * MODULI * plane;
     const int* row_exp = p.row_exp + (int64_t)z * p.M + row0;
     const int* col_exp = p.col_exp + (int64_t)z * p.N + col0;
     const int groups = (cols + 3) / 4;
-    const int64_t total = (int64_t)rows * groups;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    const int dr = (int)(stride / groups), dc = (int)(stride % groups);
     const int so = p.sum_order ? p.sum_order[z] : 0x7fffffff;
     const bool add = p.beta != 0.0;
     double ss = 0.0, ss2 = 0.0;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / groups), c = (int)(idx % groups) * 4;
-        const uint8_t* src = res + (int64_t)r * ldr + c;
-        unsigned long long acc[4][LIMBS];
-#pragma unroll
-        for (int u = 0; u < 4; u++)
-#pragma unroll
-            for (int i = 0; i < LIMBS; i++) acc[u][i] = 0ull;
-#pragma unroll 4
-        for (int l = 0; l < t.moduli; l++) {
-            const unsigned w = *reinterpret_cast<const unsigned*>(src + l * plane);
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const unsigned b = (w >> (8 * u)) & 255u;
-#pragma unroll
-                for (int i = 0; i < LIMBS; i++) acc[u][i] += (unsigned long long)b * t.v[l][4 - LIMBS + i];
-            }
+    int cg = (int)(first % groups);
+    for (int64_t rr = first / groups; rr < rows; rr += dr) {
+        const int r = (int)rr, c = cg * 4;
+        cg += dc;
+        if (cg >= groups) {
+            cg -= groups;
+            rr++;
         }
+        const uint8_t* src = res + (int64_t)r * ldr + c;
+        unsigned word[MODULI];
+#pragma unroll
+        for (int l = 0; l < MODULI; l++) word[l] = *reinterpret_cast<const unsigned*>(src + l * plane);
         const int er = row_exp[r], grow = row0 + r;
         const double* crow = add ? in_row(p, z, grow) + col0 + c : nullptr;
         double* drow = out_row(p, z, grow) + col0 + c;
-        double val[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const int ec = c + u < cols ? col_exp[c + u] : 0;
-            unsigned w[LIMBS];  // the limbs, carried
-            unsigned long long carry = 0ull;
-#pragma unroll
-            for (int i = 0; i < LIMBS; i++) {
-                carry += acc[u][i];
-                w[i] = (unsigned)carry;
-                carry >>= 32;
-            }
-            const unsigned long long hi = (unsigned long long)w[LIMBS - 1] << 32 | w[LIMBS - 2];
-            const unsigned long long lo = LIMBS == 4 ? (unsigned long long)w[1] << 32 | w[0] : (unsigned long long)w[0] << 32;
-            val[u] = crt_value(hi, lo, t, er + ec - 2 * t.bits, p.alpha < 0.0);
-            // an infinity or NaN in the row or column (no fixed point has it)
-            if (er > 1024 || ec > 1024) val[u] = __longlong_as_double(0x7ff8000000000000ll);
-        }
-        const int gcol = col0 + c;
         // whole 32-byte sectors where the views allow it
         const bool quad = c + 3 < cols && aligned32(drow) && (!add || aligned32(crow));
-        if (add) {  // beta = 1
-            double old[4];
+        double old[4];
+        if (add) {
             if (quad) {
                 ld_global_v4(crow, old);
             } else {
 #pragma unroll
                 for (int u = 0; u < 4; u++) old[u] = c + u < cols ? crow[u] : 0.0;
             }
+        }
+        double val[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            unsigned long long acc[LIMBS] = {};
+#pragma unroll
+            for (int l = 0; l < MODULI; l++) {
+                const unsigned b = (word[l] >> (8 * u)) & 255u;
+#pragma unroll
+                for (int i = 0; i < LIMBS; i++) acc[i] += (unsigned long long)b * t.v[l][4 - LIMBS + i];
+            }
+            const int ec = c + u < cols ? col_exp[c + u] : 0;
+            unsigned w[LIMBS];  // the limbs, carried
+            unsigned long long carry = 0ull;
+#pragma unroll
+            for (int i = 0; i < LIMBS; i++) {
+                carry += acc[i];
+                w[i] = (unsigned)carry;
+                carry >>= 32;
+            }
+            val[u] = crt_value<LIMBS>(w, t, er + ec - 2 * t.bits, p.alpha < 0.0);
+            // an infinity or NaN in the row or column (no fixed point has it)
+            if (er > 1024 || ec > 1024) val[u] = __longlong_as_double(0x7ff8000000000000ll);
+        }
+        const int gcol = col0 + c;
+        if (add) {  // beta = 1
 #pragma unroll
             for (int u = 0; u < 4; u++) val[u] = old[u] + val[u];
         }
@@ -419,6 +433,18 @@ crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int c
 }
 
 // ------------------------------------------------------------------ host --
+
+using CombineKernel = void (*)(const uint8_t*, int64_t, int, int, int, int, CrtTable, TcGemmParams);
+template <int LIMBS, int FIRST, int... M>
+CombineKernel combine_of(int moduli, std::integer_sequence<int, M...>) {
+    static constexpr CombineKernel kernels[] = {crt_combine_kernel<LIMBS, FIRST + M>...};
+    return moduli >= FIRST && moduli < FIRST + (int)sizeof...(M) ? kernels[moduli - FIRST] : nullptr;
+}
+// Up to 55 bits and k <= 98304 take 17 moduli at most, 56 bits 15 at least.
+CombineKernel combine_kernel(const CrtFormat& f) {
+    return f.bits <= 55 ? combine_of<3, kCrtMinModuli>(f.moduli, std::make_integer_sequence<int, 18 - kCrtMinModuli>())
+                        : combine_of<4, 15>(f.moduli, std::make_integer_sequence<int, kCrtMaxModuli - 14>());
+}
 
 // floor(2^128 u / p) with p, u < 2^9, rounded, as four limbs.
 void fraction_limbs(unsigned u, unsigned p, unsigned (&v)[4]) {
@@ -603,6 +629,8 @@ int crt_run(const CrtProduct& p, const CrtFormat& f, const CrtPanels& c, unsigne
     });
     if (rc) return rc;
     const int sms = sm_count();
+    const CombineKernel combine = combine_kernel(f);
+    if (combine == nullptr) return SPIN_ERR_INVALID_ARG;
     for (int row0 = 0; row0 < m; row0 += (int)c.rows) {
         const int rows = std::min((int)c.rows, m - row0);
         CUtensorMap ta;
@@ -628,10 +656,7 @@ int crt_run(const CrtProduct& p, const CrtFormat& f, const CrtPanels& c, unsigne
             const int64_t total = (int64_t)rows * ((cols + 3) / 4);
             const int64_t per = std::max<int64_t>(1, (int64_t)sms * 8 / count);
             const dim3 cg((unsigned)std::min<int64_t>((total + 255) / 256, per), 1, (unsigned)count);
-            if (f.bits <= 55)
-                crt_combine_kernel<3><<<cg, 256, 0, s>>>(res, g.ldr, rows, cols, row0, col0, table, q);
-            else
-                crt_combine_kernel<4><<<cg, 256, 0, s>>>(res, g.ldr, rows, cols, row0, col0, table, q);
+            combine<<<cg, 256, 0, s>>>(res, g.ldr, rows, cols, row0, col0, table, q);
             SPIN_CUDA_TRY(cudaGetLastError());
             nl += 2;
         }

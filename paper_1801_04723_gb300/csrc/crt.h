@@ -8,6 +8,7 @@
 
 namespace spin {
 
+constexpr int kCrtMinModuli = 7;  // 27 bits at k = 1
 constexpr int kCrtMaxModuli = 20;
 constexpr int kCrtMaxBits = 63;  // signed in 64 bits
 
