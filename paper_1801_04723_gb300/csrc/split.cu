@@ -8,10 +8,14 @@
 //       column, 4 consecutive rows per lane;
 // so that every plane is written in 8-byte pieces, 256 bytes per warp.  Bound
 // by HBM (8 bytes read, 2 written per plane and entry) for the BF16 and digit
-// planes, by FP32 arithmetic (6 operations per residue) for the residues.
+// planes, by FP32 arithmetic (6 operations per residue) for the residues.  A
+// warp's rows (columns) are a loop that is not unrolled: the residues' code is
+// long, and four copies of it per side came from memory on every launch (both
+// operands of 512^2 to 15 moduli: 29 -> 12 us; of 2048^2 73 -> 63).
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "crt.h"
 #include "split.h"
@@ -65,10 +69,27 @@ __device__ __forceinline__ void count_entry(int (&count)[kSpreadSteps], double v
 }
 
 constexpr int kExpWarps = 16;
+// Loads a thread has in flight: one warp walks a row (16 warps a block of 32
+// columns), so few warps share an SM and latency bounds the pass.  Both
+// operands of 2048^2: 18.8 us, 36.6 with one load of A and four of B at a time
+// and one form of the kernel for everything; of 4096^2 50.7 and 87 us (268 MB:
+// 40 us).
+constexpr int kExpLoads = 8;
+// A load that stays before the next one: left to itself the compiler takes
+// them one by one and waits for each.
+__device__ __forceinline__ double load_now(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
 
 // Blocks [0, blocks_a): kExpWarps rows of A, a warp each; the others: 32
-// columns of B, all warps over the rows.
-template <class Side>
+// columns of B, all warps over the rows.  SPREAD: the counts of the large FP64
+// products' rule too; SUM: sums of squares (sumsq_a, sumsq_b, each may be
+// null).  Forms of their own: the counts' registers leave room for one block
+// an SM instead of three, and under a run-time condition the compiler computes
+// the squares for everyone and selects afterwards, on the FP64 pipe.
+template <class Side, bool SPREAD, bool SUM>
 __global__ void __launch_bounds__(32 * kExpWarps)
 exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restrict__ ea, int* __restrict__ eb,
                  double* sumsq_a, double* sumsq_b, int64_t sss, int* spread, const int* active, const int* valid) {
@@ -77,7 +98,7 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nv = valid ? valid[z] : 0x7fffffff;
     __shared__ int smax[kExpWarps][32];
-    __shared__ int scount[32][kSpreadSteps + 1];
+    __shared__ int scount[SPREAD ? 32 : 1][kSpreadSteps + 1];
     __shared__ double ssum[kExpWarps];
     double ss = 0.0;
     double* sum;
@@ -88,14 +109,25 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
             const double* p = A.row(z, r);
             const bool sum_row = sum != nullptr && r < nv;
             int top = 0;
-            for (int c = lane; c < k; c += 32) {
+            int c = lane;
+            for (; c + 32 * (kExpLoads - 1) < k; c += 32 * kExpLoads) {
+                double v[kExpLoads];
+#pragma unroll
+                for (int u = 0; u < kExpLoads; u++) v[u] = load_now(p + c + 32 * u);
+#pragma unroll
+                for (int u = 0; u < kExpLoads; u++) {
+                    top = max(top, exp_field(v[u]));
+                    if (SUM && sum_row && c + 32 * u < nv) ss = fma(v[u], v[u], ss);
+                }
+            }
+            for (; c < k; c += 32) {
                 const double v = p[c];
                 top = max(top, exp_field(v));
-                if (sum_row && c < nv) ss = fma(v, v, ss);
+                if (SUM && sum_row && c < nv) ss = fma(v, v, ss);
             }
             top = __reduce_max_sync(0xffffffffu, top);
             if (lane == 0) ea[(int64_t)z * m + r] = top - 1022;
-            if (spread != nullptr) {
+            if constexpr (SPREAD) {
                 int count[kSpreadSteps] = {};
                 bool nonzero = false;
                 for (int c = lane; c < k; c += 32) {
@@ -118,32 +150,32 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
         double ss4[4] = {0.0, 0.0, 0.0, 0.0};  // a dependent FP64 FMA takes 64 cycles and more here
         if (col_ok) {
             int r = warp;
-            for (; r + 3 * kExpWarps < k; r += 4 * kExpWarps) {
-                double v[4];
+            for (; r + (kExpLoads - 1) * kExpWarps < k; r += kExpLoads * kExpWarps) {
+                double v[kExpLoads];
 #pragma unroll
-                for (int u = 0; u < 4; u++) v[u] = B.row(z, r + u * kExpWarps)[c];
+                for (int u = 0; u < kExpLoads; u++) v[u] = load_now(B.row(z, r + u * kExpWarps) + c);
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
+                for (int u = 0; u < kExpLoads; u++) {
                     top = max(top, exp_field(v[u]));
-                    if (sum_col && r + u * kExpWarps < nv) ss4[u] = fma(v[u], v[u], ss4[u]);
+                    if (SUM && sum_col && r + u * kExpWarps < nv) ss4[u & 3] = fma(v[u], v[u], ss4[u & 3]);
                 }
             }
             for (; r < k; r += kExpWarps) {
                 const double v = B.row(z, r)[c];
                 top = max(top, exp_field(v));
-                if (sum_col && r < nv) ss4[0] = fma(v, v, ss4[0]);
+                if (SUM && sum_col && r < nv) ss4[0] = fma(v, v, ss4[0]);
             }
         }
         ss = (ss4[0] + ss4[1]) + (ss4[2] + ss4[3]);
         smax[warp][lane] = top;
-        if (spread != nullptr)
+        if constexpr (SPREAD)
             for (int i = threadIdx.x; i < 32 * (kSpreadSteps + 1); i += blockDim.x) (&scount[0][0])[i] = 0;
         __syncthreads();
         top = 0;
 #pragma unroll
         for (int w = 0; w < kExpWarps; w++) top = max(top, smax[w][lane]);
         if (warp == 0 && col_ok) eb[(int64_t)z * n + c] = top - 1022;
-        if (spread != nullptr) {
+        if constexpr (SPREAD) {
             int count[kSpreadSteps] = {};
             int nonzero = 0;
             if (col_ok)
@@ -166,7 +198,7 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
             }
         }
     }
-    if (sum != nullptr) {  // the same for the whole block
+    if (SUM && sum != nullptr) {  // the same for the whole block
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) ss += __shfl_down_sync(0xffffffffu, ss, off);
         if (lane == 0) ssum[warp] = ss;
@@ -333,12 +365,8 @@ split_kernel(Side A, Side B, const __grid_constant__ SplitTarget t, int64_t tile
         uint16_t* dst = t.a + (int64_t)z * t.planes * plane;
         const int r0 = (int)(blockIdx.x / ktiles) * kTileRows, c = (int)(blockIdx.x % ktiles) * kTileK + 4 * lane;
         if (c >= t.k) return;
-#pragma unroll
-        for (int i = warp; i < kTileRows; i += 8) {
-            const int r = r0 + i;
-            if (r >= t.rows) break;
+        auto load = [&](int r, double (&x)[4], int& e) {
             const double* p = A.row(z, t.row0 + r) + c;
-            double x[4];
             if (c + 3 < t.k && ((uintptr_t)p & 15u) == 0) {
                 const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
                 x[0] = a.x;
@@ -349,8 +377,20 @@ split_kernel(Side A, Side B, const __grid_constant__ SplitTarget t, int64_t tile
 #pragma unroll
                 for (int u = 0; u < 4; u++) x[u] = c + u < t.k ? p[u] : 0.0;
             }
-            const int e = t.ea ? t.ea[(int64_t)z * t.m + t.row0 + r] : 0;
+            e = t.ea ? t.ea[(int64_t)z * t.m + t.row0 + r] : 0;
+        };
+        const int end = min(r0 + kTileRows, t.rows);
+        double x[4], next[4];
+        int e, next_e = 0;
+        int r = r0 + warp;
+        if (r < end) load(r, x, e);
+#pragma unroll 1
+        for (; r < end; r += 8) {
+            if (r + 8 < end) load(r + 8, next, next_e);
             convert(x, e, dst + (int64_t)r * t.ld + c, plane);
+#pragma unroll
+            for (int u = 0; u < 4; u++) x[u] = next[u];
+            e = next_e;
         }
         return;
     }
@@ -368,7 +408,7 @@ split_kernel(Side A, Side B, const __grid_constant__ SplitTarget t, int64_t tile
     __syncthreads();
     const int r = r0 + 4 * lane;
     if (r >= t.k) return;
-#pragma unroll
+#pragma unroll 1
     for (int i = warp; i < kTileRows; i += 8) {
         const int c = c0 + i;
         if (c >= t.cols) break;
@@ -415,8 +455,11 @@ int exponents_sides(Side A, Side B, const SplitSource& src, int m, int n, int k,
                     double* sb, int* spread, int count, int64_t sss, cudaStream_t s) {
     const int ba = ea ? (m + kExpWarps - 1) / kExpWarps : 0, bb = eb ? (n + 31) / 32 : 0;
     if (ba + bb == 0) return SPIN_OK;
-    exponents_kernel<Side><<<dim3((unsigned)(ba + bb), (unsigned)count), 32 * kExpWarps, 0, s>>>(
-        A, B, m, n, k, ba, ea, eb, sa, sb, sss, spread, src.active, src.valid);
+    const dim3 grid((unsigned)(ba + bb), (unsigned)count);
+    auto kernel = sa != nullptr || sb != nullptr ? exponents_kernel<Side, false, true> : exponents_kernel<Side, false, false>;
+    if constexpr (std::is_same<Side, SideOne>::value)
+        if (spread != nullptr) kernel = exponents_kernel<Side, true, false>;
+    kernel<<<grid, 32 * kExpWarps, 0, s>>>(A, B, m, n, k, ba, ea, eb, sa, sb, sss, spread, src.active, src.valid);
     SPIN_CUDA_TRY(cudaGetLastError());
     return SPIN_OK;
 }
@@ -425,7 +468,8 @@ int exponents_sides(Side A, Side B, const SplitSource& src, int m, int n, int k,
 
 int launch_exponents(const SplitSource& src, int m, int n, int k, int* ea, int* eb, double* sumsq_a, double* sumsq_b,
                      int* spread, cudaStream_t s) {
-    if (src.count > 65535 || (spread != nullptr && src.count > 0)) return SPIN_ERR_INVALID_ARG;
+    if (src.count > 65535) return SPIN_ERR_INVALID_ARG;
+    if (spread != nullptr && (src.count > 0 || sumsq_a != nullptr || sumsq_b != nullptr)) return SPIN_ERR_INVALID_ARG;
     if (src.count > 0)
         return exponents_sides(SideMany{src.Av}, SideMany{src.Bv}, src, m, n, k, ea, eb, sumsq_a, sumsq_b, spread,
                                src.count, 1, s);
