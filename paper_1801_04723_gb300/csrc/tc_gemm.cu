@@ -29,7 +29,8 @@
 // SM looping over the tiles, see use_persistent_tiles), warp-specialised:
 //   warp 0      TMA producer (one lane): a ~192 KB ring of BF16 operand
 //               stages, 128-byte swizzled, mbarrier complete_tx.  Float mode:
-//               128 x 256 tiles, 4 stages of one 64-wide k-block; exact mode:
+//               128 x 256 tiles, 4 stages of one 64-wide k-block (narrower
+//               tiles and 6 stages for products of few tiles); exact mode:
 //               128 x 128 tiles, 3 stages of two k-blocks.
 //   warp 1      TMEM owner and MMA issuer (one lane): tcgen05.mma kind::f16,
 //               K = 16 per instruction, one commit per stage.
@@ -71,7 +72,7 @@ namespace {
 #ifndef SPIN_KSUB_FLOAT
 #define SPIN_KSUB_FLOAT 1
 #endif
-constexpr int kFloatBN = SPIN_FLOAT_BN;             // float-mode tile width
+constexpr int kFloatBN = SPIN_FLOAT_BN;             // float-mode tile width (large products)
 constexpr int kExactBN = SPIN_EXACT_BN;             // exact-mode tile width (small products)
 constexpr int kExactEpiWarps = SPIN_EXACT_EPI_WARPS;  // exact-mode epilogue warps (small products)
 // Large exact products use 128 x 256 tiles: an MMA of N = 256 per SM keeps
@@ -931,6 +932,17 @@ int launch_tc_gemm(const TcOperand& a, const TcOperand& b, const TcGemmParams& p
             return launch_impl<256, true, 16>(a, b, p, s);
         return launch_impl<kExactBN, true, kExactEpiWarps>(a, b, p, s);
     }
+    // The narrowest tile whose tiles of all problems run at once: until the SMs
+    // are full a wider one only makes each SM's share of D longer (an FP64
+    // column of a tile is 1 KB in and 1 KB out).  Splits and product, us, at 256,
+    // 128, 64 and 32 columns: 512^3 39.2, 30.4, 24.7, 22.6; 1024^3 49.4, 40.3,
+    // 34.9, -; 1536^3 65.6, 54.4, 71.8, -; 2048^3 88.1, 107, 162, -.  Mixed order
+    // 1000 2044 -> 1943 us.  Every output is summed in the same order.
+    const int64_t rows = (int64_t)((p.M + BM - 1) / BM) * (p.batch ? p.batch : 1), sms = sm_count();
+    auto at_once = [&](int bn) { return rows * ((p.N + bn - 1) / bn) <= sms; };
+    if (at_once(32)) return launch_impl<32, false, 8>(a, b, p, s);
+    if (at_once(64)) return launch_impl<64, false, 8>(a, b, p, s);
+    if (at_once(128)) return launch_impl<128, false, 8>(a, b, p, s);
     return launch_impl<kFloatBN, false, 8>(a, b, p, s);
 }
 
