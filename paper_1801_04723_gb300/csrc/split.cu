@@ -52,20 +52,27 @@ __device__ __forceinline__ int exp_field(double x) {
 constexpr int kSpreadSteps = 26;  // t = 0, 1, ..., 25
 constexpr int kNoSpread = 1000;
 
-// Least t of 0 .. 25 with count[t] >= (8 - g) / 8 k (count: entries whose
-// exponent is at least the largest - t).
-__device__ __forceinline__ int spread_of(const int (&count)[kSpreadSteps], int k, int top, int g) {
-    if (top == 0x7FF) return kNoSpread;  // an infinity or NaN
-    int t = kNoSpread;
-#pragma unroll
-    for (int i = kSpreadSteps - 1; i >= 0; i--)
-        if (8ll * count[i] >= (long long)(8 - g) * k) t = i;
-    return t;
+// The spread counts: per thread 32 bins of 16 bits in shared memory, bin d the
+// entries whose exponent is d below the largest (31: further, or 0), two bins a
+// word and a bank per lane, so that one shared add per entry is all (26
+// comparisons and additions in registers took 3/4 of the pass's time; a thread
+// sees at most 98304 / 16 entries).
+constexpr int kSpreadWords = 16;
+__device__ __forceinline__ void count_entry(unsigned (*bins)[32], int lane, double v, int top) {
+    const int f = exp_field(v), d = f == 0 ? 31 : min(top - f, 31);
+    atomicAdd(&bins[d >> 1][lane], 1u << ((d & 1) * 16));
 }
-__device__ __forceinline__ void count_entry(int (&count)[kSpreadSteps], double v, int top) {
-    const int f = exp_field(v), d = f == 0 ? 1 << 20 : top - f;
-#pragma unroll
-    for (int i = 0; i < kSpreadSteps; i++) count[i] += d <= i;
+// One bin after the other, from 0: the least t of 0 .. 25 with at least
+// (8 - g) / 8 k entries in bins 0 .. t.
+struct SpreadScan {
+    int seen = 0, t = kNoSpread;
+    __device__ __forceinline__ void next(int i, int count, int k, int g) {
+        seen += count;
+        if (t == kNoSpread && 8ll * seen >= (long long)(8 - g) * k) t = i;
+    }
+};
+__device__ __forceinline__ bool not_zero(double v) {
+    return ((unsigned)__double2hiint(v) << 1 | (unsigned)__double2loint(v)) != 0u;  // no FP64 operation
 }
 
 constexpr int kExpWarps = 16;
@@ -86,9 +93,9 @@ __device__ __forceinline__ double load_now(const double* p) {
 // Blocks [0, blocks_a): kExpWarps rows of A, a warp each; the others: 32
 // columns of B, all warps over the rows.  SPREAD: the counts of the large FP64
 // products' rule too; SUM: sums of squares (sumsq_a, sumsq_b, each may be
-// null).  Forms of their own: the counts' registers leave room for one block
-// an SM instead of three, and under a run-time condition the compiler computes
-// the squares for everyone and selects afterwards, on the FP64 pipe.
+// null).  Forms of their own: under a run-time condition the compiler computes
+// the squares for everyone and selects afterwards, on the FP64 pipe, and the
+// counts take 32 KB of shared memory.
 template <class Side, bool SPREAD, bool SUM>
 __global__ void __launch_bounds__(32 * kExpWarps)
 exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restrict__ ea, int* __restrict__ eb,
@@ -98,7 +105,9 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nv = valid ? valid[z] : 0x7fffffff;
     __shared__ int smax[kExpWarps][32];
-    __shared__ int scount[SPREAD ? 32 : 1][kSpreadSteps + 1];
+    __shared__ int scount[SPREAD ? 32 : 1][kSpreadSteps + 1];  // the last one: the column has a nonzero entry
+    __shared__ unsigned bins[SPREAD ? kExpWarps : 1][kSpreadWords][32];
+    static_assert(kSpreadSteps % 2 == 0 && kSpreadSteps / 2 <= kExpWarps && kSpreadSteps < 2 * kSpreadWords, "bins");
     __shared__ double ssum[kExpWarps];
     double ss = 0.0;
     double* sum;
@@ -128,17 +137,29 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
             top = __reduce_max_sync(0xffffffffu, top);
             if (lane == 0) ea[(int64_t)z * m + r] = top - 1022;
             if constexpr (SPREAD) {
-                int count[kSpreadSteps] = {};
-                bool nonzero = false;
-                for (int c = lane; c < k; c += 32) {
-                    const double v = p[c];
-                    nonzero |= v != 0.0;
-                    count_entry(count, v, top);
-                }
 #pragma unroll
-                for (int i = 0; i < kSpreadSteps; i++) count[i] = __reduce_add_sync(0xffffffffu, count[i]);
+                for (int j = 0; j < kSpreadWords; j++) bins[warp][j][lane] = 0u;
+                bool nonzero = top != 0;
+                if (!nonzero)  // zeros and subnormals
+                    for (int c = lane; c < k; c += 32) nonzero |= not_zero(p[c]);
+                int c = lane;
+                for (; c + 32 * (kExpLoads - 1) < k; c += 32 * kExpLoads) {
+                    double v[kExpLoads];
+#pragma unroll
+                    for (int u = 0; u < kExpLoads; u++) v[u] = load_now(p + c + 32 * u);
+#pragma unroll
+                    for (int u = 0; u < kExpLoads; u++) count_entry(bins[warp], lane, v[u], top);
+                }
+                for (; c < k; c += 32) count_entry(bins[warp], lane, p[c], top);
+                SpreadScan scan;  // a level per lane
+                for (int j = 0; j < kSpreadSteps / 2; j++) {
+                    const unsigned w = bins[warp][j][lane];
+                    scan.next(2 * j, __reduce_add_sync(0xffffffffu, (int)(w & 0xffffu)), k, lane);
+                    scan.next(2 * j + 1, __reduce_add_sync(0xffffffffu, (int)(w >> 16)), k, lane);
+                }
+                const int t = top == 0x7FF ? kNoSpread : scan.t;  // an infinity or NaN
                 const bool any = __any_sync(0xffffffffu, nonzero);
-                if (lane >= 1 && lane <= kSpreadLevels && any) atomicMax(&spread[lane - 1], spread_of(count, k, top, lane));
+                if (lane >= 1 && lane <= kSpreadLevels && any) atomicMax(&spread[lane - 1], t);
             }
         }
     } else {
@@ -168,32 +189,50 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
         }
         ss = (ss4[0] + ss4[1]) + (ss4[2] + ss4[3]);
         smax[warp][lane] = top;
-        if constexpr (SPREAD)
-            for (int i = threadIdx.x; i < 32 * (kSpreadSteps + 1); i += blockDim.x) (&scount[0][0])[i] = 0;
+        if constexpr (SPREAD) {
+#pragma unroll
+            for (int j = 0; j < kSpreadWords; j++) bins[warp][j][lane] = 0u;
+            if (warp == 0) scount[lane][kSpreadSteps] = 0;
+        }
         __syncthreads();
         top = 0;
 #pragma unroll
         for (int w = 0; w < kExpWarps; w++) top = max(top, smax[w][lane]);
         if (warp == 0 && col_ok) eb[(int64_t)z * n + c] = top - 1022;
         if constexpr (SPREAD) {
-            int count[kSpreadSteps] = {};
-            int nonzero = 0;
-            if (col_ok)
-                for (int r = warp; r < k; r += kExpWarps) {
-                    const double v = B.row(z, r)[c];
-                    nonzero |= v != 0.0;
-                    count_entry(count, v, top);
-                }
+            if (col_ok) {
+                bool nonzero = top != 0;
+                if (!nonzero)
+                    for (int r = warp; r < k; r += kExpWarps) nonzero |= not_zero(B.row(z, r)[c]);
+                int r = warp;
+                for (; r + (kExpLoads - 1) * kExpWarps < k; r += kExpLoads * kExpWarps) {
+                    double v[kExpLoads];
 #pragma unroll
-            for (int i = 0; i < kSpreadSteps; i++)
-                if (count[i]) atomicAdd(&scount[lane][i], count[i]);
-            if (nonzero) scount[lane][kSpreadSteps] = 1;
+                    for (int u = 0; u < kExpLoads; u++) v[u] = load_now(B.row(z, r + u * kExpWarps) + c);
+#pragma unroll
+                    for (int u = 0; u < kExpLoads; u++) count_entry(bins[warp], lane, v[u], top);
+                }
+                for (; r < k; r += kExpWarps) count_entry(bins[warp], lane, B.row(z, r)[c], top);
+                if (nonzero) scount[lane][kSpreadSteps] = 1;
+            }
+            __syncthreads();
+            if (warp < kSpreadSteps / 2) {  // a word of bins per warp, a column per lane
+                int lo = 0, hi = 0;
+#pragma unroll
+                for (int w = 0; w < kExpWarps; w++) {
+                    const unsigned x = bins[w][warp][lane];
+                    lo += (int)(x & 0xffffu);
+                    hi += (int)(x >> 16);
+                }
+                scount[lane][2 * warp] = lo;
+                scount[lane][2 * warp + 1] = hi;
+            }
             __syncthreads();
             if (warp >= 1 && warp <= kSpreadLevels) {  // a level per warp, a column per lane
-#pragma unroll
-                for (int i = 0; i < kSpreadSteps; i++) count[i] = scount[lane][i];
+                SpreadScan scan;
+                for (int i = 0; i < kSpreadSteps; i++) scan.next(i, scount[lane][i], k, warp);
                 const bool wanted = col_ok && scount[lane][kSpreadSteps];
-                const int t = __reduce_max_sync(0xffffffffu, wanted ? spread_of(count, k, top, warp) : 0);
+                const int t = __reduce_max_sync(0xffffffffu, wanted ? (top == 0x7FF ? kNoSpread : scan.t) : 0);
                 if (lane == 0) atomicMax(&spread[kSpreadLevels + warp - 1], t);
             }
         }
