@@ -452,7 +452,8 @@ size_t spin_workspace_bytes(int64_t n, const spin_opts* opts);
 /* The leaf order the library picks for n and a precision when leaf = 0:
  * n itself for n <= 128, else the autotuned choice for n's size class
  * (ceil(log2 n); a class above the largest tuned one reuses it), else a
- * built-in default (plain: 512 for n >= 16384, else 256; mixed: 128). */
+ * built-in default (plain: 128, or 256 where 128 would leave leaves of under
+ * about 86 rows above order 256; mixed: 128). */
 int spin_default_leaf(int64_t n, int precision);
 
 /* Predicted time (seconds) of one plain FP64 inversion of order n with the

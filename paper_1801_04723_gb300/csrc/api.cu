@@ -869,8 +869,9 @@ __global__ void synth_sdd_kernel(double* A, int64_t n, uint64_t seed) {
 // levels are too small to fill 152 SMs (left), and Gauss-Jordan leaves run on
 // one cluster of at most 16 SMs at the FP64 rate plus a per-pivot latency
 // (right).  Model, per recursion node: six products (n1, n2 split), each
-//   t = launch + max(ceil(tiles / 152) * 2 * TM * TM * k / P_sm, 2 m n k / P_gpu)
-// with the product kernel's TM x TM tiles (64, 32 or 16) and P_sm = 4 flops/clock at 2.07 GHz (P_gpu = 152 P_sm,
+//   t = launch + max(ceil(tiles / 152) * 2 * rows * cols * k / P_sm, 2 m n k / P_gpu,
+//                    k * 64 clocks)       (an output's chain of dependent FMAs)
+// with the product kernel's tiles (rows x cols) and P_sm = 4 flops/clock at 2.07 GHz (P_gpu = 152 P_sm,
 // 1.259 TFLOP/s, the measured DFMA rate); per leaf of order L on C = min(16,
 // 2^ceil(log2 L)) CTAs, L pivot steps of
 //   a + b T                           (L <= 256: columns over the cluster, T
@@ -888,10 +889,10 @@ constexpr double kModelACol = 0.36e-6, kModelBCol = 0.125e-6, kModelAPull = 3.46
 constexpr double kModelG = 0.44e-9;
 
 double model_gemm(int64_t m, int64_t n, int64_t k) {
-    const int64_t tm = gemm_f64_tile_size(m, n, 1);
-    const double tiles = (double)((m + tm - 1) / tm) * (double)((n + tm - 1) / tm);
-    const double wave = std::ceil(tiles / 152.0) * 2.0 * (double)(tm * tm) * (double)k / kModelPsm;
-    return kModelLaunch + std::max(wave, 2.0 * (double)m * (double)n * (double)k / kModelPgpu);
+    const F64Tile t = gemm_f64_tile_size(m, n, 1);
+    const double tiles = (double)((m + t.rows - 1) / t.rows) * (double)((n + t.cols - 1) / t.cols);
+    const double wave = std::ceil(tiles / 152.0) * 2.0 * (double)(t.rows * t.cols) * (double)k / kModelPsm;
+    return kModelLaunch + std::max({wave, 2.0 * (double)m * (double)n * (double)k / kModelPgpu, 64.0 * (double)k / kModelClock});
 }
 
 double model_leaf(int64_t L) {
@@ -911,12 +912,25 @@ double model_fp64(int64_t n, int64_t leaf) {
            model_gemm(n1, n2, n2) + model_gemm(n2, n1, n1) + model_gemm(n2, n1, n2) + model_gemm(n1, n1, n2);
 }
 
+// Rows of a leaf block of order n at this leaf, about.
+int64_t leaf_rows(int64_t n, int64_t leaf) {
+    while (n > leaf) n = (n + 1) / 2;
+    return n;
+}
+
+// Pivoting is confined to a leaf, so a default of smaller leaves refuses
+// matrices that a larger one inverts: 64 is no default, and above order 256
+// leaves of about 86 rows at least are.  It costs up to a few percent (ms at 64 and 128: order 777 1.518, 1.564; 3000 46.9, 47.1;
+// 8192 29.95, 30.48), more where 128 would leave 65 to 85 rows and 256 is taken
+// (128 and 256: order 300 0.343, 0.438; 5000 13.6, 15.2).
+constexpr int64_t kDefaultLeafRows = 86;
 int model_best_leaf(int64_t n) {
-    static const int cands[] = {64, 128, 256, 512, 1024, 2048};
-    int best = 64;
+    static const int cands[] = {128, 256, 512, 1024, 2048};
+    int best = 128;
     double bt = 1e300;
     for (int L : cands) {
         if (L > n) break;
+        if (n > 256 && L < 256 && leaf_rows(n, L) < kDefaultLeafRows) continue;
         const double t = model_fp64(n, L);
         if (t < bt) {
             bt = t;

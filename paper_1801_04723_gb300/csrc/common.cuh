@@ -103,8 +103,11 @@ struct BatchView {
 };
 
 // ---- kernel launchers (host) ----
-// FP64 product tile size (64, 32 or 16) for count m x n products side by side.
-int gemm_f64_tile_size(int64_t m, int64_t n, int64_t count);
+// FP64 product tile for count m x n products side by side.
+struct F64Tile {
+    int rows, cols;
+};
+F64Tile gemm_f64_tile_size(int64_t m, int64_t n, int64_t count);
 // The tile SPIN_F64_TILE forces (64, 32 or 16; for measurement), else 0.
 int forced_f64_tile();
 // gate (optional, device int): the product runs only while *gate != 0.

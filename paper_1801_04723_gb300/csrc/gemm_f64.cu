@@ -10,10 +10,10 @@
 // the rate of the SMs it occupies.  A 64x64 output tile per 256-thread CTA,
 // 4x4 register tile per thread, k-step 16 staged through double-buffered
 // shared memory, gives 16 independent FMAs per thread per k-slice and needs
-// ~0.25 B of L2 traffic per FMA -- far under any memory roof.  Products too
-// small to give every SM a 64x64 tile (the deep recursion levels: at n =
-// 1024 the three levels have 64, 16 and 4 such tiles) take 32x32 or 16x16
-// tiles instead.  Every output is one FMA chain over k in order, whatever
+// ~0.25 B of L2 traffic per FMA -- far under any memory roof.  Where the last
+// wave of 64x64 tiles would leave SMs idle (most products of a few hundred to
+// a few thousand rows) a product takes 32x32, 16x16, 8x16 or 8x8 tiles
+// instead.  Every output is one FMA chain over k in order, whatever
 // the tile, so the tile size never changes a result bit.  Operands are
 // arbitrary strided views (no alignment beyond 8 B).
 #include <math.h>
@@ -119,41 +119,44 @@ __device__ __forceinline__ void gemm_f64_tile(int64_t m, int64_t n, int64_t k, d
     }
 }
 
-// An 8 x 16 output tile per 128-thread CTA, one output per thread: products
-// whose 16 x 16 tiles leave SMs idle (128^3 has 64 of them).  Each SM
-// sub-partition then runs one chain of dependent FMAs (64 cycles each), which
-// is also all its FP64 unit can take.  Same order of operations (k in order,
-// zero padding to a multiple of BK) as the other tiles.
-constexpr int SM_ROWS = 8, SM_COLS = 16, SM_NT = SM_ROWS * SM_COLS;
+// An 8 x 16 or 8 x 8 output tile per CTA, one output per thread: products whose
+// 16 x 16 tiles leave SMs idle (128^3 has 64 of them) or fill their last wave
+// badly (256^3: 256 on 152 SMs).  A warp's chain of dependent FMAs (64 cycles
+// each) is also all that an SM sub-partition's FP64 unit can take.  Same order
+// of operations (k in order, zero padding to a multiple of BK) as the other
+// tiles.
+constexpr int SM_ROWS = 8;
+template <int COLS>
 __device__ __forceinline__ void gemm_f64_small_tile(int64_t m, int64_t n, int64_t k, double alpha,
                                                     const double* __restrict__ A, int64_t lda,
                                                     const double* __restrict__ B, int64_t ldb, double beta,
                                                     const double* C, int64_t ldc, double* D, int64_t ldd,
                                                     int64_t tile_m, int64_t tile_n) {
     constexpr int KS = 2 * BK;  // two k-steps per stage
+    constexpr int THREADS = SM_ROWS * COLS, AR = THREADS / KS, AP = SM_ROWS / AR, BP = KS / SM_ROWS;
     __shared__ double As[2][KS][SM_ROWS + 1];
-    __shared__ double Bs[2][KS][SM_COLS];
-    const int tid = threadIdx.x, tx = tid % SM_COLS, ty = tid / SM_COLS;
-    const int64_t m0 = tile_m * SM_ROWS, n0 = tile_n * SM_COLS;
-    const int a_kk = tid % KS, a_r = tid / KS;  // A: 4 rows per pass
-    double ra[2], rb[4];
+    __shared__ double Bs[2][KS][COLS];
+    const int tid = threadIdx.x, tx = tid % COLS, ty = tid / COLS;
+    const int64_t m0 = tile_m * SM_ROWS, n0 = tile_n * COLS;
+    const int a_kk = tid % KS, a_r = tid / KS;  // A: AR rows per pass
+    double ra[AP], rb[BP];
     auto load_regs = [&](int64_t k0) {
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int64_t r = m0 + a_r + 4 * i, c = k0 + a_kk;
+        for (int i = 0; i < AP; i++) {
+            const int64_t r = m0 + a_r + AR * i, c = k0 + a_kk;
             ra[i] = (r < m && c < k) ? A[r * lda + c] : 0.0;
         }
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            const int64_t r = k0 + ty + 8 * i, c = n0 + tx;
+        for (int i = 0; i < BP; i++) {
+            const int64_t r = k0 + ty + SM_ROWS * i, c = n0 + tx;
             rb[i] = (r < k && c < n) ? B[r * ldb + c] : 0.0;
         }
     };
     auto store_smem = [&](int buf) {
 #pragma unroll
-        for (int i = 0; i < 2; i++) As[buf][a_kk][a_r + 4 * i] = ra[i];
+        for (int i = 0; i < AP; i++) As[buf][a_kk][a_r + AR * i] = ra[i];
 #pragma unroll
-        for (int i = 0; i < 4; i++) Bs[buf][ty + 8 * i][tx] = rb[i];
+        for (int i = 0; i < BP; i++) Bs[buf][ty + SM_ROWS * i][tx] = rb[i];
     };
     double acc = 0.0;
     const int64_t kpad = (k + BK - 1) / BK * BK;
@@ -217,22 +220,25 @@ gemm_f64_kernel(int64_t m, int64_t n, int64_t k, double alpha, const double* __r
     gemm_f64_tile<TM>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_m, tile_n);
 }
 
-__global__ void __launch_bounds__(SM_NT)
+template <int COLS>
+__global__ void __launch_bounds__(SM_ROWS * COLS)
 gemm_f64_small_kernel(int64_t m, int64_t n, int64_t k, double alpha, const double* __restrict__ A, int64_t lda,
                       const double* __restrict__ B, int64_t ldb, double beta, const double* C, int64_t ldc, double* D,
-                      int64_t ldd) {
-    gemm_f64_small_tile(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, blockIdx.y, blockIdx.x);
+                      int64_t ldd, const int* gate) {
+    if (gate != nullptr && *gate == 0) return;
+    gemm_f64_small_tile<COLS>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, blockIdx.y, blockIdx.x);
 }
 
 // Batched form: problem blockIdx.z uses the views described by the BatchView
 // operands (same shape for every problem, per-problem base and leading dim).
-__global__ void __launch_bounds__(SM_NT)
+template <int COLS>
+__global__ void __launch_bounds__(SM_ROWS * COLS)
 gemm_f64_small_batched_kernel(int64_t m, int64_t n, int64_t k, double alpha, BatchView a, BatchView b, double beta,
                               BatchView c, BatchView d) {
     const int z = blockIdx.z;
     const int64_t lda = a.ld_of(z), ldb = b.ld_of(z), ldd = d.ld_of(z);
     const int64_t ldc = beta != 0.0 ? c.ld_of(z) : 0;
-    gemm_f64_small_tile(m, n, k, alpha, a.ptr(z, lda), lda, b.ptr(z, ldb), ldb, beta,
+    gemm_f64_small_tile<COLS>(m, n, k, alpha, a.ptr(z, lda), lda, b.ptr(z, ldb), ldb, beta,
                         beta != 0.0 ? c.ptr(z, ldc) : nullptr, ldc, const_cast<double*>(d.ptr(z, ldd)), ldd, blockIdx.y,
                         blockIdx.x);
 }
@@ -278,35 +284,31 @@ int tile_group() {
     return g;
 }
 
-// Whether `count` m x n products with tm-row tiles are better off with 8 x 16
-// tiles: the same rule as between the square ones (the busiest SM's FMAs, at
-// least 1.25 times fewer).  128^3: 10.8 -> 7.3 us; 256^3 (256 tiles of 16 x 16,
-// 512 of 8 x 16: 512 FMAs per k on the busiest SM either way) keeps 16 x 16.
-bool use_small_tiles(int64_t m, int64_t n, int64_t count, int tm) {
-    if (tm != 16 || forced_tile() != 0) return false;
-    const double t16 = (double)((m + 15) / 16) * (double)((n + 15) / 16) * (double)count;
-    const double ts = (double)((m + SM_ROWS - 1) / SM_ROWS) * (double)((n + SM_COLS - 1) / SM_COLS) * (double)count;
-    return std::ceil(ts / 152.0) * SM_NT * 1.25 <= std::ceil(t16 / 152.0) * 256.0;
-}
-
 }  // namespace
 
 int forced_f64_tile() { return forced_tile(); }
 
-// Tile size for an m x n product (count of them side by side): the one
-// whose busiest SM has the fewest FMAs, ceil(tiles / 152) * TM^2 per
-// k, larger tiles preferred unless a smaller one is at least 1.25x better
-// (a smaller tile keeps fewer FMAs in flight per thread).
-int gemm_f64_tile_size(int64_t m, int64_t n, int64_t count) {
+// Tile for an m x n product (count of them side by side): the one whose
+// busiest SM has the fewest FMAs, ceil(tiles / 152) * rows * cols per k, larger
+// tiles preferred unless a smaller one has 1 % fewer: all of them keep the FP64
+// pipe equally busy, so that count is the time (within 3 % of ceil(tiles / 152)
+// rows cols k / (2 per clock) plus 4 us).  us with 64, 32, 16 rows, 8 x 16 and
+// 8 x 8: 128^3 -, 35.6, 11.1, 7.6, 7.4; 200^3 -, 56.4, 29.1, 21.9, 18.9; 256^3
+// -, 69.1, 35.3, 34.4, 30.7; 300^3 -, 81.7, 60.5, 50.1, 50.6; 512^3 -, 257.9,
+// 229.2, 228.6, 229.6; 1024^3 2046, 1791, 1736, 1740, 1748 (at 64 rows until a
+// smaller tile was 25 % better, 512^3 took 258 and 1024^3 2046).
+F64Tile gemm_f64_tile_size(int64_t m, int64_t n, int64_t count) {
     const int forced = forced_tile();
-    if (forced) return forced;
-    int best = 64;
+    if (forced) return {forced, forced};
+    constexpr F64Tile tiles[] = {{64, 64}, {32, 32}, {16, 16}, {8, 16}, {8, 8}};
+    F64Tile best = tiles[0];
     double best_cost = 0.0;
-    for (int tm : {64, 32, 16}) {
-        const double tiles = (double)((m + tm - 1) / tm) * (double)((n + tm - 1) / tm) * (double)count;
-        const double cost = std::ceil(tiles / 152.0) * tm * tm;
-        if (tm == 64 || cost * 1.25 <= best_cost) {
-            best = tm;
+    for (const F64Tile& t : tiles) {
+        const int64_t rows = (m + t.rows - 1) / t.rows;
+        const double num = (double)rows * (double)((n + t.cols - 1) / t.cols) * (double)count;
+        const double cost = std::ceil(num / 152.0) * t.rows * t.cols;
+        if (t.rows == 64 || (rows <= 65535 && cost * 1.01 <= best_cost)) {  // blockIdx.y
+            best = t;
             best_cost = cost;
         }
     }
@@ -316,21 +318,15 @@ int gemm_f64_tile_size(int64_t m, int64_t n, int64_t count) {
 int launch_gemm_f64_batched(int64_t m, int64_t n, int64_t k, double alpha, const BatchView& a, const BatchView& b,
                             double beta, const BatchView& c, const BatchView& d, int count, cudaStream_t s) {
     if (m <= 0 || n <= 0 || count <= 0) return SPIN_OK;
-    const int tm = gemm_f64_tile_size(m, n, count);
-    if (use_small_tiles(m, n, count, tm) && count <= 65535) {
-        const dim3 g((unsigned)((n + SM_COLS - 1) / SM_COLS), (unsigned)((m + SM_ROWS - 1) / SM_ROWS), (unsigned)count);
-        gemm_f64_small_batched_kernel<<<g, SM_NT, 0, s>>>(m, n, k, alpha, a, b, beta, c, d);
-        SPIN_CUDA_TRY(cudaGetLastError());
-        return SPIN_OK;
-    }
-    dim3 grid((unsigned)((n + tm - 1) / tm), (unsigned)((m + tm - 1) / tm), (unsigned)count);
+    const F64Tile t = gemm_f64_tile_size(m, n, count);
+    const dim3 grid((unsigned)((n + t.cols - 1) / t.cols), (unsigned)((m + t.rows - 1) / t.rows), (unsigned)count);
     if (grid.y > 65535u || grid.z > 65535u) return SPIN_ERR_INVALID_ARG;
-    if (tm == 64)
-        gemm_f64_batched_kernel<64><<<grid, NT, 0, s>>>(m, n, k, alpha, a, b, beta, c, d);
-    else if (tm == 32)
-        gemm_f64_batched_kernel<32><<<grid, NT, 0, s>>>(m, n, k, alpha, a, b, beta, c, d);
-    else
-        gemm_f64_batched_kernel<16><<<grid, NT, 0, s>>>(m, n, k, alpha, a, b, beta, c, d);
+    auto kernel = t.rows == 64   ? gemm_f64_batched_kernel<64>
+                  : t.rows == 32 ? gemm_f64_batched_kernel<32>
+                  : t.rows == 16 ? gemm_f64_batched_kernel<16>
+                  : t.cols == 16 ? gemm_f64_small_batched_kernel<16>
+                                 : gemm_f64_small_batched_kernel<8>;
+    kernel<<<grid, t.rows >= 16 ? NT : t.rows * t.cols, 0, s>>>(m, n, k, alpha, a, b, beta, c, d);
     SPIN_CUDA_TRY(cudaGetLastError());
     return SPIN_OK;
 }
@@ -339,21 +335,16 @@ int launch_gemm_f64(int64_t m, int64_t n, int64_t k, double alpha, const double*
                     const double* B, int64_t ldb, double beta, const double* C, int64_t ldc, double* D,
                     int64_t ldd, cudaStream_t s, const int* gate) {
     if (m <= 0 || n <= 0) return SPIN_OK;
-    const int tm = gemm_f64_tile_size(m, n, 1);
-    if (gate == nullptr && use_small_tiles(m, n, 1, tm)) {
-        const dim3 g((unsigned)((n + SM_COLS - 1) / SM_COLS), (unsigned)((m + SM_ROWS - 1) / SM_ROWS));
-        gemm_f64_small_kernel<<<g, SM_NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd);
-        SPIN_CUDA_TRY(cudaGetLastError());
-        return SPIN_OK;
-    }
-    dim3 grid((unsigned)((n + tm - 1) / tm), (unsigned)((m + tm - 1) / tm));
+    const F64Tile t = gemm_f64_tile_size(m, n, 1);
+    const dim3 grid((unsigned)((n + t.cols - 1) / t.cols), (unsigned)((m + t.rows - 1) / t.rows));
     if (grid.y > 65535u) return SPIN_ERR_INVALID_ARG;
-    if (tm == 64)
-        gemm_f64_kernel<64><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group(), gate);
-    else if (tm == 32)
-        gemm_f64_kernel<32><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group(), gate);
-    else
-        gemm_f64_kernel<16><<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group(), gate);
+    if (t.rows < 16) {
+        auto kernel = t.cols == 16 ? gemm_f64_small_kernel<16> : gemm_f64_small_kernel<8>;
+        kernel<<<grid, t.rows * t.cols, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, gate);
+    } else {
+        auto kernel = t.rows == 64 ? gemm_f64_kernel<64> : t.rows == 32 ? gemm_f64_kernel<32> : gemm_f64_kernel<16>;
+        kernel<<<grid, NT, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, tile_group(), gate);
+    }
     SPIN_CUDA_TRY(cudaGetLastError());
     return SPIN_OK;
 }

@@ -1,4 +1,4 @@
-"""Products of few 16 x 16 tiles run on 8 x 16 ones, one output per thread.
+"""Products of few 16 x 16 tiles run on 8 x 16 or 8 x 8 ones, one output per thread.
 An output's operations do not depend on the tile, so every bit equals the same
 output's inside a product large enough for the wide tiles."""
 import pytest
@@ -10,7 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("m,n,k", [(1, 1, 1), (7, 15, 16), (8, 16, 17), (9, 17, 33), (24, 300, 40), (64, 64, 64),
-                                   (5, 2000, 31), (100, 128, 129), (128, 128, 128), (200, 200, 200)])
+                                   (5, 2000, 31), (100, 128, 129), (128, 128, 128), (200, 200, 200),
+                                   (250, 257, 64), (301, 299, 48), (512, 512, 33)])
 @pytest.mark.parametrize("alpha,beta", [(1.0, 0.0), (-1.0, 1.0), (-1.0, 0.0)])
 def test_small_tiles_equal_wide_tiles_bit_by_bit(m, n, k, alpha, beta):
     g = torch.Generator(device="cuda")
