@@ -6,24 +6,27 @@
 // the sum itself exact.  Whether that is as accurate as 53-bit floating point
 // depends on the entries: an entry is off by at most 2^-63 of its row's (or
 // column's) largest, so the residue form's error is at most
-//     k 2^-62 rowmax_i colmax_j,
-// the FP64 kernel's k 2^-53 G_ij with G_ij = sum_k |a_ik| |b_kj|.  The first is
-// the smaller one wherever G_ij >= 2^-9 rowmax_i colmax_j.  A lower bound of
-// G_ij for every output comes from the sizes of the entries alone: sorted by
-// size, the g-th eighth of a row (g = 1 .. 7) is at least 2^-(s_g + 1) of the
-// row's largest, s_g from its exponents, and the worst a column can do is to
-// pair its eighths in the opposite order (the rearrangement inequality), so
+//     2^-63 (S_i + T_j) rowmax_i colmax_j,   S_i = sum_k |a_ik| / rowmax_i,
+// T_j alike, the FP64 kernel's k 2^-53 G_ij with G_ij = sum_k |a_ik| |b_kj|.
+// The first is the smaller one wherever k G_ij >= 2^-10 (S_i + T_j) rowmax_i
+// colmax_j.  A lower bound of G_ij for every output comes from the sizes of the
+// entries alone: sorted by size, the g-th eighth of a row (g = 1 .. 7) is at
+// least 2^-(s_g + 1) of the row's largest, s_g from its exponents, and the worst
+// a column can do is to pair its eighths in the opposite order (the
+// rearrangement inequality), so
 //     G_ij >= (k / 8) sum_{g=1..6} 2^-(s_g + 1) 2^-(t_{7-g} + 1) rowmax_i colmax_j
 // and
-//     k sum_{g=1..6} 2^-(s_g + t_{7-g}) >= 2^-4
+//     k^2 sum_{g=1..6} 2^-(s_g + t_{7-g}) >= 2^-5 (S + T)
 // is enough for every output.  The exponents pass finds the largest s_g and
-// t_g of the operands, a one-thread kernel compares, and either the residue
-// product or the FP64 kernel runs (the other one's launches return at once):
-// operands with an infinity or NaN, mostly empty ones and widely spread ones
-// keep the FP64 kernel, without a host read.  A Gram matrix and its inverse
-// pass by 5 bits and more; a strictly diagonally dominant one (entries U(-1, 1)
-// beside a diagonal n, its inverse's diagonal 4 n times the entries beside it)
-// by 1.
+// t_g of the operands and bounds S and T, a one-thread kernel compares, and
+// either the residue product or the FP64 kernel runs (the other one's launches
+// return at once): operands with an infinity or NaN, mostly empty ones and
+// widely spread ones keep the FP64 kernel, without a host read.  A Gram matrix
+// and its inverse pass by 5 bits and more; a strictly diagonally dominant one
+// (entries U(-1, 1) beside a diagonal n, its inverse's diagonal 4 n times the
+// entries beside it) by 2 at n = 8192 and k = 4096, at k = 512 it does not
+// (S + T = 2 k, which any operands have, would pass one bit less: order 8192
+// took 60.2 ms that way, and 36.3 this way).
 #include "crt.h"
 #include "f64_residues.h"
 #include "split.h"
@@ -32,14 +35,15 @@ namespace spin {
 namespace {
 
 constexpr int kMinBits = 63;
-constexpr size_t kHeader = 256;  // spread[2 * kSpreadLevels], use[2] (residues, FP64 kernel)
-constexpr int kUse = 2 * kSpreadLevels;
+constexpr size_t kHeader = 256;  // spread[2 * kSpreadInts], use[2] (residues, FP64 kernel)
+constexpr int kUse = 2 * kSpreadInts;
 
 __global__ void choose_form_kernel(const int* spread, double k, int* use) {
     double sum = 0.0;
     for (int g = 1; g < kSpreadLevels; g++)
-        sum += ldexp(1.0, -min(spread[g - 1] + spread[kSpreadLevels + 6 - g], 1000));
-    const int residues = k * sum >= 0.0625;
+        sum += ldexp(1.0, -min(spread[g - 1] + spread[kSpreadInts + 6 - g], 1000));
+    const double mass = ldexp((double)spread[kSpreadLevels] + (double)spread[kSpreadInts + kSpreadLevels], -14);
+    const int residues = k * k * sum >= 0.03125 * mass;
     use[0] = residues;
     use[1] = !residues;
 }
@@ -67,7 +71,7 @@ int f64_residue_decide(const F64Product& p, void* arena, F64Plan* plan, cudaStre
     plan->ea = (int*)(base + kHeader);
     plan->eb = plan->ea + p.m;
     plan->rest = base + kHeader + exps_bytes(p.m, p.n);
-    SPIN_CUDA_TRY(cudaMemsetAsync(head, 0, 2 * kSpreadLevels * sizeof(int), s));
+    SPIN_CUDA_TRY(cudaMemsetAsync(head, 0, 2 * kSpreadInts * sizeof(int), s));
     SplitSource src;
     src.A = p.A;
     src.lda = p.lda;

@@ -63,12 +63,20 @@ __device__ __forceinline__ void count_entry(unsigned (*bins)[32], int lane, doub
     atomicAdd(&bins[d >> 1][lane], 1u << ((d & 1) * 16));
 }
 // One bin after the other, from 0: the least t of 0 .. 25 with at least
-// (8 - g) / 8 k entries in bins 0 .. t.
+// (8 - g) / 8 k entries in bins 0 .. t, and an upper bound of the sum of the
+// entries' sizes over the largest, in units of 2^-14 (an entry of bin d is
+// below 2^(1 - d) of the largest; every other one counts a unit).
 struct SpreadScan {
-    int seen = 0, t = kNoSpread;
+    int seen = 0, t = kNoSpread, mass = 0;
     __device__ __forceinline__ void next(int i, int count, int k, int g) {
         seen += count;
+        mass += count * max(16384 >> max(i - 1, 0), 1);
         if (t == kNoSpread && 8ll * seen >= (long long)(8 - g) * k) t = i;
+    }
+    // entry g of the result: a level, or behind them the sum
+    __device__ __forceinline__ int result(int k, int g, int top) const {
+        if (g > kSpreadLevels) return mass + (k - seen);
+        return top == 0x7FF ? kNoSpread : t;  // an infinity or NaN
     }
 };
 __device__ __forceinline__ bool not_zero(double v) {
@@ -157,9 +165,8 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
                     scan.next(2 * j, __reduce_add_sync(0xffffffffu, (int)(w & 0xffffu)), k, lane);
                     scan.next(2 * j + 1, __reduce_add_sync(0xffffffffu, (int)(w >> 16)), k, lane);
                 }
-                const int t = top == 0x7FF ? kNoSpread : scan.t;  // an infinity or NaN
                 const bool any = __any_sync(0xffffffffu, nonzero);
-                if (lane >= 1 && lane <= kSpreadLevels && any) atomicMax(&spread[lane - 1], t);
+                if (lane >= 1 && lane <= kSpreadInts && any) atomicMax(&spread[lane - 1], scan.result(k, lane, top));
             }
         }
     } else {
@@ -228,12 +235,12 @@ exponents_kernel(Side A, Side B, int m, int n, int k, int blocks_a, int* __restr
                 scount[lane][2 * warp + 1] = hi;
             }
             __syncthreads();
-            if (warp >= 1 && warp <= kSpreadLevels) {  // a level per warp, a column per lane
+            if (warp >= 1 && warp <= kSpreadInts) {  // a level per warp, a column per lane
                 SpreadScan scan;
                 for (int i = 0; i < kSpreadSteps; i++) scan.next(i, scount[lane][i], k, warp);
                 const bool wanted = col_ok && scount[lane][kSpreadSteps];
-                const int t = __reduce_max_sync(0xffffffffu, wanted ? (top == 0x7FF ? kNoSpread : scan.t) : 0);
-                if (lane == 0) atomicMax(&spread[kSpreadLevels + warp - 1], t);
+                const int t = __reduce_max_sync(0xffffffffu, wanted ? scan.result(k, warp, top) : 0);
+                if (lane == 0) atomicMax(&spread[kSpreadInts + warp - 1], t);
             }
         }
     }

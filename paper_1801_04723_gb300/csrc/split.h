@@ -25,12 +25,13 @@ struct SplitSource {
 // Exponents e with |a_ik| < 2^e for every row i of A (k entries) and every
 // column j of B: ea (m per problem, or null: not wanted), eb (n per problem,
 // or null), += sums of squares (optional, one entry per problem).  spread
-// (optional, device int[2 * kSpreadLevels], count = 0 only): entry g - 1 of A's
+// (optional, device int[2 * kSpreadInts], count = 0 only): entry g - 1 of A's
 // half is raised to the largest over the rows (of B's half: over the columns)
 // of the least t of 0 .. 25 such that 8 - g eighths of the row's exponents are
-// at least its largest - t; 1000 where none is or an entry is not finite; rows
-// of zeros do not count.
-constexpr int kSpreadLevels = 7;
+// at least its largest - t; 1000 where none is or an entry is not finite; the
+// last entry to the largest bound of a row's sum of sizes over its largest
+// size, in units of 2^-14.  Rows of zeros do not count.
+constexpr int kSpreadLevels = 7, kSpreadInts = kSpreadLevels + 1;
 int launch_exponents(const SplitSource& src, int m, int n, int k, int* ea, int* eb, double* sumsq_a, double* sumsq_b,
                      int* spread, cudaStream_t s);
 
