@@ -305,12 +305,12 @@ __device__ __forceinline__ double crt_value(unsigned (&w)[LIMBS], const CrtTable
     const unsigned long long m = (prod >> 11) + ((prod >> 10) & 1ull);  // 53 bits, or 2^53
     const int e = 11 + t.pe - lz - one + scale;                         // value = m 2^e
     const int be = e + 52 + 1023;
-    double v;
+    const unsigned long long sign = (unsigned long long)(neg != (flip != 0u)) << 63;
     if (be >= 1 && be <= 2045)
-        v = __longlong_as_double((long long)(((unsigned long long)(be - 1) << 52) + m));
-    else
-        v = ldexp((double)m, e);
-    return neg != (flip != 0u) ? -v : v;
+        return __longlong_as_double((long long)((((unsigned long long)(be - 1) << 52) + m) | sign));
+    double v;  // where it stands: not computed for everyone and selected afterwards
+    asm volatile("cvt.rn.f64.u64 %0, %1;" : "=d"(v) : "l"(m));
+    return __longlong_as_double(__double_as_longlong(ldexp(v, e)) | (long long)sign);
 }
 
 // 4 columns of a row per thread.  p: the whole product (views, epilogue);
@@ -320,10 +320,12 @@ __device__ __forceinline__ double crt_value(unsigned (&w)[LIMBS], const CrtTable
 // Bound by instructions (about 200 per output, 39 to 80 of them 32 x 32 + 64
 // bit multiply-adds): the number of moduli is a template argument, so the words
 // of a thread's four outputs (and of C) are all requested before the first is
-// used and the constants are immediate.  4096^2 outputs of 15 moduli with C:
-// 187 us, 344 with four words in flight in a run-time loop and the indices by a
-// division each (540 MB: 80 us).  Four blocks an SM spill: 64 registers.
-template <int LIMBS, int MODULI>
+// used and the constants are immediate; SUM (the sum of squares) is one as well,
+// as the compiler computes squares nobody asked for on the FP64 pipe.  4096^2
+// outputs of 15 moduli with C: 169 us, 187 without SUM apart, 344 with four words
+// in flight in a run-time loop and the indices by a division each (540 MB: 80
+// us).  Four blocks an SM spill: 64 registers.
+template <int LIMBS, int MODULI, bool SUM>
 __global__ void __launch_bounds__(256, 2)
 crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int cols, int row0, int col0,
                    const __grid_constant__ CrtTable t, const __grid_constant__ TcGemmParams p) {
@@ -337,7 +339,9 @@ crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int c
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     const int dr = (int)(stride / groups), dc = (int)(stride % groups);
     const int so = p.sum_order ? p.sum_order[z] : 0x7fffffff;
-    const bool add = p.beta != 0.0;
+    // alpha = +-1, beta = 0 or 1, told apart by their bits: an FP64 compare is
+    // made again for every output
+    const bool add = (unsigned)__double2hiint(p.beta) << 1 != 0u, minus = __double2hiint(p.alpha) < 0;
     double ss = 0.0, ss2 = 0.0;
     int cg = (int)(first % groups);
     for (int64_t rr = first / groups; rr < rows; rr += dr) {
@@ -384,21 +388,21 @@ crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int c
                 w[i] = (unsigned)carry;
                 carry >>= 32;
             }
-            val[u] = crt_value<LIMBS>(w, t, er + ec - 2 * t.bits, p.alpha < 0.0);
+            val[u] = crt_value<LIMBS>(w, t, er + ec - 2 * t.bits, minus);
             // an infinity or NaN in the row or column (no fixed point has it)
             if (er > 1024 || ec > 1024) val[u] = __longlong_as_double(0x7ff8000000000000ll);
         }
         const int gcol = col0 + c;
         if (add) {  // beta = 1
 #pragma unroll
-            for (int u = 0; u < 4; u++) val[u] = old[u] + val[u];
+            for (int u = 0; u < 4; u++) val[u] = add_now(old[u], val[u]);
         }
         if (p.add_identity && (unsigned)(grow - gcol) < 4u) {
 #pragma unroll
             for (int u = 0; u < 4; u++)
                 if (gcol + u == grow) val[u] = add_now(val[u], 1.0);
         }
-        if (p.sumsq && grow < so) {
+        if (SUM && grow < so) {
             if (c + 3 < cols && gcol + 3 < so) {
                 ss = fma(val[0], val[0], ss);
                 ss2 = fma(val[1], val[1], ss2);
@@ -418,7 +422,7 @@ crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int c
                 if (c + u < cols) drow[u] = val[u];
         }
     }
-    if (p.sumsq) {
+    if (SUM) {
         __shared__ double part[8];
         ss += ss2;
 #pragma unroll
@@ -435,15 +439,18 @@ crt_combine_kernel(const uint8_t* __restrict__ res, int64_t ldr, int rows, int c
 // ------------------------------------------------------------------ host --
 
 using CombineKernel = void (*)(const uint8_t*, int64_t, int, int, int, int, CrtTable, TcGemmParams);
-template <int LIMBS, int FIRST, int... M>
+template <int LIMBS, bool SUM, int FIRST, int... M>
 CombineKernel combine_of(int moduli, std::integer_sequence<int, M...>) {
-    static constexpr CombineKernel kernels[] = {crt_combine_kernel<LIMBS, FIRST + M>...};
+    static constexpr CombineKernel kernels[] = {crt_combine_kernel<LIMBS, FIRST + M, SUM>...};
     return moduli >= FIRST && moduli < FIRST + (int)sizeof...(M) ? kernels[moduli - FIRST] : nullptr;
 }
 // Up to 55 bits and k <= 98304 take 17 moduli at most, 56 bits 15 at least.
-CombineKernel combine_kernel(const CrtFormat& f) {
-    return f.bits <= 55 ? combine_of<3, kCrtMinModuli>(f.moduli, std::make_integer_sequence<int, 18 - kCrtMinModuli>())
-                        : combine_of<4, 15>(f.moduli, std::make_integer_sequence<int, kCrtMaxModuli - 14>());
+CombineKernel combine_kernel(const CrtFormat& f, bool sum) {
+    const auto few = std::make_integer_sequence<int, 18 - kCrtMinModuli>();
+    const auto many = std::make_integer_sequence<int, kCrtMaxModuli - 14>();
+    if (f.bits <= 55)
+        return sum ? combine_of<3, true, kCrtMinModuli>(f.moduli, few) : combine_of<3, false, kCrtMinModuli>(f.moduli, few);
+    return sum ? combine_of<4, true, 15>(f.moduli, many) : combine_of<4, false, 15>(f.moduli, many);
 }
 
 // floor(2^128 u / p) with p, u < 2^9, rounded, as four limbs.
@@ -629,7 +636,7 @@ int crt_run(const CrtProduct& p, const CrtFormat& f, const CrtPanels& c, unsigne
     });
     if (rc) return rc;
     const int sms = sm_count();
-    const CombineKernel combine = combine_kernel(f);
+    const CombineKernel combine = combine_kernel(f, q.sumsq != nullptr);
     if (combine == nullptr) return SPIN_ERR_INVALID_ARG;
     for (int row0 = 0; row0 < m; row0 += (int)c.rows) {
         const int rows = std::min((int)c.rows, m - row0);
