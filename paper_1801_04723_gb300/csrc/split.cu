@@ -364,7 +364,7 @@ struct ToResidues {
                 int d;
                 if (q + 1 < PIECES) {
                     d = (int)((unsigned)v << (32 - kPiece)) >> (32 - kPiece);  // low 14 bits, signed
-                    v = (v - d) >> kPiece;
+                    v = (v >> kPiece) + (d < 0 ? 1 : 0);  // (v - d) / 2^14; v - d may be 2^63 at 63 bits
                 } else {
                     d = (int)v;
                 }

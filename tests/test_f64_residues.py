@@ -97,3 +97,22 @@ def test_non_finite_entries(spin, bad):
     Y, info2 = fp64_kernel_inverse(spin, A, check=False)
     assert info["status"] == info2["status"] == 2
     assert (info["fail_leaf"], info["fail_col"]) == (info2["fail_leaf"], info2["fail_col"])
+
+
+def test_entries_just_below_a_power_of_two(spin):
+    """Positive entries within 8 units of their last place below the power of
+    two that bounds their row (column): the largest 63-bit integers."""
+    g = torch.Generator(device="cuda:0").manual_seed(11)
+    A = torch.rand((N, N), generator=g, dtype=torch.float64, device="cuda:0").mul_(2.0).sub_(1.0)
+    A.diagonal().add_(200.0)
+    for j in range(1, 10):
+        x = 1.0 - j * 2.0 ** -53
+        A[2200 + 64 * j, 7 * j] = x
+        A[2210 + 64 * j, 7 * j] = -x
+        A[9 * j, 2300 + 32 * j] = x
+        A[9 * j, 2310 + 32 * j] = -x
+    X, info, (top, _), _ = products_by_residues(spin, A)
+    assert info["status"] == 0 and top == 6
+    Y, _ = fp64_kernel_inverse(spin, A)
+    assert not torch.equal(X, Y)
+    assert bounds.elementwise_ok(X.cpu().numpy(), Y.cpu().numpy(), A.cpu().numpy())
