@@ -355,11 +355,13 @@ __device__ __forceinline__ void leaf_gj_col_body(const double* __restrict__ src,
             const int mh = __reduce_max_sync(FULL, m);
             double val = 1.0;
             int about = 0;  // of this lane's best row: its position, row, whether others tie with it
+            int seen = 0;   // (position 0 of row 0 is a word of zeros too)
 #pragma unroll
             for (int t = 0; t < T; t++)
                 if (h[t] == m) {
                     val = v[t];
-                    about = pos[t] | (lane + 32 * t) << 10 | (about != 0 ? 1 << 30 : 0);
+                    about = pos[t] | (lane + 32 * t) << 10 | seen;
+                    seen = 1 << 30;
                 }
             double inv;
             int quick = recip_int(val, &inv);

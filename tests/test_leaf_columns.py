@@ -61,3 +61,17 @@ def test_same_bits_as_the_batched_leaf(spin, L, kind):
     assert few[2].item() == status[0].item()
     if info[0].item() == 0:
         assert torch.equal(X, Y[0]) and torch.equal(X, Z[2])
+
+
+@pytest.mark.parametrize("apart", [0.0, 2.0 ** -52, -(2.0 ** -52)])
+@pytest.mark.parametrize("L,row", [(L, row) for L in (33, 64, 65, 128, 256) for row in (32, 64, 96, 224) if row < L])
+def test_first_pivot_tied_with_a_row_of_its_lane(spin, L, row, apart):
+    """Rows 0 and 32 t, which one lane holds, have the largest entries of column
+    0: equal ones (the lower row is the pivot) or one unit in the last place apart."""
+    A = np.random.default_rng(L + row).uniform(-0.5, 0.5, (L, L))
+    A[0, 0], A[row, 0] = 1.0 + 2.0 ** -50, -(1.0 + 2.0 ** -50 + apart)
+    A = torch.from_numpy(A).cuda()
+    X = spin.leaf_inverse(A)
+    Y, _ = spin.invert_batched([A] * 80, leaf=L, schedule="lockstep")  # no clusters of columns
+    torch.cuda.synchronize()
+    assert torch.equal(X, Y[0])
