@@ -548,8 +548,8 @@ int spin_gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha,
  * BF16; 8 * slices - 1 bits in all); digit products (<= 2^14) are summed
  * exactly in FP32 runs of 1024, the runs in int32, and each slice-pair group
  * is scaled into the FP64 result (slice pairs (t, u) with t + u < slices).
- * For 4 slices and more (and k <= 98304) the same fixed-point integers, at
- * least 8 * slices - 5 bits of them, are multiplied modulo several coprime
+ * For 4 slices and more (and k <= 98304) the same fixed-point integers (at
+ * least 8 * slices - 1 bits) are multiplied modulo several coprime
  * numbers instead and the whole sum is put together from its residues: fewer
  * tensor-core products, no pair left out, a smaller error; a row of A or a
  * column of B that holds an infinity or NaN then gives NaN.  The refinement residual

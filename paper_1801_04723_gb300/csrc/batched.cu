@@ -387,7 +387,8 @@ int64_t tc_min_batched() {
 }
 
 // Split-plane bytes per matrix for a bucket of order n: the largest level
-// product (bf16x3 planes, or digit planes for the top Schur complements),
+// product (bf16x3 planes, or room for the top Schur complements' residues: a
+// bucket of one matrix needs crt_min_bytes, larger ones pack better with more),
 // the residual's digit planes of X and the update's three planes of X and R.
 size_t mixed_scratch_per(int64_t n, int64_t leaf, int fp64_levels, int sr) {
     size_t need = 0;
@@ -395,8 +396,10 @@ size_t mixed_scratch_per(int64_t n, int64_t leaf, int fp64_levels, int sr) {
         const int64_t n1 = split_order(n);
         const size_t ld1 = (size_t)tc_ld(n1);
         need = std::max(need, 2 * 2 * (size_t)n1 * ld1 * 2);  // bf16x3: 2 planes of m and n rows
-        if (fp64_levels > 0)
+        if (fp64_levels > 0) {
             need = std::max(need, (size_t)kSchurSlices * 2 * (size_t)n1 * ld1 * 2 + 2 * (size_t)n1 * 4 + 512);
+            need = std::max(need, crt_min_bytes(n1, n1, n1, fp64_class_moduli(n1, kSchurSlices)));
+        }
     }
     const size_t ld = (size_t)tc_ld(n);
     need = std::max(need, (size_t)sr * (size_t)n * ld * 2 + (size_t)n * 4 + 512);  // residual: X digits
@@ -412,10 +415,10 @@ size_t mixed_cache_per(int64_t n, int sr) {
 // residual is one mostly empty 128 x 256 tile per modulus, and the digit
 // form's 21 pairs, packed into a few exact runs, are cheaper: 256 matrices of
 // order 96 / 128 take 1.58 / 2.65 ms with digits, 1.74 / 2.87 ms with
-// residues; 192 of order 160 3.62 against 2.99 ms, 32 of order 1024 14.3
-// against 13.1 ms.  The Schur complements (28 pairs, 15 moduli) are cheaper by
-// residues at every order that reaches the tensor cores (128 matrices of
-// order 192, Schur order 32 at the second level: 2.84 -> 2.64 ms).
+// residues of one modulus fewer; 192 of order 160 3.62 against 2.99 ms, 32 of
+// order 1024 14.3 against 13.1 ms.  The Schur complements (28 pairs, 16 moduli)
+// are cheaper by residues at every order that reaches the tensor cores (128
+// matrices of order 192, Schur order 32 at the second level: 2.84 -> 2.64 ms).
 bool residual_by_residues(int64_t n, int slices) { return n > 128 && fp64_class_moduli(n, slices) > 0; }
 
 struct BMix {

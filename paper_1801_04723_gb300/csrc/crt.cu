@@ -8,9 +8,9 @@
 // exactly, and the Chinese remainder theorem gives the whole sum, as long as
 // the product of the moduli exceeds twice its largest magnitude (Ozaki,
 // Uchino and Imamura, "Ozaki Scheme II", 2025, on INT8 units, whose rate on
-// GB300 is far below BF16's).  Nothing is left out of the sum, so fewer bits
-// give the same error (crt_bits_for_slices), and the number of tensor-core
-// products falls from 21 to 13 or 14 for s = 6, from 28 to 15 or 16 for s = 7.
+// GB300 is far below BF16's).  Nothing is left out of the sum, and the number
+// of tensor-core products falls from 21 to 13 or 14 for s = 6 (up to 15 above
+// k = 32768), from 28 to 15 or 16 for s = 7 (17).
 //
 // Three kernels:
 //   split    (split.cu) FP64 -> N BF16 planes of signed residues (|r| <= 128,
@@ -315,8 +315,9 @@ __device__ __forceinline__ double crt_value(unsigned (&w)[LIMBS], const CrtTable
 
 // 4 columns of a row per thread.  p: the whole product (views, epilogue);
 // (row0, col0): the panel pair's origin; rows x cols its size.  LIMBS 32-bit
-// limbs of the fraction: 3 leave an error of 2^-84 P, i.e. below 2^-60 of the
-// largest entries' product for the formats that use it (bits <= 55).
+// limbs of the fraction: 3 leave an error of 2^-84 P, i.e. below 2^-75 k of the
+// largest entries' product for the formats that use it (bits <= 55, P at most
+// 2^9 times the least for them).
 // Bound by instructions (about 200 per output, 39 to 80 of them 32 x 32 + 64
 // bit multiply-adds): the number of moduli is a template argument, so the words
 // of a thread's four outputs (and of C) are all requested before the first is
@@ -448,7 +449,7 @@ CombineKernel combine_of(int moduli, std::integer_sequence<int, M...>) {
 CombineKernel combine_kernel(const CrtFormat& f, bool sum) {
     const auto few = std::make_integer_sequence<int, 18 - kCrtMinModuli>();
     const auto many = std::make_integer_sequence<int, kCrtMaxModuli - 14>();
-    if (f.bits <= 55)
+    if (f.bits <= kCrtFewBits)
         return sum ? combine_of<3, true, kCrtMinModuli>(f.moduli, few) : combine_of<3, false, kCrtMinModuli>(f.moduli, few);
     return sum ? combine_of<4, true, 15>(f.moduli, many) : combine_of<4, false, 15>(f.moduli, many);
 }
@@ -684,7 +685,7 @@ CrtFormat crt_format(int64_t k, int min_bits) {
         const int bits = (int)std::floor((log2p - 1.0 - std::log2((double)k) - 1e-9) / 2.0);
         if (bits >= min_bits) {
             f.moduli = l + 1;
-            f.bits = std::min(bits, kCrtMaxBits);
+            f.bits = std::min(bits, min_bits <= kCrtFewBits ? kCrtFewBits : kCrtMaxBits);
             return f;
         }
     }

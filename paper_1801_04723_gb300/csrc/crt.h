@@ -8,9 +8,10 @@
 
 namespace spin {
 
-constexpr int kCrtMinModuli = 7;  // 27 bits at k = 1
+constexpr int kCrtMinModuli = 8;  // 31 bits at k = 1
 constexpr int kCrtMaxModuli = 20;
 constexpr int kCrtMaxBits = 63;  // signed in 64 bits
+constexpr int kCrtFewBits = 55;  // up to here 96-bit fractions and four pieces do (crt.cu, split.cu)
 
 // Pairwise coprime, in falling order; signed residues |r| <= 128.
 __host__ __device__ constexpr int crt_modulus(int l) {
@@ -21,20 +22,22 @@ __host__ __device__ constexpr int crt_modulus(int l) {
 
 // Moduli and fixed-point bits per operand for an inner dimension k: the
 // fewest moduli whose product exceeds twice the largest |sum| at bits >=
-// min_bits, then every bit that they allow (at most kCrtMaxBits).  0 moduli:
-// none fits.
+// min_bits, then every bit that they allow (at most kCrtFewBits for a min_bits
+// up to it, kCrtMaxBits above).  0 moduli: none fits.
 struct CrtFormat {
     int moduli;
     int bits;
 };
 CrtFormat crt_format(int64_t k, int min_bits);
 
-// Bits that stand in for s 8-bit digit slices (pairs t + u < s): an FP64
-// simulation of the residual product (Householder SPD matrices of condition
-// 1e3 and Gram matrices, n = 512, s = 4, 5, 6) gives the residue form at 8 s
-// - 5 bits 0.65 to 0.88 of the digit form's error, which is mostly that of
-// the pairs it leaves out.
-inline int crt_bits_for_slices(int s) { return 8 * s - 5; }
+// Bits that stand in for s 8-bit digit slices (pairs t + u < s): the digits'
+// own, so the operands are the same fixed-point integers and nothing is left
+// out of their product: for every operand the residue form's error is the
+// digit form's less that of the pairs it leaves out.  Fewer bits would be
+// worse for operands whose rows are full of entries near the largest (four
+// bits fewer, one modulus fewer: 4.8 times the digit form's error for normal
+// entries at k = 128, where the operands' rounding is all of it).
+inline int crt_bits_for_slices(int s) { return 8 * s - 1; }
 
 // One operand's or the whole product's device memory.
 //   exps       one int per row of A / column of B, for all of them

@@ -59,8 +59,9 @@ void tc_pairs_ozaki(TcGemmParams& p, int slices) {
     p.chunk_kb = 16;  // runs of 1024: every partial sum is an integer of magnitude <= 2^24, exact in FP32
 }
 
-// The digit-slice residual's error relative to ||A||_F ||X||_F with s 8-bit
-// slices at order n.  An exact CPU simulation of the product (Householder
+// The residual's error relative to ||A||_F ||X||_F with s 8-bit digit slices
+// at order n, which bounds the residue form's, too (the same integers, nothing
+// left out).  An exact CPU simulation of the product (Householder
 // SPD matrices of condition 1e3 and approximate inverses, n = 1024, every
 // pair product exact, compared with an 80-bit reference) gives
 // 0.62 sqrt(n) 2^-(8s-1) for s = 6 and 0.67 sqrt(n) 2^-(8s-1) for s = 7;
@@ -232,8 +233,7 @@ int gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha, const double* A, 
 }
 
 int fp64_class_moduli(int64_t k, int slices) {
-    const int n = crt_format(k, crt_bits_for_slices(slices)).moduli;
-    return n > 0 && n < slices * (slices + 1) / 2 ? n : 0;
+    return slices >= 4 ? crt_format(k, crt_bits_for_slices(slices)).moduli : 0;
 }
 
 size_t fp64_class_bytes(int64_t m, int64_t n, int64_t k, int slices) {

@@ -8,8 +8,9 @@
 
 namespace spin {
 
-constexpr int kSchurSlices = 7;  // digit slices of the FP64-class Schur complements (55 bits)
-constexpr int kLevelSlices = 4;  // digit slices of the level products in SPIN_MIXED_DIGITS (31 bits)
+// What the FP64-class products are as accurate as, in 8-bit digit slices.
+constexpr int kSchurSlices = 7;  // Schur complements (55 bits)
+constexpr int kLevelSlices = 4;  // level products in SPIN_MIXED_DIGITS (31 bits)
 constexpr int kMaxResidualSlices = 7;
 
 // Digit slices of the refinement residual R = I - A X.  The error of the
@@ -54,11 +55,11 @@ int gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha, const double* A, 
 
 // FP64-class product (the Schur complements, the refinement residual, the
 // level products of SPIN_MIXED_DIGITS): as accurate as s digit slices, by
-// residues (crt.cu) where those take fewer tensor-core products -- s >= 4: at
-// n = 2048, 9 instead of 10 for s = 4, 11 instead of 15, 13 instead of 21 and
-// 15 instead of 28 for s = 7 (n = 2048: 0.79 -> 0.40 ms at s = 7; the n = 16384
-// mixed inversion 380 -> 273 ms) -- else by digits (s <= 3, and k beyond 96
-// runs of 1024).
+// residues (crt.cu) for s >= 4, else by digits (s <= 3, and k beyond 96 runs of
+// 1024).  At n = 2048 the residues take as many tensor-core products for s = 4
+// (10), 12 instead of 15, 14 instead of 21 and 16 instead of 28 for s = 7, and
+// their drain is cheaper: us by digits and by residues, s = 4 to 7: 425, 528,
+// 656, 784 and 227, 256, 279, 307; n = 512: 107, 124, 140, 157 and 30, 30, 31, 35.
 int fp64_class_moduli(int64_t k, int slices);       // 0: digits
 size_t fp64_class_bytes(int64_t m, int64_t n, int64_t k, int slices);  // an arena that needs no panels
 double fp64_class_products(int64_t k, int slices);  // tensor-core products of m x n x k

@@ -490,7 +490,8 @@ int split_sides(Side A, Side B, const SplitTarget& t, int count, const int* acti
         default:
             if (t.planes < 1 || t.planes > kCrtMaxModuli || t.bits < 1 || t.bits > kCrtMaxBits)
                 return SPIN_ERR_INVALID_ARG;
-            if (t.bits <= 4 * kPiece - 1)
+            static_assert(kCrtFewBits <= 4 * kPiece - 1, "pieces");
+            if (t.bits <= kCrtFewBits)
                 return split_with(A, B, t, ToResidues<4>{t.bits, t.planes}, count, active, s);
             return split_with(A, B, t, ToResidues<5>{t.bits, t.planes}, count, active, s);
     }

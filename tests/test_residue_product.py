@@ -89,3 +89,54 @@ def test_panels_change_no_bit(spin, n):
     Y, info2 = spin.invert(A, precision="bf16x3", workspace=ws)
     assert info["refine_iters"] == info2["refine_iters"]
     assert torch.equal(X, Y)
+
+
+def exact_product(A, B):
+    """A B in extended precision, rows in blocks."""
+    L = np.longdouble
+    return np.stack([(A[i].astype(L)[:, None] * B.astype(L)).sum(axis=0) for i in range(A.shape[0])])
+
+
+@pytest.mark.parametrize("slices", [4, 5, 6, 7])
+@pytest.mark.parametrize("k", [64, 128, 256, 512, 2048, 8192])
+def test_bits_of_the_digit_slices(spin, k, slices):
+    """Dense operands: the error is that of rounding them to the 8 s - 1 bits of
+    s digit slices, nothing more: independent uniform errors of up to half a
+    unit u = 2^-(8 s - 1) of the row's (column's) power of two, so a standard
+    deviation of u / sqrt(12) sqrt(4^e_i |b_j|^2 + 4^f_j |a_i|^2) per output,
+    plus the rounding of the result.  The digit form has that error and the
+    pairs it leaves out."""
+    rng = np.random.default_rng(k + slices)
+    m, n = 96, 80
+    A, B = rng.standard_normal((m, k)), rng.standard_normal((k, n))
+    D = spin.gemm_ozaki(dev(A), dev(B), slices=slices)
+    torch.cuda.synchronize()
+    want = exact_product(A, B)
+    u = 2.0 ** -(8 * slices - 1)
+    ei, fj = np.frexp(np.abs(A).max(axis=1))[1], np.frexp(np.abs(B).max(axis=0))[1]
+    var = u * u / 12 * (4.0 ** ei[:, None] * (B * B).sum(axis=0) + 4.0 ** fj * (A * A).sum(axis=1)[:, None])
+    var += (2.0 ** -53 * np.abs(want.astype(float))) ** 2
+    z = (D.cpu().numpy() - want).astype(float) / np.sqrt(var)
+    # 7680 outputs sharing 176 rows and columns: the root mean square is within 3 % of its expectation
+    assert np.sqrt(np.mean(z * z)) <= 1.05
+    assert np.abs(z).max() <= 7.0
+
+
+@pytest.mark.parametrize("slices", [4, 5, 6])
+@pytest.mark.parametrize("family", ["spd", "sdd"])
+@pytest.mark.parametrize("n", [64, 80, 96, 130, 160, 300])
+def test_residual_within_its_error_model(spin, n, family, slices):
+    """The refinement certifies with 0.7 sqrt(n) 2^-(8 s - 1) as the residual's
+    error relative to |A|_F |X|_F."""
+    rng = np.random.default_rng(n + slices)
+    if family == "spd":
+        G = rng.standard_normal((n, n))
+        A = G @ G.T / n + 0.3 * np.eye(n)
+    else:
+        A = rng.uniform(-1, 1, (n, n)) + n * np.eye(n)
+    X = np.linalg.inv(A)
+    R = spin.gemm_ozaki(dev(A), dev(X), slices=slices, alpha=-1.0, add_identity=True)
+    torch.cuda.synchronize()
+    want = np.eye(n) - exact_product(A, X)
+    err = np.linalg.norm((R.cpu().numpy() - want).astype(float)) / np.linalg.norm(A) / np.linalg.norm(X)
+    assert err <= 0.7 * np.sqrt(n) * 2.0 ** -(8 * slices - 1)
