@@ -490,6 +490,8 @@ struct MixLayout {
     size_t scratch;       // least bytes of the split arena
     size_t side_scratch;  // split arena of the side stream (overlapped schedule), else 0
     size_t preferred;     // total, and an arena in which the refinement's products need no panels
+    bool digits;          // residuals by digits: the least arena has no room for the residues (orders below
+                          // 40); decided here, so that a larger workspace gives the same result
     int sr;  // digit slices that the certifying residuals stand for
     int s0;  // those of the first residual (<= sr)
 };
@@ -518,6 +520,7 @@ MixLayout mix_layout(int64_t n, int64_t leaf, const spin_opts& o) {
     // both operands of the residual
     sc = round256(sc) + round256((size_t)L.sr * (size_t)n * (size_t)tc_ld(n) * 2);
     L.scratch = sc;
+    L.digits = std::max(fp64_class_least(n, n, n, L.s0), fp64_class_least(n, n, n, L.sr)) > L.scratch;
     // the side stream's products (II and C21 of every level: at most n2 x n1 x n1)
     size_t side = 0;
     if (overlap) {
@@ -531,7 +534,7 @@ MixLayout mix_layout(int64_t n, int64_t leaf, const spin_opts& o) {
     L.off_side = L.off_exps + round256((size_t)n * sizeof(int));
     L.off_scratch = L.off_side + L.side_scratch;
     L.total = L.off_scratch + L.scratch;
-    const size_t full = round256(fp64_class_bytes(n, n, n, L.sr));
+    const size_t full = L.digits ? 0 : round256(fp64_class_bytes(n, n, n, L.sr));
     L.preferred = L.off_scratch + std::max(L.scratch, std::min(full, kFp64ClassArena));
     return L;
 }
@@ -606,6 +609,7 @@ int refine(Run& r, StreamState* st, const double* A, int64_t lda, double* X, int
             x.sumsq_d = &norms[2];
             x.a_exps = exps;
             x.a_known = it > 0;
+            x.digits = L.digits;
             ProfScope ps(r.prof, s, SPIN_KERNEL_RESIDUAL, -1, n, n, n, fp64_class_products(n, s_it) * f, 24.0 * n * n,
                          act);
             RET(gemm_fp64_class(n, n, n, -1.0, A, lda, X, ldx, 0.0, nullptr, 0, R, n, s_it, 1, x, scratch,

@@ -124,7 +124,7 @@ int plan_bf16x3(int64_t m, int64_t n, int64_t k, void* scratch, size_t bytes, Sp
 
 int plan_ozaki(int64_t m, int64_t n, int64_t k, int slices, void* scratch, size_t bytes, SplitPlan* sp) {
     if (slices < 1 || slices > 7) return SPIN_ERR_INVALID_ARG;
-    if (bytes < ozaki_scratch_bytes(m, n, k, slices)) return SPIN_ERR_INVALID_ARG;
+    if (bytes < ozaki_scratch_bytes(m, n, k, slices) - 512) return SPIN_ERR_INVALID_ARG;  // the alignments take 271
     sp->ld = tc_ld(k);
     sp->a = (uint16_t*)align_up((uintptr_t)scratch, 256);
     sp->b = sp->a + (int64_t)slices * m * sp->ld;
@@ -236,6 +236,11 @@ int fp64_class_moduli(int64_t k, int slices) {
     return slices >= 4 ? crt_format(k, crt_bits_for_slices(slices)).moduli : 0;
 }
 
+size_t fp64_class_least(int64_t m, int64_t n, int64_t k, int slices) {
+    const int mods = fp64_class_moduli(k, slices);
+    return mods ? crt_min_bytes(m, n, k, mods) : ozaki_scratch_bytes(m, n, k, slices);
+}
+
 size_t fp64_class_bytes(int64_t m, int64_t n, int64_t k, int slices) {
     const int mods = fp64_class_moduli(k, slices);
     return mods ? crt_full_bytes(m, n, k, mods) : ozaki_scratch_bytes(m, n, k, slices);
@@ -252,8 +257,7 @@ int gemm_fp64_class(int64_t m, int64_t n, int64_t k, double alpha, const double*
                     cudaStream_t s) {
     if (m <= 0 || n <= 0) return SPIN_OK;
     if (k <= 0) return SPIN_ERR_INVALID_ARG;
-    const int mods = fp64_class_moduli(k, slices);
-    if (mods && scratch_bytes >= crt_min_bytes(m, n, k, mods)) {
+    if (!x.digits && fp64_class_moduli(k, slices) > 0) {
         CrtProduct p = {};
         p.m = m;
         p.n = n;
@@ -288,8 +292,9 @@ int gemm_fp64_class(int64_t m, int64_t n, int64_t k, double alpha, const double*
     src.B = B;
     src.ldb = ldb;
     src.active = x.active;
-    if ((rc = launch_exponents(src, (int)m, (int)n, (int)k, sp.ea, sp.eb, x.a_known ? nullptr : x.sumsq_a, x.sumsq_b,
-                               nullptr, s)))
+    if (x.a_exps != nullptr) sp.ea = x.a_exps;
+    if ((rc = launch_exponents(src, (int)m, (int)n, (int)k, x.a_known ? nullptr : sp.ea, sp.eb,
+                               x.a_known ? nullptr : x.sumsq_a, x.sumsq_b, nullptr, s)))
         return rc;
     if ((rc = launch_split(src,
                            SplitTarget{SPLIT_DIGITS, slices, 0, (int)m, (int)n, (int)k, 0, (int)m, 0, (int)n, sp.ea,
@@ -359,8 +364,8 @@ extern "C" int spin_gemm_ozaki(int64_t m, int64_t n, int64_t k, double alpha, co
     int rc = ensure_test_err();
     if (rc) return rc;
     // everything in one panel where the device has the memory, else in the
-    // panels that fit the digit form's arena
-    const size_t need = ozaki_scratch_bytes(m, n, k, slices);
+    // panels that fit the digit form's arena (the least one, where that is more)
+    const size_t need = std::max(ozaki_scratch_bytes(m, n, k, slices), fp64_class_least(m, n, k, slices));
     rc = g_test_scratch.reserve(std::max(need, std::min(fp64_class_bytes(m, n, k, slices), kFp64ClassArena)));
     if (rc == SPIN_ERR_OOM) rc = g_test_scratch.reserve(need);
     if (rc) return rc;

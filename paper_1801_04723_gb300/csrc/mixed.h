@@ -61,10 +61,11 @@ int gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha, const double* A, 
 // their drain is cheaper: us by digits and by residues, s = 4 to 7: 425, 528,
 // 656, 784 and 227, 256, 279, 307; n = 512: 107, 124, 140, 157 and 30, 30, 31, 35.
 int fp64_class_moduli(int64_t k, int slices);       // 0: digits
+size_t fp64_class_least(int64_t m, int64_t n, int64_t k, int slices);  // the least arena
 size_t fp64_class_bytes(int64_t m, int64_t n, int64_t k, int slices);  // an arena that needs no panels
 double fp64_class_products(int64_t k, int slices);  // tensor-core products of m x n x k
 // The residue form runs in panels in any arena of at least the digit form's
-// size; library-owned arenas are made larger, up to this, to save the panels'
+// size (from order 40 on); library-owned arenas are made larger, up to this, to save the panels'
 // repeated splits and launches at small orders.
 constexpr size_t kFp64ClassArena = (size_t)2 << 30;
 struct Fp64ClassExtra {
@@ -73,6 +74,7 @@ struct Fp64ClassExtra {
     double* sumsq_b = nullptr;
     double* sumsq_d = nullptr;
     int* a_exps = nullptr;        // optional, device: m row exponents of A, kept between products
+    bool digits = false;          // by digits for every s: the arena may be too small for the residues
     bool a_known = false;         // a_exps and *sumsq_a are there from an earlier product with this A
 };
 int gemm_fp64_class(int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda, const double* B,

@@ -140,3 +140,20 @@ def test_residual_within_its_error_model(spin, n, family, slices):
     want = np.eye(n) - exact_product(A, X)
     err = np.linalg.norm((R.cpu().numpy() - want).astype(float)) / np.linalg.norm(A) / np.linalg.norm(X)
     assert err <= 0.7 * np.sqrt(n) * 2.0 ** -(8 * slices - 1)
+
+
+@pytest.mark.parametrize("n", [3, 16, 20, 32, 33, 34, 35, 36, 37, 38, 39, 40, 48, 64, 65, 96, 127])
+def test_small_orders_in_the_least_workspace(spin, n):
+    """The form of the residual depends on the order alone: the certified residual is that of the
+    library's own buffer, up to the order in which its n^2 squares are added (n^2 2^-53)."""
+    g = torch.Generator(device="cuda:0").manual_seed(n)
+    G = torch.randn((n, n), generator=g, dtype=torch.float64, device="cuda:0")
+    A = G @ G.T / n + 0.5 * torch.eye(n, dtype=torch.float64, device="cuda:0")
+    for tol, slices in ((1e-4, 0), (1e-10, 0), (1e-13, 7)):
+        kw = dict(precision="bf16x3", leaf=16, residual_slices=slices)
+        X, info = spin.invert(A, tol=tol, **kw)
+        ws = torch.empty(spin.workspace_bytes(n, **kw), dtype=torch.uint8, device="cuda:0")
+        Y, info2 = spin.invert(A, tol=tol, workspace=ws, **kw)
+        assert info["refine_iters"] == info2["refine_iters"]
+        assert abs(info["rel_residual"] - info2["rel_residual"]) <= 1e-10 * info["rel_residual"]
+        assert torch.equal(X, Y)
