@@ -211,7 +211,8 @@ int spin_invert_ex(const double* A, int64_t lda, double* X, int64_t ldx, int64_t
  * graph: each matrix's stopping decision is taken on the device, so the
  * result of a matrix does not depend on the others in the batch, and the
  * call returns once the graph is enqueued (with opts->blocking, once it has
- * run).  count <= 65535, n[i] <= 65536.
+ * run).  count <= 65535, n[i] <= 65536.  SPIN_ERR_CUDA, with nothing done, while
+ * the stream is being captured.
  */
 int spin_invert_batched(const double* const* A, const int64_t* lda, double* const* X, const int64_t* n,
                         int count, const spin_opts* opts, int* info_dev, spin_stream_t stream);

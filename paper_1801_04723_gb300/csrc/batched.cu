@@ -1339,6 +1339,12 @@ extern "C" int spin_invert_batched(const double* const* A, const int64_t* lda, d
     }
     if (count > 65535) return SPIN_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    // A capturing stream takes no graph launch.  Refused before anything is
+    // done: the addresses' copy would be captured, not made, and the plan
+    // would take them for uploaded.
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    SPIN_CUDA_TRY(cudaStreamIsCapturing(s, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone) SPIN_CUDA_TRY(cudaErrorStreamCaptureUnsupported);
     std::lock_guard<std::mutex> lk(g_bmu);
     BatchPlan& p = g_plans[s];
     std::vector<uint64_t> key = make_key(n, count, o);
