@@ -171,8 +171,12 @@ int spin_invert(const double* A, double* X, int64_t n, int64_t lda, int leaf, sp
  * A workspace larger than spin_workspace_bytes is put to use: the mixed forms
  * then need fewer panels, and FP64 inversions above order 4096 have room for
  * the tensor-core form of their large products (with exactly that size they
- * run on the FP64 pipe; without a caller's workspace the library keeps an
- * arena of at most 8 GB per stream for them).
+ * run on the FP64 pipe).
+ * Library-owned memory, kept per stream: the workspace, for the mixed forms up
+ * to 2 GB more than spin_workspace_bytes, and for FP64 inversions above order
+ * 4096 an arena of at most 8 GB.  Both extras are taken only where the device
+ * has them free, and the arenas are given back when another allocation of the
+ * library fails for want of memory.
  * Schedule: the recursion (Algorithm 2's driver) is a DAG of product and
  * leaf launches over views of X, A and the workspace, on the stream and, up
  * to order 8192 in FP64, a second library stream (II, then C21, beside the

@@ -121,6 +121,7 @@ struct StreamState {
     Profiler prof;
     void* ws = nullptr;
     size_t ws_bytes = 0;
+    size_t ws_refused_at = 0;           // free device memory when a larger workspace was last refused
     cudaStream_t side = nullptr;        // second stream of the overlapped schedule
     std::vector<cudaEvent_t> events;    // its fork / join events (one per use within a call)
     int32_t* info_dev = nullptr;   // CTL_BYTES: info record + refinement control
@@ -131,6 +132,9 @@ struct StreamState {
     int* err_dev = nullptr;        // device: tensor-core bounded-wait failures
     unsigned char* f64_arena = nullptr;  // large FP64 products by residues (two halves on two streams)
     size_t f64_arena_bytes = 0;
+    size_t f64_refused_at = 0;
+    bool f64_captured = false;     // a caller's capture holds the arena
+    std::mutex f64_mu;             // held while a call enqueues with it
     int last_mixed = 0;            // host: the latest call refined (mixed precision)
     int last_pretransformed = 0;   // host: the latest call went through the butterfly transform
     // The schedule as a CUDA graph: the previous call's arguments, and the
@@ -165,48 +169,92 @@ int get_state(cudaStream_t s, StreamState** out) {
     return SPIN_OK;
 }
 
-int ensure_ws(StreamState* st, size_t bytes) {
-    if (bytes <= st->ws_bytes) return SPIN_OK;
-    if (st->ws) {
+}  // namespace
+
+// Gives the idle arenas of large FP64 products on this device back to it.
+// False when there was none.  An arena that a caller's own graph may hold, or
+// that another thread is enqueuing with, stays.
+bool release_f64_arenas() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    bool any = false;
+    std::lock_guard<std::mutex> lk(g_mu);
+    for (auto& e : g_states) {
+        StreamState& st = e.second;
+        if (e.first.first != dev) continue;
+        std::unique_lock<std::mutex> mine(st.f64_mu, std::try_to_lock);
+        if (!mine.owns_lock() || st.f64_arena == nullptr || st.f64_captured) continue;
+        if (!any && cudaDeviceSynchronize() != cudaSuccess) return false;  // work enqueued with them
+        cudaFree(st.f64_arena);
+        st.f64_arena = nullptr;
+        st.f64_arena_bytes = 0;
+        any = true;
+    }
+    return any;
+}
+
+void* optional_malloc(size_t bytes, size_t* refused_at) {
+    size_t avail = 0, total = 0;
+    void* p = nullptr;
+    if (cudaMemGetInfo(&avail, &total) == cudaSuccess && avail >= bytes && avail > *refused_at) {
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        *refused_at = avail;
+    }
+    cudaGetLastError();
+    return nullptr;
+}
+
+namespace {
+
+// The stream's workspace: at least `need` bytes, `want` where the device has
+// them.  One that is large enough is never given up for a larger one that may
+// not be had: a change of address loses the captured schedule, and freeing
+// waits for the device.
+int ensure_ws(StreamState* st, size_t need, size_t want) {
+    if (st->ws_bytes >= want) return SPIN_OK;
+    const bool enough = st->ws != nullptr && st->ws_bytes >= need;
+    if (!enough && st->ws != nullptr) {
         cudaFree(st->ws);
         st->ws = nullptr;
         st->ws_bytes = 0;
     }
-    if (bytes == 0) return SPIN_OK;
-    if (cudaMalloc(&st->ws, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return SPIN_ERR_OOM;
+    void* p = want > need ? optional_malloc(want, &st->ws_refused_at) : nullptr;
+    if (p == nullptr) {
+        if (enough || need == 0) return SPIN_OK;
+        want = need;
+        if (device_malloc(&p, need) != cudaSuccess) {
+            cudaGetLastError();
+            return SPIN_ERR_OOM;
+        }
     }
-    st->ws_bytes = bytes;
+    if (st->ws != nullptr) cudaFree(st->ws);
+    st->ws = p;
+    st->ws_bytes = want;
     return SPIN_OK;
 }
 
 // The arena of large FP64 products for inversions of order n on this stream:
 // what the top level needs at once, up to a bound, less when the device has
 // less (panels), none when it has too little or no product is large enough
-// (the FP64 kernel runs).  Kept for later calls, as the workspace is.
+// (the FP64 kernel runs).  Kept for later calls, as the workspace is, until an
+// allocation that a call cannot do without fails.  With st->f64_mu held.
 size_t ensure_f64_arena(StreamState* st, int64_t n, int64_t leaf, bool two_streams) {
     const int64_t n1 = split_order(n), n2 = n - n1;
     if (n <= leaf || n2 <= kF64ResidueTop || f64_residue_moduli(n1) == 0) return 0;
     const size_t parts = two_streams ? 2 : 1;
     const size_t least = f64_residue_bytes(n1, n1, n1, true);
+    const size_t have = st->f64_arena_bytes / parts / 256 * 256;
     size_t want = std::max(least, std::min(f64_residue_bytes(n1, n1, n1, false), kF64ResidueArena / parts));
-    if (st->f64_arena_bytes >= parts * want) return st->f64_arena_bytes / parts / 256 * 256;
-    if (st->f64_arena) {
-        cudaFree(st->f64_arena);
-        st->f64_arena = nullptr;
-        st->f64_arena_bytes = 0;
-    }
-    for (; want >= least; want /= 2) {
+    for (; want > have && want >= least; want /= 2) {
         want = (want + 255) / 256 * 256;
-        if (cudaMalloc(&st->f64_arena, parts * want) == cudaSuccess) {
-            st->f64_arena_bytes = parts * want;
-            return want;
-        }
-        cudaGetLastError();
-        st->f64_arena = nullptr;
+        void* p = optional_malloc(parts * want, &st->f64_refused_at);
+        if (p == nullptr) continue;
+        if (st->f64_arena) cudaFree(st->f64_arena);
+        st->f64_arena = (unsigned char*)p;
+        st->f64_arena_bytes = parts * want;
+        return want;
     }
-    return 0;
+    return have >= least ? have : 0;
 }
 
 struct Run {
@@ -784,7 +832,7 @@ int enqueue(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, con
         ws_bytes = o.workspace_bytes;
     } else {
         const size_t want = preferred_bytes(n, leaf, o, need);
-        if (want == need || ensure_ws(st, want) != SPIN_OK) RET(ensure_ws(st, need));
+        RET(ensure_ws(st, need, want));
         ws = (unsigned char*)st->ws;
         ws_bytes = std::min(st->ws_bytes, want);
     }
@@ -792,12 +840,18 @@ int enqueue(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, con
     // caller's workspace holds beyond `need`
     void* f64_arena = nullptr;
     size_t f64_bytes = 0;  // per stream
+    std::unique_lock<std::mutex> f64_lock(st->f64_mu, std::defer_lock);
     if (!mixed) {
         const int64_t top = o.pretransform != 0 ? rbt_padded_order(n, kRbtDepth) : n;
         const bool two = overlap_schedule(top, o.precision, o.schedule);
         if (o.workspace == nullptr) {
+            f64_lock.lock();
             f64_bytes = ensure_f64_arena(st, top, leaf, two);
-            f64_arena = st->f64_arena;
+            f64_arena = f64_bytes > 0 ? st->f64_arena : nullptr;
+            cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+            if (f64_bytes > 0 && cudaStreamIsCapturing(s, &capturing) == cudaSuccess &&
+                capturing != cudaStreamCaptureStatusNone)
+                st->f64_captured = true;
         } else if (top > leaf && top - split_order(top) > kF64ResidueTop) {
             const size_t used = round256(need);
             if (o.workspace_bytes > used) f64_bytes = (o.workspace_bytes - used) / (two ? 2 : 1) / 256 * 256;
@@ -1017,7 +1071,7 @@ int spin_autotune_leaf(int64_t n, int precision, const int* candidates, int ncan
     double* A = nullptr;
     double* X = nullptr;
     const size_t bytes = (size_t)n * (size_t)n * sizeof(double);
-    if (cudaMalloc(&A, bytes) != cudaSuccess || cudaMalloc(&X, bytes) != cudaSuccess) {
+    if (device_malloc(&A, bytes) != cudaSuccess || device_malloc(&X, bytes) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(A);
         return SPIN_ERR_OOM;
@@ -1123,8 +1177,8 @@ int spin_invert_host(const double* A_host, int64_t lda, double* X_host, int64_t 
         if (st->hostX) cudaFree(st->hostX);
         st->hostA = st->hostX = nullptr;
         st->host_elems = 0;
-        if (cudaMalloc(&st->hostA, elems * sizeof(double)) != cudaSuccess ||
-            cudaMalloc(&st->hostX, elems * sizeof(double)) != cudaSuccess) {
+        if (device_malloc(&st->hostA, elems * sizeof(double)) != cudaSuccess ||
+            device_malloc(&st->hostX, elems * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             return SPIN_ERR_OOM;
         }
@@ -1170,7 +1224,7 @@ int spin_leaf_inverse(const double* A, int64_t lda, double* X, int64_t ldx, int6
     double* scratch = nullptr;
     const size_t need = leaf_scratch_elems(n) * sizeof(double);
     if (need) {
-        RET(ensure_ws(st, need));
+        RET(ensure_ws(st, need, need));
         scratch = (double*)st->ws;
     }
     int32_t* info = info_dev ? info_dev : st->info_dev;

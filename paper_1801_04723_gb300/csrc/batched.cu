@@ -830,12 +830,12 @@ int build_plan(BatchPlan& p, const int64_t* n, int count, const spin_opts& o, cu
     }
     if (p.persistent) set_tile_caps(p.buckets);
     std::vector<double*> hw(count);
-    if (cudaMalloc(&p.ws, ws_total * sizeof(double)) != cudaSuccess) {
+    if (device_malloc(&p.ws, ws_total * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return SPIN_ERR_OOM;
     }
     if (mixed) {
-        if (cudaMalloc(&p.arena, std::max<size_t>(p.arena_bytes, 256)) != cudaSuccess) {
+        if (device_malloc(&p.arena, std::max<size_t>(p.arena_bytes, 256)) != cudaSuccess) {
             cudaGetLastError();
             return SPIN_ERR_OOM;
         }
@@ -1164,7 +1164,7 @@ extern "C" int spin_test_persistent_timeout(double limit_ms, int* status0, int* 
                  o_ptr = take(4 * count * 8), o_rec = take(count * INFO_WORDS * 4), o_ctl = take(done_bytes + 256),
                  o_st = take(st.size() * sizeof(PStage)), o_start = take(start.size() * 8);
     unsigned char* d = nullptr;
-    if (cudaMalloc(&d, off) != cudaSuccess) {
+    if (device_malloc(&d, off) != cudaSuccess) {
         cudaGetLastError();
         return SPIN_ERR_OOM;
     }
@@ -1466,7 +1466,7 @@ struct PersistBatchRun {
             cudaFree(d);
             d = nullptr;
             bytes = 0;
-            if (cudaMalloc(&d, off) != cudaSuccess) {
+            if (device_malloc(&d, off) != cudaSuccess) {
                 cudaGetLastError();
                 return SPIN_ERR_OOM;
             }
@@ -1554,7 +1554,7 @@ extern "C" int spin_autotune_batched_persistent(const int64_t* orders, int count
     double* A = nullptr;
     double* X = nullptr;
     unsigned long long* clk = nullptr;
-    if (cudaMalloc(&A, elems * sizeof(double)) != cudaSuccess || cudaMalloc(&X, elems * sizeof(double)) != cudaSuccess ||
+    if (device_malloc(&A, elems * sizeof(double)) != cudaSuccess || device_malloc(&X, elems * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&clk, nb * sizeof(unsigned long long)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(A);
@@ -1710,7 +1710,7 @@ extern "C" int spin_autotune_batched_leaf(const int64_t* orders, int count, int 
         double* X = nullptr;
         void* host = nullptr;
         const size_t nn = (size_t)n * (size_t)n;
-        if (cudaMalloc(&A, nn * k * sizeof(double)) != cudaSuccess || cudaMalloc(&X, nn * k * sizeof(double)) != cudaSuccess ||
+        if (device_malloc(&A, nn * k * sizeof(double)) != cudaSuccess || device_malloc(&X, nn * k * sizeof(double)) != cudaSuccess ||
             cudaMallocHost(&host, bucket_host_bytes(k)) != cudaSuccess) {
             cudaGetLastError();
             cudaFree(A);
@@ -1736,7 +1736,7 @@ extern "C" int spin_autotune_batched_leaf(const int64_t* orders, int count, int 
             o.leaf = (int)L;
             const size_t wsb = bucket_bytes(n, k, o);
             void* ws = nullptr;
-            if (cudaMalloc(&ws, wsb) != cudaSuccess) {
+            if (device_malloc(&ws, wsb) != cudaSuccess) {
                 cudaGetLastError();
                 rc = SPIN_ERR_OOM;
                 break;

@@ -102,6 +102,23 @@ struct BatchView {
     __device__ __forceinline__ const double* ptr(int z, int64_t l) const { return base[z] + r0 * l + c0; }
 };
 
+// ---- device memory (host) ----
+// The arenas that the library keeps for large FP64 products and can do without
+// (api.cu): released where they are idle; true when there was one.
+bool release_f64_arenas();
+// cudaMalloc, once more after release_f64_arenas() when the device is out of memory.
+template <class T>
+cudaError_t device_malloc(T** p, size_t bytes) {
+    const cudaError_t e = cudaMalloc((void**)p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    return release_f64_arenas() ? cudaMalloc((void**)p, bytes) : e;
+}
+// An allocation that a call can do without: null when the device has too
+// little free, or no more than when it last refused (so that a shortage costs
+// a query per call, no failing allocation and no synchronisation).
+void* optional_malloc(size_t bytes, size_t* refused_at);
+
 // ---- kernel launchers (host) ----
 // FP64 product tile for count m x n products side by side.
 struct F64Tile {

@@ -82,16 +82,25 @@ int first_residual_slices_for(int64_t n, double tol, int sr) {
     return sr;
 }
 
-int MixScratch::reserve(size_t bytes) {
-    if (bytes <= cap) return SPIN_OK;
-    if (base) cudaFree(base);
-    base = nullptr;
-    cap = 0;
-    if (cudaMalloc(&base, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return SPIN_ERR_OOM;
+int MixScratch::reserve(size_t need, size_t want) {
+    if (want <= cap) return SPIN_OK;
+    if (need > cap) {  // one that is large enough stays until a larger one is there
+        if (base) cudaFree(base);
+        base = nullptr;
+        cap = 0;
     }
-    cap = bytes;
+    void* p = want > need ? optional_malloc(want, &refused_at) : nullptr;
+    if (p == nullptr) {
+        if (need <= cap) return SPIN_OK;
+        want = need;
+        if (device_malloc(&p, need) != cudaSuccess) {
+            cudaGetLastError();
+            return SPIN_ERR_OOM;
+        }
+    }
+    if (base) cudaFree(base);
+    base = p;
+    cap = want;
     return SPIN_OK;
 }
 
@@ -346,7 +355,8 @@ extern "C" int spin_gemm_bf16x3(int64_t m, int64_t n, int64_t k, double alpha, c
     std::lock_guard<std::mutex> lk(g_mix_mu);
     int rc = ensure_test_err();
     if (rc) return rc;
-    rc = g_test_scratch.reserve(bf16x3_scratch_bytes(m, n, k));
+    const size_t need = bf16x3_scratch_bytes(m, n, k);
+    rc = g_test_scratch.reserve(need, need);
     if (rc) return rc;
     return gemm_bf16x3(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, g_test_scratch.base, g_test_scratch.cap,
                        g_test_err, (cudaStream_t)stream);
@@ -366,8 +376,7 @@ extern "C" int spin_gemm_ozaki(int64_t m, int64_t n, int64_t k, double alpha, co
     // everything in one panel where the device has the memory, else in the
     // panels that fit the digit form's arena (the least one, where that is more)
     const size_t need = std::max(ozaki_scratch_bytes(m, n, k, slices), fp64_class_least(m, n, k, slices));
-    rc = g_test_scratch.reserve(std::max(need, std::min(fp64_class_bytes(m, n, k, slices), kFp64ClassArena)));
-    if (rc == SPIN_ERR_OOM) rc = g_test_scratch.reserve(need);
+    rc = g_test_scratch.reserve(need, std::max(need, std::min(fp64_class_bytes(m, n, k, slices), kFp64ClassArena)));
     if (rc) return rc;
     Fp64ClassExtra x;
     x.sumsq_d = sumsq_dev;

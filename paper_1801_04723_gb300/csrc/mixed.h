@@ -42,7 +42,8 @@ void tc_pairs_ozaki(TcGemmParams& p, int slices);  // digit pairs t + u < slices
 struct MixScratch {
     void* base = nullptr;
     size_t cap = 0;
-    int reserve(size_t bytes);
+    size_t refused_at = 0;
+    int reserve(size_t need, size_t want);  // at least need bytes, want where the device has them
 };
 
 size_t bf16x3_scratch_bytes(int64_t m, int64_t n, int64_t k);

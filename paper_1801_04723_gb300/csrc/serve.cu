@@ -338,6 +338,7 @@ void worker_loop(spin_server* sv, int slot) {
             release_group(g, m, s, true);
             cudaStreamSynchronize(s);
             cudaMemPoolTrimTo(sv->pool, 0);
+            release_f64_arenas();
             if (!alloc_group(sv, g, m, batched, s)) {
                 release_group(g, m, s, true);
                 cudaStreamSynchronize(s);
