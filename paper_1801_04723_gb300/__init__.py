@@ -24,6 +24,7 @@ from .binding import (  # noqa: F401
     gemm_bf16x3,
     gemm_ozaki,
     take_device_error,
+    batched_leaf_exchange_timeout,
     leaf_exchange_timeout,
     persistent_wait_timeout,
     autotune_batched_persistent,

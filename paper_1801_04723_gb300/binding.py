@@ -206,8 +206,9 @@ def lib():
         L.spin_schedule_stats.restype = ctypes.c_int
         L.spin_take_device_error.argtypes = [vp]
         L.spin_take_device_error.restype = ctypes.c_int
-        L.spin_test_leaf_timeout.argtypes = [i64, ctypes.c_int, ctypes.c_double]
-        L.spin_test_leaf_timeout.restype = ctypes.c_int
+        for hook in (L.spin_test_leaf_timeout, L.spin_test_batched_leaf_timeout):
+            hook.argtypes = [i64, ctypes.c_int, ctypes.c_double]
+            hook.restype = ctypes.c_int
         L.spin_test_persistent_timeout.argtypes = [ctypes.c_double, ctypes.POINTER(ctypes.c_int),
                                                    ctypes.POINTER(ctypes.c_int)]
         L.spin_test_persistent_timeout.restype = ctypes.c_int
@@ -485,6 +486,11 @@ def take_device_error(stream=None) -> int:
 def leaf_exchange_timeout(order: int, mute_rank: int, limit_ms: float) -> int:
     """Status of a leaf whose CTA mute_rank sends nothing (spin_test_leaf_timeout)."""
     return int(lib().spin_test_leaf_timeout(int(order), int(mute_rank), float(limit_ms)))
+
+
+def batched_leaf_exchange_timeout(order: int, mute_rank: int, limit_ms: float) -> int:
+    """The same of the batched paths' leaf with its rows over a cluster (spin_test_batched_leaf_timeout)."""
+    return int(lib().spin_test_batched_leaf_timeout(int(order), int(mute_rank), float(limit_ms)))
 
 
 def persistent_wait_timeout(limit_ms: float):

@@ -287,7 +287,7 @@ __device__ __forceinline__ void leaf_gj_pull_body(const double* __restrict__ src
 // row, so that every step delivers the same byte count.
 __device__ __forceinline__ void leaf_gj_push_body(const double* __restrict__ src, int64_t lds,
                                                   double* __restrict__ dst, int64_t ldd, int L, int R, int32_t* info,
-                                                  int leaf_index) {
+                                                  int leaf_index, const LeafWait& lw) {
     const int C = (int)tc::cluster_nctarank();
     const int rank = (int)tc::cluster_ctarank();
     const int tid = threadIdx.x;
@@ -321,8 +321,9 @@ __device__ __forceinline__ void leaf_gj_push_body(const double* __restrict__ src
     // fenced for the copy engine by the compute threads before a barrier the
     // messenger has passed) to the other CTAs' slot s: one bulk copy per
     // peer, by the messenger lanes.
+    const bool muted = rank == lw.mute_rank;
     auto send_row = [&](int s) {
-        if (mt >= 0 && mt < C && mt != rank) {
+        if (mt >= 0 && mt < C && mt != rank && !muted) {
             const uint32_t src_row = tc::smem_u32(slots + ((size_t)s * C + rank) * LS);
             tc::bulk_copy_to_peer(tc::mapa_u32(src_row, (uint32_t)mt), src_row, row_bytes,
                                   tc::mapa_u32(tc::smem_u32(&bars[s]), (uint32_t)mt));
@@ -339,7 +340,7 @@ __device__ __forceinline__ void leaf_gj_push_body(const double* __restrict__ src
                 mine.inv = inv;
                 mine.pos = c.pos;
                 mine.phys = c.phys;
-            } else {
+            } else if (!muted) {
                 const uint32_t a = tc::mapa_u32(tc::smem_u32(&infos[s * C + rank]), (uint32_t)mt);
                 const uint32_t b = tc::mapa_u32(tc::smem_u32(&bars[s]), (uint32_t)mt);
                 tc::st_async_v2_b64(a, c.key, (uint64_t)__double_as_longlong(c.val), b);
@@ -388,7 +389,7 @@ __device__ __forceinline__ void leaf_gj_push_body(const double* __restrict__ src
     double prev_inv = 0.0;
     for (int k = 0; k < L; k++) {
         const int s = k & 1;
-        const bool ok = slot_wait(&bars[s], (uint32_t)(k >> 1) & 1u, kLeafWaitLimitNs);
+        const bool ok = slot_wait(&bars[s], (uint32_t)(k >> 1) & 1u, lw.limit_ns);
         if (__syncthreads_or(!ok)) {  // also makes this CTA's own slot entries visible
             if (tid == 0) record_failure(info, SPIN_ERR_TIMEOUT, leaf_index, k);
             break;
@@ -508,9 +509,9 @@ leaf_gj_cta_kernel(BatchView srcv, BatchView dstv, int L, int32_t* info_base, in
 template <bool ROWS_IN_SMEM, bool PUSH>
 __device__ __forceinline__ void leaf_gj_body(const double* __restrict__ src, int64_t lds, double* __restrict__ dst,
                                              int64_t ldd, double* __restrict__ gwork, int L, int R, int32_t* info,
-                                             int leaf_index) {
+                                             int leaf_index, const LeafWait& lw) {
     if constexpr (PUSH)
-        leaf_gj_push_body(src, lds, dst, ldd, L, R, info, leaf_index);
+        leaf_gj_push_body(src, lds, dst, ldd, L, R, info, leaf_index, lw);
     else
         leaf_gj_pull_body<ROWS_IN_SMEM>(src, lds, dst, ldd, gwork, L, R, info, leaf_index);
 }
@@ -528,12 +529,12 @@ leaf_gj_kernel(const double* __restrict__ src, int64_t lds, double* __restrict__
 template <bool ROWS_IN_SMEM, bool PUSH>
 __global__ void __launch_bounds__(PUSH ? NT + kMessengers : NT, 2)
 leaf_gj_batched_kernel(BatchView src, BatchView dst, double* __restrict__ gwork, int64_t gwork_stride, int L, int R,
-                       int32_t* info, int leaf_index) {
+                       int32_t* info, int leaf_index, LeafWait lw) {
     const int z = blockIdx.y;
     const int64_t lds = src.ld_of(z), ldd = dst.ld_of(z);
     leaf_gj_body<ROWS_IN_SMEM, PUSH>(src.ptr(z, lds), lds, const_cast<double*>(dst.ptr(z, ldd)), ldd,
                                      ROWS_IN_SMEM ? nullptr : gwork + (int64_t)z * gwork_stride, L, R,
-                                     info + (int64_t)z * INFO_WORDS, leaf_index);
+                                     info + (int64_t)z * INFO_WORDS, leaf_index, lw);
 }
 
 struct LeafConfig {
@@ -739,7 +740,7 @@ bool launch_leaf_col_batched(const BatchView& src, const BatchView& dst, int64_t
 template <bool S, bool P>
 int launch_leaf_batched_impl(const BatchView& src, const BatchView& dst, const LeafConfig& c, int64_t L,
                              double* scratch, int64_t stride, int32_t* info, int leaf_index, int count,
-                             cudaStream_t s) {
+                             cudaStream_t s, LeafWait lw = LeafWait()) {
     static PerDeviceOnce attrs;
     auto kern = leaf_gj_batched_kernel<S, P>;
     {
@@ -758,7 +759,7 @@ int launch_leaf_batched_impl(const BatchView& src, const BatchView& dst, const L
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    SPIN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, src, dst, scratch, stride, (int)L, c.R, info, leaf_index));
+    SPIN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, src, dst, scratch, stride, (int)L, c.R, info, leaf_index, lw));
     return SPIN_OK;
 }
 
@@ -812,44 +813,65 @@ int launch_leaf_gj(const double* A, int64_t lda, double* X, int64_t ldx, int64_t
 
 }  // namespace spin
 
-// Test hook: the identity of order L (2 <= L <= 256, the pushed-row form, on
-// its widest cluster) with the CTA of rank mute_rank sending nothing and the
-// exchange waits limited to limit_ms.  The other CTAs' waits for step 0 run
-// out, the muted CTA's wait for step 1 does, every CTA leaves, and the info
-// record gets SPIN_ERR_TIMEOUT.  Remote writes happen only in the first
-// exchange, while every CTA still waits.  Returns the recorded status.
+namespace {
+
+// The status that an inversion of the identity of order L leaves behind, with
+// the CTA of rank mute_rank sending nothing and the exchange waits limited to
+// limit_ms: launch(A, X, info, views, wait) on the legacy stream.  The other
+// CTAs' waits for the first exchange run out, the muted CTA's next one does,
+// every CTA leaves, and the info record gets SPIN_ERR_TIMEOUT.  (The identity:
+// the muted CTA has a valid pivot in the first step.)  Remote writes happen
+// only in the first exchange, while every CTA still waits.
+template <class Launch>
+int leaf_timeout(int64_t L, int mute_rank, double limit_ms, Launch launch) {
+    double* block = nullptr;  // A, X, their addresses, the info record
+    const size_t elems = (size_t)L * (size_t)L, bytes = (2 * elems + 2) * sizeof(double) + spin::INFO_WORDS * sizeof(int32_t);
+    if (cudaMalloc(&block, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return SPIN_ERR_OOM;
+    }
+    double *A = block, *X = block + elems;
+    double** views = (double**)(block + 2 * elems);
+    int32_t* info = (int32_t*)(block + 2 * elems + 2);
+    std::vector<double> I(elems, 0.0);
+    for (int64_t i = 0; i < L; i++) I[(size_t)i * (size_t)L + (size_t)i] = 1.0;
+    double* const host_views[2] = {A, X};
+    spin::LeafWait lw;
+    lw.limit_ns = (uint64_t)(limit_ms * 1e6);
+    lw.mute_rank = mute_rank;
+    int32_t h[spin::INFO_WORDS] = {0, 0, 0, 0};
+    int rc = SPIN_ERR_CUDA;
+    if (cudaMemcpy(A, I.data(), elems * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
+        cudaMemcpy(views, host_views, sizeof host_views, cudaMemcpyHostToDevice) == cudaSuccess &&
+        cudaMemset(info, 0, sizeof h) == cudaSuccess)
+        rc = launch(A, X, info, views, lw);
+    if (rc == SPIN_OK && cudaMemcpy(h, info, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) rc = SPIN_ERR_CUDA;
+    cudaFree(block);
+    return rc == SPIN_OK ? h[spin::INFO_STATUS] : rc;
+}
+
+}  // namespace
+
+// Test hooks: the single inversions' leaf, columns over its cluster, and the
+// batched paths' leaf of 128 < L <= 256, rows over the narrowest cluster that
+// holds them.
 extern "C" int spin_test_leaf_timeout(int64_t L, int mute_rank, double limit_ms) {
     using namespace spin;
     if (L < 2 || L > kColMaxL || !(limit_ms > 0.0) || limit_ms > 4000.0) return SPIN_ERR_INVALID_ARG;
     ColConfig c;
     if (!col_config(L, &c) || mute_rank < 0 || mute_rank * c.w >= L) return SPIN_ERR_INVALID_ARG;
-    double* A = nullptr;
-    double* X = nullptr;
-    int32_t* info = nullptr;
-    const size_t bytes = (size_t)L * (size_t)L * sizeof(double);
-    if (cudaMalloc(&A, bytes) != cudaSuccess || cudaMalloc(&X, bytes) != cudaSuccess ||
-        cudaMalloc(&info, INFO_WORDS * sizeof(int32_t)) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(A);
-        cudaFree(X);
-        return SPIN_ERR_OOM;
-    }
-    {  // the identity: the muted CTA gets past step 0 (a valid pivot) and waits at step 1
-        std::vector<double> I((size_t)L * (size_t)L, 0.0);
-        for (int64_t i = 0; i < L; i++) I[(size_t)i * (size_t)L + (size_t)i] = 1.0;
-        cudaMemcpy(A, I.data(), bytes, cudaMemcpyHostToDevice);
-    }
-    cudaMemset(info, 0, INFO_WORDS * sizeof(int32_t));
-    LeafWait lw;
-    lw.limit_ns = (uint64_t)(limit_ms * 1e6);
-    lw.mute_rank = mute_rank;
-    int rc = launch_leaf_col(A, L, X, L, c, L, info, 0, 0, lw);
-    int32_t h[INFO_WORDS] = {0, 0, 0, 0};
-    if (rc == SPIN_OK) {
-        if (cudaMemcpy(h, info, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) rc = SPIN_ERR_CUDA;
-    }
-    cudaFree(A);
-    cudaFree(X);
-    cudaFree(info);
-    return rc == SPIN_OK ? h[INFO_STATUS] : rc;
+    return leaf_timeout(L, mute_rank, limit_ms, [&](double* A, double* X, int32_t* info, double**, LeafWait lw) {
+        return launch_leaf_col(A, L, X, L, c, L, info, 0, 0, lw);
+    });
+}
+
+extern "C" int spin_test_batched_leaf_timeout(int64_t L, int mute_rank, double limit_ms) {
+    using namespace spin;
+    if (L < 2 || L > kPushMaxL || !(limit_ms > 0.0) || limit_ms > 4000.0) return SPIN_ERR_INVALID_ARG;
+    const LeafConfig c = leaf_config(L, false, true);
+    if (!c.push || c.C < 2 || mute_rank < 0 || mute_rank >= c.C) return SPIN_ERR_INVALID_ARG;
+    return leaf_timeout(L, mute_rank, limit_ms, [&](double*, double*, int32_t* info, double** views, LeafWait lw) {
+        const BatchView src{(const double* const*)views, nullptr, L, 0, 0}, dst{(const double* const*)(views + 1), nullptr, L, 0, 0};
+        return launch_leaf_batched_impl<true, true>(src, dst, c, L, nullptr, 0, info, 0, 1, 0, lw);
+    });
 }
