@@ -757,6 +757,7 @@ int crt_product(const CrtProduct& p, void* arena, size_t bytes, cudaStream_t s, 
         if (p.sumsq_b) q.sumsq_b = p.sumsq_b + z;
         if (p.sumsq_d) q.sumsq_d = p.sumsq_d + z;
         if (p.a_exps) q.a_exps = p.a_exps + (int64_t)z * p.m;
+        if (p.b_exps) q.b_exps = p.b_exps + (int64_t)z * p.n;
         if (p.a_exps_out) q.a_exps_out = p.a_exps_out + (int64_t)z * p.m;
         if (!choose_panels(q.m, q.n, q.k, f.moduli, q.count, bytes, &c)) return SPIN_ERR_INVALID_ARG;
         const int rc = crt_run(q, f, c, base, s, launches);

@@ -74,7 +74,7 @@ struct CrtProduct {
     double* sumsq_b;
     double* sumsq_d;
     const int* a_exps;    // optional, device: row exponents of A from an earlier product with the same A
-    const int* b_exps;    // optional, device (with a_exps): column exponents of B
+    const int* b_exps;    // optional, device (with a_exps): column exponents of B, n per problem
     int* a_exps_out;      // optional, device: m ints per problem, where they are kept (else in the arena)
     int* err;
 };
