@@ -445,13 +445,14 @@ CombineKernel combine_of(int moduli, std::integer_sequence<int, M...>) {
     static constexpr CombineKernel kernels[] = {crt_combine_kernel<LIMBS, FIRST + M, SUM>...};
     return moduli >= FIRST && moduli < FIRST + (int)sizeof...(M) ? kernels[moduli - FIRST] : nullptr;
 }
-// Up to 55 bits and k <= 98304 take 17 moduli at most, 56 bits 15 at least.
+// For k <= 98304: 31 to 55 bits take 8 to 17 moduli, 63 bits 17 to 19 (large
+// FP64 products, which have no sum of squares).
 CombineKernel combine_kernel(const CrtFormat& f, bool sum) {
     const auto few = std::make_integer_sequence<int, 18 - kCrtMinModuli>();
-    const auto many = std::make_integer_sequence<int, kCrtMaxModuli - 14>();
+    const auto many = std::make_integer_sequence<int, kCrtMaxModuli - 16>();
     if (f.bits <= kCrtFewBits)
         return sum ? combine_of<3, true, kCrtMinModuli>(f.moduli, few) : combine_of<3, false, kCrtMinModuli>(f.moduli, few);
-    return sum ? combine_of<4, true, 15>(f.moduli, many) : combine_of<4, false, 15>(f.moduli, many);
+    return sum ? nullptr : combine_of<4, false, 17>(f.moduli, many);
 }
 
 // floor(2^128 u / p) with p, u < 2^9, rounded, as four limbs.

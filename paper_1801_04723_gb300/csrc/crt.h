@@ -9,14 +9,14 @@
 namespace spin {
 
 constexpr int kCrtMinModuli = 8;  // 31 bits at k = 1
-constexpr int kCrtMaxModuli = 20;
+constexpr int kCrtMaxModuli = 19;  // 63 bits at k = 98304
 constexpr int kCrtMaxBits = 63;  // signed in 64 bits
 constexpr int kCrtFewBits = 55;  // up to here 96-bit fractions and four pieces do (crt.cu, split.cu)
 
 // Pairwise coprime, in falling order; signed residues |r| <= 128.
 __host__ __device__ constexpr int crt_modulus(int l) {
     constexpr int p[kCrtMaxModuli] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227,
-                                      223, 217, 211, 199, 197, 193, 191, 181, 179, 173};
+                                      223, 217, 211, 199, 197, 193, 191, 181, 179};
     return p[l];
 }
 

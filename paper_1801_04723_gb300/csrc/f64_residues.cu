@@ -54,7 +54,7 @@ size_t exps_bytes(int64_t m, int64_t n) { return ((size_t)(m + n) * sizeof(int) 
 
 int f64_residue_moduli(int64_t k) {
     const CrtFormat f = crt_format(k, kMinBits);
-    return f.moduli;  // 0 where 20 moduli do not give the 63 bits of the rule above
+    return f.moduli;  // 0 where the moduli do not give the 63 bits of the rule above
 }
 
 size_t f64_residue_bytes(int64_t m, int64_t n, int64_t k, bool least) {

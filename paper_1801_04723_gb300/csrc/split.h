@@ -38,7 +38,7 @@ int launch_exponents(const SplitSource& src, int m, int n, int k, int* ea, int* 
 // What a plane holds.
 enum SplitKind {
     SPLIT_BF16,      // planes 2 or 3: hi, (mid,) lo of the value in FP32
-    SPLIT_DIGITS,    // planes 1..8: balanced base-256 digits relative to the row's exponent
+    SPLIT_DIGITS,    // planes 1..7: balanced base-256 digits relative to the row's exponent
     SPLIT_RESIDUES,  // planes: residues of the value in `bits` fixed-point bits (crt.h)
 };
 // Rows row0 .. row0 + rows - 1 of A and columns col0 .. col0 + cols - 1 of B
