@@ -61,8 +61,8 @@ WORKLOADS = {
                        "(alpha uniform in [0.1, 1]); half the requests ask for residual <= 1e-13, half for "
                        "<= 1e-10; admission by device-memory footprint under a 150 GB budget, 8 slots"),
     "mixed_digits": dict(n=32768, leaf=128, precision="digits", family="householder", seed=SEED_BASE + 2,
-                         desc="as mixed_bf16x3 but the level products are 4-slice BF16 digit products with exact "
-                              "FP32 runs (~2^-30), so the first residual usually certifies the result"),
+                         desc="as mixed_bf16x3 but the level products are fixed-point with the bits of 4 digit "
+                              "slices (~2^-30), exact on the BF16 tensor cores, so the first residual usually certifies the result"),
     "mixed_bf16x3": dict(n=32768, leaf=128, precision="bf16x3", family="householder", seed=SEED_BASE + 2,
                          desc="mixed precision, one SPD matrix A = Q diag(d) Q^T (64 Householder reflectors, "
                               "d log-uniform in [1, 1e3]), n = 32768: BF16x3 tensor-core level products, FP64 "
@@ -119,8 +119,8 @@ def parse():
                     "(one batched leaf launch, one CTA each) and print the per-pivot-step time and cycles")
     ap.add_argument("--leaf-sweep", default="", help="comma-separated orders: time every candidate leaf "
                     "(the U-shaped block-size sweep) with spin_autotune_leaf and print one JSON line")
-    ap.add_argument("--gemm-probe", type=int, default=0, help="time one digit-slice (6 slices) and one bf16x3 "
-                    "tensor-core product of this order and print one JSON line")
+    ap.add_argument("--gemm-probe", type=int, default=0, help="time one digit-slice, one FP64-class and one "
+                    "bf16x3 tensor-core product of this order and print one JSON line")
     ap.add_argument("--serve-seconds", type=float, default=60.0, help="serving: arrival window (s)")
     ap.add_argument("--serve-rate", type=float, default=200.0, help="serving: Poisson arrival rate (req/s)")
     ap.add_argument("--serve-slots", type=int, default=8)
@@ -613,7 +613,7 @@ def top_roofline(by_kind: dict, ms_step: float, steps: int, peaks: dict, peak_fp
         peak, src = tensor_peak(peaks)
         return {"kernel": top, "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": None, "peak_source": src,
-                "flops_counted": "BF16 tensor-core products actually issued (slice pairs x 2mnk)",
+                "flops_counted": "BF16 tensor-core products actually issued (slice pairs or moduli x 2mnk)",
                 "launches": d["launches"], "share_of_step": d["ms"] / (ms_step * steps)}
     return {"kernel": top, "bound": "alu", "achieved": achieved, "peak": peak_fp64, "unit": "TFLOP/s",
             "frac": achieved / peak_fp64, "traffic": None,
@@ -1149,8 +1149,9 @@ def run_serve(args, w: dict, sub: bool = False):
 
 
 def run_gemm_probe(args):
-    """One digit-slice (6 slices, 21 pairs: the refinement residual's form)
-    and one bf16x3 tensor-core product of order n, each timed 3 times after a
+    """One digit-slice product (3 slices, 6 pairs), one FP64-class product by
+    residues (6 slices' bits: the refinement residual's form; 13 to 15 BF16
+    products) and one bf16x3 tensor-core product of order n, each timed 3 times after a
     warm-up (CUDA events, splits included), with the SM clock sampled over
     the timed calls: the kernel variant switches (SPIN_TC_WIDE, SPIN_TC_PAIR)
     are compared this way, clock and all."""
@@ -1166,7 +1167,8 @@ def run_gemm_probe(args):
     D = torch.empty_like(A)
     out = {"probe": "tensor-core products", "n": n,
            "variant": {k: os.environ.get(k, "") for k in ("SPIN_TC_WIDE", "SPIN_TC_PAIR", "SPIN_TC_PERSIST")}}
-    for name, fn, pairs in (("ozaki6", lambda: spin.gemm_ozaki(A, B, slices=6, out=D), 21),
+    for name, fn, pairs in (("digits3", lambda: spin.gemm_ozaki(A, B, slices=3, out=D), 6),
+                            ("residues6", lambda: spin.gemm_ozaki(A, B, slices=6, out=D), None),
                             ("bf16x3", lambda: spin.gemm_bf16x3(A, B, out=D), 3)):
         fn()  # warm
         torch.cuda.synchronize()
@@ -1180,8 +1182,9 @@ def run_gemm_probe(args):
                 torch.cuda.synchronize()
                 times.append(e0.elapsed_time(e1))
         ms = statistics.median(times)
-        out[name] = {"ms_with_splits": ms, "bf16_tflops_incl_splits": pairs * 2.0 * n ** 3 / (ms * 1e-3) / 1e12,
-                     "clocks": clk.summary()}
+        out[name] = {"ms_with_splits": ms, "clocks": clk.summary()}
+        if pairs:
+            out[name]["bf16_tflops_incl_splits"] = pairs * 2.0 * n ** 3 / (ms * 1e-3) / 1e12
     out["device_error"] = spin.take_device_error()
     print(json.dumps(out), flush=True)
     return 0

@@ -17,7 +17,7 @@
 // per split and per product; the digit or BF16 planes of every matrix of the
 // bucket sit in one arena, one problem after the other), FP64-class Schur
 // complements at the top fp64_levels levels, then Newton-Schulz refinement
-// of every matrix with FP64-class residuals (cached digit planes of A).  The
+// of every matrix with FP64-class residuals.  The
 // refinement's stopping decisions are taken per matrix on the device
 // (refine.cu): every round is part of the captured graph and a matrix that
 // has converged is switched off, so a mixed batch is one graph replay too.

@@ -323,7 +323,7 @@ __device__ __forceinline__ double crt_value(unsigned (&w)[LIMBS], const CrtTable
 // of a thread's four outputs (and of C) are all requested before the first is
 // used and the constants are immediate; SUM (the sum of squares) is one as well,
 // as the compiler computes squares nobody asked for on the FP64 pipe.  4096^2
-// outputs of 15 moduli with C: 169 us, 187 without SUM apart, 344 with four words
+// outputs of 15 moduli with C: 169 us (16: 173), 187 without SUM apart, 344 with four words
 // in flight in a run-time loop and the indices by a division each (540 MB: 80
 // us).  Four blocks an SM spill: 64 registers.
 template <int LIMBS, int MODULI, bool SUM>
