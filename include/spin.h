@@ -171,7 +171,8 @@ int spin_invert(const double* A, double* X, int64_t n, int64_t lda, int leaf, sp
  * A workspace larger than spin_workspace_bytes is put to use: the mixed forms
  * then need fewer panels, and FP64 inversions above order 4096 have room for
  * the tensor-core form of their large products (with exactly that size they
- * run on the FP64 pipe).
+ * run on the FP64 pipe; 24 n^2 bytes more, 48 n^2 on two streams, need no
+ * panels, a fiftieth of that is the least that is put to use).
  * Library-owned memory, kept per stream: the workspace, for the mixed forms up
  * to 2 GB more than spin_workspace_bytes, and for FP64 inversions above order
  * 4096 an arena of at most 8 GB.  Both extras are taken only where the device

@@ -75,3 +75,19 @@ def test_first_pivot_tied_with_a_row_of_its_lane(spin, L, row, apart):
     Y, _ = spin.invert_batched([A] * 80, leaf=L, schedule="lockstep")  # no clusters of columns
     torch.cuda.synchronize()
     assert torch.equal(X, Y[0])
+
+
+@pytest.mark.parametrize("count", [12, 20, 38, 76])
+@pytest.mark.parametrize("kind", ["uniform", "ties", "zero_column"])
+@pytest.mark.parametrize("L", [16, 17, 32, 33, 50, 64, 65, 100, 127, 128, 200])
+def test_narrow_clusters_of_a_batch(spin, L, kind, count):
+    """More leaves at once take narrower clusters with wider panels (16 columns a
+    CTA at most), up to the count that takes one CTA a leaf."""
+    As = [torch.from_numpy(np.ascontiguousarray(matrix(kind, L, np.random.default_rng(z + L)))).cuda() for z in range(4)]
+    As = (As * 20)[:80]
+    Y, want = spin.invert_batched(As, leaf=L, schedule="lockstep")
+    X, status = spin.invert_batched(As[:count], leaf=L, schedule="lockstep")
+    torch.cuda.synchronize()
+    assert status.tolist() == want.tolist()[:count]
+    if status[0].item() == 0:
+        assert all(torch.equal(x, y) for x, y in zip(X, Y))
