@@ -849,9 +849,8 @@ int enqueue(const double* A, int64_t lda, double* X, int64_t ldx, int64_t n, con
             f64_bytes = ensure_f64_arena(st, top, leaf, two);
             f64_arena = f64_bytes > 0 ? st->f64_arena : nullptr;
             cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-            if (f64_bytes > 0 && cudaStreamIsCapturing(s, &capturing) == cudaSuccess &&
-                capturing != cudaStreamCaptureStatusNone)
-                st->f64_captured = true;
+            if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) cudaGetLastError();
+            if (f64_bytes > 0 && capturing != cudaStreamCaptureStatusNone) st->f64_captured = true;
         } else if (top > leaf && top - split_order(top) > kF64ResidueTop) {
             const size_t used = round256(need);
             if (o.workspace_bytes > used) f64_bytes = (o.workspace_bytes - used) / (two ? 2 : 1) / 256 * 256;
